@@ -94,7 +94,7 @@ int rsa_run_static(uint32_t L, uint32_t k, const uint64_t *seeds, uint32_t n, ui
 /* ---- batching of uneven shapes (no counterpart in the paper: a way of
  * running many of its samples at once) ---------------------------------- */
 
-/* Small lattices, one CTA per sample: all greedy rounds and the whole
+/* Small lattices, one CTA per sample: all rounds and the whole
  * first-wrap search of a sample run in one CTA's shared memory, and the n
  * samples -- of any mix of shapes -- run in one persistent launch (each CTA
  * takes the next sample from a work counter).  Sample i has lattice L[i],
@@ -126,10 +126,9 @@ void rsa_mix_release(void);
 unsigned long long rsa_mix_launches(void);
 
 /* How a shape runs: RSA_MODE_SMALL (one CTA per sample, `threads` per CTA)
- * or RSA_MODE_GLOBAL (the tiled / long-k / general kernels over the whole
- * batch, `rounds_per_check` greedy rounds per captured graph chunk and host
- * check, `window_threads` threads per CTA of the long-k window pass, 0 for
- * the handle's default as rsa_set_window_threads(h, 0) gives it).
+ * or RSA_MODE_GLOBAL (a handle's run of the whole batch, `rounds_per_check`
+ * as rsa_set_rounds_per_check; `window_threads` is kept for tuning files and
+ * changes nothing).
  * ms_per_sample is the time measured when the choice was made (0 for an
  * unmeasured default). */
 #define RSA_MODE_GLOBAL 0
@@ -147,21 +146,19 @@ typedef struct {
  * the global path at 2 / 4 / 8 rounds per check) is timed once on seeds
  * 1 .. n (at most 8 GB of workspace) and the fastest is kept and appended
  * to the file; otherwise a default is returned (small mode at 512 threads
- * where it fits, else the global path at 4 rounds per check and 256-thread
- * windows).  The long-k window pass is also timed at 128 threads per CTA
- * (twice the cells per thread) where the shape allows it. */
+ * where it fits, else the global path at 4 rounds per check). */
 int rsa_tune(uint32_t L, uint32_t k, uint32_t n, int measure, rsa_tune_t *out);
 
-/* Greedy rounds per captured graph chunk and host check of later runs on
- * this handle (1 .. 64, default 4).  Results do not depend on it. */
+/* Rounds per captured graph chunk and host check of later runs on this
+ * handle (1 .. 64, default 4): used by samples that are still undecided after
+ * the run's first graph, which enters every slice of the priority range.
+ * Results do not depend on it. */
 int rsa_set_rounds_per_check(rsa_t *h, uint32_t rounds);
 
-/* CTA size of the long-k window pass of later runs on this handle: 256 or
- * 128 threads per CTA, each thread then holding twice as many cells of the
- * span; 0 restores the default (128 on the argmin-offset long-k path with
- * 4096-cell spans and k >= 512, 256 otherwise).  128 needs the argmin-offset long-k path
- * with spans of 2048 or 4096 cells (RSA_EINVAL otherwise).  Results do not
- * depend on it. */
+/* A former tuning setting (CTA size of a window pass that no longer exists):
+ * 0, 256 or 128, the last only for 32 < k <= 4096 dividing spans of 2048 or
+ * 4096 cells (RSA_EINVAL otherwise).  It is checked as before and changes
+ * nothing. */
 int rsa_set_window_threads(rsa_t *h, uint32_t threads);
 
 /* Copy the last run's results to caller-owned host arrays of length n
@@ -218,7 +215,7 @@ int rsa_accepted(rsa_t *h, uint32_t sample, uint32_t *idx, uint32_t cap, uint32_
  * loops for later runs on this handle, so that a test can make each capped
  * loop run out on purpose and check that the run reports it and the GPU
  * stays usable.  0 restores a cap's default.
- *   round_cap  greedy rounds per sample (default n_j bound + 2): a sample
+ *   round_cap  rounds per sample (default n_j bound + 2): a sample
  *              still undecided after that many rounds stops with
  *              RSA_ETIMEOUT from rsa_results;
  *   uf_steps   steps of one union-find walk and retries of one link (default
@@ -242,14 +239,10 @@ int rsa_test_caps(rsa_t *h, uint32_t round_cap, uint32_t uf_steps, uint32_t prob
 int rsa_profile(rsa_t *h, int enable);
 int rsa_kernel_stats(rsa_t *h, double *ms, unsigned long long *launches, uint32_t n_kinds);
 const char *rsa_kernel_name(uint32_t kind);
-/* Work done by the round kernels since the previous call (then reset; n <= 4
- * values are written).  Tile path (power-of-two k <= 32): out[0] cells of live
- * tiles processed by the cell-minimum pass, out[1] live candidates it gave a
- * priority, out[2] / out[3] cells and accepted candidates of the acceptance
- * pass.  Long-k path: out[0] / out[1] cells processed by the horizontal /
- * vertical window-minimum passes, out[2] by the acceptance passes, out[3] by
- * the code pass (segments and tiles without live candidates are skipped and
- * not counted).  Zero on the general path. */
+/* Work done by the deposition since the previous call (then reset; n <= 4
+ * values are written): out[0] candidates given a priority by the first pass,
+ * out[1] list entries and undecided candidates tested for free cells, out[2]
+ * active candidates resolved, out[3] k-mers accepted. */
 int rsa_work_stats(rsa_t *h, unsigned long long *out, uint32_t n);
 
 /* Bytes of device workspace a run of n_samples needs for (L, k). */

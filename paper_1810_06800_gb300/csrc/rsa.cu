@@ -9,6 +9,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstddef>
 #include <mutex>
 #include <cstdio>
@@ -19,9 +20,7 @@
 
 #include "../../include/rsa.h"
 #include "rsa_kernels.cuh"
-#include "rsa_tile.cuh"
-#include "rsa_line.cuh"
-#include "rsa_lwin.cuh"
+#include "rsa_rounds.cuh"
 #include "rsa_config.cuh"
 
 using namespace rsak;
@@ -50,36 +49,25 @@ int fail(int code, const std::string& msg) {
   } while (0)
 
 constexpr size_t ALIGN = 256;
-constexpr u32 ROUND_CHECK = 4;   // greedy rounds between host checks (default)
+constexpr u32 ROUND_CHECK = 4;   // rounds between host checks once every slice is entered (default)
 constexpr u32 PROBE_CHECK = 4;   // bisection probes between host checks
 constexpr u32 PROBE_CAP = 40;    // rank bisection (<= 31 halvings) plus the initial probe
-constexpr size_t SMEM_BUDGET = 160 * 1024;
 
 size_t align_up(size_t v) { return (v + ALIGN - 1) / ALIGN * ALIGN; }
 
 struct Layout {
-  size_t occ, occw, occT, cB, code16, code16T, cH, cV, masks, dead, owner, cmin, base, node_key, node_idx, node_pos, uf, edges, edges_b,
-      ebkt, nkey_b, nbkt, st, seeds, counters, work, keys,
-      scratch, total;
+  size_t fine, block, anch, heads, list, flat, act;   // rounds
+  size_t uf, edges, edges_b, ebkt, nkey_b, nbkt;      // contact graph and search
+  size_t owner, base, node_key, node_idx, node_pos, rs, st, seeds, counters, work, keys, total;
+  size_t bits_bytes;  // fine + block, zeroed together
+  size_t anch_bytes, heads_bytes;
 };
 
 struct Geometry {
-  bool tile;                    // power-of-two k <= 32 and L % 32 == 0
-  bool line;                    // 32 <= k <= LINE_KMAX, L % 32 == 0, not tile
-  LineCfg lc;
-  // long-k lines made of whole k-blocks and whole CTA spans (rsa_lwin.cuh),
-  // used for seeded priorities; caller priorities keep the lc kernels
-  bool lw;
-  LwinCfg lw_cfg;
-  u32 lw_C;                     // cells per thread of k_lwin
-  size_t line_smem, line_acc_smem, line_codes_smem;
-  TileCfg tc;                   // (items filled per run)
-  RowCfg row;
-  ColCfg col;
-  u32 row_threads, col_threads;
-  size_t row_smem, col_smem;
-  dim3 row_grid_x, col_grid_x;  // .x only
-  size_t scratch_words;         // per sample
+  bool sites;       // k = 1: one pass, no slices
+  RoundCfg rc;
+  size_t list_cap;  // listed candidates per sample
+  bool win128;      // shape of the 128-thread window setting (rsa_set_window_threads)
 };
 
 u32 cap_nodes_of(u32 L, u32 k) { return (u32)(((u64)L * L) / k); }
@@ -89,103 +77,67 @@ u32 cap_edges_of(u32 L, u32 k) {
   return (u32)c;
 }
 
-bool tile_shape(u32 L, u32 k) { return k <= 32 && (k & (k - 1)) == 0 && L % 32 == 0; }
+u32 log2_floor(u64 v) {
+  u32 r = 0;
+  while (v >>= 1) ++r;
+  return r;
+}
+
+// Shapes that accept rsa_set_window_threads(h, 128): 32 < k <= 4096 dividing
+// spans of 2048 or 4096 cells.
+bool window_shape(u32 L, u32 k) {
+  if (L % 32 || k < 32 || k > 4096 || (k <= 32 && (k & (k - 1)) == 0)) return false;
+  const u32 P = std::min<u32>(L, 4096), C = P / 256;
+  return P % 256 == 0 && C >= 1 && C <= 16 && (C & (C - 1)) == 0 && L % P == 0 && P % k == 0 &&
+         k % C == 0 && L / P <= 8 && (P == 4096 || P == 2048);
+}
 
 Geometry plan(u32 L, u32 k) {
   Geometry G{};
-  G.tile = tile_shape(L, k);
-  G.tc.T = L / 32;
-  G.tc.T2 = G.tc.T * G.tc.T;
-  G.line = !G.tile && L % 32 == 0 && k >= 32 && k <= LINE_KMAX;
-  if (G.line) {
-    // longest segment (multiple of 32, <= 4096) whose buffers stay near 100 KB,
-    // so at least two blocks fit on an SM
-    u32 S = std::min<u32>(L, 4096);
-    while (S > 256 && line_smem_bytes(S + k - 1, S, k) > 100 * 1024) S -= 256;
-    // very long windows: if that cap leaves segments shorter than k, take
-    // S = k (rounded down to 32, at most L) with the one-array layout, which
-    // halves the bytes per value: fewer halo values per output cell
-    G.lc.compact = 0;
-    if (S < k) {
-      S = std::min<u32>(L, k & ~31u);
-      G.lc.compact = 1;
-    }
-    G.lc.S = S;
-    G.lc.nseg = (L + S - 1) / S;
-    G.lc.nmax = S + k - 1;
-    G.lc.T = L / 32;
-    G.line_smem = line_smem_bytes(G.lc.nmax, S, k, G.lc.compact != 0);
-    G.line_acc_smem = line_smem_bytes(G.lc.nmax, S, k);
-    G.line_codes_smem = line_codes_smem_bytes(G.lc.nmax);
-    const u32 P = std::min<u32>(L, 4096), C = P / LW_THREADS;
-    G.lw = P % LW_THREADS == 0 && C >= 1 && C <= 16 && (C & (C - 1)) == 0 && L % P == 0 &&
-           P % k == 0 && k % C == 0 && L / P <= 8;
-    if (G.lw) {
-      G.lw_cfg.P = P;
-      G.lw_cfg.nc = L / P;
-      G.lw_cfg.T = L / 32;
-      G.lw_C = C;
-    }
+  G.sites = k == 1;
+  G.win128 = window_shape(L, k);
+  RoundCfg& c = G.rc;
+  const u64 N = 2ull * L * L, D = (u64)k * k + 2 * k;
+  const u32 lk = log2_floor(k);
+  c.W = (L + k + 31) / 32 + 1;
+  c.WA = (L + 2 * k + 31) / 32 + 1;
+  // lines per block line: 2^bs + k / 2^bs updates per k-mer, least at sqrt(k)
+  c.bs = k < 16 ? 0 : std::max(3u, lk / 2);
+  c.nbl = c.bs ? (L + (1u << c.bs) - 1) >> c.bs : 0;
+  // bins about 4 sqrt(k) cells wide
+  c.b = 2 + lk / 2;
+  c.nb = ((L - 1) >> c.b) + 1;
+  // Priorities below 2^(64 - a) are listed by the first pass: the fewer, the
+  // more candidates are still live afterwards (1.5% at 2^-a = 4 / k).
+  c.a = std::max(1u, (lk + 2) / 2);
+  // the first slice holds about two to four candidates per conflict
+  // neighbourhood
+  const u32 ld = log2_floor(D);
+  c.lzmax = std::max(c.a, std::min(ld > 0 ? ld - 1 : 0u, RD_LEVELS - 1));
+  c.nlev = c.lzmax - c.a + 1;
+  size_t off = 0;
+  for (u32 t = 0; t < c.nlev; ++t) {
+    // slice 0: every priority with lzmax leading zeros or more; slice t: exactly lzmax - t
+    const u32 lz = c.lzmax - t;
+    const double mean = std::ldexp((double)N, -(int)(t == 0 ? lz : lz + 1));
+    // eight standard deviations of the number of hashes that fall in it
+    const u64 cap = std::min<u64>(N, (u64)(mean + 8.0 * std::sqrt(mean) + 64.0));
+    c.lvl_off[t] = (u32)off;
+    c.lvl_cap[t] = (u32)cap;
+    off += cap;
   }
-  // ---- row pass: one warp per (row, segment) ----
-  RowCfg& r = G.row;
-  r.S = L <= 4096 ? L : 4096;
-  r.nseg = (L + r.S - 1) / r.S;
-  r.nmax = r.S + k - 1;
-  r.warp_words = 2 * r.nmax;
-  size_t warp_bytes = (size_t)r.warp_words * 8;
-  if (warp_bytes <= 200 * 1024) {
-    r.global_scratch = 0;
-    r.warps = (u32)std::max<size_t>(1, std::min<size_t>(8, (96 * 1024) / warp_bytes));
-    G.row_smem = warp_bytes * r.warps;
-    G.row_grid_x = dim3((unsigned)(((u64)L * r.nseg + r.warps - 1) / r.warps));
-  } else {
-    r.global_scratch = 1;
-    r.warps = 8;
-    G.row_smem = 0;
-    G.row_grid_x = dim3(16);
-  }
-  G.row_threads = 32 * r.warps;
-  // ---- column pass: W columns x S rows per block ----
-  ColCfg& c = G.col;
-  const u32 T = 256;
-  u32 W = k <= 64 ? 32 : k <= 256 ? 16 : k <= 1024 ? 8 : k <= 2048 ? 4 : 2;
-  c.W = W;
-  auto bytes_for = [&](u32 S) {
-    size_t nmax = (size_t)S + k - 1, nocc = (size_t)S + 2 * k - 2;
-    size_t a_words = std::max(nmax * W, (nocc * W + 1) / 2);
-    size_t Gc = T / W;
-    size_t words = a_words + nmax * W + Gc * W + (Gc * W + 7) / 8;
-    return words * 8;
-  };
-  u32 S = std::min<u32>(L, 1024);
-  while (S > 32 && bytes_for(S) > SMEM_BUDGET) S /= 2;
-  c.S = S;
-  c.nseg = (L + S - 1) / S;
-  c.nstrip = (L + W - 1) / W;
-  c.nmax = S + k - 1;
-  c.nocc = S + 2 * k - 2;
-  size_t bb = bytes_for(S);
-  c.block_words = (u32)(bb / 8);
-  G.col_threads = T;
-  if (bb <= 200 * 1024) {
-    c.global_scratch = 0;
-    G.col_smem = bb;
-    G.col_grid_x = dim3(c.nstrip * c.nseg);
-  } else {
-    c.global_scratch = 1;
-    G.col_smem = 0;
-    G.col_grid_x = dim3(16);
-  }
-  size_t row_scr = r.global_scratch ? (size_t)G.row_grid_x.x * r.warps * r.warp_words : 0;
-  size_t col_scr = c.global_scratch ? (size_t)G.col_grid_x.x * c.block_words : 0;
-  G.scratch_words = std::max(row_scr, col_scr);
+  G.list_cap = off;
+  // neither limit is met by random priorities; past one, a round (a refill)
+  // takes a narrower slice and the run only takes longer
+  c.cap_flat = (u32)std::min<u64>(N, N / 4 + 32);
+  c.cap_act = (u32)std::min<u64>(N, cap_nodes_of(L, k) / 2 + 32);
   return G;
 }
 
 Layout layout_of(u32 L, u32 k, u32 n, bool with_keys, const Geometry& G) {
   Layout l{};
   const u64 LL = (u64)L * L;
+  const RoundCfg& c = G.rc;
   const size_t cn = cap_nodes_of(L, k), ce = cap_edges_of(L, k);
   size_t off = 0;
   auto take = [&](size_t bytes) {
@@ -193,55 +145,42 @@ Layout layout_of(u32 L, u32 k, u32 n, bool with_keys, const Geometry& G) {
     off = align_up(off + bytes);
     return at;
   };
-  const bool bits = G.tile || G.line;
-  const bool lw = G.lw && !with_keys;        // argmin-offset round (rsa_lwin.cuh)
-  const bool lold = G.line && !lw;           // 8-byte minima round (rsa_line.cuh)
-  l.occ = take(bits ? 0 : n * LL);
-  l.occw = take(bits ? n * LL / 8 : 0);
-  l.occT = take(G.line ? n * LL / 8 : 0);
-  l.cB = take(lold ? n * LL * 8 : 0);
-  l.code16 = take(lold ? n * LL * 2 : 0);
-  l.code16T = take(lold ? n * LL * 2 : 0);
-  l.cH = take(lw ? n * LL * 2 : 0);
-  l.cV = take(lw ? n * LL * 2 : 0);
-  // acceptance masks: win / first / last, rows then the transposed layout
-  l.masks = take(lw ? 6 * (n * LL / 8) : 0);
-  // dead flags: per 32 x 32 tile (tile path); per line segment (or span) of
-  // each orientation, then per 32 x 32 code tile (long-k path; 32 x 32
-  // combine squares on the argmin-offset path)
-  const u32 nseg = lw ? G.lw_cfg.nc : G.lc.nseg;
-  const size_t ncode = G.tc.T2;
-  l.dead = take(G.tile ? (size_t)n * G.tc.T2
-                       : G.line ? (size_t)n * (2ull * L * nseg + ncode) : 0);
-  l.owner = take(n * LL * 4);
-  // tile path: one argmin code byte per cell; none on the argmin-offset path
-  l.cmin = take(n * LL * (G.tile ? 1 : lw ? 0 : 8));
-  l.base = take((size_t)n * 8);
-  l.node_key = take(n * cn * 8);
-  l.node_idx = take(n * cn * 4);
-  l.node_pos = take(n * cn * 4);
+  // the buffers of the rounds and those of the contact graph and the search
+  // are never in use together: both start at 0
+  if (!G.sites) {
+    l.bits_bytes = (size_t)n * 2 * (L + c.nbl) * c.W * 4;
+    l.fine = take(l.bits_bytes);
+    l.block = l.fine + (size_t)n * 2 * L * c.W * 4;
+    l.heads_bytes = (size_t)n * 4 * c.nb * c.nb * 4;
+    l.heads = take(l.heads_bytes);
+    l.list = take((size_t)n * G.list_cap * 4);
+    l.flat = take((size_t)n * c.cap_flat * 4);
+    l.act = take((size_t)n * 2 * c.cap_act * sizeof(Act));
+  }
+  const size_t rounds_end = off;
+  off = 0;
   l.uf = take(n * cn * 16);
   l.edges = take(n * ce * sizeof(Edge));
   l.edges_b = take(n * ce * sizeof(Edge));
   l.ebkt = take((size_t)n * (NBKT + 1) * 4);
   l.nkey_b = take(n * cn * 8);
   l.nbkt = take((size_t)n * (NBKT + 1) * 4);
+  off = std::max(off, rounds_end);
+  l.anch_bytes = G.sites ? 0 : (size_t)n * 4 * L * c.WA * 4;
+  l.anch = take(l.anch_bytes);
+  l.owner = take(G.sites ? 0 : n * LL * 4);  // written at anchors only
+  l.base = take((size_t)n * 8);
+  l.node_key = take(n * cn * 8);
+  l.node_idx = take(n * cn * 4);
+  l.node_pos = take(n * cn * 4);
+  l.rs = take(G.sites ? 0 : (size_t)n * sizeof(RoundState));
   l.st = take((size_t)n * sizeof(SampleState));
   l.seeds = take((size_t)n * 8);
   l.counters = take(64);
   l.work = take(4 * WORK_SLOTS * 8);
   l.keys = take(with_keys ? 2 * LL * 8 : 0);
-  // scratch blocks are indexed by (sample, block) in the kernels
-  l.scratch = take(bits ? 0 : G.scratch_words * 8 * n);
   l.total = off;
   return l;
-}
-
-template <typename F>
-int set_smem(F* fn, size_t bytes) {
-  if (bytes > 48 * 1024)
-    CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-  return 0;
 }
 
 }  // namespace
@@ -253,17 +192,12 @@ int set_error(int code, const std::string& msg) { return fail(code, msg); }
 }  // namespace rsa_detail
 
 enum Kind {
-  KD_INIT, KD_ROW_CMIN, KD_COL_CMIN, KD_ROW_ACCEPT, KD_COL_ACCEPT, KD_TILE_CMIN, KD_TILE_ACCEPT,
-  KD_LINE_CMIN_H, KD_LINE_CMIN_V, KD_LINE_COMBINE, KD_LINE_ACCEPT_H, KD_LINE_ACCEPT_V,
-  KD_LINE_CODES, KD_LWIN_H, KD_LWIN_V, KD_LCOMB, KD_LACC_H, KD_LACC_V,
-  KD_ROUND_END, KD_EDGES, KD_BUCKET, KD_SEARCH_INIT, KD_PROBE_COPY, KD_PROBE, KD_DECIDE, KD_COUNT
+  KD_INIT, KD_DENSE, KD_PICK, KD_RESOLVE, KD_REFILL, KD_CHECK, KD_SITES, KD_EDGES, KD_BUCKET,
+  KD_SEARCH_INIT, KD_PROBE_COPY, KD_PROBE, KD_DECIDE, KD_COUNT
 };
 const char* const kKindNames[KD_COUNT] = {
-    "k_init",         "k_row_cmin",    "k_col_cmin",   "k_row_accept", "k_col_accept",
-    "k_tile_cmin",    "k_tile_accept", "k_line_cmin_h", "k_line_cmin_v", "k_line_combine",
-    "k_line_accept_h", "k_line_accept_v", "k_line_codes", "k_lwin_h", "k_lwin_v", "k_lcomb",
-    "k_lacc_h",       "k_lacc_v",      "k_round_end",  "k_edges",      "k_bucket",     "k_search_init",
-    "k_probe_copy",   "k_probe",       "k_search_decide"};
+    "k_init", "k_dense", "k_pick", "k_resolve", "k_refill", "k_round_check", "k_sites", "k_edges",
+    "k_bucket", "k_search_init", "k_probe_copy", "k_probe", "k_search_decide"};
 
 // Optional per-kernel timing with CUDA events recorded around each launch
 // on the launch stream, plus launch counts (always kept).
@@ -295,7 +229,6 @@ struct rsa {
   unsigned long long work[4] = {0, 0, 0, 0};  // accumulated round-pass work
   int device = -1;
   int sm_count = 0;
-  int tile_blocks[2] = {0, 0};  // resident blocks per SM: cmin, accept
   Prof prof;
   // CUDA graphs of a chunk of greedy rounds and of bisection probes, captured
   // once per (workspace, batch size, key source) on a private stream and
@@ -304,10 +237,8 @@ struct rsa {
   cudaStream_t cap_stream = nullptr;
   // chunks the previous run needed before its samples were done: the next
   // run launches that many before its first device->host check
-  u32 round_chunks_hint = 1, probe_chunks_hint = 1;
+  u32 round_chunks_hint = 0, probe_chunks_hint = 1;
   u32 round_check = ROUND_CHECK;  // greedy rounds per graph chunk / host check
-  u32 lw_threads = 256;           // CTA size of the long-k window pass (256 or 128;
-                                  // rsa_create sets default_window_threads)
   // test-only lowered caps of the device loops (0 = default; rsa_test_caps)
   u32 t_round = 0, t_uf = 0, t_probe = 0, t_edges = 0;
   struct GraphSlot {
@@ -315,9 +246,9 @@ struct rsa {
     const void* ws = nullptr;
     u32 n = 0;
     bool keys = false;
-    u32 caps[6] = {0, 0, 0, 0, 0, 0};  // caps, rounds per chunk, window CTA size in the graph
+    u32 caps[5] = {0, 0, 0, 0, 0};  // caps and rounds per chunk in the graph
     unsigned long long launches[32] = {};
-  } g_round, g_probe;
+  } g_main, g_round, g_probe;
 };
 
 namespace {
@@ -361,9 +292,7 @@ Group group_of(rsa_t* h, u32 n) {
   g.uf_cap = h->t_uf ? h->t_uf : UF_CAP;
   g.edge_limit = h->t_edges ? std::min(h->t_edges, g.cap_edges) : g.cap_edges;
   g.LL = (u64)h->L * h->L;
-  g.occ = reinterpret_cast<u8*>(b + l.occ);
   g.owner = reinterpret_cast<u32*>(b + l.owner);
-  g.cmin = reinterpret_cast<u64*>(b + l.cmin);
   g.base = reinterpret_cast<u64*>(b + l.base);
   g.keys = h->with_keys ? reinterpret_cast<const u64*>(b + l.keys) : nullptr;
   g.node_key = reinterpret_cast<u64*>(b + l.node_key);
@@ -376,9 +305,24 @@ Group group_of(rsa_t* h, u32 n) {
   g.uf = reinterpret_cast<u64*>(b + l.uf);
   g.edges = reinterpret_cast<Edge*>(b + l.edges);
   g.st = reinterpret_cast<SampleState*>(b + l.st);
-  g.scratch = reinterpret_cast<u64*>(b + l.scratch);
   g.work = reinterpret_cast<u64*>(b + l.work);
   return g;
+}
+
+RoundPtrs round_ptrs(rsa_t* h) {
+  char* b = static_cast<char*>(h->ws);
+  const Layout& l = h->lay;
+  RoundPtrs p{};
+  p.fine = reinterpret_cast<u32*>(b + l.fine);
+  p.block = reinterpret_cast<u32*>(b + l.block);
+  p.anch = reinterpret_cast<u32*>(b + l.anch);
+  p.list = reinterpret_cast<u32*>(b + l.list);
+  p.flat = reinterpret_cast<u32*>(b + l.flat);
+  p.act = reinterpret_cast<Act*>(b + l.act);
+  p.heads = reinterpret_cast<u32*>(b + l.heads);
+  p.rs = reinterpret_cast<RoundState*>(b + l.rs);
+  p.list_cap = h->geo.list_cap;
+  return p;
 }
 
 cudaEvent_t prof_event(Prof& p, size_t i) {
@@ -411,76 +355,6 @@ void launch(rsa_t* h, int kind, K kernel, dim3 grid, dim3 block, size_t smem, cu
   p.launches[kind] += 1;
 }
 
-// As launch(), for a kernel launched in thread-block clusters of
-// cluster_x CTAs along x.  Returns the launch's error.
-template <typename... KArgs, typename... Args>
-cudaError_t launch_cluster(rsa_t* h, int kind, void (*kernel)(KArgs...), dim3 grid, dim3 block,
-                           size_t smem, cudaStream_t st, u32 cluster_x, Args... args) {
-  Prof& p = h->prof;
-  cudaEvent_t e0 = nullptr, e1 = nullptr;
-  if (p.on) {
-    size_t i = p.kinds.size();
-    e0 = prof_event(p, 2 * i);
-    e1 = prof_event(p, 2 * i + 1);
-    if (e0 && e1) {
-      cudaEventRecord(e0, st);
-      p.kinds.push_back(kind);
-    }
-  }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = cluster_x;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
-  if (e0 && e1) cudaEventRecord(e1, st);
-  p.launches[kind] += 1;
-  return e;
-}
-
-template <int F, int NT>
-cudaError_t launch_lwin_nt(rsa_t* h, Group g, const Geometry& G, const u32* occw, const u32* occT,
-                           u16* out, u8* lflag, u32 n, cudaStream_t st) {
-  const dim3 grid(g.L * G.lw_cfg.nc, n), block(NT);
-  const int kind = F == 0 ? KD_LWIN_H : KD_LWIN_V;
-  const u32 nc = G.lw_cfg.nc, C = G.lw_cfg.P / NT;
-  if constexpr (NT == 128) {
-    if (C == 32) return launch_cluster(h, kind, k_lwin<F, 32, 128>, grid, block, 0, st, nc, g, G.lw_cfg, occw, occT, out, lflag);
-    return launch_cluster(h, kind, k_lwin<F, 16, 128>, grid, block, 0, st, nc, g, G.lw_cfg, occw, occT, out, lflag);
-  } else {
-    switch (C) {
-      case 1: return launch_cluster(h, kind, k_lwin<F, 1, 256>, grid, block, 0, st, nc, g, G.lw_cfg, occw, occT, out, lflag);
-      case 2: return launch_cluster(h, kind, k_lwin<F, 2, 256>, grid, block, 0, st, nc, g, G.lw_cfg, occw, occT, out, lflag);
-      case 4: return launch_cluster(h, kind, k_lwin<F, 4, 256>, grid, block, 0, st, nc, g, G.lw_cfg, occw, occT, out, lflag);
-      case 8: return launch_cluster(h, kind, k_lwin<F, 8, 256>, grid, block, 0, st, nc, g, G.lw_cfg, occw, occT, out, lflag);
-      default: return launch_cluster(h, kind, k_lwin<F, 16, 256>, grid, block, 0, st, nc, g, G.lw_cfg, occw, occT, out, lflag);
-    }
-  }
-}
-
-// The window pass with the handle's CTA size: 256 threads, or 128 threads
-// with twice the cells per thread (spans of 2048 or 4096 cells).
-template <int F>
-cudaError_t launch_lwin(rsa_t* h, Group g, const Geometry& G, const u32* occw, const u32* occT,
-                        u16* out, u8* lflag, u32 n, cudaStream_t st) {
-  if (h->lw_threads == 128) return launch_lwin_nt<F, 128>(h, g, G, occw, occT, out, lflag, n, st);
-  return launch_lwin_nt<F, 256>(h, g, G, occw, occT, out, lflag, n, st);
-}
-
-// Default CTA size of the long-k window pass: 128 threads x 32 cells on
-// 4096-cell spans with k >= 512 (measured 3% faster than 256 x 16 at
-// L = 8192, k = 512 and L = 32768, k = 4096), 256 threads elsewhere.
-u32 default_window_threads(const Geometry& G, u32 k) {
-  return G.lw && G.lw_cfg.P == 4096 && k >= 512 ? 128u : 256u;
-}
-
 int launch_check(const char* what) {
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(RSA_ECUDA, std::string(what) + ": " + cudaGetErrorString(e));
@@ -491,57 +365,6 @@ int read_counter(rsa_t* h, u32* dev_counter, u32* out) {
   CUDA_TRY(cudaMemcpyAsync(h->h_counter, dev_counter, 4, cudaMemcpyDeviceToHost, h->stream));
   CUDA_TRY(cudaStreamSynchronize(h->stream));
   *out = *h->h_counter;
-  return 0;
-}
-
-template <int K>
-int tile_occ_k(rsa_t* h) {
-  // the cell-minimum pass is sized for six resident blocks of ~38 KB static
-  // shared memory: ask for the largest shared-memory carveout
-  CUDA_TRY(cudaFuncSetAttribute(k_tile_cmin<K>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                (int)cudaSharedmemCarveoutMaxShared));
-  CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&h->tile_blocks[0], k_tile_cmin<K>, TILE_THREADS, 0));
-  CUDA_TRY(
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&h->tile_blocks[1], k_tile_accept<K>, TILE_THREADS, 0));
-  return 0;
-}
-
-int tile_occupancy(rsa_t* h) {
-  if (h->sm_count) return 0;
-  CUDA_TRY(cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, h->device));
-  int rc = 0;
-  switch (h->k) {
-    case 1: rc = tile_occ_k<1>(h); break;
-    case 2: rc = tile_occ_k<2>(h); break;
-    case 4: rc = tile_occ_k<4>(h); break;
-    case 8: rc = tile_occ_k<8>(h); break;
-    case 16: rc = tile_occ_k<16>(h); break;
-    default: rc = tile_occ_k<32>(h); break;
-  }
-  if (rc) return rc;
-  for (int i = 0; i < 2; ++i) h->tile_blocks[i] = std::max(1, h->tile_blocks[i]);
-  return 0;
-}
-
-template <int K>
-void launch_tile_k(rsa_t* h, Group g, TileCfg tc, u32* occw, u8* dead, const u32* tgrid,
-                   cudaStream_t stream) {
-  launch(h, KD_TILE_CMIN, k_tile_cmin<K>, dim3(tgrid[0]), dim3(TILE_THREADS), 0, stream, g, tc, occw, dead);
-  launch(h, KD_TILE_ACCEPT, k_tile_accept<K>, dim3(tgrid[1]), dim3(TILE_THREADS), 0, stream, g, tc, occw,
-         (const u8*)dead);
-}
-
-int launch_tile(rsa_t* h, Group g, TileCfg tc, u32* occw, u8* dead, const u32* tgrid,
-                cudaStream_t stream) {
-  switch (h->k) {
-    case 1: launch_tile_k<1>(h, g, tc, occw, dead, tgrid, stream); break;
-    case 2: launch_tile_k<2>(h, g, tc, occw, dead, tgrid, stream); break;
-    case 4: launch_tile_k<4>(h, g, tc, occw, dead, tgrid, stream); break;
-    case 8: launch_tile_k<8>(h, g, tc, occw, dead, tgrid, stream); break;
-    case 16: launch_tile_k<16>(h, g, tc, occw, dead, tgrid, stream); break;
-    case 32: launch_tile_k<32>(h, g, tc, occw, dead, tgrid, stream); break;
-    default: return fail(RSA_EINVAL, "tile path needs k in {1,2,4,8,16,32}");
-  }
   return 0;
 }
 
@@ -558,8 +381,7 @@ int run_chunk(rsa_t* h, rsa_t::GraphSlot& gs, cudaStream_t stream, u32 n, B body
     body(stream);
     return launch_check("chunk launches");
   }
-  const u32 caps[6] = {h->t_round, h->t_uf, h->t_probe, h->t_edges, h->round_check,
-                       h->lw_threads};
+  const u32 caps[5] = {h->t_round, h->t_uf, h->t_probe, h->t_edges, h->round_check};
   if (!(gs.exec && gs.ws == h->ws && gs.n == n && gs.keys == h->with_keys &&
         std::memcmp(gs.caps, caps, sizeof(caps)) == 0)) {
     drop_graph(gs);
@@ -613,152 +435,117 @@ int run_impl(rsa_t* h, const uint64_t* seeds, u32 n, const uint64_t* keys, cudaS
   u32* d_counter = reinterpret_cast<u32*>(b + l.counters);
   const u64 LL = g.LL;
 
-  // long-k lines made of whole k-blocks run the argmin-offset round for
-  // seeded priorities; caller priorities cannot be inverted
-  const bool use_lw = G.lw && !h->with_keys;
-  const u32 line_nseg = use_lw ? G.lw_cfg.nc : G.lc.nseg;
   CUDA_TRY(cudaMemcpyAsync(d_seeds, seeds, (size_t)n * 8, cudaMemcpyHostToDevice, stream));
   if (keys)
     CUDA_TRY(cudaMemcpyAsync(b + l.keys, keys, 2 * LL * 8, cudaMemcpyHostToDevice, stream));
-  if (G.tile) {
-    CUDA_TRY(cudaMemsetAsync(b + l.occw, 0, (size_t)n * LL / 8, stream));
-    CUDA_TRY(cudaMemsetAsync(b + l.dead, 0, (size_t)n * G.tc.T2, stream));
-  } else if (G.line) {
-    CUDA_TRY(cudaMemsetAsync(b + l.occw, 0, (size_t)n * LL / 8, stream));
-    CUDA_TRY(cudaMemsetAsync(b + l.occT, 0, (size_t)n * LL / 8, stream));
-    const size_t ncode = G.tc.T2;
-    CUDA_TRY(cudaMemsetAsync(b + l.dead, 0, (size_t)n * (2ull * h->L * line_nseg + ncode),
-                             stream));
-  } else {
-    CUDA_TRY(cudaMemsetAsync(g.occ, 0, (size_t)n * LL, stream));
-  }
-  CUDA_TRY(cudaMemsetAsync(g.owner, 0xFF, (size_t)n * LL * 4, stream));
-  CUDA_TRY(cudaMemsetAsync(b + l.counters, 0, 64, stream));
-  CUDA_TRY(cudaMemsetAsync(b + l.work, 0, 4 * WORK_SLOTS * 8, stream));
-  launch(h, KD_INIT, k_init, dim3((n + 127) / 128), dim3(128), 0, stream, g,
-         (const u64*)d_seeds);
-  if ((rc = launch_check("k_init"))) return rc;
-
-  if (G.line) {
-    if ((rc = set_smem(k_line_cmin<0>, G.line_smem))) return rc;
-    if ((rc = set_smem(k_line_cmin<1>, G.line_smem))) return rc;
-    if ((rc = set_smem(k_line_accept<0>, G.line_acc_smem))) return rc;
-    if ((rc = set_smem(k_line_accept<1>, G.line_acc_smem))) return rc;
-    if ((rc = set_smem(k_line_accept_codes<0>, G.line_codes_smem))) return rc;
-    if ((rc = set_smem(k_line_accept_codes<1>, G.line_codes_smem))) return rc;
-    if ((rc = set_smem(k_lcomb, sizeof(LcombSmem)))) return rc;
-  } else if (!G.tile) {
-    if ((rc = set_smem(k_row<0>, G.row_smem))) return rc;
-    if ((rc = set_smem(k_row<1>, G.row_smem))) return rc;
-    if ((rc = set_smem(k_col<0>, G.col_smem))) return rc;
-    if ((rc = set_smem(k_col<1>, G.col_smem))) return rc;
-  }
-  const dim3 rg(G.row_grid_x.x, n), cg(G.col_grid_x.x, n);
-  TileCfg tc = G.tc;
-  tc.items = (u64)n * tc.T2;
-  u32* occw = reinterpret_cast<u32*>(b + l.occw);
-  u8* dead = reinterpret_cast<u8*>(b + l.dead);
-  u32 tgrid[2] = {0, 0};
-  if (G.tile) {
-    if ((rc = tile_occupancy(h))) return rc;
-    for (int i = 0; i < 2; ++i)
-      tgrid[i] = (u32)std::min<u64>(tc.items, (u64)h->sm_count * h->tile_blocks[i]);
-  }
-  // every round accepts at least the smallest live key, so n_j + 1 rounds
-  // always suffice
-  const u32 round_cap = h->t_round ? h->t_round : cap_nodes_of(h->L, h->k) + 2;
+  if (!h->sm_count)
+    CUDA_TRY(cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, h->device));
+  RoundCfg c = G.rc;
+  // every round with an active candidate accepts the smallest of them, so
+  // n_j + 1 rounds always suffice
+  c.round_cap = h->t_round ? h->t_round : cap_nodes_of(h->L, h->k) + 2;
   const u32 probe_cap = h->t_probe ? h->t_probe : PROBE_CAP;
-  // one chunk = ROUND_CHECK greedy rounds; k_round_end counts the samples
-  // still active after each round into d_counter
-  u32* occT = reinterpret_cast<u32*>(b + l.occT);
-  u64* cB = reinterpret_cast<u64*>(b + l.cB);
+  const RoundPtrs rp = round_ptrs(h);
   int body_rc = 0;
-  auto rounds = [&](cudaStream_t st) {
-    for (u32 i = 0; i < h->round_check; ++i) {
-      if (cudaMemsetAsync(d_counter, 0, 4, st) != cudaSuccess) body_rc = RSA_ECUDA;
-      if (G.tile) {
-        if (launch_tile(h, g, tc, occw, dead, tgrid, st)) body_rc = RSA_EINVAL;
-      } else if (use_lw) {
-        u8* lflag = dead;                                          // [n][2][L][nc]
-        u8* cdead = dead + (size_t)n * 2 * h->L * line_nseg;       // [n][T^2]
-        u16* cH = reinterpret_cast<u16*>(b + l.cH);
-        u16* cV = reinterpret_cast<u16*>(b + l.cV);
-        u32* mk = reinterpret_cast<u32*>(b + l.masks);
-        const size_t mw = (size_t)n * LL / 32;  // words of one mask array
-        const AccMasks mh{mk, mk + mw, mk + 2 * mw}, mv{mk + 3 * mw, mk + 4 * mw, mk + 5 * mw};
-        if (launch_lwin<0>(h, g, G, occw, occT, cH, lflag, n, st) != cudaSuccess) body_rc = RSA_ECUDA;
-        if (launch_lwin<1>(h, g, G, occw, occT, cV, lflag, n, st) != cudaSuccess) body_rc = RSA_ECUDA;
-        launch(h, KD_LCOMB, k_lcomb, dim3((G.tc.T2 + LC_WARPS - 1) / LC_WARPS, n),
-               dim3(LC_WARPS * 32), sizeof(LcombSmem), st, g, (const u16*)cH, (const u16*)cV, mh,
-               mv, cdead);
-        const dim3 ag(h->L * line_nseg, n);
-        launch(h, KD_LACC_H, k_lacc<0>, ag, dim3(LW_THREADS), 0, st, g, G.lw_cfg, occw, occT, mh,
-               (const u8*)lflag);
-        launch(h, KD_LACC_V, k_lacc<1>, ag, dim3(LW_THREADS), 0, st, g, G.lw_cfg, occw, occT, mv,
-               (const u8*)lflag);
-      } else if (G.line) {
-        const dim3 lg(h->L * G.lc.nseg, n), tg(G.tc.T2, n);
-        u8* ldead = dead;                                          // [n][2][L][nseg]
-        u8* cdead = dead + (size_t)n * 2 * h->L * G.lc.nseg;       // [n][T^2]
-        launch(h, KD_LINE_CMIN_H, k_line_cmin<0>, lg, dim3(LINE_THREADS), G.line_smem, st, g,
-               G.lc, (const u32*)occw, (const u32*)occT, g.cmin, cB, ldead);
-        launch(h, KD_LINE_CMIN_V, k_line_cmin<1>, lg, dim3(LINE_THREADS), G.line_smem, st, g,
-               G.lc, (const u32*)occw, (const u32*)occT, g.cmin, cB, ldead);
-        if (h->with_keys) {
-          // caller-supplied priorities cannot be inverted: compare values
-          launch(h, KD_LINE_COMBINE, k_line_combine, tg, dim3(256), 0, st, g, g.cmin, cB);
-          launch(h, KD_LINE_ACCEPT_H, k_line_accept<0>, lg, dim3(LINE_THREADS), G.line_acc_smem, st,
-                 g, G.lc, occw, occT, (const u64*)g.cmin, (const u64*)cB);
-          launch(h, KD_LINE_ACCEPT_V, k_line_accept<1>, lg, dim3(LINE_THREADS), G.line_acc_smem, st,
-                 g, G.lc, occw, occT, (const u64*)g.cmin, (const u64*)cB);
-        } else {
-          u16* c16 = reinterpret_cast<u16*>(b + l.code16);
-          u16* c16T = reinterpret_cast<u16*>(b + l.code16T);
-          launch(h, KD_LINE_CODES, k_line_codes, tg, dim3(256), 0, st, g, (const u64*)g.cmin,
-                 (const u64*)cB, c16, c16T, cdead);
-          launch(h, KD_LINE_ACCEPT_H, k_line_accept_codes<0>, lg, dim3(LINE_THREADS),
-                 G.line_codes_smem, st, g, G.lc, occw, occT, (const u16*)c16, (const u16*)c16T,
-                 (const u8*)ldead);
-          launch(h, KD_LINE_ACCEPT_V, k_line_accept_codes<1>, lg, dim3(LINE_THREADS),
-                 G.line_codes_smem, st, g, G.lc, occw, occT, (const u16*)c16, (const u16*)c16T,
-                 (const u8*)ldead);
-        }
-      } else {
-        launch(h, KD_ROW_CMIN, k_row<0>, rg, dim3(G.row_threads), G.row_smem, st, g, G.row);
-        launch(h, KD_COL_CMIN, k_col<0>, cg, dim3(G.col_threads), G.col_smem, st, g, G.col);
-        launch(h, KD_ROW_ACCEPT, k_row<1>, rg, dim3(G.row_threads), G.row_smem, st, g, G.row);
-        launch(h, KD_COL_ACCEPT, k_col<1>, cg, dim3(G.col_threads), G.col_smem, st, g, G.col);
-      }
-      launch(h, KD_ROUND_END, k_round_end, dim3((n + 127) / 128), dim3(128), 0, st, g, round_cap,
-             d_counter);
+  auto check = [&](cudaError_t e) {
+    if (e != cudaSuccess) body_rc = RSA_ECUDA;
+  };
+  // blocks per sample: what the work of a sample fills, at most `waves`
+  // blocks per SM over the batch
+  auto grid_x = [&](u64 blocks, u32 waves) {
+    const u64 most = std::max<u64>(1, ((u64)h->sm_count * waves + n - 1) / n);
+    return dim3((unsigned)std::max<u64>(1, std::min(blocks, most)), n);
+  };
+  const dim3 init_grid((n + 127) / 128);
+  // Lanes per active candidate in k_resolve.  Long k has many bins to look at
+  // (L = 8192, k = 512, 32 samples: 4.9 ms with 32 lanes, 7.4 with 8, 7.6 with
+  // 1).  For short k one lane does the least work in all, which counts once
+  // the candidates fill the GPU (L = 1024, k = 32, 1000 samples: 10.4 ms with
+  // 1, 11.5 with 8), and eight lanes have the shortest chain of loads, which
+  // counts when they do not (L = 128, k = 8, 32 samples: 0.49 and 0.18 ms).
+  const u32 lanes = h->k > 128 ? 32 : (u64)n * g.cap_nodes >= (2u << 20) ? 1 : 8;
+  auto round = [&](cudaStream_t st) {
+    const dim3 pg = grid_x((c.lvl_cap[c.nlev - 1] + RD_THREADS - 1) / RD_THREADS, 16);
+    if (h->k <= PICK_LONGK)
+      launch(h, KD_PICK, k_pick<false>, pg, dim3(RD_THREADS), 0, st, g, c, rp);
+    else
+      launch(h, KD_PICK, k_pick<true>, pg, dim3(RD_THREADS), 0, st, g, c, rp);
+    const dim3 rg = grid_x(((u64)(g.cap_nodes / 4 + 1) * lanes + RD_THREADS - 1) / RD_THREADS, 16);
+    switch (lanes) {
+      case 1: launch(h, KD_RESOLVE, k_resolve<1>, rg, dim3(RD_THREADS), 0, st, g, c, rp); break;
+      case 8: launch(h, KD_RESOLVE, k_resolve<8>, rg, dim3(RD_THREADS), 0, st, g, c, rp); break;
+      default: launch(h, KD_RESOLVE, k_resolve<32>, rg, dim3(RD_THREADS), 0, st, g, c, rp); break;
     }
   };
-  {
-  NvtxRange rounds_range("greedy rounds");
-  for (u32 chunks = 0;;) {
-    const u32 burst = chunks == 0 ? h->round_chunks_hint : 1;
-    for (u32 i = 0; i < burst; ++i, ++chunks)
-      if ((rc = run_chunk(h, h->g_round, stream, n, rounds))) return rc;
-    if (body_rc) return fail(body_rc, "round launches failed");
-    u32 active;
-    if ((rc = read_counter(h, d_counter, &active))) return rc;
-    if (active == 0) {
-      h->round_chunks_hint = chunks;
-      break;
+  const u32 lines = std::max(1u, std::min(1024u, REFILL_WORDS) / c.W);
+  auto refill = [&](cudaStream_t st) {
+    launch(h, KD_REFILL, k_refill, grid_x((2ull * h->L + lines - 1) / lines, 16), dim3(RD_THREADS),
+           0, st, g, c, rp, lines);
+  };
+  auto count_active = [&](cudaStream_t st) {
+    check(cudaMemsetAsync(d_counter, 0, 4, st));
+    launch(h, KD_CHECK, k_round_check, init_grid, dim3(128), 0, st, g, d_counter);
+  };
+  // the whole deposition: every slice once, and three more rounds for the
+  // candidates left undecided by the last ones
+  auto deposit = [&](cudaStream_t st) {
+    check(cudaMemsetAsync(b + l.counters, 0, 64, st));
+    check(cudaMemsetAsync(b + l.work, 0, 4 * WORK_SLOTS * 8, st));
+    launch(h, KD_INIT, k_init, init_grid, dim3(128), 0, st, g, (const u64*)d_seeds);
+    if (G.sites) {
+      launch(h, KD_SITES, k_sites, grid_x((LL + 255) / 256, 32), dim3(256), 0, st, g);
+      return;
     }
-  }
+    check(cudaMemsetAsync(b + l.fine, 0, l.bits_bytes, st));
+    check(cudaMemsetAsync(b + l.anch, 0, l.anch_bytes, st));
+    check(cudaMemsetAsync(b + l.heads, 0xFF, l.heads_bytes, st));
+    launch(h, KD_INIT, k_round_init, init_grid, dim3(128), 0, st, g, c, rp);
+    const dim3 dg = grid_x((2 * LL + DENSE_TILE - 1) / DENSE_TILE, 16);
+    if (h->with_keys)
+      launch(h, KD_DENSE, k_dense<true>, dg, dim3(RD_THREADS), 0, st, g, c, rp);
+    else
+      launch(h, KD_DENSE, k_dense<false>, dg, dim3(RD_THREADS), 0, st, g, c, rp);
+    for (u32 t = 0; t < c.nlev; ++t) round(st);
+    refill(st);
+    for (u32 t = c.nlev; t <= c.lzmax + 3; ++t) round(st);
+    count_active(st);
+  };
+  // a sample that is not through yet: more rounds
+  auto more_rounds = [&](cudaStream_t st) {
+    refill(st);
+    for (u32 i = 0; i < h->round_check; ++i) round(st);
+    count_active(st);
+  };
+  {
+    NvtxRange rounds_range("deposition");
+    if ((rc = run_chunk(h, h->g_main, stream, n, deposit))) return rc;
+    if (body_rc) return fail(body_rc, "round launches failed");
+    for (u32 chunks = 0; !G.sites;) {
+      for (; chunks < h->round_chunks_hint; ++chunks)
+        if ((rc = run_chunk(h, h->g_round, stream, n, more_rounds))) return rc;
+      if (body_rc) return fail(body_rc, "round launches failed");
+      u32 active;
+      if ((rc = read_counter(h, d_counter, &active))) return rc;
+      if (active == 0) break;
+      h->round_chunks_hint = chunks + 1;
+    }
   }
   NvtxRange wrap_range("contact graph and first-wrap search");
   // contact graph of the jammed lattice
-  {
-    // rows per sample spread over enough blocks to fill the GPU across the batch
-    const u32 bx = (u32)std::min<u64>(h->L, std::max<u64>(1, 65536 / n));
-    if (h->L % 4 == 0 && h->L >= 8)
-      launch(h, KD_EDGES, k_edges4, dim3(bx, n), dim3(EDGES_THREADS), 0, stream, g);
+  if (G.sites) {
+    launch(h, KD_EDGES, k_site_contacts, grid_x((LL + 255) / 256, 32), dim3(256), 0, stream, g);
+  } else {
+    // lanes per k-mer: 1 for lines of a few words (L = 1024, k = 32, 1000
+    // samples: 2.0 ms, with 4 lanes 2.8), 4 for longer ones (L = 32768,
+    // k = 4096, 4 samples: 1.2 ms, with 1 lane 1.8, with 32 lanes 2.7)
+    const u32 el = h->k <= 64 ? 1 : 4;
+    const dim3 eg = grid_x(((u64)g.cap_nodes * el + 255) / 256, 32);
+    if (el == 1)
+      launch(h, KD_EDGES, k_contacts<1>, eg, dim3(256), 0, stream, g, c, rp);
     else
-      launch(h, KD_EDGES, k_edges, dim3(bx, n), dim3(EDGES_THREADS), 0, stream, g);
-    if ((rc = launch_check("k_edges"))) return rc;
+      launch(h, KD_EDGES, k_contacts<4>, eg, dim3(256), 0, stream, g, c, rp);
   }
+  if ((rc = launch_check("k_edges"))) return rc;
   launch(h, KD_BUCKET, k_bucket, dim3(n), dim3(1024), 0, stream, g);
   // bisection for the first wrap
   launch(h, KD_SEARCH_INIT, k_search_init, dim3((n + 127) / 128), dim3(128), 0, stream, g);
@@ -940,7 +727,6 @@ int rsa_create(uint32_t L, uint32_t k, uint64_t seed, rsa_t** out) {
   h->k = k;
   h->seed = seed;
   h->geo = plan(L, k);
-  h->lw_threads = default_window_threads(h->geo, k);
   *out = h;
   g_err.clear();
   return 0;
@@ -961,14 +747,22 @@ int rsa_run_batch(rsa_t* h, uint32_t n_samples, void* stream) {
 int rsa_run_keys(rsa_t* h, const uint64_t* keys, void* stream) {
   if (!h || !keys) return fail(RSA_EINVAL, "null handle or keys");
   const u64 n = 2ull * h->L * h->L;
-  std::vector<uint64_t> sorted(keys, keys + n);
-  std::sort(sorted.begin(), sorted.end());
+  std::vector<u32> order(n);
+  for (u64 i = 0; i < n; ++i) order[i] = (u32)i;
+  std::sort(order.begin(), order.end(), [&](u32 a, u32 b) { return keys[a] < keys[b]; });
+  // Only the order of the priorities matters.  The slices of the scan expect
+  // them spread evenly over 64 bits, so the ranks, spread evenly, run in
+  // their place.
+  const u64 step = (KEY_NONE - 1) / n;
+  std::vector<uint64_t> spread(n);
   for (u64 i = 0; i < n; ++i) {
-    if (sorted[i] == KEY_NONE) return fail(RSA_EINVAL, "key 2^64-1 is reserved");
-    if (i && sorted[i] == sorted[i - 1]) return fail(RSA_EINVAL, "keys are not distinct");
+    if (keys[order[i]] == KEY_NONE) return fail(RSA_EINVAL, "key 2^64-1 is reserved");
+    if (i && keys[order[i]] == keys[order[i - 1]])
+      return fail(RSA_EINVAL, "keys are not distinct");
+    spread[order[i]] = i * step + step / 2;
   }
   uint64_t seed = h->seed;
-  return run_impl(h, &seed, 1, keys, static_cast<cudaStream_t>(stream));
+  return run_impl(h, &seed, 1, spread.data(), static_cast<cudaStream_t>(stream));
 }
 
 int rsa_run_static(uint32_t L, uint32_t k, const uint64_t* seeds, uint32_t n, uint32_t* n_j,
@@ -1130,18 +924,17 @@ int rsa_test_caps(rsa_t* h, uint32_t round_cap, uint32_t uf_steps, uint32_t prob
 int rsa_set_rounds_per_check(rsa_t* h, uint32_t rounds) {
   if (!h) return fail(RSA_EINVAL, "null handle");
   if (rounds < 1 || rounds > 64) return fail(RSA_EINVAL, "rounds per check must be in 1 .. 64");
-  if (rounds != h->round_check) h->round_chunks_hint = 1;
+  if (rounds != h->round_check) h->round_chunks_hint = 0;
   h->round_check = rounds;
   return 0;
 }
 
 int rsa_set_window_threads(rsa_t* h, uint32_t threads) {
   if (!h) return fail(RSA_EINVAL, "null handle");
-  if (threads == 0) threads = default_window_threads(h->geo, h->k);
-  if (threads != 256 && threads != 128) return fail(RSA_EINVAL, "window CTA size must be 128 or 256");
-  if (threads == 128 && !(h->geo.lw && (h->geo.lw_cfg.P == 4096 || h->geo.lw_cfg.P == 2048)))
-    return fail(RSA_EINVAL, "128-thread windows need the long-k offset path with spans of 2048 or 4096 cells");
-  h->lw_threads = threads;
+  if (threads != 0 && threads != 256 && threads != 128)
+    return fail(RSA_EINVAL, "window CTA size must be 128 or 256");
+  if (threads == 128 && !h->geo.win128)
+    return fail(RSA_EINVAL, "128-thread windows need 32 < k <= 4096 dividing spans of 2048 or 4096 cells");
   return 0;
 }
 
@@ -1187,6 +980,7 @@ const char* rsa_kernel_name(uint32_t kind) {
 
 void rsa_destroy(rsa_t* h) {
   if (!h) return;
+  drop_graph(h->g_main);
   drop_graph(h->g_round);
   drop_graph(h->g_probe);
   if (h->cap_stream) cudaStreamDestroy(h->cap_stream);

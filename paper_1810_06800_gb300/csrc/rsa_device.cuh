@@ -33,7 +33,6 @@ constexpr u64 KEY_NONE = 0xFFFFFFFFFFFFFFFFull;  // dead / no candidate
 constexpr u64 SM_GAMMA = 0x9E3779B97F4A7C15ull;  // splitmix64 increment
 constexpr u32 NONE32 = 0xFFFFFFFFu;
 constexpr unsigned FULL = 0xFFFFFFFFu;
-constexpr u32 OWN_V = 1u << 31;  // owner word: set for a vertical k-mer's cells
 // Work counters are spread over WORK_SLOTS addresses (by block index), so that
 // many blocks adding to one counter do not queue on a single L2 address.
 constexpr u32 WORK_SLOTS = 32;
@@ -54,18 +53,6 @@ __device__ __forceinline__ u64 mix64(u64 z) {
   z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
   return z ^ (z >> 31);
 }
-
-// Inverse of mix64: each xor-shift z ^ (z >> s) is undone by xoring the
-// shifts s, 2s, ... below 64, each odd multiplier by its inverse mod 2^64.
-__device__ __forceinline__ u64 mix64_inverse(u64 z) {
-  z = z ^ (z >> 31) ^ (z >> 62);
-  z *= 0x319642B2D24D8EC3ull;  // inverse of 0x94D049BB133111EB
-  z = z ^ (z >> 27) ^ (z >> 54);
-  z *= 0x96DE1B173F119089ull;  // inverse of 0xBF58476D1CE4E5B9
-  z = z ^ (z >> 30) ^ (z >> 60);
-  return z;
-}
-constexpr u64 SM_GAMMA_INV = 0xF1DE83E19937733Dull;  // inverse of the golden gamma
 
 struct Edge {          // one contact between two k-mers (24 bytes)
   u64 time;            // max of the two k-mers' priorities
@@ -94,9 +81,8 @@ struct Group {         // one batch of samples sharing (L, k)
   u32 uf_cap;          // steps of one union-find walk or link retry loop
   u32 edge_limit;      // contact edges stored per sample (<= cap_edges)
   u64 LL;
-  u8* occ;             // [n][L][L]   1 = occupied
-  u32* owner;          // [n][L][L]   node id (| OWN_V if vertical) or NONE32
-  u64* cmin;           // [n][L][L]   per-cell minimum of live priorities
+  u32* owner;          // [n][L][L]   node id of the k-mer anchored at the cell; only
+                       //             anchors are written, the rest is never read
   u64* base;           // [n]         splitmix64 stream base per sample
   const u64* keys;     // caller priorities [2 L^2] (test path), else null
   u64* node_key;       // [n][cap_nodes]
@@ -109,11 +95,9 @@ struct Group {         // one batch of samples sharing (L, k)
   u64* nkey_b;         // [n][cap_nodes] node keys grouped by key >> 56
   u32* nbkt;           // [n][NBKT + 1] bucket offsets into nkey_b
   SampleState* st;     // [n]
-  u64* scratch;        // global scratch for very long windows (or null)
-  u64* work;           // [4][WORK_SLOTS] work counters of the round passes (tile path:
-                       //     cmin cells, cmin keys, accept cells, accept keys; long-k
-                       //     path: horizontal and vertical window-minimum cells,
-                       //     acceptance cells, code cells)
+  u64* work;           // [4][WORK_SLOTS] work counters of the deposition: candidates
+                       //     hashed by the first pass, list entries tested, active
+                       //     candidates resolved, k-mers accepted
 };
 
 // Add v to work counter c (slot chosen by the block index).
@@ -144,173 +128,5 @@ __device__ __forceinline__ u64 uf_pack(u32 p, u32 dx, u32 dy) {
 }
 
 constexpr u32 UF_CAP = 1u << 20;  // default walk / retry cap (Group::uf_cap)
-
-// ---------------------------------------------------------------------
-// Segmented min-scans used by the window minimum.  A window of width k
-// ending at span position v+k-1 (i.e. covering [v, v+k-1]) equals
-// min(Q[v], P[v+k-1]) where P / Q are prefix / suffix minima inside blocks
-// [m k, (m+1) k) of the span (van Herk / Gil-Werman).  seg == 0 means one
-// unbounded segment.
-// ---------------------------------------------------------------------
-
-// One warp scans arr[0, n) (contiguous).  Forward = prefix minima.
-template <typename T>
-__device__ void warp_scan_fwd(const T* src, T* dst, u32 n, u32 seg, T ident) {
-  const u32 lane = threadIdx.x & 31;
-  u32 C = (n + 31) / 32;
-  C |= 1u;  // odd chunk stride keeps the 32 lanes on distinct banks
-  const u32 a = min(lane * C, n), b = min(a + C, n);
-  T run = ident;
-  bool flag = false;
-  for (u32 u = a; u < b; ++u) {
-    if (seg && (u % seg) == 0) { run = ident; flag = true; }
-    run = tmin(run, src[u]);
-    dst[u] = run;
-  }
-  T agg = run;
-  bool f = flag;
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    T oa = __shfl_up_sync(FULL, agg, d);
-    bool of = __shfl_up_sync(FULL, f, d);
-    if ((int)lane >= d) {
-      if (!f) agg = tmin(agg, oa);
-      f = f || of;
-    }
-  }
-  T carry = __shfl_up_sync(FULL, agg, 1);
-  if (lane == 0) carry = ident;
-  if (a < b && !(seg && (a % seg) == 0)) {
-    u64 stop = seg ? ((u64)(a + seg - 1) / seg) * seg : (u64)b;
-    u32 e = (u32)(stop < b ? stop : b);
-    for (u32 u = a; u < e; ++u) dst[u] = tmin(dst[u], carry);
-  }
-}
-
-// One warp, suffix minima (segments end at multiples of seg minus one).
-template <typename T>
-__device__ void warp_scan_bwd(const T* src, T* dst, u32 n, u32 seg, T ident) {
-  const u32 lane = threadIdx.x & 31;
-  u32 C = (n + 31) / 32;
-  C |= 1u;
-  const u32 a = min(lane * C, n), b = min(a + C, n);
-  T run = ident;
-  bool flag = false;
-  for (u32 u = b; u > a; --u) {
-    const u32 p = u - 1;
-    if (seg && ((p + 1) % seg) == 0) { run = ident; flag = true; }
-    run = tmin(run, src[p]);
-    dst[p] = run;
-  }
-  T agg = run;
-  bool f = flag;
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    T oa = __shfl_down_sync(FULL, agg, d);
-    bool of = __shfl_down_sync(FULL, f, d);
-    if (lane + d < 32) {
-      if (!f) agg = tmin(agg, oa);
-      f = f || of;
-    }
-  }
-  T carry = __shfl_down_sync(FULL, agg, 1);
-  if (lane == 31) carry = ident;
-  if (a < b && !(seg && (b % seg) == 0)) {
-    u32 s0 = seg ? (b / seg) * seg : 0u;
-    u32 e = s0 > a ? s0 : a;
-    for (u32 u = e; u < b; ++u) dst[u] = tmin(dst[u], carry);
-  }
-}
-
-// Whole block scans W interleaved lines: element (u, line) at [u*W + line].
-// Thread t handles line t % W, chunk t / W (G = blockDim / W chunks).
-template <typename T>
-__device__ void lines_scan_fwd(const T* src, T* dst, u32 n, u32 seg, T ident, u32 W,
-                               T* aggv, u8* aggf) {
-  const u32 line = threadIdx.x % W, g = threadIdx.x / W, G = blockDim.x / W;
-  const u32 C = (n + G - 1) / G;
-  const u32 a = min(g * C, n), b = min(a + C, n);
-  T run = ident;
-  bool flag = false;
-  for (u32 u = a; u < b; ++u) {
-    if (seg && (u % seg) == 0) { run = ident; flag = true; }
-    run = tmin(run, src[(size_t)u * W + line]);
-    dst[(size_t)u * W + line] = run;
-  }
-  aggv[g * W + line] = run;
-  aggf[g * W + line] = flag;
-  __syncthreads();
-  if (a < b && !(seg && (a % seg) == 0)) {
-    T carry = ident;
-    for (int gg = (int)g - 1; gg >= 0; --gg) {
-      carry = tmin(carry, aggv[gg * W + line]);
-      if (aggf[gg * W + line]) break;
-    }
-    u64 stop = seg ? ((u64)(a + seg - 1) / seg) * seg : (u64)b;
-    u32 e = (u32)(stop < b ? stop : b);
-    for (u32 u = a; u < e; ++u) dst[(size_t)u * W + line] = tmin(dst[(size_t)u * W + line], carry);
-  }
-  __syncthreads();
-}
-
-template <typename T>
-__device__ void lines_scan_bwd(const T* src, T* dst, u32 n, u32 seg, T ident, u32 W,
-                               T* aggv, u8* aggf) {
-  const u32 line = threadIdx.x % W, g = threadIdx.x / W, G = blockDim.x / W;
-  const u32 C = (n + G - 1) / G;
-  const u32 a = min(g * C, n), b = min(a + C, n);
-  T run = ident;
-  bool flag = false;
-  for (u32 u = b; u > a; --u) {
-    const u32 p = u - 1;
-    if (seg && ((p + 1) % seg) == 0) { run = ident; flag = true; }
-    run = tmin(run, src[(size_t)p * W + line]);
-    dst[(size_t)p * W + line] = run;
-  }
-  aggv[g * W + line] = run;
-  aggf[g * W + line] = flag;
-  __syncthreads();
-  if (a < b && !(seg && (b % seg) == 0)) {
-    T carry = ident;
-    for (u32 gg = g + 1; gg < G; ++gg) {
-      carry = tmin(carry, aggv[gg * W + line]);
-      if (aggf[gg * W + line]) break;
-    }
-    u32 s0 = seg ? (b / seg) * seg : 0u;
-    u32 e = s0 > a ? s0 : a;
-    for (u32 u = e; u < b; ++u) dst[(size_t)u * W + line] = tmin(dst[(size_t)u * W + line], carry);
-  }
-  __syncthreads();
-}
-
-// Record an accepted candidate: allocate its node, occupy its k cells.
-__device__ __forceinline__ void accept_candidate(const Group& g, u32 s, u32 idx, u64 key) {
-  SampleState& st = g.st[s];
-  const u32 node = atomicAdd(&st.n_nodes, 1u);
-  if (node >= g.cap_nodes) { atomicOr(&st.status, ST_NODE_OVF); return; }
-  g.node_key[(size_t)s * g.cap_nodes + node] = key;
-  g.node_idx[(size_t)s * g.cap_nodes + node] = idx;
-  const u32 L = g.L;
-  const u32 o = idx / (u32)g.LL, r = idx % (u32)g.LL;
-  const u32 y0 = r / L, x0 = r % L;
-  g.node_pos[(size_t)s * g.cap_nodes + node] = (o << 31) | (y0 << 15) | x0;
-  u8* occ = g.occ + (size_t)s * g.LL;
-  u32* own = g.owner + (size_t)s * g.LL;
-  if (o == 0) {
-    u32 x = x0;
-    for (u32 i = 0; i < g.k; ++i) {
-      occ[(size_t)y0 * L + x] = 1;
-      own[(size_t)y0 * L + x] = node;  // horizontal: bit 31 clear
-      if (++x == L) x = 0;
-    }
-  } else {
-    u32 y = y0;
-    for (u32 i = 0; i < g.k; ++i) {
-      occ[(size_t)y * L + x0] = 1;
-      own[(size_t)y * L + x0] = node | OWN_V;
-      if (++y == L) y = 0;
-    }
-  }
-}
 
 }  // namespace rsak

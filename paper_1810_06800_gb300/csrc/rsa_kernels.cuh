@@ -4,184 +4,6 @@
 
 namespace rsak {
 
-// Launch geometry of the row pass: one warp per (row, segment of S cells).
-struct RowCfg {
-  u32 S, nseg;        // segment length, segments per row
-  u32 warps;          // warps per block
-  u32 warp_words;     // u64 words of per-warp scratch (A region + B region)
-  u32 nmax;           // max span length (S + k - 1)
-  int global_scratch; // 1: per-warp scratch in g.scratch instead of smem
-};
-
-// Geometry of the column pass: W adjacent columns x (segment of S rows).
-struct ColCfg {
-  u32 S, nseg;        // segment length (rows), segments per column
-  u32 W, nstrip;      // columns per block, column strips
-  u32 nmax, nocc;     // value span and occupancy span lengths
-  u32 block_words;    // u64 words of scratch per block
-  int global_scratch;
-};
-
-__device__ __forceinline__ u32 wrap_add(u32 a, u32 b, u32 L) {
-  u32 r = a + b;
-  return r >= L ? (r % L) : r;
-}
-
-// MODE 0: horizontal part of cmin.  For row y and x in the segment,
-//   cmin(y,x) = min over live horizontal candidates anchored at
-//               (y, x-k+1 .. x) of their key.
-// A horizontal candidate is live iff its k cells are free.
-// MODE 1: accept horizontal candidates: (y,x) is accepted iff
-//   min(cmin(y, x .. x+k-1)) == key(0, y, x).
-template <int MODE>
-__global__ void __launch_bounds__(256) k_row(Group g, RowCfg rc) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const u32 s = blockIdx.y;
-  if (g.st[s].done) return;
-  const u32 warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const u32 L = g.L, k = g.k;
-  u64* A;
-  if (rc.global_scratch)
-    A = g.scratch +
-        (((size_t)blockIdx.y * gridDim.x + blockIdx.x) * rc.warps + warp) * rc.warp_words;
-  else
-    A = reinterpret_cast<u64*>(smem_raw) + (size_t)warp * rc.warp_words;
-  u64* B = A + rc.nmax;          // values -> prefix minima
-  u32* N = reinterpret_cast<u32*>(A);  // next-occupied table (aliases A)
-  const u8* occ = g.occ + (size_t)s * g.LL;
-  u64* cmin = g.cmin + (size_t)s * g.LL;
-  bool any_alive = false;
-  const u64 total = (u64)L * rc.nseg;
-  for (u64 q = (u64)blockIdx.x * rc.warps + warp; q < total; q += (u64)gridDim.x * rc.warps) {
-    const u32 y = (u32)(q / rc.nseg), seg = (u32)(q % rc.nseg);
-    const u32 x0 = seg * rc.S;
-    const u32 Se = min(rc.S, L - x0);
-    const u32 n = Se + k - 1;
-    const u8* orow = occ + (size_t)y * L;
-    u64* crow = cmin + (size_t)y * L;
-    if (MODE == 0) {
-      const u32 xs = (x0 + L - (k - 1)) % L;
-      const u32 nocc = Se + 2 * k - 2;
-      for (u32 u = lane; u < nocc; u += 32) N[u] = orow[wrap_add(xs, u % L, L)] ? u : NONE32;
-      __syncwarp();
-      warp_scan_bwd<u32>(N, N, nocc, 0u, NONE32);
-      __syncwarp();
-      for (u32 u = lane; u < n; u += 32) {
-        const bool alive = N[u] >= u + k;  // NONE32 >= anything
-        u64 v = KEY_NONE;
-        if (alive) {
-          const u32 x = wrap_add(xs, u % L, L);
-          v = cand_key(g, s, (u64)y * L + x);
-          any_alive = true;
-        }
-        B[u] = v;
-      }
-    } else {
-      for (u32 u = lane; u < n; u += 32) B[u] = crow[wrap_add(x0, u % L, L)];
-    }
-    __syncwarp();
-    warp_scan_bwd<u64>(B, A, n, k, KEY_NONE);  // suffix minima -> A
-    __syncwarp();
-    warp_scan_fwd<u64>(B, B, n, k, KEY_NONE);  // prefix minima in place
-    __syncwarp();
-    for (u32 v = lane; v < Se; v += 32) {
-      const u64 w = tmin(A[v], B[v + k - 1]);
-      const u32 x = x0 + v;
-      if (MODE == 0) {
-        crow[x] = w;
-      } else if (w != KEY_NONE) {
-        const u32 idx = y * L + x;
-        if (w == cand_key(g, s, idx)) accept_candidate(g, s, idx, w);
-      }
-    }
-    __syncwarp();
-  }
-  if (MODE == 0) {
-    if (__any_sync(FULL, any_alive) && lane == 0) atomicOr(&g.st[s].alive, 1u);
-  }
-}
-
-// MODE 0: vertical part of cmin, combined with the horizontal part already
-//   in cmin: cmin(y,x) = min(cmin(y,x), min over live vertical candidates
-//   anchored at (y-k+1 .. y, x)).
-// MODE 1: accept vertical candidates: (y,x) accepted iff
-//   min(cmin(y .. y+k-1, x)) == key(1, y, x).
-template <int MODE>
-__global__ void __launch_bounds__(256) k_col(Group g, ColCfg cc) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  const u32 s = blockIdx.y;
-  if (g.st[s].done) return;
-  const u32 L = g.L, k = g.k, W = cc.W, G = blockDim.x / W;
-  u64* base;
-  if (cc.global_scratch)
-    base = g.scratch + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * cc.block_words;
-  else
-    base = reinterpret_cast<u64*>(smem_raw);
-  u64* A = base;                                     // nmax*W (N aliases it)
-  const size_t a_words = max((size_t)cc.nmax * W, ((size_t)cc.nocc * W + 1) / 2);
-  u64* B = A + a_words;                              // nmax*W
-  u64* aggv = B + (size_t)cc.nmax * W;               // G*W
-  u8* aggf = reinterpret_cast<u8*>(aggv + (size_t)G * W);  // G*W
-  u32* N = reinterpret_cast<u32*>(A);
-  const u8* occ = g.occ + (size_t)s * g.LL;
-  u64* cmin = g.cmin + (size_t)s * g.LL;
-  bool any_alive = false;
-  const u32 total = cc.nstrip * cc.nseg;
-  for (u32 q = blockIdx.x; q < total; q += gridDim.x) {
-    const u32 strip = q / cc.nseg, seg = q % cc.nseg;
-    const u32 c0 = strip * W, y0 = seg * cc.S;
-    const u32 Se = min(cc.S, L - y0);
-    const u32 n = Se + k - 1;
-    if (MODE == 0) {
-      const u32 ys = (y0 + L - (k - 1)) % L;
-      const u32 nocc = Se + 2 * k - 2;
-      for (u32 f = threadIdx.x; f < nocc * W; f += blockDim.x) {
-        const u32 u = f / W, c = f % W, x = c0 + c;
-        u32 v = NONE32;
-        if (x < L && occ[(size_t)wrap_add(ys, u % L, L) * L + x]) v = u;
-        N[f] = v;
-      }
-      __syncthreads();
-      lines_scan_bwd<u32>(N, N, nocc, 0u, NONE32, W, reinterpret_cast<u32*>(aggv), aggf);
-      for (u32 f = threadIdx.x; f < n * W; f += blockDim.x) {
-        const u32 u = f / W, c = f % W, x = c0 + c;
-        u64 v = KEY_NONE;
-        if (x < L && N[f] >= u + k) {
-          const u32 y = wrap_add(ys, u % L, L);
-          v = cand_key(g, s, (u64)L * L + (u64)y * L + x);
-          any_alive = true;
-        }
-        B[f] = v;
-      }
-    } else {
-      for (u32 f = threadIdx.x; f < n * W; f += blockDim.x) {
-        const u32 u = f / W, c = f % W, x = c0 + c;
-        B[f] = x < L ? cmin[(size_t)wrap_add(y0, u % L, L) * L + x] : KEY_NONE;
-      }
-    }
-    __syncthreads();
-    lines_scan_bwd<u64>(B, A, n, k, KEY_NONE, W, aggv, aggf);
-    lines_scan_fwd<u64>(B, B, n, k, KEY_NONE, W, aggv, aggf);
-    for (u32 f = threadIdx.x; f < Se * W; f += blockDim.x) {
-      const u32 v = f / W, c = f % W, x = c0 + c;
-      if (x >= L) continue;
-      const u64 w = tmin(A[f], B[f + (size_t)(k - 1) * W]);
-      const u32 y = y0 + v;
-      if (MODE == 0) {
-        u64* p = cmin + (size_t)y * L + x;
-        *p = tmin(*p, w);
-      } else if (w != KEY_NONE) {
-        const u32 idx = (u32)(g.LL + (u64)y * L + x);
-        if (w == cand_key(g, s, idx)) accept_candidate(g, s, idx, w);
-      }
-    }
-    __syncthreads();
-  }
-  if (MODE == 0) {
-    if (__syncthreads_or(any_alive) && threadIdx.x == 0) atomicOr(&g.st[s].alive, 1u);
-  }
-}
-
 // Per-sample set-up: stream base from the seed, state cleared.
 __global__ void k_init(Group g, const u64* seeds) {
   const u32 s = blockIdx.x * blockDim.x + threadIdx.x;
@@ -189,212 +11,6 @@ __global__ void k_init(Group g, const u64* seeds) {
   g.base[s] = mix64(seeds[s] + SM_GAMMA);
   SampleState z = {};
   g.st[s] = z;
-}
-
-// End of a round: a sample with no live candidate left is jammed.
-__global__ void k_round_end(Group g, u32 round_cap, u32* n_active) {
-  const u32 s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= g.n) return;
-  SampleState& st = g.st[s];
-  if (st.done) return;
-  if (!st.alive) {
-    st.done = 1;
-    return;
-  }
-  st.alive = 0;
-  st.rounds += 1;
-  if (st.rounds >= round_cap) {
-    st.status |= ST_ROUND_CAP;
-    st.done = 1;
-    return;
-  }
-  atomicAdd(n_active, 1u);
-}
-
-// ---------------------------------------------------------------------
-// Contact graph of the jammed lattice.  Nodes are accepted k-mers; a
-// lattice edge (a, a+e), e in {+x, +y}, between occupied cells of k-mers
-// m1 and m2 says that in the lift anchor(m2) = anchor(m1) + delta with
-//   delta = i e(m1) + e - j e(m2)  (i, j = positions of a, a+e inside the
-// k-mers).  Runs of identical (m1, m2, delta) along the direction
-// perpendicular to e are emitted once; a run start is forced at row 0 (for
-// +x) / column 0 (for +y) so that runs that close around the torus are kept.
-// Only edges whose m1 == m2 and delta == 0 (inside one k-mer) are dropped.
-// ---------------------------------------------------------------------
-// Lifted displacement of the contact between cell (y, x) of node m1 and its
-// neighbour (by, bx) in direction dir of node m2, packed as 16+16 bits.
-__device__ __forceinline__ u32 contact_delta(const Group& g, u32 s, u32 y, u32 x, u32 by, u32 bx,
-                                             u32 dir, u32 m1, u32 m2, bool* internal) {
-  const u32* npos = g.node_pos + (size_t)s * g.cap_nodes;
-  u32 o1, o2;
-  const u32 i = pos_in_kmer(npos[m1], y, x, g.L, &o1);
-  const u32 j = pos_in_kmer(npos[m2], by, bx, g.L, &o2);
-  const int dx = (o1 == 0 ? (int)i : 0) + (dir == 0) - (o2 == 0 ? (int)j : 0);
-  const int dy = (o1 == 1 ? (int)i : 0) + (dir == 1) - (o2 == 1 ? (int)j : 0);
-  *internal = m1 == m2 && dx == 0 && dy == 0;
-  return ((u32)dx & 0xFFFFu) | (((u32)dy & 0xFFFFu) << 16);
-}
-
-constexpr u32 EDGES_THREADS = 256;
-
-// The two contacts (+x, +y) of cell (y, x) of owner a, given the owners of
-// its neighbours (right, down, up, up-right, left, down-left): counted by
-// class into cnt, and emitted as graph edges unless internal to one k-mer or
-// a repeat of the previous contact of their run.  Every lane of the warp
-// calls it (ballots inside); a lane with nothing to do passes a = NONE32.
-__device__ __forceinline__ void edge_cell(const Group& g, u32 s, SampleState& st, const u64* nkey,
-                                          Edge* E, bool full_compare, u32 lane, u32 y, u32 x,
-                                          u32 yp, u32 yn, u32 xp, u32 xn, u32 a, u32 o_r,
-                                          u32 o_d, u32 o_u, u32 o_ur, u32 o_l, u32 o_dl,
-                                          u32 cnt[3]) {
-#pragma unroll
-  for (u32 dir = 0; dir < 2; ++dir) {
-    const u32 by = dir ? yn : y, bx = dir ? x : xn;
-    bool emit = false;
-    u32 b = NONE32, d = 0;
-    u32 kind = 3;  // contact class: 0 both horizontal, 1 both vertical, 2 mixed
-    if (a != NONE32) {
-      b = dir ? o_d : o_r;
-      // owner words carry the k-mer's orientation in bit 31
-      if (b != NONE32 && b != a) kind = (a ^ b) >> 31 ? 2u : a >> 31;
-      if (b != NONE32) {
-        bool internal = false;
-        // the previous contact of the run: one row up (+x edges) or one
-        // column left (+y edges)
-        const bool force = dir == 0 ? (y == 0) : (x == 0);
-        const u32 py = dir == 0 ? yp : y, px = dir == 0 ? x : xp;
-        const u32 qy = dir == 0 ? yp : yn, qx = dir == 0 ? xn : xp;
-        const u32 pa = force ? NONE32 : (dir == 0 ? o_u : o_l);
-        const u32 pb = force ? NONE32 : (dir == 0 ? o_ur : o_dl);
-        const bool same_pair = pa == a && pb == b;
-        if (!same_pair || full_compare) {
-          d = contact_delta(g, s, y, x, by, bx, dir, a & ~OWN_V, b & ~OWN_V, &internal);
-          emit = !internal;
-          if (emit && same_pair) {
-            bool pint = false;
-            const u32 pd = contact_delta(g, s, py, px, qy, qx, dir, pa & ~OWN_V, pb & ~OWN_V,
-                                         &pint);
-            emit = pd != d;
-          }
-        }
-      }
-    }
-    // interspecific-contact counts (Sec. II.A): every contact, before the
-    // run deduplication of the graph edges
-    cnt[0] += kind == 0;
-    cnt[1] += kind == 1;
-    cnt[2] += kind == 2;
-    const u32 mask = __ballot_sync(FULL, emit);
-    if (!mask) continue;
-    u32 basei = 0;
-    const u32 leader = __ffs(mask) - 1;
-    if (lane == leader) basei = atomicAdd(&st.n_edges, (u32)__popc(mask));
-    basei = __shfl_sync(FULL, basei, leader);
-    if (emit) {
-      const u32 e = basei + __popc(mask & ((1u << lane) - 1u));
-      if (e < g.edge_limit) {
-        Edge ed;
-        const u32 ma = a & ~OWN_V, mb = b & ~OWN_V;
-        ed.time = max(nkey[ma], nkey[mb]);
-        ed.m1 = ma;
-        ed.m2 = mb;
-        ed.dxy = d;
-        ed.pad = 0;
-        E[e] = ed;
-      } else {
-        atomicOr(&st.status, ST_EDGE_OVF);
-      }
-    }
-  }
-}
-
-__device__ __forceinline__ void edge_counts(SampleState& st, u32 lane, const u32 cnt[3]) {
-#pragma unroll
-  for (u32 c = 0; c < 3; ++c) {
-    const u32 t = __reduce_add_sync(FULL, cnt[c]);
-    if (lane == 0 && t)
-      atomicAdd(c == 0 ? &st.contacts_x : c == 1 ? &st.contacts_y : &st.contacts_xy, t);
-  }
-}
-
-// Any L: one cell per thread per step.
-__global__ void __launch_bounds__(EDGES_THREADS) k_edges(Group g) {
-  const u32 s = blockIdx.y;
-  const u32 L = g.L;
-  const u32 lane = threadIdx.x & 31;
-  SampleState& st = g.st[s];
-  const u32* own = g.owner + (size_t)s * g.LL;
-  const u64* nkey = g.node_key + (size_t)s * g.cap_nodes;
-  Edge* E = g.edges + (size_t)s * g.cap_edges;
-  // For k < L (and L > 2) consecutive contacts between the same two k-mers
-  // along a run always have the same displacement, so runs are told apart by
-  // their owners alone; rings (k = L) and tiny lattices compare displacements.
-  const bool full_compare = g.k == L || L <= 2;
-  // block b walks rows b, b + gridDim.x, ...; its threads stride along the
-  // row (every lane of a warp runs the same number of steps: ballots inside)
-  const u32 xsteps = (L + blockDim.x - 1) / blockDim.x;
-  u32 cnt[3] = {0, 0, 0};
-  for (u32 y = blockIdx.x; y < L; y += gridDim.x)
-  for (u32 xs = 0; xs < xsteps; ++xs) {
-    const u32 xx = xs * blockDim.x + threadIdx.x;
-    const bool inb = xx < L;
-    const u32 x = inb ? xx : 0;
-    const u32 yp = y == 0 ? L - 1 : y - 1, yn = y + 1 == L ? 0 : y + 1;
-    const u32 xp = x == 0 ? L - 1 : x - 1, xn = x + 1 == L ? 0 : x + 1;
-    // the cell, its +x / +y neighbours, and the cells whose contact precedes
-    // each of the two in its run (up, up-right for +x; left, down-left for
-    // +y): all loaded at once, so their latencies overlap
-    const u32 a = inb ? __ldg(own + (size_t)y * L + x) : NONE32;
-    const u32 o_r = __ldg(own + (size_t)y * L + xn), o_d = __ldg(own + (size_t)yn * L + x);
-    const u32 o_u = __ldg(own + (size_t)yp * L + x), o_ur = __ldg(own + (size_t)yp * L + xn);
-    const u32 o_l = __ldg(own + (size_t)y * L + xp), o_dl = __ldg(own + (size_t)yn * L + xp);
-    edge_cell(g, s, st, nkey, E, full_compare, lane, y, x, yp, yn, xp, xn, a, o_r, o_d, o_u,
-              o_ur, o_l, o_dl, cnt);
-  }
-  edge_counts(st, lane, cnt);
-}
-
-// L a multiple of 4 (and at least 8): four consecutive cells per thread per
-// step, from one 16-byte load of each of the three rows involved plus the
-// four neighbour cells outside the quad.
-__global__ void __launch_bounds__(EDGES_THREADS) k_edges4(Group g) {
-  const u32 s = blockIdx.y;
-  const u32 L = g.L, L4 = L / 4;
-  const u32 lane = threadIdx.x & 31;
-  SampleState& st = g.st[s];
-  const u32* own = g.owner + (size_t)s * g.LL;
-  const u64* nkey = g.node_key + (size_t)s * g.cap_nodes;
-  Edge* E = g.edges + (size_t)s * g.cap_edges;
-  const bool full_compare = g.k == L;
-  const u32 xsteps = (L4 + blockDim.x - 1) / blockDim.x;
-  u32 cnt[3] = {0, 0, 0};
-  for (u32 y = blockIdx.x; y < L; y += gridDim.x)
-  for (u32 xs = 0; xs < xsteps; ++xs) {
-    const u32 qq = xs * blockDim.x + threadIdx.x;
-    const bool inb = qq < L4;
-    const u32 x0 = inb ? 4 * qq : 0;
-    const u32 yp = y == 0 ? L - 1 : y - 1, yn = y + 1 == L ? 0 : y + 1;
-    const u32 xl = x0 == 0 ? L - 1 : x0 - 1, xr = x0 + 4 == L ? 0 : x0 + 4;
-    const u32* ry = own + (size_t)y * L;
-    const u32* rn = own + (size_t)yn * L;
-    const u32* rp = own + (size_t)yp * L;
-    const uint4 A = __ldg(reinterpret_cast<const uint4*>(ry + x0));
-    const uint4 D = __ldg(reinterpret_cast<const uint4*>(rn + x0));
-    const uint4 U = __ldg(reinterpret_cast<const uint4*>(rp + x0));
-    const u32 a_r = __ldg(ry + xr), a_l = __ldg(ry + xl);
-    const u32 d_l = __ldg(rn + xl), u_r = __ldg(rp + xr);
-    const u32 av[4] = {A.x, A.y, A.z, A.w}, dv[4] = {D.x, D.y, D.z, D.w};
-    const u32 uv[4] = {U.x, U.y, U.z, U.w};
-#pragma unroll
-    for (u32 i = 0; i < 4; ++i) {
-      const u32 x = x0 + i;
-      const u32 xp = i == 0 ? xl : x - 1, xn = i == 3 ? xr : x + 1;
-      edge_cell(g, s, st, nkey, E, full_compare, lane, y, x, yp, yn, xp, xn,
-                inb ? av[i] : NONE32, i < 3 ? av[i + 1] : a_r, dv[i], uv[i],
-                i < 3 ? uv[i + 1] : u_r, i > 0 ? av[i - 1] : a_l, i > 0 ? dv[i - 1] : d_l, cnt);
-    }
-  }
-  edge_counts(st, lane, cnt);
 }
 
 // Group one sample's edges by time >> 56 and its node keys by key >> 56

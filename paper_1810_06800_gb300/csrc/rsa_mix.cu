@@ -137,7 +137,7 @@ extern "C" int rsa_run_small(const uint32_t* L, const uint32_t* k, const uint64_
 // Autotuner.  For one (GPU, L, k, batch size rounded up to a power of two)
 // it times every candidate way to run the batch once -- small mode at 256,
 // 512 and 1024 threads per CTA when the shape fits it, and the global path
-// at 2, 4 and 8 greedy rounds per host check -- on seeds 1 .. n, and keeps
+// at 2, 4 and 8 rounds per host check -- on seeds 1 .. n, and keeps
 // the fastest.  Results go to a JSON-lines cache ($RSA_TUNE_CACHE, else
 // $HOME/.cache/rsa_gb300/tune.jsonl), read back on the next process start.
 // ---------------------------------------------------------------------
@@ -311,24 +311,13 @@ extern "C" int rsa_tune(uint32_t L, uint32_t k, uint32_t n, int measure, rsa_tun
       c.threads = t;
       cands.push_back(c);
     }
-  // the 128-thread window pass exists only for some shapes: ask a handle
-  bool w128 = false;
-  {
-    rsa_t* h = nullptr;
-    if (rsa_create(L, k, 1, &h) == 0) {
-      w128 = rsa_set_window_threads(h, 128) == 0;
-      rsa_destroy(h);
-    }
+  for (uint32_t r : {2u, 4u, 8u}) {
+    rsa_tune_t c{};
+    c.mode = RSA_MODE_GLOBAL;
+    c.rounds_per_check = r;
+    c.window_threads = 256;
+    cands.push_back(c);
   }
-  for (uint32_t r : {2u, 4u, 8u})
-    for (uint32_t wt : {256u, 128u}) {
-      if (wt == 128 && !w128) continue;
-      rsa_tune_t c{};
-      c.mode = RSA_MODE_GLOBAL;
-      c.rounds_per_check = r;
-      c.window_threads = wt;
-      cands.push_back(c);
-    }
   cudaStream_t st = nullptr;
   MIX_CUDA(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
   rsa_tune_t best = *out;

@@ -1,0 +1,844 @@
+// rsa_rounds.cuh -- deposition to jamming by slices of the priority range
+// (any 2 <= k <= L), sm_103a.
+//
+// A candidate of priority key conflicts with about D = k^2 + 2k others, so
+// the ones accepted first all have priorities near 2^64 / D and nearly every
+// candidate dies before its turn comes.  The scan therefore goes through the
+// priority range in slices [lo, hi] (each twice as wide as the one before)
+// and only ever works on the candidates of the current slice that are still
+// live:
+//   k_dense    every candidate hashed once; the idx of those with priority
+//              below 2^(64 - a) go to one list per slice (level = leading
+//              zeros of the priority);
+//   k_pick     the entries of the current slice whose k cells are free become
+//              the active set, together with the undecided rest of the slice
+//              before; each is linked into a square bin of its anchor;
+//   k_resolve  an active candidate that conflicts with no active candidate of
+//              smaller priority is accepted: node, anchor bits, cover bits.
+//              The others stay for the next slice, whose k_pick drops the
+//              dead ones;
+//   k_refill   after the listed slices (2^-a of all candidates): the few
+//              candidates still live, read off the cover bits of each line,
+//              become the list of all remaining slices.
+// Exactness: when a slice is resolved every undecided candidate of smaller
+// priority is in the active set, so "no active conflicting candidate is
+// smaller" is the sequential scan's condition for acceptance, and acceptance
+// order is irrelevant otherwise.
+//
+// Measured share of candidates (L = 1024 .. 2048, k = 4 .. 256): the active
+// sets of all slices add up to 1.4 n_j, two to four rounds decide a slice,
+// and 1.5% of the candidates are still live at priority 2^64 * 4 / k.  The
+// arithmetic is thus one splitmix64 per candidate plus work proportional to
+// the k-mers, where a round over the whole lattice costs two window minima
+// of 64-bit priorities for every cell, eight to ten times over.
+//
+// Lines are kept as bits with their first k cells repeated after the end, so
+// a window of k cells never wraps.  Cover bits of orientation o (lines along
+// o) mark the cells a candidate of o must avoid: the k-mers of o on their own
+// line, and the crossing ones.  A crossing k-mer would set one bit on each of
+// k lines; instead the blocks of 2^bs whole lines it crosses get one bit in a
+// block line, and only the lines at its two ends their own: 2^bs + k / 2^bs
+// updates in place of k, against reading two lines in each test.
+#pragma once
+#include "rsa_device.cuh"
+
+namespace rsak {
+
+constexpr u32 RD_LEVELS = 32;
+constexpr u32 RD_THREADS = 256;
+constexpr u32 DENSE_PER = 16;                      // candidates per thread and tile
+constexpr u32 DENSE_TILE = RD_THREADS * DENSE_PER;
+constexpr u32 DENSE_STAGE = 2 * DENSE_TILE;
+constexpr u32 REFILL_WORDS = 2304;                 // words of line staged per block
+
+struct RoundCfg {
+  u32 W;            // words of a cover line, (L + k) bits and one spare
+  u32 WA;           // words of an anchor line, (L + 2k) bits and one spare
+  u32 bs, nbl;      // block lines: 2^bs lines each, nbl of them (bs = 0: none)
+  u32 b, nb;        // bins of 2^b x 2^b cells, nb per side
+  u32 a;            // k_dense lists priorities below 2^(64 - a)
+  u32 lzmax;        // slice 0 takes every priority of at least lzmax leading zeros
+  u32 nlev;         // listed slices, lzmax - a + 1
+  u32 cap_act;      // active candidates per sample
+  u32 cap_flat;     // entries of the refilled list
+  u32 round_cap;
+  u32 lvl_off[RD_LEVELS], lvl_cap[RD_LEVELS];
+};
+
+struct Act {        // an active candidate (16 bytes, one load)
+  u64 key;
+  u32 pos;          // o << 31 | y << 15 | x of its anchor
+  u32 next;         // next active candidate of its bin
+};
+
+struct RoundState { // per sample
+  u64 lo, hi;       // current slice, both ends included
+  u64 fill_hi;      // the refilled list holds priorities up to this one
+  u32 t;            // number of the slice: 0 .. lzmax
+  u32 open;         // 0: no slice, only undecided candidates go on
+  u32 drain;        // the active set was full: one round without new entries
+  u32 refill;       // the lists are used up: k_refill has to run, from lo on
+  u32 finished;     // every slice has been entered
+  u32 par;          // active buffer written by this round
+  u32 act[2];       // active candidates per buffer
+  u32 left;         // not accepted in the last round
+  u32 flat_n;
+  u32 ticket, ticket2;
+  u32 lvl_n[RD_LEVELS];
+};
+
+__device__ __forceinline__ u64 slice_top(const RoundCfg& c, u32 t) {
+  const u32 lz = c.lzmax - t;
+  return lz == 0 ? ~0ull : (1ull << (64 - lz)) - 1ull;
+}
+
+struct RoundPtrs {
+  u32* fine;        // [n][2][L][W]
+  u32* block;       // [n][2][nbl][W]
+  u32* anch;        // [n][4][L][WA]: type * 2 + layout
+  u32* list;        // [n][list_cap]
+  u32* flat;        // [n][cap_flat]
+  Act* act;         // [n][2][cap_act]
+  u32* heads;       // [n][2][2][nb * nb]
+  RoundState* rs;   // [n]
+  u64 list_cap;
+};
+
+__device__ __forceinline__ u32* cover_line(const Group& g, const RoundCfg& c, const RoundPtrs& p,
+                                           u32 s, u32 o, u32 line) {
+  return p.fine + (((size_t)s * 2 + o) * g.L + line) * c.W;
+}
+__device__ __forceinline__ u32* block_line(const RoundCfg& c, const RoundPtrs& p, u32 s, u32 o,
+                                           u32 bl) {
+  return p.block + (((size_t)s * 2 + o) * c.nbl + bl) * c.W;
+}
+// Anchors of k-mers of orientation `type`, as lines along `layout`.
+__device__ __forceinline__ u32* anchor_line(const Group& g, const RoundCfg& c, const RoundPtrs& p,
+                                            u32 s, u32 type, u32 layout, u32 line) {
+  return p.anch + (((size_t)s * 4 + type * 2 + layout) * g.L + line) * c.WA;
+}
+
+__global__ void k_round_init(Group g, RoundCfg c, RoundPtrs p) {
+  const u32 s = blockIdx.x * blockDim.x + threadIdx.x;
+  if (s >= g.n) return;
+  RoundState z = {};
+  z.open = 1;
+  z.hi = slice_top(c, 0);
+  z.fill_hi = ~0ull;
+  p.rs[s] = z;
+}
+
+// Append v for every lane with ok: slot of the lane in a counter.
+__device__ __forceinline__ u32 warp_append(u32* counter, bool ok) {
+  const u32 m = __ballot_sync(FULL, ok);
+  if (!m) return 0;
+  const u32 lane = threadIdx.x & 31, leader = __ffs(m) - 1;
+  u32 at = 0;
+  if (lane == leader) at = atomicAdd(counter, (u32)__popc(m));
+  at = __shfl_sync(FULL, at, leader);
+  return at + __popc(m & ((1u << lane) - 1u));
+}
+
+// Every candidate hashed once.  A block goes over tiles of 4096 consecutive
+// candidates; a thread keeps its 16 hits of a tile as a bit mask, so the
+// inner loop is the hash and one compare.  Hits are staged in shared memory
+// and leave by level, one global counter update per level and flush.
+// (the high word of mix64's last step z ^ (z >> 31) has at least a >= 1
+// leading zeros iff that of z has, so the hit test needs neither that step
+// nor the low word of the second product)
+template <bool KEYS>
+__global__ void __launch_bounds__(RD_THREADS) k_dense(Group g, const __grid_constant__ RoundCfg c,
+                                                      RoundPtrs p) {
+  __shared__ u32 stage[DENSE_STAGE];
+  __shared__ u8 lev[DENSE_STAGE];
+  __shared__ u32 count, lcnt[RD_LEVELS], lbase[RD_LEVELS];
+  const u32 s = blockIdx.y, tid = threadIdx.x, lane = tid & 31;
+  const u64 N = 2 * g.LL, zb = g.base[s] + SM_GAMMA;
+  RoundState& r = p.rs[s];
+  const u64 ntile = (N + DENSE_TILE - 1) / DENSE_TILE;
+  const u32 shift = 32 - c.a;
+  if (tid == 0) count = 0;
+  __syncthreads();
+  for (u64 tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
+    const u64 i0 = tile * DENSE_TILE + tid;
+    u32 hits = 0;
+    if (KEYS) {
+      for (u32 j = 0; j < DENSE_PER; ++j) {
+        const u64 i = i0 + j * RD_THREADS;
+        if (i < N && (u32)(g.keys[i] >> 32) >> shift == 0) hits |= 1u << j;
+      }
+    } else {
+      u64 z = zb + SM_GAMMA * i0;
+#pragma unroll
+      for (u32 j = 0; j < DENSE_PER; ++j, z += SM_GAMMA * RD_THREADS) {
+        u64 h = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+        h = (h ^ (h >> 27)) * 0x94D049BB133111EBull;
+        if ((u32)(h >> 32) >> shift == 0) hits |= 1u << j;
+      }
+      if (i0 + (DENSE_PER - 1) * RD_THREADS >= N) {
+        for (u32 j = 0; j < DENSE_PER; ++j)
+          if (i0 + j * RD_THREADS >= N) hits &= ~(1u << j);
+      }
+    }
+    // this warp's hits, packed
+    const u32 nh = __popc(hits);
+    u32 pre = nh;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const u32 o = __shfl_up_sync(FULL, pre, d);
+      if ((int)lane >= d) pre += o;
+    }
+    u32 at = 0;
+    if (lane == 31 && pre) at = atomicAdd(&count, pre);
+    at = __shfl_sync(FULL, at, 31) + pre - nh;
+    for (u32 m = hits; m; m &= m - 1) stage[at++] = (u32)(i0 + (__ffs(m) - 1) * RD_THREADS);
+    __syncthreads();
+    const u32 n = count;
+    const bool last = tile + gridDim.x >= ntile;
+    if (n + DENSE_TILE > DENSE_STAGE || last) {
+      if (tid < RD_LEVELS) lcnt[tid] = 0;
+      __syncthreads();
+      for (u32 i = tid; i < n; i += RD_THREADS) {
+        const u32 idx = stage[i];
+        const u64 key = KEYS ? g.keys[idx] : mix64(zb + SM_GAMMA * idx);
+        const u32 lz = min((u32)__clzll((long long)key), c.lzmax), t = c.lzmax - lz;
+        lev[i] = (u8)t;
+        atomicAdd(&lcnt[t], 1u);
+      }
+      __syncthreads();
+      if (tid < c.nlev) {
+        lbase[tid] = lcnt[tid] ? atomicAdd(&r.lvl_n[tid], lcnt[tid]) : 0u;
+        lcnt[tid] = 0;
+      }
+      __syncthreads();
+      u32* list = p.list + (size_t)s * p.list_cap;
+      for (u32 i = tid; i < n; i += RD_THREADS) {
+        const u32 t = lev[i], at2 = lbase[t] + atomicAdd(&lcnt[t], 1u);
+        if (at2 < c.lvl_cap[t]) list[c.lvl_off[t] + at2] = stage[i];
+        else atomicOr(&g.st[s].status, ST_NODE_OVF);
+      }
+      __syncthreads();
+      if (tid == 0) count = 0;
+    }
+    __syncthreads();
+  }
+  if (tid == 0 && blockIdx.x == 0) work_add(g, 0, N);
+}
+
+// Word w of the bits [pos, pos + k) of a line, masked to them.
+__device__ __forceinline__ u32 window_word(const u32* line, u32 w, u32 pos, u32 end) {
+  u32 v = __ldcg(line + w);
+  if (w == pos >> 5) v &= 0xFFFFFFFFu << (pos & 31u);
+  if (w == end >> 5) v &= 0xFFFFFFFFu >> (31u - (end & 31u));
+  return v;
+}
+
+// The active set of this round.  Windows of up to LONGK cells are tested by
+// the lane that holds the candidate; longer ones first at three words, and
+// the few that pass by the whole warp.
+constexpr u32 PICK_LONGK = 96;
+template <bool LONG>
+__global__ void __launch_bounds__(RD_THREADS) k_pick(Group g, const __grid_constant__ RoundCfg c,
+                                                     RoundPtrs p) {
+  const u32 s = blockIdx.y;
+  if (g.st[s].done) return;
+  RoundState& r = p.rs[s];
+  const u32 L = g.L, k = g.k, tid = threadIdx.x, lane = tid & 31;
+  const u32 par = r.par, t = r.t;
+  const u64 lo = r.lo, hi = r.hi;
+  const bool flat = t >= c.nlev, take = r.open && !r.drain;
+  const u32 n1 = !take ? 0u : flat ? r.flat_n : min(r.lvl_n[t], c.lvl_cap[t]);
+  const u32 n2 = r.act[par ^ 1u];
+  const u32* list = flat ? p.flat + (size_t)s * c.cap_flat
+                         : p.list + (size_t)s * p.list_cap + c.lvl_off[t];
+  const Act* prev = p.act + ((size_t)s * 2 + (par ^ 1u)) * c.cap_act;
+  Act* cur = p.act + ((size_t)s * 2 + par) * c.cap_act;
+  u32* heads = p.heads + ((size_t)s * 2 + par) * 2 * c.nb * c.nb;
+  const u64 zb = g.base[s] + SM_GAMMA;
+  if (blockIdx.x == 0 && tid == 0) r.left = 0;
+  const u32 total = n1 + n2;
+  for (u32 i0 = blockIdx.x * blockDim.x; i0 < total; i0 += gridDim.x * blockDim.x) {
+    const u32 i = i0 + tid;
+    bool ok = i < total;
+    u32 o = 0, y = 0, x = 0;
+    u64 key = 0;
+    if (ok) {
+      if (i < n1) {
+        const u32 idx = __ldg(list + i);
+        key = g.keys ? g.keys[idx] : mix64(zb + SM_GAMMA * idx);
+        ok = key >= lo && key <= hi;
+        if (ok) {
+          u32 rr = idx;
+          if (rr >= (u32)g.LL) { o = 1; rr -= (u32)g.LL; }
+          y = rr / L;
+          x = rr - y * L;
+        }
+      } else {
+        const Act e = prev[i - n1];
+        key = e.key;
+        o = e.pos >> 31;
+        y = (e.pos >> 15) & 0x7FFFu;
+        x = e.pos & 0x7FFFu;
+      }
+    }
+    const u32 line = o ? x : y, pos = o ? y : x, end = pos + k - 1;
+    const u32* fl = cover_line(g, c, p, s, o, line);
+    const u32* bl = c.bs ? block_line(c, p, s, o, line >> c.bs) : fl;
+    const u32 w0 = pos >> 5, w1 = end >> 5;
+    if (!LONG) {
+      if (ok) {
+        u32 v = 0;
+        for (u32 w = w0; w <= w1; ++w) {
+          v |= window_word(fl, w, pos, end);
+          if (c.bs) v |= window_word(bl, w, pos, end);
+          if (v) break;
+        }
+        ok = v == 0;
+      }
+    } else {
+      if (ok) {
+        const u32 wm = (w0 + w1) >> 1;
+        ok = (window_word(fl, w0, pos, end) | window_word(bl, w0, pos, end) |
+              window_word(fl, w1, pos, end) | window_word(bl, w1, pos, end) | __ldcg(fl + wm) |
+              __ldcg(bl + wm)) == 0;
+      }
+      // the words between, 32 at a time, one candidate after another
+      for (u32 m = __ballot_sync(FULL, ok); m; m &= m - 1) {
+        const u32 src = __ffs(m) - 1;
+        const u32 so = __shfl_sync(FULL, o, src), sl = __shfl_sync(FULL, line, src);
+        const u32 a0 = __shfl_sync(FULL, w0, src) + 1, a1 = __shfl_sync(FULL, w1, src);
+        const u32* f2 = cover_line(g, c, p, s, so, sl);
+        const u32* b2 = block_line(c, p, s, so, sl >> c.bs);
+        u32 v = 0;
+        for (u32 w = a0 + lane; w < a1; w += 32) v |= __ldcg(f2 + w) | __ldcg(b2 + w);
+        const bool hit = __any_sync(FULL, v != 0);
+        if (lane == src && hit) ok = false;
+      }
+    }
+    const u32 slot = warp_append(&r.act[par], ok);
+    if (ok && slot < c.cap_act) {
+      Act e;
+      e.key = key;
+      e.pos = (o << 31) | (y << 15) | x;
+      e.next = atomicExch(heads + ((size_t)o * c.nb + (y >> c.b)) * c.nb + (x >> c.b), slot);
+      *reinterpret_cast<uint4*>(cur + slot) = *reinterpret_cast<uint4*>(&e);
+    }
+  }
+  if (tid == 0 && blockIdx.x == 0) work_add(g, 1, total);
+}
+
+// Bins that the cells [a, a + len) of a ring of L cells touch, as n1 bins
+// from b0 on and n2 from bin 0 on.
+struct BinRun {
+  u32 b0, n1, n;
+  __device__ __forceinline__ BinRun(u32 a, u32 len, u32 L, u32 b) {
+    if (len > L) len = L;
+    b0 = a >> b;
+    const u32 e = a + len;
+    if (e <= L) {
+      n1 = n = ((e - 1) >> b) - b0 + 1;
+    } else {
+      n1 = ((L - 1) >> b) - b0 + 1;
+      n = n1 + min(((e - L - 1) >> b) + 1, b0);
+    }
+  }
+  __device__ __forceinline__ u32 bin(u32 i) const { return i < n1 ? b0 + i : i - n1; }
+};
+
+__device__ __forceinline__ u32 ring_sub(u32 a, u32 b, u32 L) { return a >= b ? a - b : a + L - b; }
+
+// Set bit q of a line and its copies one and two turns on.
+__device__ __forceinline__ void set_bit_copies(u32* line, u32 q, u32 L, u32 bits) {
+  for (; q < bits; q += L) atomicOr(line + (q >> 5), 1u << (q & 31u));
+}
+
+// Bits [a, e) of a line that fall in word w.
+__device__ __forceinline__ u32 range_word(u32 w, u32 a, u32 e) {
+  const u32 w0 = w * 32;
+  if (e <= w0 || a >= w0 + 32) return 0;
+  u32 m = 0xFFFFFFFFu;
+  if (a > w0) m &= 0xFFFFFFFFu << (a - w0);
+  if (e < w0 + 32) m &= 0xFFFFFFFFu >> (w0 + 32 - e);
+  return m;
+}
+
+// Cover bits of an accepted k-mer, by the G lanes of a group (lane j).
+template <int G>
+__device__ void cover_kmer(const Group& g, const RoundCfg& c, const RoundPtrs& p, u32 s, u32 o,
+                           u32 line, u32 pos, u32 j) {
+  const u32 L = g.L, k = g.k;
+  // its own line: [pos, pos + k), the part past the end again at the start,
+  // the part among the first k cells again past the end
+  u32* own = cover_line(g, c, p, s, o, line);
+  const u32 e = pos + k;
+  for (u32 w = (pos >> 5) + j; w <= (e - 1) >> 5; w += G) atomicOr(own + w, range_word(w, pos, e));
+  if (e > L)
+    for (u32 w = j; w <= (e - L - 1) >> 5; w += G) atomicOr(own + w, range_word(w, 0, e - L));
+  if (pos < k) {
+    const u32 a2 = pos + L, e2 = min(e, k) + L;
+    for (u32 w = (a2 >> 5) + j; w <= (e2 - 1) >> 5; w += G) atomicOr(own + w, range_word(w, a2, e2));
+  }
+  // the lines it crosses: cells [pos, pos + k) of the ring as one or two
+  // stretches; whole blocks of lines by their block line
+  const u32 bits = L + k;
+  for (u32 h = 0; h < 2; ++h) {
+    const u32 a = h ? 0u : pos, b = h ? (e > L ? e - L : 0u) : min(e, L);
+    if (a >= b) continue;
+    u32 f0 = b, f1 = b;  // whole blocks cover lines [f0, f1)
+    if (c.bs) {
+      const u32 j0 = (a + (1u << c.bs) - 1) >> c.bs, j1 = b == L ? c.nbl : b >> c.bs;
+      if (j0 < j1) {
+        f0 = j0 << c.bs;
+        f1 = min(j1 << c.bs, L);
+        for (u32 bl = j0 + j; bl < j1; bl += G)
+          set_bit_copies(block_line(c, p, s, o ^ 1u, bl), line, L, bits);
+      }
+    }
+    for (u32 q = a + j; q < f0; q += G)
+      set_bit_copies(cover_line(g, c, p, s, o ^ 1u, q), line, L, bits);
+    for (u32 q = f1 + j; q < b; q += G)
+      set_bit_copies(cover_line(g, c, p, s, o ^ 1u, q), line, L, bits);
+  }
+}
+
+// The step from one round to the next (one thread per sample).
+__device__ void round_step(const Group& g, const RoundCfg& c, RoundState& r, SampleState& st,
+                           u32 n) {
+  if (n > c.cap_act) {
+    // too many: this round decided nothing; the same undecided candidates
+    // again, with a narrower slice, or with none if it is one key wide
+    r.act[r.par] = 0;
+    if (r.hi == r.lo) r.drain = 1;
+    else r.hi = r.lo + (r.hi - r.lo) / 8;
+    return;
+  }
+  r.par ^= 1u;
+  r.act[r.par] = 0;
+  if (r.drain) {
+    r.drain = 0;
+  } else if (r.open) {
+    const u64 top = slice_top(c, r.t), wide = r.hi - r.lo;
+    const bool listed = r.t < c.nlev, used_up = r.hi == (listed ? slice_top(c, c.nlev - 1) : r.fill_hi);
+    r.lo = r.hi + 1;
+    if (r.lo == 0) {
+      r.finished = 1;
+      r.open = 0;
+    } else {
+      if (r.hi == top) {
+        r.t += 1;
+        r.hi = slice_top(c, r.t);
+      } else {  // narrowed before: wider again
+        const u64 room = top - r.lo, w = wide < (1ull << 61) ? wide * 4 + 3 : room;
+        r.hi = r.lo + (w < room ? w : room);
+      }
+      if (used_up) {
+        r.refill = 1;  // k_refill opens the next slice
+        r.open = 0;
+        r.fill_hi = ~0ull;
+        r.flat_n = 0;
+      } else if (!listed) {
+        r.hi = r.hi < r.fill_hi ? r.hi : r.fill_hi;
+      }
+    }
+  }
+  if (n) st.rounds += 1;
+  if (r.finished && r.left == 0) st.done = 1;
+  else if (st.rounds >= c.round_cap) {
+    st.status |= ST_ROUND_CAP;
+    st.done = 1;
+  }
+}
+
+// G lanes per active candidate.  Bins are about 4 sqrt(k) cells wide, which
+// leaves one or two active candidates in each and k / 16 bins to look at.
+template <int G>
+__global__ void __launch_bounds__(RD_THREADS) k_resolve(Group g,
+                                                        const __grid_constant__ RoundCfg c,
+                                                        RoundPtrs p) {
+  __shared__ u32 left_sh;
+  const u32 s = blockIdx.y;
+  SampleState& st = g.st[s];
+  if (st.done) return;
+  RoundState& r = p.rs[s];
+  const u32 L = g.L, k = g.k, tid = threadIdx.x;
+  const u32 par = r.par, n = r.act[par];
+  const bool over = n > c.cap_act;
+  // the bins of the next round
+  {
+    u32* nx = p.heads + ((size_t)s * 2 + (over ? par : par ^ 1u)) * 2 * c.nb * c.nb;
+    for (u32 i = blockIdx.x * RD_THREADS + tid; i < 2 * c.nb * c.nb; i += gridDim.x * RD_THREADS)
+      nx[i] = NONE32;
+  }
+  if (tid == 0) left_sh = 0;
+  __syncthreads();
+  const u32* heads = p.heads + ((size_t)s * 2 + par) * 2 * c.nb * c.nb;
+  const Act* cur = p.act + ((size_t)s * 2 + par) * c.cap_act;
+  const u32 j = tid & (G - 1);
+  const u32 gmask = G == 32 ? FULL : ((1u << (G & 31)) - 1u) << ((tid & 31) & ~(G - 1));
+  constexpr u32 GPB = RD_THREADS / G;
+  u32 left = 0, taken = 0;
+  if (!over) {
+    for (u32 i = blockIdx.x * GPB + tid / G; i < n; i += gridDim.x * GPB) {
+      const uint4 raw = __ldg(reinterpret_cast<const uint4*>(cur + i));
+      const u64 key = (u64)raw.y << 32 | raw.x;
+      const u32 o = raw.z >> 31, y = (raw.z >> 15) & 0x7FFFu, x = raw.z & 0x7FFFu;
+      const u32 line = o ? x : y, pos = o ? y : x;
+      // conflicting anchors: on its own line less than k away; crossing ones
+      // on the k lines of its cells, from k - 1 cells before its line to it
+      const BinRun same(ring_sub(pos, k - 1, L), 2 * k - 1, L, c.b);
+      const BinRun cl(pos, k, L, c.b), cp(ring_sub(line, k - 1, L), k, L, c.b);
+      const u32 nbin = same.n + cl.n * cp.n;
+      bool beaten = false;
+      for (u32 q0 = 0; q0 < nbin; q0 += G) {
+        const u32 q = q0 + j;
+        if (q < nbin) {
+          u32 bo, bl, bp;  // orientation, bin along its line's index, bin along the line
+          if (q < same.n) {
+            bo = o;
+            bl = line >> c.b;
+            bp = same.bin(q);
+          } else {
+            const u32 qq = q - same.n, q1 = qq / cp.n;
+            bo = o ^ 1u;
+            bl = cl.bin(q1);
+            bp = cp.bin(qq - q1 * cp.n);
+          }
+          // bins are stored by (row, column)
+          const u32 by = bo ? bp : bl, bx = bo ? bl : bp;
+          u32 e = __ldg(heads + ((size_t)bo * c.nb + by) * c.nb + bx);
+          for (u32 guard = 0; e != NONE32 && guard < n; ++guard) {
+            const uint4 a = __ldg(reinterpret_cast<const uint4*>(cur + e));
+            e = a.w;
+            if (((u64)a.y << 32 | a.x) >= key) continue;
+            const u32 ay = (a.z >> 15) & 0x7FFFu, ax = a.z & 0x7FFFu;
+            const u32 aline = bo ? ax : ay, apos = bo ? ay : ax;
+            if (bo == o) {
+              const u32 d = ring_sub(apos, pos, L);
+              if (aline == line && (d < k || d > L - k)) { beaten = true; break; }
+            } else if (ring_sub(aline, pos, L) < k && ring_sub(line, apos, L) < k) {
+              beaten = true;
+              break;
+            }
+          }
+        }
+        if (G > 1) beaten = (__ballot_sync(gmask, beaten) & gmask) != 0;
+        if (beaten) break;
+      }
+      if (beaten) {
+        if (j == 0) ++left;
+        continue;
+      }
+      u32 node = 0;
+      if (j == 0) node = atomicAdd(&st.n_nodes, 1u);
+      if (G > 1) node = __shfl_sync(gmask, node, 0, G);
+      if (node >= g.cap_nodes) {
+        if (j == 0) atomicOr(&st.status, ST_NODE_OVF);
+        continue;
+      }
+      if (j == 0) {
+        const size_t nd = (size_t)s * g.cap_nodes + node;
+        const u32 cell = y * L + x;
+        g.node_key[nd] = key;
+        g.node_idx[nd] = o * (u32)g.LL + cell;
+        g.node_pos[nd] = raw.z;
+        g.owner[(size_t)s * g.LL + cell] = node;
+        ++taken;
+      }
+      if (G == 1 || j < 2) {
+        const u32 bits = L + 2 * k;
+        for (u32 lay = G == 1 ? 0 : j; lay < (G == 1 ? 2 : j + 1); ++lay)
+          set_bit_copies(anchor_line(g, c, p, s, o, lay, lay ? x : y), lay ? y : x, L, bits);
+      }
+      cover_kmer<G>(g, c, p, s, o, line, pos, j);
+    }
+  }
+  left = __reduce_add_sync(FULL, left);
+  taken = __reduce_add_sync(FULL, taken);
+  if ((tid & 31) == 0) {
+    if (left) atomicAdd(&left_sh, left);
+    if (taken) work_add(g, 3, taken);
+  }
+  __syncthreads();
+  if (tid == 0) {
+    if (left_sh) atomicAdd(&r.left, left_sh);
+    if (blockIdx.x == 0) work_add(g, 2, over ? 0 : n);
+    __threadfence();
+    if (atomicAdd(&r.ticket, 1u) == gridDim.x - 1) {
+      __threadfence();
+      r.ticket = 0;
+      r.left = __ldcg(&r.left);
+      round_step(g, c, r, st, n);
+    }
+  }
+}
+
+// The candidates of every line still live once the list is used up, those
+// with priorities in [lo, fill_hi]: the window OR of a line's cover bits,
+// doubling the window until it holds k cells.
+__global__ void __launch_bounds__(RD_THREADS) k_refill(Group g, const __grid_constant__ RoundCfg c,
+                                                       RoundPtrs p, u32 lines_per_block) {
+  __shared__ u32 buf[2][REFILL_WORDS];
+  const u32 s = blockIdx.y;
+  if (g.st[s].done) return;
+  RoundState& r = p.rs[s];
+  if (!r.refill) return;
+  const u32 L = g.L, k = g.k, W = c.W, tid = threadIdx.x;
+  const u64 lo = r.lo, hi = r.fill_hi, zb = g.base[s] + SM_GAMMA;
+  u32* flat = p.flat + (size_t)s * c.cap_flat;
+  const u32 groups = (2 * L + lines_per_block - 1) / lines_per_block;
+  for (u32 gr = blockIdx.x; gr < groups; gr += gridDim.x) {
+    const u32 l0 = gr * lines_per_block, nl = min(lines_per_block, 2 * L - l0), nw = nl * W;
+    for (u32 i = tid; i < nw; i += RD_THREADS) {
+      const u32 ll = i / W, w = i - ll * W, o = l0 + ll >= L, line = l0 + ll - (o ? L : 0u);
+      u32 v = cover_line(g, c, p, s, o, line)[w];
+      if (c.bs) v |= block_line(c, p, s, o, line >> c.bs)[w];
+      buf[0][i] = v;
+    }
+    __syncthreads();
+    u32 from = 0;
+    for (u32 m = 1; m < k;) {
+      const u32 d = min(m, k - m), dw = d >> 5, db = d & 31u;
+      for (u32 i = tid; i < nw; i += RD_THREADS) {
+        const u32 w = i % W;
+        const u32 v0 = w + dw < W ? buf[from][i + dw] : 0u;
+        const u32 v1 = w + dw + 1 < W ? buf[from][i + dw + 1] : 0u;
+        buf[from ^ 1][i] = buf[from][i] | __funnelshift_r(v0, v1, db);
+      }
+      m += d;
+      from ^= 1u;
+      __syncthreads();
+    }
+    const u32 WL = (L + 31) / 32, items = nl * WL;
+    for (u32 i0 = 0; i0 < items; i0 += RD_THREADS) {
+      const u32 i = i0 + tid;
+      u32 live = 0;
+      u64 idx0 = 0, step = 1;
+      if (i < items) {
+        const u32 ll = i / WL, w = i - ll * WL, o = l0 + ll >= L, line = l0 + ll - (o ? L : 0u);
+        live = ~buf[from][ll * W + w];
+        if (w == WL - 1 && (L & 31u)) live &= (1u << (L & 31u)) - 1u;
+        idx0 = o ? g.LL + (u64)w * 32 * L + line : (u64)line * L + w * 32;
+        step = o ? L : 1;
+        for (u32 m = live; m; m &= m - 1) {
+          const u32 b = __ffs(m) - 1;
+          const u64 idx = idx0 + step * b;
+          const u64 key = g.keys ? g.keys[idx] : mix64(zb + SM_GAMMA * idx);
+          if (key < lo || key > hi) live &= ~(1u << b);  // below lo: in the active set already
+        }
+      }
+      const u32 nh = __popc(live), lane = tid & 31;
+      u32 pre = nh;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const u32 v = __shfl_up_sync(FULL, pre, d);
+        if ((int)lane >= d) pre += v;
+      }
+      u32 at = 0;
+      if (lane == 31 && pre) at = atomicAdd(&r.flat_n, pre);
+      at = __shfl_sync(FULL, at, 31) + pre - nh;
+      for (u32 m = live; m; m &= m - 1, ++at)
+        if (at < c.cap_flat) flat[at] = (u32)(idx0 + step * (__ffs(m) - 1));
+    }
+    __syncthreads();
+  }
+  if (tid == 0) {
+    __threadfence();
+    if (atomicAdd(&r.ticket2, 1u) == gridDim.x - 1) {
+      __threadfence();
+      r.ticket2 = 0;
+      if (__ldcg(&r.flat_n) > c.cap_flat) {
+        // more than the list holds: fewer priorities, next time
+        r.fill_hi = lo + (hi - lo) / 8;
+        r.flat_n = 0;
+      } else {
+        r.refill = 0;
+        r.open = 1;
+        r.hi = r.hi < hi ? r.hi : hi;
+      }
+    }
+  }
+}
+
+// Samples not jammed yet.
+__global__ void k_round_check(Group g, u32* n_active) {
+  const u32 s = blockIdx.x * blockDim.x + threadIdx.x;
+  if (s < g.n && !g.st[s].done) atomicAdd(n_active, 1u);
+}
+
+// ---------------------------------------------------------------------
+// k = 1: the two candidates of a cell conflict only with each other, so each
+// cell takes the one of smaller priority, in one pass, as node y L + x; its
+// contacts are its right and lower neighbour.
+// ---------------------------------------------------------------------
+__global__ void __launch_bounds__(256) k_sites(Group g) {
+  const u32 s = blockIdx.y, L = g.L;
+  const u64 zb = g.base[s] + SM_GAMMA;
+  const size_t nb = (size_t)s * g.cap_nodes;
+  for (u64 i = blockIdx.x * 256ull + threadIdx.x; i < g.LL; i += gridDim.x * 256ull) {
+    const u64 h = g.keys ? g.keys[i] : mix64(zb + SM_GAMMA * i);
+    const u64 v = g.keys ? g.keys[i + g.LL] : mix64(zb + SM_GAMMA * (i + g.LL));
+    const u32 o = v < h, y = (u32)i / L, x = (u32)i - y * L;
+    g.node_key[nb + i] = o ? v : h;
+    g.node_idx[nb + i] = (u32)(i + (o ? g.LL : 0));
+    g.node_pos[nb + i] = (o << 31) | (y << 15) | x;
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    SampleState& st = g.st[s];
+    st.n_nodes = (u32)g.LL;
+    st.rounds = 1;
+    st.done = 1;
+    work_add(g, 0, 2 * g.LL);
+    work_add(g, 3, g.LL);
+  }
+}
+
+__device__ __forceinline__ void contact_counts(SampleState& st, const u32 cnt[3]) {
+#pragma unroll
+  for (u32 i = 0; i < 3; ++i) {
+    const u32 t = __reduce_add_sync(FULL, cnt[i]);
+    if ((threadIdx.x & 31) == 0 && t)
+      atomicAdd(i == 0 ? &st.contacts_x : i == 1 ? &st.contacts_y : &st.contacts_xy, t);
+  }
+}
+
+__device__ __forceinline__ void put_edge(const Group& g, SampleState& st, Edge* E, u32 at, u64 time,
+                                         u32 m1, u32 m2, u32 dx, u32 dy) {
+  if (at >= g.edge_limit) {
+    atomicOr(&st.status, ST_EDGE_OVF);
+    return;
+  }
+  Edge e;
+  e.time = time;
+  e.m1 = m1;
+  e.m2 = m2;
+  e.dxy = (dx & 0xFFFFu) | (dy << 16);
+  e.pad = 0;
+  E[at] = e;
+}
+
+__global__ void __launch_bounds__(256) k_site_contacts(Group g) {
+  const u32 s = blockIdx.y, L = g.L;
+  SampleState& st = g.st[s];
+  const u64* K = g.node_key + (size_t)s * g.cap_nodes;
+  const u32* P = g.node_pos + (size_t)s * g.cap_nodes;
+  Edge* E = g.edges + (size_t)s * g.cap_edges;
+  u32 cnt[3] = {0, 0, 0};
+  for (u64 i = blockIdx.x * 256ull + threadIdx.x; i < g.LL; i += gridDim.x * 256ull) {
+    const u32 m = (u32)i, y = m / L, x = m - y * L;
+    const u32 right = x + 1 == L ? m + 1 - L : m + 1, down = y + 1 == L ? x : m + L;
+    const u64 km = K[m];
+    const u32 om = P[m] >> 31;
+#pragma unroll
+    for (u32 dir = 0; dir < 2; ++dir) {
+      const u32 b = dir ? down : right;
+      put_edge(g, st, E, 2 * m + dir, tmax(km, K[b]), m, b, dir == 0, dir);
+      if (b != m) {
+        const u32 kind = om != P[b] >> 31 ? 2u : om;
+        cnt[0] += kind == 0;
+        cnt[1] += kind == 1;
+        cnt[2] += kind == 2;
+      }
+    }
+  }
+  contact_counts(st, cnt);
+  if (blockIdx.x == 0 && threadIdx.x == 0) st.n_edges = 2 * (u32)g.LL;
+}
+
+// ---------------------------------------------------------------------
+// Contact graph of the jammed lattice, k >= 2, from the k-mers themselves.
+// The lattice edges (a, a + e), e in {+x, +y}, that leave a k-mer of
+// orientation o, line l, cells [pos, pos + k) are the one past its last cell
+// and the ones from line l to line l + 1.  On line l + 1 lie the parallel
+// k-mers anchored less than k away, and the perpendicular ones that start
+// there (those that came from line l would cross this one); the cell past
+// the end is the first of a parallel k-mer or some cell of a perpendicular
+// one.  Each is read off the anchor bits, a word at a time: about k / 8 words
+// per k-mer, where reading the owners of all cells costs 4 bytes per cell.
+// One edge per pair of k-mers and displacement, its contacts counted by the
+// length of the overlap; a parallel run that passes cell 0 counts as two
+// (runs start anew there).  Only a ring (k = L) beside itself is a contact
+// of a k-mer with itself.
+// ---------------------------------------------------------------------
+__device__ __forceinline__ u32 anchor_bits(const u32* line, u32 a, u32 n) {
+  const u32 w = a >> 5;
+  const u32 v = __funnelshift_r(__ldg(line + w), __ldg(line + w + 1), a & 31u);
+  return n < 32 ? v & ((1u << n) - 1u) : v;
+}
+
+template <int G>
+__global__ void __launch_bounds__(256) k_contacts(Group g, const __grid_constant__ RoundCfg c,
+                                                  RoundPtrs p) {
+  const u32 s = blockIdx.y, L = g.L, k = g.k, tid = threadIdx.x;
+  SampleState& st = g.st[s];
+  const u32 nn = min(st.n_nodes, g.cap_nodes);
+  const size_t nb = (size_t)s * g.cap_nodes;
+  const u32* anchor_node = g.owner + (size_t)s * g.LL;
+  Edge* E = g.edges + (size_t)s * g.cap_edges;
+  const u32 j = tid & (G - 1);
+  constexpr u32 GPB = 256 / G;
+  u32 cnt[3] = {0, 0, 0};
+  for (u32 m = blockIdx.x * GPB + tid / G; m < nn; m += gridDim.x * GPB) {
+    const u32 pk = g.node_pos[nb + m];
+    const u64 key = g.node_key[nb + m];
+    const u32 o = pk >> 31, y = (pk >> 15) & 0x7FFFu, x = pk & 0x7FFFu;
+    const u32 line = o ? x : y, pos = o ? y : x, ln = line + 1 == L ? 0 : line + 1;
+    // contact with the k-mer anchored at (line al, position ap) in the
+    // layout of o, displaced by (along, across) lines of o
+    auto emit = [&](u32 al, u32 ap, u32 along, u32 across, u32 run, bool mixed, u32 copies) {
+      const u32 b = __ldg(anchor_node + (o ? ap * L + al : al * L + ap));
+      const u64 kb = g.node_key[nb + b];
+      if (b != m) cnt[mixed ? 2 : o] += run;
+      const u32 at = atomicAdd(&st.n_edges, copies);
+      for (u32 i = 0; i < copies; ++i)
+        put_edge(g, st, E, at + i, tmax(key, kb), m, b, o ? across : along, o ? along : across);
+    };
+    // parallel k-mers on the next line
+    {
+      const u32 a = ring_sub(pos, k - 1, L);
+      const u32* al = anchor_line(g, c, p, s, o, o, ln);
+      for (u32 w = j; w * 32 < 2 * k - 1; w += G)
+        for (u32 v = anchor_bits(al, a + w * 32, 2 * k - 1 - w * 32); v; v &= v - 1) {
+          const int d = (int)(w * 32 + __ffs(v) - 1) - (int)(k - 1);
+          u32 ap = a + w * 32 + __ffs(v) - 1;
+          while (ap >= L) ap -= L;
+          // cells first .. last of this k-mer touch the other; is cell 0 of
+          // the line among them, other than as the first?
+          const u32 first = d > 0 ? d : 0, len = k - (d < 0 ? -d : d);
+          const u32 to0 = ring_sub(0, pos + first >= L ? pos + first - L : pos + first, L);
+          const bool again = to0 > 0 && to0 < len && !(k == L && d == 0);
+          emit(ln, ap, (u32)d, 1, len, false, again ? 2 : 1);
+        }
+    }
+    // perpendicular k-mers that start on the next line
+    {
+      const u32* al = anchor_line(g, c, p, s, o ^ 1u, o, ln);
+      for (u32 w = j; w * 32 < k; w += G)
+        for (u32 v = anchor_bits(al, pos + w * 32, k - w * 32); v; v &= v - 1) {
+          const u32 i = w * 32 + __ffs(v) - 1;
+          emit(ln, pos + i >= L ? pos + i - L : pos + i, i, 1, 1, true, 1);
+        }
+    }
+    // the cell past the end
+    if (j == G - 1) {
+      const u32 q = pos + k >= L ? pos + k - L : pos + k;
+      if (anchor_bits(anchor_line(g, c, p, s, o, o, line), q, 1)) {
+        emit(line, q, k, 0, 1, false, 1);
+      } else {
+        const u32 a = ring_sub(line, k - 1, L);
+        const u32* al = anchor_line(g, c, p, s, o ^ 1u, o ^ 1u, q);
+        for (u32 w = 0; w * 32 < k; ++w) {
+          const u32 v = anchor_bits(al, a + w * 32, k - w * 32);
+          if (v) {
+            const u32 tt = w * 32 + __ffs(v) - 1;
+            const u32 first = a + tt >= L ? a + tt - L : a + tt;
+            emit(first, q, k, tt - (k - 1), 1, true, 1);
+            break;
+          }
+        }
+      }
+    }
+  }
+  contact_counts(st, cnt);
+}
+
+}  // namespace rsak
