@@ -19,8 +19,8 @@
 #include <vector>
 
 #include "../../include/rsa.h"
-#include "rsa_kernels.cuh"
 #include "rsa_rounds.cuh"
+#include "rsa_search.cuh"
 #include "rsa_config.cuh"
 
 using namespace rsak;
@@ -50,23 +50,28 @@ int fail(int code, const std::string& msg) {
 
 constexpr size_t ALIGN = 256;
 constexpr u32 ROUND_CHECK = 4;   // rounds between host checks once every slice is entered (default)
-constexpr u32 PROBE_CHECK = 4;   // bisection probes between host checks
-constexpr u32 PROBE_CAP = 40;    // rank bisection (<= 31 halvings) plus the initial probe
+constexpr u32 PROBE_CAP = 96;    // a threshold bisection of 64-bit times, at its worst, and the last window
+
+// The loop counters and, behind them, the work counters.
+constexpr size_t READ_BYTES = ALIGN + 4 * WORK_SLOTS * 8;
 
 size_t align_up(size_t v) { return (v + ALIGN - 1) / ALIGN * ALIGN; }
 
 struct Layout {
   size_t fine, block, anch, heads, list, flat, act;   // rounds
-  size_t uf, edges, edges_b, ebkt, nkey_b, nbkt;      // contact graph and search
+  size_t uf, etime, elink, ehist, win;                // contact graph and search
   size_t owner, base, node_key, node_idx, node_pos, rs, st, seeds, counters, work, keys, total;
   size_t bits_bytes;  // fine + block, zeroed together
-  size_t anch_bytes, heads_bytes;
+  size_t anch_bytes, heads_bytes, ehist_bytes;
 };
 
 struct Geometry {
   bool sites;       // k = 1: one pass, no slices
   RoundCfg rc;
   size_t list_cap;  // listed candidates per sample
+  SearchCfg sc;
+  u32 win_pow2;     // sc.win_cap rounded up to a power of two
+  u32 probes;       // probes that bring the window of a large graph to the last
   bool win128;      // shape of the 128-thread window setting (rsa_set_window_threads)
 };
 
@@ -92,8 +97,27 @@ bool window_shape(u32 L, u32 k) {
          k % C == 0 && L / P <= 8 && (P == 4096 || P == 2048);
 }
 
+void plan_search(u32 L, u32 k, Geometry& G) {
+  const u32 cn = cap_nodes_of(L, k), ce = cap_edges_of(L, k);
+  SearchCfg& c = G.sc;
+  c.win_cap = std::min(FIN_EDGES, ce);
+  c.hashed = cn > 2 * FIN_EDGES;
+  c.ids = c.hashed ? 2 * FIN_EDGES : cn;
+  G.win_pow2 = 1;
+  while (G.win_pow2 < c.win_cap) G.win_pow2 <<= 1;
+  // n_c / n_j runs from 0.59 (k = 1) to 0.86 (k = 4096), within 0.04 either
+  // way; an edge is there by then with about the square of that chance
+  const double f = 0.59 + 0.0225 * std::log2((double)k);
+  c.q0 = (u32)(65536 * (f - 0.04) * (f - 0.04));
+  c.q1 = std::min(64000u, (u32)(65536 * (f + 0.04) * (f + 0.04)));
+  // edges per k-mer of capacity: 2 at k = 1, 1.7 at k = 4, 1 from 32 on
+  const double edges = (double)cn * (k == 1 ? 2.0 : k <= 8 ? 1.7 : 1.0) * 0.16 * f;
+  G.probes = ce <= c.win_cap ? 0 : 3 + (u32)std::max(0.0, std::ceil(std::log2(edges / c.win_cap)));
+}
+
 Geometry plan(u32 L, u32 k) {
   Geometry G{};
+  plan_search(L, k, G);
   G.sites = k == 1;
   G.win128 = window_shape(L, k);
   RoundCfg& c = G.rc;
@@ -160,11 +184,11 @@ Layout layout_of(u32 L, u32 k, u32 n, bool with_keys, const Geometry& G) {
   const size_t rounds_end = off;
   off = 0;
   l.uf = take(n * cn * 16);
-  l.edges = take(n * ce * sizeof(Edge));
-  l.edges_b = take(n * ce * sizeof(Edge));
-  l.ebkt = take((size_t)n * (NBKT + 1) * 4);
-  l.nkey_b = take(n * cn * 8);
-  l.nbkt = take((size_t)n * (NBKT + 1) * 4);
+  l.etime = take(n * ce * 8);
+  l.elink = take(n * ce * 16);
+  l.ehist_bytes = G.probes ? (size_t)n * (EHIST + SUB_BINS) * 4 : 0;
+  l.ehist = take(l.ehist_bytes);
+  l.win = take((size_t)n * G.sc.win_cap * sizeof(WinEdge));
   off = std::max(off, rounds_end);
   l.anch_bytes = G.sites ? 0 : (size_t)n * 4 * L * c.WA * 4;
   l.anch = take(l.anch_bytes);
@@ -176,8 +200,8 @@ Layout layout_of(u32 L, u32 k, u32 n, bool with_keys, const Geometry& G) {
   l.rs = take(G.sites ? 0 : (size_t)n * sizeof(RoundState));
   l.st = take((size_t)n * sizeof(SampleState));
   l.seeds = take((size_t)n * 8);
-  l.counters = take(64);
-  l.work = take(4 * WORK_SLOTS * 8);
+  l.counters = take(READ_BYTES);  // loop counters, then the work counters
+  l.work = l.counters + ALIGN;
   l.keys = take(with_keys ? 2 * LL * 8 : 0);
   l.total = off;
   return l;
@@ -192,12 +216,12 @@ int set_error(int code, const std::string& msg) { return fail(code, msg); }
 }  // namespace rsa_detail
 
 enum Kind {
-  KD_INIT, KD_DENSE, KD_PICK, KD_RESOLVE, KD_REFILL, KD_CHECK, KD_SITES, KD_EDGES, KD_BUCKET,
-  KD_SEARCH_INIT, KD_PROBE_COPY, KD_PROBE, KD_DECIDE, KD_COUNT
+  KD_INIT, KD_DENSE, KD_PICK, KD_RESOLVE, KD_REFILL, KD_CHECK, KD_SITES, KD_EDGES,
+  KD_SEARCH_INIT, KD_PROBE_COPY, KD_PROBE, KD_COLLECT, KD_FINISH, KD_RANK, KD_COUNT
 };
 const char* const kKindNames[KD_COUNT] = {
     "k_init", "k_dense", "k_pick", "k_resolve", "k_refill", "k_round_check", "k_sites", "k_edges",
-    "k_bucket", "k_search_init", "k_probe_copy", "k_probe", "k_search_decide"};
+    "k_search_init", "k_probe_copy", "k_probe", "k_collect", "k_finish", "k_rank"};
 
 // Optional per-kernel timing with CUDA events recorded around each launch
 // on the launch stream, plus launch counts (always kept).
@@ -225,7 +249,7 @@ struct rsa {
   u32 last_n = 0;
   bool with_keys = false;
   cudaStream_t stream = nullptr;
-  u32* h_counter = nullptr;  // pinned, 64 bytes: loop counters, configuration bits
+  u32* h_counter = nullptr;  // pinned, READ_BYTES: loop and work counters, configuration bits
   unsigned long long work[4] = {0, 0, 0, 0};  // accumulated round-pass work
   int device = -1;
   int sm_count = 0;
@@ -235,9 +259,9 @@ struct rsa {
   // replayed on the run's stream
   bool use_graphs = true;
   cudaStream_t cap_stream = nullptr;
-  // chunks the previous run needed before its samples were done: the next
-  // run launches that many before its first device->host check
-  u32 round_chunks_hint = 0, probe_chunks_hint = 1;
+  // rounds after the last slice in the run's first graph: more once a run
+  // has needed more
+  u32 drain = 3;
   u32 round_check = ROUND_CHECK;  // greedy rounds per graph chunk / host check
   // test-only lowered caps of the device loops (0 = default; rsa_test_caps)
   u32 t_round = 0, t_uf = 0, t_probe = 0, t_edges = 0;
@@ -246,9 +270,9 @@ struct rsa {
     const void* ws = nullptr;
     u32 n = 0;
     bool keys = false;
-    u32 caps[5] = {0, 0, 0, 0, 0};  // caps and rounds per chunk in the graph
+    u32 caps[6] = {0, 0, 0, 0, 0, 0};  // caps, rounds per chunk and after the last slice
     unsigned long long launches[32] = {};
-  } g_main, g_round, g_probe;
+  } g_main, g_round, g_search, g_probe;
 };
 
 namespace {
@@ -298,12 +322,11 @@ Group group_of(rsa_t* h, u32 n) {
   g.node_key = reinterpret_cast<u64*>(b + l.node_key);
   g.node_idx = reinterpret_cast<u32*>(b + l.node_idx);
   g.node_pos = reinterpret_cast<u32*>(b + l.node_pos);
-  g.edges_b = reinterpret_cast<Edge*>(b + l.edges_b);
-  g.ebkt = reinterpret_cast<u32*>(b + l.ebkt);
-  g.nkey_b = reinterpret_cast<u64*>(b + l.nkey_b);
-  g.nbkt = reinterpret_cast<u32*>(b + l.nbkt);
   g.uf = reinterpret_cast<u64*>(b + l.uf);
-  g.edges = reinterpret_cast<Edge*>(b + l.edges);
+  g.etime = reinterpret_cast<u64*>(b + l.etime);
+  g.elink = reinterpret_cast<uint4*>(b + l.elink);
+  g.ehist = l.ehist_bytes ? reinterpret_cast<u32*>(b + l.ehist) : nullptr;
+  g.win = reinterpret_cast<WinEdge*>(b + l.win);
   g.st = reinterpret_cast<SampleState*>(b + l.st);
   g.work = reinterpret_cast<u64*>(b + l.work);
   return g;
@@ -361,10 +384,12 @@ int launch_check(const char* what) {
   return 0;
 }
 
-int read_counter(rsa_t* h, u32* dev_counter, u32* out) {
-  CUDA_TRY(cudaMemcpyAsync(h->h_counter, dev_counter, 4, cudaMemcpyDeviceToHost, h->stream));
+int read_counters(rsa_t* h, u32* active, u32* open) {
+  const char* from = static_cast<const char*>(h->ws) + h->lay.counters;
+  CUDA_TRY(cudaMemcpyAsync(h->h_counter, from, READ_BYTES, cudaMemcpyDeviceToHost, h->stream));
   CUDA_TRY(cudaStreamSynchronize(h->stream));
-  *out = *h->h_counter;
+  *active = h->h_counter[0];
+  *open = h->h_counter[1];
   return 0;
 }
 
@@ -381,7 +406,7 @@ int run_chunk(rsa_t* h, rsa_t::GraphSlot& gs, cudaStream_t stream, u32 n, B body
     body(stream);
     return launch_check("chunk launches");
   }
-  const u32 caps[5] = {h->t_round, h->t_uf, h->t_probe, h->t_edges, h->round_check};
+  const u32 caps[6] = {h->t_round, h->t_uf, h->t_probe, h->t_edges, h->round_check, h->drain};
   if (!(gs.exec && gs.ws == h->ws && gs.n == n && gs.keys == h->with_keys &&
         std::memcmp(gs.caps, caps, sizeof(caps)) == 0)) {
     drop_graph(gs);
@@ -422,7 +447,7 @@ int run_impl(rsa_t* h, const uint64_t* seeds, u32 n, const uint64_t* keys, cudaS
   NvtxRange run_range("rsa_run");
   int rc;
   CUDA_TRY(cudaGetDevice(&h->device));
-  if (!h->h_counter) CUDA_TRY(cudaMallocHost(&h->h_counter, 64));
+  if (!h->h_counter) CUDA_TRY(cudaMallocHost(&h->h_counter, READ_BYTES));
   h->with_keys = keys != nullptr;
   if ((rc = ensure_workspace(h, n, h->with_keys))) return rc;
   h->stream = stream;
@@ -489,8 +514,7 @@ int run_impl(rsa_t* h, const uint64_t* seeds, u32 n, const uint64_t* keys, cudaS
   // the whole deposition: every slice once, and three more rounds for the
   // candidates left undecided by the last ones
   auto deposit = [&](cudaStream_t st) {
-    check(cudaMemsetAsync(b + l.counters, 0, 64, st));
-    check(cudaMemsetAsync(b + l.work, 0, 4 * WORK_SLOTS * 8, st));
+    check(cudaMemsetAsync(b + l.counters, 0, READ_BYTES, st));
     launch(h, KD_INIT, k_init, init_grid, dim3(128), 0, st, g, (const u64*)d_seeds);
     if (G.sites) {
       launch(h, KD_SITES, k_sites, grid_x((LL + 255) / 256, 32), dim3(256), 0, st, g);
@@ -507,7 +531,7 @@ int run_impl(rsa_t* h, const uint64_t* seeds, u32 n, const uint64_t* keys, cudaS
       launch(h, KD_DENSE, k_dense<false>, dg, dim3(RD_THREADS), 0, st, g, c, rp);
     for (u32 t = 0; t < c.nlev; ++t) round(st);
     refill(st);
-    for (u32 t = c.nlev; t <= c.lzmax + 3; ++t) round(st);
+    for (u32 t = c.nlev; t <= c.lzmax + h->drain; ++t) round(st);
     count_active(st);
   };
   // a sample that is not through yet: more rounds
@@ -516,73 +540,76 @@ int run_impl(rsa_t* h, const uint64_t* seeds, u32 n, const uint64_t* keys, cudaS
     for (u32 i = 0; i < h->round_check; ++i) round(st);
     count_active(st);
   };
-  {
-    NvtxRange rounds_range("deposition");
-    if ((rc = run_chunk(h, h->g_main, stream, n, deposit))) return rc;
-    if (body_rc) return fail(body_rc, "round launches failed");
-    for (u32 chunks = 0; !G.sites;) {
-      for (; chunks < h->round_chunks_hint; ++chunks)
-        if ((rc = run_chunk(h, h->g_round, stream, n, more_rounds))) return rc;
-      if (body_rc) return fail(body_rc, "round launches failed");
-      u32 active;
-      if ((rc = read_counter(h, d_counter, &active))) return rc;
-      if (active == 0) break;
-      h->round_chunks_hint = chunks + 1;
-    }
-  }
-  NvtxRange wrap_range("contact graph and first-wrap search");
-  // contact graph of the jammed lattice
-  if (G.sites) {
-    launch(h, KD_EDGES, k_site_contacts, grid_x((LL + 255) / 256, 32), dim3(256), 0, stream, g);
-  } else {
-    // lanes per k-mer: 1 for lines of a few words (L = 1024, k = 32, 1000
-    // samples: 2.0 ms, with 4 lanes 2.8), 4 for longer ones (L = 32768,
-    // k = 4096, 4 samples: 1.2 ms, with 1 lane 1.8, with 32 lanes 2.7)
-    const u32 el = h->k <= 64 ? 1 : 4;
-    const dim3 eg = grid_x(((u64)g.cap_nodes * el + 255) / 256, 32);
-    if (el == 1)
-      launch(h, KD_EDGES, k_contacts<1>, eg, dim3(256), 0, stream, g, c, rp);
-    else
-      launch(h, KD_EDGES, k_contacts<4>, eg, dim3(256), 0, stream, g, c, rp);
-  }
-  if ((rc = launch_check("k_edges"))) return rc;
-  launch(h, KD_BUCKET, k_bucket, dim3(n), dim3(1024), 0, stream, g);
-  // bisection for the first wrap
-  launch(h, KD_SEARCH_INIT, k_search_init, dim3((n + 127) / 128), dim3(128), 0, stream, g);
-  {
-    u32 bx = (u32)std::min<u64>(((u64)g.cap_nodes + 255) / 256, 1024);
-    launch(h, KD_SEARCH_INIT, k_uf_identity, dim3(bx, n), dim3(256), 0, stream, g);
-  }
-  if ((rc = launch_check("search init"))) return rc;
-  // enough blocks per sample to fill the GPU across the batch, no more
-  const u64 per_sample = std::max<u64>(8, 16384 / n);
-  const u32 copy_bx = (u32)std::min<u64>(((u64)g.cap_nodes + 255) / 256, per_sample);
-  const u32 probe_bx = (u32)std::min<u64>(((u64)g.cap_edges + 255) / 256, per_sample);
+  const SearchCfg& sc = G.sc;
+  // blocks per sample over its k-mers and its edges
+  const dim3 node_grid = grid_x(((u64)g.cap_nodes + 255) / 256, 32);
+  const dim3 edge_grid = grid_x(((u64)g.cap_edges + 1023) / 1024, 16);
+  const size_t fin_smem = finish_smem(sc, G.win_pow2);
+  // the same limit for every shape: handles run on several threads at once
+  CUDA_TRY(cudaFuncSetAttribute(k_finish, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)FIN_SMEM_MAX));
   auto probes = [&](cudaStream_t st) {
-    for (u32 i = 0; i < PROBE_CHECK; ++i) {
-      if (cudaMemsetAsync(d_counter + 1, 0, 4, st) != cudaSuccess) body_rc = RSA_ECUDA;
-      launch(h, KD_PROBE_COPY, k_probe_copy, dim3(copy_bx, n), dim3(256), 0, st, g);
-      launch(h, KD_PROBE, k_probe, dim3(probe_bx, n), dim3(256), 0, st, g);
-      launch(h, KD_DECIDE, k_search_decide, dim3(n), dim3(256), 0, st, g, probe_cap,
-             d_counter + 1);
+    check(cudaMemsetAsync(d_counter + 1, 0, 4, st));
+    for (u32 i = 0; i < G.probes; ++i) {
+      launch(h, KD_PROBE_COPY, k_probe_copy, node_grid, dim3(256), 0, st, g);
+      launch(h, KD_PROBE, k_probe, edge_grid, dim3(256), 0, st, g, sc, probe_cap);
     }
+    launch(h, KD_COLLECT, k_collect, edge_grid, dim3(256), 0, st, g, sc);
+    launch(h, KD_FINISH, k_finish, dim3(n), dim3(FIN_THREADS), fin_smem, st, g, sc, G.win_pow2,
+           probe_cap, d_counter + 1);
+    launch(h, KD_RANK, k_rank, node_grid, dim3(256), 0, st, g);
   };
-  for (u32 chunks = 0; chunks * PROBE_CHECK < probe_cap + PROBE_CHECK;) {
-    const u32 burst = chunks == 0 ? h->probe_chunks_hint : 1;
-    for (u32 i = 0; i < burst; ++i, ++chunks)
-      if ((rc = run_chunk(h, h->g_probe, stream, n, probes))) return rc;
-    if (body_rc) return fail(body_rc, "probe launches failed");
-    u32 open;
-    if ((rc = read_counter(h, d_counter + 1, &open))) return rc;
-    if (open == 0) {
-      h->probe_chunks_hint = chunks;
-      break;
+  // contact graph of the jammed lattice and the search for the first wrap
+  auto search = [&](cudaStream_t st) {
+    if (l.ehist_bytes) check(cudaMemsetAsync(b + l.ehist, 0, l.ehist_bytes, st));
+    launch(h, KD_SEARCH_INIT, k_graph_init, init_grid, dim3(128), 0, st, g,
+           (const u32*)d_counter);
+    if (G.sites) {
+      launch(h, KD_EDGES, k_site_contacts, grid_x((LL + 255) / 256, 32), dim3(256), 0, st, g);
+    } else {
+      // lanes per k-mer: 1 for lines of a few words (L = 1024, k = 32, 1000
+      // samples: 2.0 ms, with 4 lanes 2.8), 4 for longer ones (L = 32768,
+      // k = 4096, 4 samples: 1.2 ms, with 1 lane 1.8, with 32 lanes 2.7)
+      const u32 el = h->k <= 64 ? 1 : 4;
+      const dim3 eg = grid_x(((u64)g.cap_nodes * el + 255) / 256, 32);
+      if (el == 1)
+        launch(h, KD_EDGES, k_contacts<1>, eg, dim3(256), 0, st, g, c, rp);
+      else
+        launch(h, KD_EDGES, k_contacts<4>, eg, dim3(256), 0, st, g, c, rp);
     }
+    launch(h, KD_SEARCH_INIT, k_search_init, dim3(n), dim3(256), 0, st, g, sc);
+    probes(st);
+  };
+  auto whole = [&](cudaStream_t st) {
+    deposit(st);
+    search(st);
+  };
+  u32 active = 0, open = 0;
+  if ((rc = run_chunk(h, h->g_main, stream, n, whole))) return rc;
+  if (body_rc) return fail(body_rc, "launches failed");
+  if ((rc = read_counters(h, &active, &open))) return rc;
+  if (active) {
+    // the search of the first graph was left out
+    NvtxRange rounds_range("more rounds");
+    if (h->drain < 16) h->drain += 2;
+    while (active) {
+      if ((rc = run_chunk(h, h->g_round, stream, n, more_rounds))) return rc;
+      if (body_rc) return fail(body_rc, "round launches failed");
+      if ((rc = read_counters(h, &active, &open))) return rc;
+    }
+    if ((rc = run_chunk(h, h->g_search, stream, n, search))) return rc;
+    if (body_rc) return fail(body_rc, "search launches failed");
+    if ((rc = read_counters(h, &active, &open))) return rc;
+  }
+  while (open) {
+    NvtxRange wrap_range("more probes");
+    if ((rc = run_chunk(h, h->g_probe, stream, n, probes))) return rc;
+    if (body_rc) return fail(body_rc, "probe launches failed");
+    if ((rc = read_counters(h, &active, &open))) return rc;
   }
   // round-pass work counters of this run (for throughput accounting)
-  unsigned long long wk[4 * WORK_SLOTS];
-  CUDA_TRY(cudaMemcpyAsync(wk, b + l.work, sizeof(wk), cudaMemcpyDeviceToHost, stream));
-  CUDA_TRY(cudaStreamSynchronize(stream));
+  const unsigned long long* wk =
+      reinterpret_cast<const unsigned long long*>(reinterpret_cast<const char*>(h->h_counter) + ALIGN);
   for (u32 i = 0; i < 4 * WORK_SLOTS; ++i) h->work[i / WORK_SLOTS] += wk[i];
   return 0;
 }
@@ -689,8 +716,20 @@ int configuration(rsa_t* h, uint32_t sample, uint32_t m, uint32_t* counts, uint3
   Group g = group_of(h, h->last_n);
   const u32 bx = (u32)std::min<u64>(((u64)g.cap_edges + 255) / 256, 2048);
   const u32 nb = (u32)std::min<u64>(((u64)nj + 256) / 256, 1024);
-  k_select_key<<<1, 1024, 0, stream>>>(g, sample, m);
-  k_cfg_init<<<nb, 256, 0, stream>>>(g, sample);
+  const bool at_wrap = m == st[sample].nc;
+  if (!at_wrap) {
+    u64* keys_out = cfg_uf(g, sample);
+    if (g.cap_nodes >= EHIST) {
+      u32* bins = cfg_size(g, sample);
+      const u32 kb = std::min(nb, 152u);
+      CUDA_TRY(cudaMemsetAsync(bins, 0, (EHIST + 4) * 4, stream));
+      k_key_bins<<<kb, 256, 0, stream>>>(g, sample, m, bins);
+      k_key_select<<<kb, 256, 0, stream>>>(g, sample, m, bins, keys_out);
+    } else {
+      k_key_select<<<1, 256, 0, stream>>>(g, sample, m, nullptr, keys_out);
+    }
+  }
+  k_cfg_init<<<nb, 256, 0, stream>>>(g, sample, at_wrap);
   k_cfg_union<<<bx, 256, 0, stream>>>(g, sample);
   if (counts) {
     k_cfg_count<<<nb, 256, 0, stream>>>(g, sample);
@@ -702,9 +741,8 @@ int configuration(rsa_t* h, uint32_t sample, uint32_t m, uint32_t* counts, uint3
   CUDA_TRY(cudaMemcpyAsync(h->h_counter + 12, b + so + offsetof(SampleState, wdirs), 4,
                            cudaMemcpyDeviceToHost, stream));
   if (counts)
-    CUDA_TRY(cudaMemcpyAsync(counts,
-                             b + h->lay.edges + (size_t)sample * g.cap_edges * sizeof(Edge),
-                             ((size_t)m + 1) * sizeof(uint32_t), cudaMemcpyDeviceToHost, stream));
+    CUDA_TRY(cudaMemcpyAsync(counts + 1, cfg_hist(g, sample), (size_t)m * sizeof(uint32_t),
+                             cudaMemcpyDeviceToHost, stream));
   CUDA_TRY(cudaStreamSynchronize(stream));
   const u32 w = h->h_counter[12];
   if (w & CFG_CAPPED) return fail(RSA_ETIMEOUT, "union-find walk cap reached");
@@ -787,7 +825,7 @@ int rsa_run_static(uint32_t L, uint32_t k, const uint64_t* seeds, uint32_t n, ui
   h.use_graphs = false;  // plain launches only: nothing is created or allocated
   h.bound_ptr = ws;  // the run's buffers (all re-initialised by the run) live here
   h.bound_bytes = STATIC_WS_BYTES;
-  alignas(8) u32 counter[16] = {};  // pageable host words for the loop checks
+  alignas(8) u32 counter[READ_BYTES / 4] = {};  // pageable host words for the loop checks
   h.h_counter = counter;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   rc = run_impl(&h, seeds, n, nullptr, st);
@@ -924,8 +962,7 @@ int rsa_test_caps(rsa_t* h, uint32_t round_cap, uint32_t uf_steps, uint32_t prob
 int rsa_set_rounds_per_check(rsa_t* h, uint32_t rounds) {
   if (!h) return fail(RSA_EINVAL, "null handle");
   if (rounds < 1 || rounds > 64) return fail(RSA_EINVAL, "rounds per check must be in 1 .. 64");
-  if (rounds != h->round_check) h->round_chunks_hint = 0;
-  h->round_check = rounds;
+    h->round_check = rounds;
   return 0;
 }
 
@@ -982,6 +1019,7 @@ void rsa_destroy(rsa_t* h) {
   if (!h) return;
   drop_graph(h->g_main);
   drop_graph(h->g_round);
+  drop_graph(h->g_search);
   drop_graph(h->g_probe);
   if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
   for (cudaEvent_t e : h->prof.pool) cudaEventDestroy(e);

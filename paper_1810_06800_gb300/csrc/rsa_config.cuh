@@ -10,9 +10,9 @@
 // The k-mers tried first are the ones with the smallest keys, so the first m
 // accepted k-mers are the nodes with key <= T_m, the m-th smallest node key,
 // and the lattice edges among them are the contact-graph edges with time
-// (the larger key of their two ends) <= T_m.  One pass of the bisection
-// machinery at that threshold gives both answers:
-//   k_select_key   T_m by an 8-bit radix select over the node keys;
+// (the larger key of their two ends) <= T_m:
+//   k_key_bins, k_key_select   T_m: a histogram of the keys over all blocks,
+//                  then the keys of one bin and a radix select among them;
 //   k_cfg_init     identity union-find, zero sizes and histogram;
 //   k_cfg_union    union the edges with time <= T_m; an edge that closes a
 //                  cycle of non-zero winding adds its directions;
@@ -22,90 +22,172 @@
 // cycle of the clusters, so "some closed cycle has a != 0" is "the clusters
 // wind along x", whatever order the edges are united in.
 // Scratch (the sample's search state is no longer needed): union-find words
-// in the first half of its uf slot, sizes (u32) in the second half, the
-// histogram (u32) in its unsorted edge array.
+// in the first half of its uf slot; sizes (u32) in the third quarter and the
+// histogram (u32, entry s - 1 for size s) in the fourth; for the select, the
+// key bins in the second half and the keys of one bin in the first.
 #pragma once
-#include "rsa_kernels.cuh"
+#include "rsa_search.cuh"
 
 namespace rsak {
 
 constexpr u32 CFG_CAPPED = 1u << 31;  // wdirs bit: a union-find walk hit its cap
 
-__device__ __forceinline__ u64* cfg_uf(const Group& g, u32 s) {
+__host__ __device__ __forceinline__ u64* cfg_uf(const Group& g, u32 s) {
   return g.uf + (size_t)s * 2 * g.cap_nodes;
 }
-__device__ __forceinline__ u32* cfg_size(const Group& g, u32 s) {
+__host__ __device__ __forceinline__ u32* cfg_size(const Group& g, u32 s) {
   return reinterpret_cast<u32*>(g.uf + ((size_t)s * 2 + 1) * g.cap_nodes);
 }
-__device__ __forceinline__ u32* cfg_hist(const Group& g, u32 s) {
-  return reinterpret_cast<u32*>(g.edges + (size_t)s * g.cap_edges);
+__host__ __device__ __forceinline__ u32* cfg_hist(const Group& g, u32 s) {
+  return cfg_size(g, s) + g.cap_nodes;
 }
 
-// T_m (1 <= m <= n_j) into st.sel: eight passes, each fixing the next 8 bits
-// of the answer from a histogram of the keys that share the bits fixed so far.
-__global__ void __launch_bounds__(1024) k_select_key(Group g, u32 s, u32 m) {
+// Keys per time_bin; the last block finds the bin that holds rank m.  bins:
+// EHIST + 4 words, zero before; bins[EHIST ..]: ticket, bin, rank in it, keys
+// gathered.
+__global__ void __launch_bounds__(256) k_key_bins(Group g, u32 s, u32 m, u32* bins) {
+  __shared__ u32 h[EHIST];
+  __shared__ u32 part[256];
+  __shared__ u32 last_sh;
+  const u32 tid = threadIdx.x;
+  const u32 nn = min(g.st[s].n_nodes, g.cap_nodes);
+  const u64* K = g.node_key + (size_t)s * g.cap_nodes;
+  for (u32 i = tid; i < EHIST; i += 256) h[i] = 0;
+  __syncthreads();
+  for (u32 i = blockIdx.x * 256 + tid; i < nn; i += gridDim.x * 256)
+    atomicAdd(&h[time_bin(K[i])], 1u);
+  __syncthreads();
+  for (u32 i = tid; i < EHIST; i += 256)
+    if (h[i]) atomicAdd(&bins[i], h[i]);
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) last_sh = atomicAdd(&bins[EHIST], 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last_sh) return;
+  __threadfence();
+  constexpr u32 PER = EHIST / 256;
+  u32 sum = 0;
+  for (u32 i = 0; i < PER; ++i) sum += __ldcg(bins + tid * PER + i);
+  part[tid] = sum;
+  __syncthreads();
+  for (u32 d = 1; d < 256; d <<= 1) {
+    const u32 o = tid >= d ? part[tid - d] : 0u;
+    __syncthreads();
+    part[tid] += o;
+    __syncthreads();
+  }
+  u32 a = part[tid] - sum;
+  for (u32 i = 0; i < PER; ++i) {
+    const u32 v = __ldcg(bins + tid * PER + i);
+    if (a < m && m <= a + v) {
+      bins[EHIST + 1] = tid * PER + i;
+      bins[EHIST + 2] = m - a;
+    }
+    a += v;
+  }
+  if (tid == 0) {
+    bins[EHIST] = 0;
+    bins[EHIST + 3] = 0;
+  }
+}
+
+// The keys of that bin into `out`; the last block selects the one of the
+// rank, T_m, into st.sel: eight passes, each fixing the next 8 bits of the
+// answer from a histogram of the keys that share the bits fixed so far.
+// Without bins, one block selects the key of rank m from all.
+__global__ void __launch_bounds__(256) k_key_select(Group g, u32 s, u32 m, u32* bins, u64* out) {
   __shared__ u32 hist[256];
   __shared__ u64 pre_sh;
-  __shared__ u32 rank_sh;
+  __shared__ u32 rank_sh, last_sh;
+  const u32 tid = threadIdx.x;
   SampleState& st = g.st[s];
   const u32 nn = min(st.n_nodes, g.cap_nodes);
-  const u64* K = g.node_key + (size_t)s * g.cap_nodes;
-  u64 pre = 0, mask = 0;
-  u32 rank = m;
-  for (int shift = 56; shift >= 0; shift -= 8) {
-    for (u32 i = threadIdx.x; i < 256; i += blockDim.x) hist[i] = 0;
+  const u64* from = g.node_key + (size_t)s * g.cap_nodes;
+  u32 cnt = nn, rank = m;
+  if (bins) {
+    const u32 bin = bins[EHIST + 1];
+    for (u32 i = blockIdx.x * 256 + tid; i < nn; i += gridDim.x * 256) {
+      const u64 k = from[i];
+      if (time_bin(k) == bin) out[atomicAdd(&bins[EHIST + 3], 1u)] = k;
+    }
+    __threadfence();
     __syncthreads();
-    for (u32 i = threadIdx.x; i < nn; i += blockDim.x) {
-      const u64 kk = K[i];
+    if (tid == 0) last_sh = atomicAdd(&bins[EHIST], 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last_sh) return;
+    __threadfence();
+    cnt = __ldcg(bins + EHIST + 3);
+    rank = bins[EHIST + 2];
+    from = out;
+  }
+  u64 pre = 0, mask = 0;
+  for (int shift = 56; shift >= 0; shift -= 8) {
+    hist[tid] = 0;
+    __syncthreads();
+    for (u32 i = tid; i < cnt; i += 256) {
+      const u64 kk = __ldcg(from + i);
       if ((kk & mask) == pre) atomicAdd(&hist[(u32)(kk >> shift) & 255u], 1u);
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-      u32 d = 0, below = 0;
-      while (d < 255 && below + hist[d] < rank) below += hist[d++];
-      rank_sh = rank - below;
-      pre_sh = pre | ((u64)d << shift);
+    // inclusive prefix of the 256 counts by the first warp
+    if (tid < 32) {
+      u32 v[8], sum = 0;
+      for (u32 i = 0; i < 8; ++i) { v[i] = hist[tid * 8 + i]; sum += v[i]; }
+      u32 inc = sum;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const u32 o = __shfl_up_sync(FULL, inc, d);
+        if ((int)tid >= d) inc += o;
+      }
+      u32 a = inc - sum;
+      for (u32 i = 0; i < 8; ++i) {
+        if (a < rank && rank <= a + v[i]) {
+          rank_sh = rank - a;
+          pre_sh = pre | ((u64)(tid * 8 + i) << shift);
+        }
+        a += v[i];
+      }
     }
     __syncthreads();
     rank = rank_sh;
     pre = pre_sh;
     mask |= 255ull << shift;
-    __syncthreads();
   }
-  if (threadIdx.x == 0) {
-    st.sel = pre;
-    st.wdirs = 0;
-  }
+  if (tid == 0) st.sel = pre;
 }
 
-__global__ void k_cfg_init(Group g, u32 s) {
-  const u32 nn = min(g.st[s].n_nodes, g.cap_nodes);
+// at_wrap: the configuration of the first wrap, T_m = T_c.
+__global__ void k_cfg_init(Group g, u32 s, bool at_wrap) {
+  SampleState& st = g.st[s];
+  const u32 nn = min(st.n_nodes, g.cap_nodes);
   u64* W = cfg_uf(g, s);
   u32* size = cfg_size(g, s);
   u32* hist = cfg_hist(g, s);
-  for (u32 m = blockIdx.x * blockDim.x + threadIdx.x; m <= nn; m += gridDim.x * blockDim.x) {
-    if (m < nn) {
-      W[m] = uf_pack(m, 0, 0);
-      size[m] = 0;
-    }
+  for (u32 m = blockIdx.x * blockDim.x + threadIdx.x; m < nn; m += gridDim.x * blockDim.x) {
+    W[m] = uf_pack(m, 0, 0);
+    size[m] = 0;
     hist[m] = 0;
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    st.wdirs = 0;
+    if (at_wrap) st.sel = st.tc;
   }
 }
 
-__global__ void k_cfg_union(Group g, u32 s) {
+__global__ void __launch_bounds__(256) k_cfg_union(Group g, u32 s) {
   SampleState& st = g.st[s];
   const u64 T = st.sel;
-  const u32* eb = g.ebkt + (size_t)s * (NBKT + 1);
-  const u32 e1 = eb[(u32)(T >> 56) + 1];
-  const Edge* E = g.edges_b + (size_t)s * g.cap_edges;
+  const u32 ne = min(st.n_edges, g.edge_limit);
+  const u64* E = g.etime + (size_t)s * g.cap_edges;
+  const uint4* K = g.elink + (size_t)s * g.cap_edges;
   u64* W = cfg_uf(g, s);
   bool capped = false;
   u32 dirs = 0;
-  for (u32 i = blockIdx.x * blockDim.x + threadIdx.x; i < e1; i += gridDim.x * blockDim.x) {
-    const Edge e = E[i];
-    if (e.time > T) continue;
+  for (u32 i = blockIdx.x * blockDim.x + threadIdx.x; i < ne; i += gridDim.x * blockDim.x) {
+    if (E[i] > T) continue;
+    const uint4 e = K[i];
     u32 mis = 0;
-    if (uf_union(W, e.m1, e.m2, e.dxy, &capped, g.uf_cap, &mis))
+    if (uf_union(W, e.x, e.y, e.z, &capped, g.uf_cap, &mis))
       dirs |= ((mis & 0xFFFFu) ? 1u : 0u) | ((mis >> 16) ? 2u : 0u);
   }
   if (capped) dirs |= CFG_CAPPED;
@@ -113,7 +195,7 @@ __global__ void k_cfg_union(Group g, u32 s) {
   if ((threadIdx.x & 31) == 0 && dirs) atomicOr(&st.wdirs, dirs);
 }
 
-__global__ void k_cfg_count(Group g, u32 s) {
+__global__ void __launch_bounds__(256) k_cfg_count(Group g, u32 s) {
   SampleState& st = g.st[s];
   const u64 T = st.sel;
   const u32 nn = min(st.n_nodes, g.cap_nodes);
@@ -136,7 +218,7 @@ __global__ void k_cfg_hist(Group g, u32 s) {
   u32* hist = cfg_hist(g, s);
   for (u32 m = blockIdx.x * blockDim.x + threadIdx.x; m < nn; m += gridDim.x * blockDim.x) {
     const u32 c = size[m];
-    if (c) atomicAdd(&hist[c], 1u);
+    if (c) atomicAdd(&hist[c - 1], 1u);
   }
 }
 

@@ -36,7 +36,8 @@ constexpr unsigned FULL = 0xFFFFFFFFu;
 // Work counters are spread over WORK_SLOTS addresses (by block index), so that
 // many blocks adding to one counter do not queue on a single L2 address.
 constexpr u32 WORK_SLOTS = 32;
-constexpr u32 NBKT = 256;  // time buckets (top 8 bits of a priority)
+constexpr u32 EHIST = 2048;  // bins of time_bin
+
 
 // status bits (per sample), mapped to RSA_E* codes by the host
 constexpr u32 ST_NODE_OVF = 1u;     // more accepted k-mers than L^2/k (bug)
@@ -54,26 +55,22 @@ __device__ __forceinline__ u64 mix64(u64 z) {
   return z ^ (z >> 31);
 }
 
-struct Edge {          // one contact between two k-mers (24 bytes)
-  u64 time;            // max of the two k-mers' priorities
-  u32 m1, m2;          // node ids (acceptance order)
-  u32 dxy;             // lifted anchor(m2) - anchor(m1): low 16 dx, high 16 dy
-  u32 pad;
-};
-
-struct SampleState {   // one per sample, 128 bytes
+struct SampleState {   // one per sample
   u32 n_nodes, n_edges, rounds, probes;
-  u32 done, alive, status, wrap;
-  u64 lo, hi, mid;
-  u32 cnt_lo, cnt_hi, cnt_mid, lo_valid;
-  u32 cur, sdone, nc, hi_ok;
+  u32 done, status, sdone, wrap;            // wrap: the current probe closed one
+  u64 lo, hi, mid, next_mid;                // window (lo, hi] of the search
+  u32 cur, hi_ok, ready, step;
+  u32 count_a, count_b, in_win, ticket;     // edges of (lo, mid], (mid, hi], (lo, hi]
+  u32 win_n, ranked, nc, wdirs;             // wdirs: configuration pass, winding bits
   u32 contacts_x, contacts_y, contacts_xy;  // lattice edges between different
                                             // k-mers: both H, both V, mixed
-  u32 wdirs;                                // configuration pass: winding bits
+  u32 pad;
+  u64 tc;                                   // priority of the k-mer that first wraps
   u64 sel;                                  // configuration pass: m-th key
-  u32 pad[4];
 };
-static_assert(sizeof(SampleState) == 128, "SampleState is 128 bytes");
+static_assert(sizeof(SampleState) == 144, "SampleState is 144 bytes");
+
+struct WinEdge;
 
 struct Group {         // one batch of samples sharing (L, k)
   u32 L, k, n;
@@ -89,16 +86,23 @@ struct Group {         // one batch of samples sharing (L, k)
   u32* node_idx;       // [n][cap_nodes]  accepted candidate idx
   u32* node_pos;       // [n][cap_nodes]  o << 31 | y0 << 15 | x0 of the anchor
   u64* uf;             // [n][2][cap_nodes] union-find words
-  Edge* edges;         // [n][cap_edges]
-  Edge* edges_b;       // [n][cap_edges] edges grouped by time >> 56
-  u32* ebkt;           // [n][NBKT + 1] bucket offsets into edges_b
-  u64* nkey_b;         // [n][cap_nodes] node keys grouped by key >> 56
-  u32* nbkt;           // [n][NBKT + 1] bucket offsets into nkey_b
+  u64* etime;          // [n][cap_edges] contact edges: max of the two priorities,
+  uint4* elink;        // [n][cap_edges] and node ids, lifted anchor(m2) - anchor(m1)
+                       //                as 16-bit dx, dy
+  u32* ehist;          // [n][EHIST + SUB_BINS] edges per time_bin, per sub-bin of the
+                       //                window; null where no graph can be large
+  WinEdge* win;        // [n][win_cap]
   SampleState* st;     // [n]
   u64* work;           // [4][WORK_SLOTS] work counters of the deposition: candidates
                        //     hashed by the first pass, list entries tested, active
                        //     candidates resolved, k-mers accepted
 };
+
+// Monotone bin of a priority: 32 bins per power of two.
+__device__ __forceinline__ u32 time_bin(u64 t) {
+  const u32 lz = (u32)__clzll((long long)(t | 1));
+  return (63 - lz) * 32 + (lz == 63 ? 0u : (u32)((t << (lz + 1)) >> 59));
+}
 
 // Add v to work counter c (slot chosen by the block index).
 __device__ __forceinline__ void work_add(const Group& g, u32 c, u64 v) {

@@ -40,7 +40,7 @@
 // block line, and only the lines at its two ends their own: 2^bs + k / 2^bs
 // updates in place of k, against reading two lines in each test.
 #pragma once
-#include "rsa_device.cuh"
+#include "rsa_search.cuh"
 
 namespace rsak {
 
@@ -116,6 +116,15 @@ __device__ __forceinline__ u32* block_line(const RoundCfg& c, const RoundPtrs& p
 __device__ __forceinline__ u32* anchor_line(const Group& g, const RoundCfg& c, const RoundPtrs& p,
                                             u32 s, u32 type, u32 layout, u32 line) {
   return p.anch + (((size_t)s * 4 + type * 2 + layout) * g.L + line) * c.WA;
+}
+
+// Per-sample set-up: stream base from the seed, state cleared.
+__global__ void k_init(Group g, const u64* seeds) {
+  const u32 s = blockIdx.x * blockDim.x + threadIdx.x;
+  if (s >= g.n) return;
+  g.base[s] = mix64(seeds[s] + SM_GAMMA);
+  SampleState z = {};
+  g.st[s] = z;
 }
 
 __global__ void k_round_init(Group g, RoundCfg c, RoundPtrs p) {
@@ -701,27 +710,46 @@ __device__ __forceinline__ void contact_counts(SampleState& st, const u32 cnt[3]
   }
 }
 
-__device__ __forceinline__ void put_edge(const Group& g, SampleState& st, Edge* E, u32 at, u64 time,
+// Edge `at` of a sample: times and links apart, so that a probe reads 8 bytes
+// of the edges it leaves out.
+__device__ __forceinline__ void put_edge(const Group& g, u32 s, SampleState& st, u32 at, u64 time,
                                          u32 m1, u32 m2, u32 dx, u32 dy) {
   if (at >= g.edge_limit) {
     atomicOr(&st.status, ST_EDGE_OVF);
     return;
   }
-  Edge e;
-  e.time = time;
-  e.m1 = m1;
-  e.m2 = m2;
-  e.dxy = (dx & 0xFFFFu) | (dy << 16);
-  e.pad = 0;
-  E[at] = e;
+  const size_t i = (size_t)s * g.cap_edges + at;
+  g.etime[i] = time;
+  g.elink[i] = make_uint4(m1, m2, (dx & 0xFFFFu) | (dy << 16), 0);
 }
+
+// Histogram of a block's edge times, added to the sample's at the end.
+struct TimeHist {
+  u32* h;
+  __device__ __forceinline__ TimeHist(const Group& g, u32* sh) : h(g.ehist ? sh : nullptr) {
+    if (h)
+      for (u32 i = threadIdx.x; i < EHIST; i += blockDim.x) h[i] = 0;
+    __syncthreads();
+  }
+  __device__ __forceinline__ void add(u64 time, u32 copies) {
+    if (h) atomicAdd(&h[time_bin(time)], copies);
+  }
+  __device__ __forceinline__ void flush(const Group& g, u32 s) {
+    __syncthreads();
+    if (h)
+      for (u32 i = threadIdx.x; i < EHIST; i += blockDim.x)
+        if (h[i]) atomicAdd(&g.ehist[(size_t)s * (EHIST + SUB_BINS) + i], h[i]);
+  }
+};
 
 __global__ void __launch_bounds__(256) k_site_contacts(Group g) {
   const u32 s = blockIdx.y, L = g.L;
   SampleState& st = g.st[s];
   const u64* K = g.node_key + (size_t)s * g.cap_nodes;
   const u32* P = g.node_pos + (size_t)s * g.cap_nodes;
-  Edge* E = g.edges + (size_t)s * g.cap_edges;
+  __shared__ u32 hist_sh[EHIST];
+  if (st.sdone) return;
+  TimeHist hist(g, hist_sh);
   u32 cnt[3] = {0, 0, 0};
   for (u64 i = blockIdx.x * 256ull + threadIdx.x; i < g.LL; i += gridDim.x * 256ull) {
     const u32 m = (u32)i, y = m / L, x = m - y * L;
@@ -731,7 +759,9 @@ __global__ void __launch_bounds__(256) k_site_contacts(Group g) {
 #pragma unroll
     for (u32 dir = 0; dir < 2; ++dir) {
       const u32 b = dir ? down : right;
-      put_edge(g, st, E, 2 * m + dir, tmax(km, K[b]), m, b, dir == 0, dir);
+      const u64 time = tmax(km, K[b]);
+      put_edge(g, s, st, 2 * m + dir, time, m, b, dir == 0, dir);
+      hist.add(time, 1);
       if (b != m) {
         const u32 kind = om != P[b] >> 31 ? 2u : om;
         cnt[0] += kind == 0;
@@ -741,6 +771,7 @@ __global__ void __launch_bounds__(256) k_site_contacts(Group g) {
     }
   }
   contact_counts(st, cnt);
+  hist.flush(g, s);
   if (blockIdx.x == 0 && threadIdx.x == 0) st.n_edges = 2 * (u32)g.LL;
 }
 
@@ -773,7 +804,9 @@ __global__ void __launch_bounds__(256) k_contacts(Group g, const __grid_constant
   const u32 nn = min(st.n_nodes, g.cap_nodes);
   const size_t nb = (size_t)s * g.cap_nodes;
   const u32* anchor_node = g.owner + (size_t)s * g.LL;
-  Edge* E = g.edges + (size_t)s * g.cap_edges;
+  __shared__ u32 hist_sh[EHIST];
+  if (st.sdone) return;
+  TimeHist hist(g, hist_sh);
   const u32 j = tid & (G - 1);
   constexpr u32 GPB = 256 / G;
   u32 cnt[3] = {0, 0, 0};
@@ -789,8 +822,10 @@ __global__ void __launch_bounds__(256) k_contacts(Group g, const __grid_constant
       const u64 kb = g.node_key[nb + b];
       if (b != m) cnt[mixed ? 2 : o] += run;
       const u32 at = atomicAdd(&st.n_edges, copies);
+      const u64 time = tmax(key, kb);
+      hist.add(time, copies);
       for (u32 i = 0; i < copies; ++i)
-        put_edge(g, st, E, at + i, tmax(key, kb), m, b, o ? across : along, o ? along : across);
+        put_edge(g, s, st, at + i, time, m, b, o ? across : along, o ? along : across);
     };
     // parallel k-mers on the next line
     {
@@ -839,6 +874,7 @@ __global__ void __launch_bounds__(256) k_contacts(Group g, const __grid_constant
     }
   }
   contact_counts(st, cnt);
+  hist.flush(g, s);
 }
 
 }  // namespace rsak
