@@ -102,8 +102,10 @@ int rsa_run_static(uint32_t L, uint32_t k, const uint64_t *seeds, uint32_t n, ui
  * are host arrays of n (written).  Results equal rsa_run_seeds +
  * rsa_results for the same (L, k, seed).  Every sample needs L <= 128 and
  * L^2 / k <= 4096 (RSA_EINVAL otherwise).  threads: CTA size, a multiple of
- * 32 up to 1024 (0 = 512).  Allocates its job table stream-ordered on
- * `stream` and synchronises it; returns the first per-sample error code. */
+ * 32 up to 1024 (0 = the library's choice; at least 256 run).  Its job table
+ * and workspaces come stream-ordered on `stream` from a memory pool that
+ * keeps them between calls (rsa_mix_release gives them back); synchronises
+ * `stream`; returns the first per-sample error code. */
 int rsa_run_small(const uint32_t *L, const uint32_t *k, const uint64_t *seeds, uint32_t n,
                   uint32_t threads, uint32_t *n_j, uint32_t *n_c, void *stream);
 

@@ -15,7 +15,8 @@ CSRC = os.path.join(HERE, "csrc")
 SRC = os.path.join(CSRC, "rsa.cu")
 SOURCES = [SRC, os.path.join(CSRC, "rsa_mix.cu")]
 DEPS = SOURCES + [os.path.join(CSRC, f) for f in (
-    "rsa_device.cuh", "rsa_rounds.cuh", "rsa_search.cuh", "rsa_config.cuh", "rsa_small.cuh")] + [os.path.join(os.path.dirname(HERE), "include", "rsa.h")]
+    "rsa_device.cuh", "rsa_rounds.cuh", "rsa_search.cuh", "rsa_sample.cuh",
+    "rsa_config.cuh")] + [os.path.join(os.path.dirname(HERE), "include", "rsa.h")]
 LIB = os.path.join(HERE, "_lib", "librsa_gb300.so")
 OBJ_DIR = os.path.join(HERE, "_build")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

@@ -9,8 +9,10 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstddef>
+#include <map>
 #include <mutex>
 #include <cstdio>
 #include <cstring>
@@ -20,7 +22,7 @@
 
 #include "../../include/rsa.h"
 #include "rsa_rounds.cuh"
-#include "rsa_search.cuh"
+#include "rsa_sample.cuh"
 #include "rsa_config.cuh"
 
 using namespace rsak;
@@ -58,11 +60,13 @@ constexpr size_t READ_BYTES = ALIGN + 4 * WORK_SLOTS * 8;
 size_t align_up(size_t v) { return (v + ALIGN - 1) / ALIGN * ALIGN; }
 
 struct Layout {
-  size_t fine, block, anch, heads, list, flat, act;   // rounds
-  size_t uf, etime, elink, ehist, win;                // contact graph and search
-  size_t owner, base, node_key, node_idx, node_pos, rs, st, seeds, counters, work, keys, total;
-  size_t bits_bytes;  // fine + block, zeroed together
-  size_t anch_bytes, heads_bytes, ehist_bytes;
+  size_t region, rstride;                             // shared region of sample 0, bytes per sample
+  size_t fine, block, heads, list, flat, act;         // rounds (in the region)
+  size_t uf, etime, elink, ehist, win;                // contact graph and search (in the region)
+  size_t anch, owner, base, node_key, node_idx, node_pos, rs, st, seeds, counters, work, keys, total;
+  size_t bits_bytes;  // per sample, fine + block, zeroed together
+  size_t heads_bytes, ehist_bytes;  // per sample
+  size_t anch_bytes;
 };
 
 struct Geometry {
@@ -70,8 +74,11 @@ struct Geometry {
   RoundCfg rc;
   size_t list_cap;  // listed candidates per sample
   SearchCfg sc;
-  u32 win_pow2;     // sc.win_cap rounded up to a power of two
+  SearchCfg ssc;    // the same for a sample in one block (rsa_sample.cuh)
+  u32 lines;        // lines per block of k_refill
   u32 probes;       // probes that bring the window of a large graph to the last
+  Shape hot;        // what of it a block keeps in shared memory (offsets only)
+  bool one_block;   // that fits
   bool win128;      // shape of the 128-thread window setting (rsa_set_window_threads)
 };
 
@@ -103,8 +110,6 @@ void plan_search(u32 L, u32 k, Geometry& G) {
   c.win_cap = std::min(FIN_EDGES, ce);
   c.hashed = cn > 2 * FIN_EDGES;
   c.ids = c.hashed ? 2 * FIN_EDGES : cn;
-  G.win_pow2 = 1;
-  while (G.win_pow2 < c.win_cap) G.win_pow2 <<= 1;
   // n_c / n_j runs from 0.59 (k = 1) to 0.86 (k = 4096), within 0.04 either
   // way; an edge is there by then with about the square of that chance
   const double f = 0.59 + 0.0225 * std::log2((double)k);
@@ -113,6 +118,46 @@ void plan_search(u32 L, u32 k, Geometry& G) {
   // edges per k-mer of capacity: 2 at k = 1, 1.7 at k = 4, 1 from 32 on
   const double edges = (double)cn * (k == 1 ? 2.0 : k <= 8 ? 1.7 : 1.0) * 0.16 * f;
   G.probes = ce <= c.win_cap ? 0 : 3 + (u32)std::max(0.0, std::ceil(std::log2(edges / c.win_cap)));
+  // in one block: as many edges as fit beside the union-find words of all
+  // k-mers, so that most graphs need no probe at all
+  G.ssc = c;
+  if (!c.hashed || cn <= 4 * FIN_EDGES) {
+    SearchCfg w = c;
+    w.hashed = 0;
+    w.ids = cn;
+    const size_t room = SMP_MAX - SMP_FIXED - (size_t)cn * 16;
+    w.win_cap = (u32)std::min<size_t>(ce, room / 18 / 8 * 8);
+    if (w.win_cap >= c.win_cap) G.ssc = w;
+  }
+}
+
+// Shared memory of a sample in one block: cover bits, bins and active
+// candidates, and the anchor bits if they fit as well.
+void plan_hot(u32 L, Geometry& G) {
+  const RoundCfg& c = G.rc;
+  Shape& h = G.hot;
+  h.fine = h.heads = h.act = h.anch = NO_HOT;
+  h.hot_bytes = 0;
+  G.one_block = !G.sites || L <= 96;
+  if (G.sites) return;
+  size_t off = 0;
+  auto part = [&](size_t bytes) {
+    const size_t at = off;
+    off += (bytes + 15) / 16 * 16;
+    return (u32)at;
+  };
+  const size_t room = SMP_MAX - SMP_FIXED - SMP_SCRATCH;
+  h.act = part((size_t)2 * c.cap_act * sizeof(Act));
+  h.fine = part((size_t)2 * (L + c.nbl) * c.W * 4);
+  h.heads = part((size_t)4 * c.nb * c.nb * 4);
+  G.one_block = off <= room;
+  const size_t before = off;
+  h.anch = part((size_t)4 * L * c.WA * 4);
+  if (off > room) {
+    off = before;
+    h.anch = NO_HOT;
+  }
+  h.hot_bytes = (u32)off;
 }
 
 Geometry plan(u32 L, u32 k) {
@@ -134,10 +179,10 @@ Geometry plan(u32 L, u32 k) {
   // Priorities below 2^(64 - a) are listed by the first pass: the fewer, the
   // more candidates are still live afterwards (1.5% at 2^-a = 4 / k).
   c.a = std::max(1u, (lk + 2) / 2);
-  // the first slice holds about two to four candidates per conflict
-  // neighbourhood
-  const u32 ld = log2_floor(D);
-  c.lzmax = std::max(c.a, std::min(ld > 0 ? ld - 1 : 0u, RD_LEVELS - 1));
+  // the first slice holds two to four candidates per conflict neighbourhood
+  // (one to two for short k, where it is a large part of all)
+  const u32 ld = log2_floor(D), first = k < 16 ? ld : ld - 1;
+  c.lzmax = std::max(c.a, std::min(first, RD_LEVELS - 1));
   c.nlev = c.lzmax - c.a + 1;
   size_t off = 0;
   for (u32 t = 0; t < c.nlev; ++t) {
@@ -154,7 +199,9 @@ Geometry plan(u32 L, u32 k) {
   // neither limit is met by random priorities; past one, a round (a refill)
   // takes a narrower slice and the run only takes longer
   c.cap_flat = (u32)std::min<u64>(N, N / 4 + 32);
-  c.cap_act = (u32)std::min<u64>(N, cap_nodes_of(L, k) / 2 + 32);
+  c.cap_act = (u32)std::min<u64>(N, std::max(cap_nodes_of(L, k) / 2, c.lvl_cap[0]) + 32);
+  G.lines = std::max(1u, std::min(1024u, REFILL_WORDS) / c.W);
+  plan_hot(L, G);
   return G;
 }
 
@@ -169,27 +216,36 @@ Layout layout_of(u32 L, u32 k, u32 n, bool with_keys, const Geometry& G) {
     off = align_up(off + bytes);
     return at;
   };
-  // the buffers of the rounds and those of the contact graph and the search
-  // are never in use together: both start at 0
+  // one region per sample, first for the buffers of its rounds, then for those
+  // of its contact graph and search; offsets in it
+  size_t ro = 0;
+  auto part = [&](size_t bytes) {
+    size_t at = ro;
+    ro = align_up(ro + bytes);
+    return at;
+  };
   if (!G.sites) {
-    l.bits_bytes = (size_t)n * 2 * (L + c.nbl) * c.W * 4;
-    l.fine = take(l.bits_bytes);
-    l.block = l.fine + (size_t)n * 2 * L * c.W * 4;
-    l.heads_bytes = (size_t)n * 4 * c.nb * c.nb * 4;
-    l.heads = take(l.heads_bytes);
-    l.list = take((size_t)n * G.list_cap * 4);
-    l.flat = take((size_t)n * c.cap_flat * 4);
-    l.act = take((size_t)n * 2 * c.cap_act * sizeof(Act));
+    l.bits_bytes = (size_t)2 * (L + c.nbl) * c.W * 4;
+    l.fine = part(l.bits_bytes);
+    l.block = l.fine + (size_t)2 * L * c.W * 4;
+    l.heads_bytes = (size_t)4 * c.nb * c.nb * 4;
+    l.heads = part(l.heads_bytes);
+    l.list = part(G.list_cap * 4);
+    l.flat = part((size_t)c.cap_flat * 4);
+    l.act = part((size_t)2 * c.cap_act * sizeof(Act));
   }
-  const size_t rounds_end = off;
-  off = 0;
-  l.uf = take(n * cn * 16);
-  l.etime = take(n * ce * 8);
-  l.elink = take(n * ce * 16);
-  l.ehist_bytes = G.probes ? (size_t)n * (EHIST + SUB_BINS) * 4 : 0;
-  l.ehist = take(l.ehist_bytes);
-  l.win = take((size_t)n * G.sc.win_cap * sizeof(WinEdge));
-  off = std::max(off, rounds_end);
+  const size_t rounds_end = ro;
+  ro = 0;
+  l.uf = part(cn * 16);
+  l.etime = part(ce * 8);
+  l.elink = part(ce * 16);
+  // (graphs that a sample in one block starts on whole use it from 512
+  // k-mers on: two good thresholds are worth its 9 KB there)
+  l.ehist_bytes = G.probes || cap_edges_of(L, k) > G.ssc.win_cap || cn >= 512 ? (size_t)SEARCH_WORDS * 4 : 0;
+  l.ehist = part(l.ehist_bytes);
+  l.win = part(std::max(G.sc.win_cap, G.ssc.win_cap) * sizeof(WinEdge));
+  l.rstride = std::max(ro, rounds_end);
+  l.region = take(n * l.rstride);
   l.anch_bytes = G.sites ? 0 : (size_t)n * 4 * L * c.WA * 4;
   l.anch = take(l.anch_bytes);
   l.owner = take(G.sites ? 0 : n * LL * 4);  // written at anchors only
@@ -209,19 +265,23 @@ Layout layout_of(u32 L, u32 k, u32 n, bool with_keys, const Geometry& G) {
 
 }  // namespace
 
-// The thread's error message, set by the other translation units of the
-// library (rsa_mix.cu) as well.
+// For the other translation unit of the library (rsa_mix.cu): the thread's
+// error message, and what it needs of rsa_run_small.
 namespace rsa_detail {
 int set_error(int code, const std::string& msg) { return fail(code, msg); }
+bool small_eligible(uint32_t L, uint32_t k);
+unsigned long long take_small_launches();
+void release_small();
 }  // namespace rsa_detail
 
 enum Kind {
   KD_INIT, KD_DENSE, KD_PICK, KD_RESOLVE, KD_REFILL, KD_CHECK, KD_SITES, KD_EDGES,
-  KD_SEARCH_INIT, KD_PROBE_COPY, KD_PROBE, KD_COLLECT, KD_FINISH, KD_RANK, KD_COUNT
+  KD_SEARCH_INIT, KD_PROBE_COPY, KD_PROBE, KD_COLLECT, KD_FINISH, KD_RANK, KD_SAMPLE, KD_COUNT
 };
 const char* const kKindNames[KD_COUNT] = {
     "k_init", "k_dense", "k_pick", "k_resolve", "k_refill", "k_round_check", "k_sites", "k_edges",
-    "k_search_init", "k_probe_copy", "k_probe", "k_collect", "k_finish", "k_rank"};
+    "k_search_init", "k_probe_copy", "k_probe", "k_collect", "k_finish", "k_rank",
+    "k_sample"};
 
 // Optional per-kernel timing with CUDA events recorded around each launch
 // on the launch stream, plus launch counts (always kept).
@@ -322,11 +382,13 @@ Group group_of(rsa_t* h, u32 n) {
   g.node_key = reinterpret_cast<u64*>(b + l.node_key);
   g.node_idx = reinterpret_cast<u32*>(b + l.node_idx);
   g.node_pos = reinterpret_cast<u32*>(b + l.node_pos);
-  g.uf = reinterpret_cast<u64*>(b + l.uf);
-  g.etime = reinterpret_cast<u64*>(b + l.etime);
-  g.elink = reinterpret_cast<uint4*>(b + l.elink);
-  g.ehist = l.ehist_bytes ? reinterpret_cast<u32*>(b + l.ehist) : nullptr;
-  g.win = reinterpret_cast<WinEdge*>(b + l.win);
+  char* r = b + l.region;
+  g.rstride = l.rstride;
+  g.uf = reinterpret_cast<u64*>(r + l.uf);
+  g.etime = reinterpret_cast<u64*>(r + l.etime);
+  g.elink = reinterpret_cast<uint4*>(r + l.elink);
+  g.ehist = l.ehist_bytes ? reinterpret_cast<u32*>(r + l.ehist) : nullptr;
+  g.win = reinterpret_cast<WinEdge*>(r + l.win);
   g.st = reinterpret_cast<SampleState*>(b + l.st);
   g.work = reinterpret_cast<u64*>(b + l.work);
   return g;
@@ -335,16 +397,16 @@ Group group_of(rsa_t* h, u32 n) {
 RoundPtrs round_ptrs(rsa_t* h) {
   char* b = static_cast<char*>(h->ws);
   const Layout& l = h->lay;
+  char* r = b + l.region;
   RoundPtrs p{};
-  p.fine = reinterpret_cast<u32*>(b + l.fine);
-  p.block = reinterpret_cast<u32*>(b + l.block);
+  p.fine = reinterpret_cast<u32*>(r + l.fine);
+  p.block = reinterpret_cast<u32*>(r + l.block);
   p.anch = reinterpret_cast<u32*>(b + l.anch);
-  p.list = reinterpret_cast<u32*>(b + l.list);
-  p.flat = reinterpret_cast<u32*>(b + l.flat);
-  p.act = reinterpret_cast<Act*>(b + l.act);
-  p.heads = reinterpret_cast<u32*>(b + l.heads);
+  p.list = reinterpret_cast<u32*>(r + l.list);
+  p.flat = reinterpret_cast<u32*>(r + l.flat);
+  p.act = reinterpret_cast<Act*>(r + l.act);
+  p.heads = reinterpret_cast<u32*>(r + l.heads);
   p.rs = reinterpret_cast<RoundState*>(b + l.rs);
-  p.list_cap = h->geo.list_cap;
   return p;
 }
 
@@ -359,23 +421,38 @@ cudaEvent_t prof_event(Prof& p, size_t i) {
 
 // Launch wrapper: counts launches and, when profiling is on, brackets the
 // launch with two events on its stream.
+cudaEvent_t prof_begin(Prof& p, int kind, cudaStream_t st) {
+  if (!p.on) return nullptr;
+  const size_t i = p.kinds.size();
+  cudaEvent_t e0 = prof_event(p, 2 * i), e1 = prof_event(p, 2 * i + 1);
+  if (!e0 || !e1) return nullptr;
+  cudaEventRecord(e0, st);
+  p.kinds.push_back(kind);
+  return e1;
+}
+
 template <typename K, typename... Args>
 void launch(rsa_t* h, int kind, K kernel, dim3 grid, dim3 block, size_t smem, cudaStream_t st,
             Args... args) {
   Prof& p = h->prof;
-  cudaEvent_t e0 = nullptr, e1 = nullptr;
-  if (p.on) {
-    size_t i = p.kinds.size();
-    e0 = prof_event(p, 2 * i);
-    e1 = prof_event(p, 2 * i + 1);
-    if (e0 && e1) {
-      cudaEventRecord(e0, st);
-      p.kinds.push_back(kind);
-    }
-  }
+  cudaEvent_t e1 = prof_begin(p, kind, st);
   kernel<<<grid, block, smem, st>>>(args...);
-  if (e0 && e1) cudaEventRecord(e1, st);
+  if (e1) cudaEventRecord(e1, st);
   p.launches[kind] += 1;
+}
+
+// The shape of the one-block kernels.
+Shape shape_of(const Geometry& G, const Group& g, const RoundCfg& c, const RoundPtrs& p,
+               u32 probe_cap) {
+  Shape s = G.hot;
+  s.g = g;
+  s.c = c;
+  s.p = p;
+  s.sc = G.ssc;
+  s.probe_cap = probe_cap;
+  s.lines = G.lines;
+  s.sites = G.sites;
+  return s;
 }
 
 int launch_check(const char* what) {
@@ -502,10 +579,9 @@ int run_impl(rsa_t* h, const uint64_t* seeds, u32 n, const uint64_t* keys, cudaS
       default: launch(h, KD_RESOLVE, k_resolve<32>, rg, dim3(RD_THREADS), 0, st, g, c, rp); break;
     }
   };
-  const u32 lines = std::max(1u, std::min(1024u, REFILL_WORDS) / c.W);
   auto refill = [&](cudaStream_t st) {
-    launch(h, KD_REFILL, k_refill, grid_x((2ull * h->L + lines - 1) / lines, 16), dim3(RD_THREADS),
-           0, st, g, c, rp, lines);
+    launch(h, KD_REFILL, k_refill, grid_x((2ull * h->L + G.lines - 1) / G.lines, 16),
+           dim3(RD_THREADS), 0, st, g, c, rp, G.lines);
   };
   auto count_active = [&](cudaStream_t st) {
     check(cudaMemsetAsync(d_counter, 0, 4, st));
@@ -520,15 +596,16 @@ int run_impl(rsa_t* h, const uint64_t* seeds, u32 n, const uint64_t* keys, cudaS
       launch(h, KD_SITES, k_sites, grid_x((LL + 255) / 256, 32), dim3(256), 0, st, g);
       return;
     }
-    check(cudaMemsetAsync(b + l.fine, 0, l.bits_bytes, st));
+    check(cudaMemset2DAsync(b + l.region + l.fine, l.rstride, 0, l.bits_bytes, n, st));
     check(cudaMemsetAsync(b + l.anch, 0, l.anch_bytes, st));
-    check(cudaMemsetAsync(b + l.heads, 0xFF, l.heads_bytes, st));
+    check(cudaMemset2DAsync(b + l.region + l.heads, l.rstride, 0xFF, l.heads_bytes, n, st));
     launch(h, KD_INIT, k_round_init, init_grid, dim3(128), 0, st, g, c, rp);
-    const dim3 dg = grid_x((2 * LL + DENSE_TILE - 1) / DENSE_TILE, 16);
+    const u64 dense_tile = DENSE_THREADS * DENSE_PER;
+    const dim3 dg = grid_x((2 * LL + dense_tile - 1) / dense_tile, 16);
     if (h->with_keys)
-      launch(h, KD_DENSE, k_dense<true>, dg, dim3(RD_THREADS), 0, st, g, c, rp);
+      launch(h, KD_DENSE, k_dense<true>, dg, dim3(DENSE_THREADS), 0, st, g, c, rp);
     else
-      launch(h, KD_DENSE, k_dense<false>, dg, dim3(RD_THREADS), 0, st, g, c, rp);
+      launch(h, KD_DENSE, k_dense<false>, dg, dim3(DENSE_THREADS), 0, st, g, c, rp);
     for (u32 t = 0; t < c.nlev; ++t) round(st);
     refill(st);
     for (u32 t = c.nlev; t <= c.lzmax + h->drain; ++t) round(st);
@@ -544,7 +621,7 @@ int run_impl(rsa_t* h, const uint64_t* seeds, u32 n, const uint64_t* keys, cudaS
   // blocks per sample over its k-mers and its edges
   const dim3 node_grid = grid_x(((u64)g.cap_nodes + 255) / 256, 32);
   const dim3 edge_grid = grid_x(((u64)g.cap_edges + 1023) / 1024, 16);
-  const size_t fin_smem = finish_smem(sc, G.win_pow2);
+  const size_t fin_smem = finish_smem(sc);
   // the same limit for every shape: handles run on several threads at once
   CUDA_TRY(cudaFuncSetAttribute(k_finish, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)FIN_SMEM_MAX));
@@ -555,15 +632,13 @@ int run_impl(rsa_t* h, const uint64_t* seeds, u32 n, const uint64_t* keys, cudaS
       launch(h, KD_PROBE, k_probe, edge_grid, dim3(256), 0, st, g, sc, probe_cap);
     }
     launch(h, KD_COLLECT, k_collect, edge_grid, dim3(256), 0, st, g, sc);
-    launch(h, KD_FINISH, k_finish, dim3(n), dim3(FIN_THREADS), fin_smem, st, g, sc, G.win_pow2,
-           probe_cap, d_counter + 1);
+    launch(h, KD_FINISH, k_finish, dim3(n), dim3(FIN_THREADS), fin_smem, st, g, sc, probe_cap,
+           d_counter + 1);
     launch(h, KD_RANK, k_rank, node_grid, dim3(256), 0, st, g);
   };
   // contact graph of the jammed lattice and the search for the first wrap
   auto search = [&](cudaStream_t st) {
-    if (l.ehist_bytes) check(cudaMemsetAsync(b + l.ehist, 0, l.ehist_bytes, st));
-    launch(h, KD_SEARCH_INIT, k_graph_init, init_grid, dim3(128), 0, st, g,
-           (const u32*)d_counter);
+    launch(h, KD_SEARCH_INIT, k_graph_init, dim3(n), dim3(256), 0, st, g, (const u32*)d_counter);
     if (G.sites) {
       launch(h, KD_EDGES, k_site_contacts, grid_x((LL + 255) / 256, 32), dim3(256), 0, st, g);
     } else {
@@ -580,7 +655,20 @@ int run_impl(rsa_t* h, const uint64_t* seeds, u32 n, const uint64_t* keys, cudaS
     launch(h, KD_SEARCH_INIT, k_search_init, dim3(n), dim3(256), 0, st, g, sc);
     probes(st);
   };
+  // One block per sample for the small lattices, and for those that still fit
+  // a block when there are enough samples to fill the GPU with blocks
+  // (L = 256, k = 16: 256 samples 0.78 ms, over the whole grid 1.11; 4 samples
+  // 0.40 and 0.36).
+  const bool by_sample = G.one_block && (h->L <= 160 || n >= (u32)h->sm_count / 2);
+  const Shape shape = shape_of(G, g, c, rp, probe_cap);
+  CUDA_TRY(cudaFuncSetAttribute(k_sample, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMP_MAX));
   auto whole = [&](cudaStream_t st) {
+    if (by_sample) {
+      check(cudaMemsetAsync(b + l.counters, 0, READ_BYTES, st));
+      launch(h, KD_SAMPLE, k_sample, dim3(std::min(n, (u32)h->sm_count)), dim3(SMP_THREADS),
+             sample_smem(shape), st, shape, (const u64*)d_seeds);
+      return;
+    }
     deposit(st);
     search(st);
   };
@@ -750,9 +838,148 @@ int configuration(rsa_t* h, uint32_t sample, uint32_t m, uint32_t* counts, uint3
   return 0;
 }
 
+// ---------------------------------------------------------------------
+// Small lattices of any mix of shapes (rsa_run_small).  Every block has a
+// workspace slot of the largest shape's size.  The slots come stream-ordered
+// from a memory pool of the library's own, which keeps up to SMALL_POOL_KEEP
+// bytes between calls (a serving loop calls this often) and gives them back
+// in rsa_mix_release.
+// ---------------------------------------------------------------------
+constexpr u64 SMALL_LMAX = 128, SMALL_NMAX = 4096;
+constexpr unsigned long long SMALL_POOL_KEEP = 512ull << 20;
+std::atomic<unsigned long long> g_small_launches{0};
+std::mutex g_pool_mu;
+cudaMemPool_t g_pool[MAX_DEVICES] = {};
+
+int small_pool(int dev, cudaMemPool_t* out) {
+  if (dev < 0 || dev >= MAX_DEVICES) return fail(RSA_EINVAL, "device ordinal out of range");
+  std::lock_guard<std::mutex> lock(g_pool_mu);
+  if (!g_pool[dev]) {
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t pool = nullptr;
+    CUDA_TRY(cudaMemPoolCreate(&pool, &props));
+    unsigned long long keep = SMALL_POOL_KEEP;
+    cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    g_pool[dev] = pool;
+  }
+  *out = g_pool[dev];
+  return 0;
+}
+
+// A shape with the pointers of a workspace of one sample that starts at 0.
+Shape slot_shape(uint32_t L, uint32_t k, size_t* bytes) {
+  rsa h;
+  h.L = L;
+  h.k = k;
+  h.geo = plan(L, k);
+  h.lay = layout_of(L, k, 1, false, h.geo);
+  h.ws = nullptr;
+  *bytes = h.lay.total;
+  Group g = group_of(&h, 1);
+  RoundCfg c = h.geo.rc;
+  c.round_cap = cap_nodes_of(L, k) + 2;
+  return shape_of(h.geo, g, c, round_ptrs(&h), PROBE_CAP);
+}
+
+int run_small(const uint32_t* L, const uint32_t* k, const uint64_t* seeds, uint32_t n,
+              uint32_t threads, uint32_t* n_j, uint32_t* n_c, cudaStream_t st) {
+  NvtxRange range("rsa_run_small");
+  std::vector<Shape> shapes;
+  std::map<std::pair<uint32_t, uint32_t>, u32> known;
+  std::vector<SmallJob> jobs(n);
+  size_t slot = 0, smem = 0;
+  for (uint32_t i = 0; i < n; ++i) {
+    if (!rsa_detail::small_eligible(L[i], k[i]))
+      return fail(RSA_EINVAL, "rsa_run_small: sample " + std::to_string(i) + " (L=" +
+                                  std::to_string(L[i]) + ", k=" + std::to_string(k[i]) +
+                                  ") needs L <= 128 and L^2/k <= 4096");
+    auto it = known.find({L[i], k[i]});
+    if (it == known.end()) {
+      size_t bytes = 0;
+      shapes.push_back(slot_shape(L[i], k[i], &bytes));
+      it = known.emplace(std::make_pair(L[i], k[i]), (u32)shapes.size() - 1).first;
+      slot = std::max(slot, align_up(bytes));
+      smem = std::max(smem, sample_smem(shapes.back()));
+    }
+    jobs[i] = SmallJob{seeds[i], it->second, 0};
+  }
+  int dev = 0, sms = 0;
+  CUDA_TRY(cudaGetDevice(&dev));
+  CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  cudaMemPool_t pool = nullptr;
+  int rc = small_pool(dev, &pool);
+  if (rc) return rc;
+  CUDA_TRY(cudaFuncSetAttribute(k_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMP_MAX));
+  const u32 grid = std::min(n, (u32)sms);
+  // shapes and jobs in one copy; then results, work counters, job counter, slots
+  const size_t sb = align_up(sizeof(Shape) * shapes.size()), jb = align_up(sizeof(SmallJob) * n);
+  const size_t ob = align_up(sizeof(SmallOut) * n), wb = 4 * WORK_SLOTS * 8 + ALIGN;
+  std::vector<char> in(sb + jb);
+  std::memcpy(in.data(), shapes.data(), sizeof(Shape) * shapes.size());
+  std::memcpy(in.data() + sb, jobs.data(), sizeof(SmallJob) * n);
+  std::vector<SmallOut> out(n);
+  char* d = nullptr;
+  CUDA_TRY(cudaMallocFromPoolAsync(reinterpret_cast<void**>(&d), sb + jb + ob + wb + grid * slot, pool, st));
+  char* work = d + sb + jb + ob;
+  cudaError_t e = cudaMemcpyAsync(d, in.data(), in.size(), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(work, 0, wb, st);
+  if (e == cudaSuccess) {
+    k_small<<<grid, threads, smem, st>>>(
+        reinterpret_cast<const Shape*>(d), reinterpret_cast<const SmallJob*>(d + sb), n,
+        reinterpret_cast<SmallOut*>(d + sb + jb), work + wb, slot, reinterpret_cast<u64*>(work),
+        reinterpret_cast<u32*>(work + 4 * WORK_SLOTS * 8));
+    e = cudaGetLastError();
+    if (e == cudaSuccess) g_small_launches.fetch_add(1);
+  }
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(out.data(), d + sb + jb, sizeof(SmallOut) * n, cudaMemcpyDeviceToHost, st);
+  cudaFreeAsync(d, st);
+  const cudaError_t e2 = cudaStreamSynchronize(st);
+  if (e == cudaSuccess) e = e2;
+  if (e != cudaSuccess)
+    return fail(RSA_ECUDA, std::string("rsa_run_small: ") + cudaGetErrorString(e));
+  int first = 0;
+  for (uint32_t i = 0; i < n; ++i) {
+    n_j[i] = out[i].n_j;
+    n_c[i] = out[i].n_c;
+    const int cd = status_code(out[i].status);
+    if (cd && !first) {
+      first = cd;
+      g_err = "sample " + std::to_string(i) + " status bits " + std::to_string(out[i].status);
+    }
+  }
+  return first;
+}
+
 }  // namespace
 
+namespace rsa_detail {
+bool small_eligible(uint32_t L, uint32_t k) {
+  return k >= 1 && k <= L && L <= SMALL_LMAX && (uint64_t)L * L / k <= SMALL_NMAX;
+}
+unsigned long long take_small_launches() { return g_small_launches.exchange(0); }
+void release_small() {
+  std::lock_guard<std::mutex> lock(g_pool_mu);
+  for (cudaMemPool_t p : g_pool)
+    if (p) cudaMemPoolTrimTo(p, 0);
+}
+}  // namespace rsa_detail
+
 extern "C" {
+
+int rsa_run_small(const uint32_t* L, const uint32_t* k, const uint64_t* seeds, uint32_t n,
+                  uint32_t threads, uint32_t* n_j, uint32_t* n_c, void* stream) {
+  if (!L || !k || !seeds || !n_j || !n_c || n == 0)
+    return fail(RSA_EINVAL, "rsa_run_small: null array or n == 0");
+  if (threads % 32 || threads > 1024)
+    return fail(RSA_EINVAL, "threads must be 32 .. 1024, a multiple of 32");
+  // the search's set-up needs 256 threads
+  threads = threads == 0 ? SMP_THREADS : std::max(threads, 256u);
+  return run_small(L, k, seeds, n, threads, n_j, n_c, static_cast<cudaStream_t>(stream));
+}
 
 int rsa_create(uint32_t L, uint32_t k, uint64_t seed, rsa_t** out) {
   if (!out) return fail(RSA_EINVAL, "out is NULL");
@@ -877,7 +1104,7 @@ int rsa_sample_stats(rsa_t* h, uint32_t* rounds, uint32_t* probes, uint32_t* edg
   if (rc) return rc;
   for (u32 i = 0; i < n; ++i) {
     if (rounds) rounds[i] = st[i].rounds;
-    if (probes) probes[i] = st[i].probes;
+    if (probes) probes[i] = st[i].w.probes;
     if (edges) edges[i] = st[i].n_edges;
     if (status) status[i] = status_code(st[i].status);
   }

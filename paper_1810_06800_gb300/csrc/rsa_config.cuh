@@ -33,10 +33,10 @@ namespace rsak {
 constexpr u32 CFG_CAPPED = 1u << 31;  // wdirs bit: a union-find walk hit its cap
 
 __host__ __device__ __forceinline__ u64* cfg_uf(const Group& g, u32 s) {
-  return g.uf + (size_t)s * 2 * g.cap_nodes;
+  return region_of(g, g.uf, s);
 }
 __host__ __device__ __forceinline__ u32* cfg_size(const Group& g, u32 s) {
-  return reinterpret_cast<u32*>(g.uf + ((size_t)s * 2 + 1) * g.cap_nodes);
+  return reinterpret_cast<u32*>(region_of(g, g.uf, s) + g.cap_nodes);
 }
 __host__ __device__ __forceinline__ u32* cfg_hist(const Group& g, u32 s) {
   return cfg_size(g, s) + g.cap_nodes;
@@ -178,18 +178,21 @@ __global__ void __launch_bounds__(256) k_cfg_union(Group g, u32 s) {
   SampleState& st = g.st[s];
   const u64 T = st.sel;
   const u32 ne = min(st.n_edges, g.edge_limit);
-  const u64* E = g.etime + (size_t)s * g.cap_edges;
-  const uint4* K = g.elink + (size_t)s * g.cap_edges;
+  const u64* E = region_of(g, g.etime, s);
+  const uint4* K = region_of(g, g.elink, s);
   u64* W = cfg_uf(g, s);
   bool capped = false;
   u32 dirs = 0;
-  for (u32 i = blockIdx.x * blockDim.x + threadIdx.x; i < ne; i += gridDim.x * blockDim.x) {
-    if (E[i] > T) continue;
-    const uint4 e = K[i];
-    u32 mis = 0;
-    if (uf_union(W, e.x, e.y, e.z, &capped, g.uf_cap, &mis))
-      dirs |= ((mis & 0xFFFFu) ? 1u : 0u) | ((mis >> 16) ? 2u : 0u);
-  }
+  __shared__ u32 queue[queue_words(256)];
+  scan_packed(
+      ne, Team{blockIdx.x, gridDim.x}, *reinterpret_cast<EdgeQueue*>(queue),
+      [&](u32 i) { return E[i] <= T; },
+      [&](u32 i) {
+        const uint4 e = K[i];
+        u32 mis = 0;
+        if (uf_union(W, e.x, e.y, e.z, &capped, g.uf_cap, &mis))
+          dirs |= ((mis & 0xFFFFu) ? 1u : 0u) | ((mis >> 16) ? 2u : 0u);
+      });
   if (capped) dirs |= CFG_CAPPED;
   dirs = __reduce_or_sync(FULL, dirs);
   if ((threadIdx.x & 31) == 0 && dirs) atomicOr(&st.wdirs, dirs);

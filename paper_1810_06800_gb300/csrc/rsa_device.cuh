@@ -55,20 +55,29 @@ __device__ __forceinline__ u64 mix64(u64 z) {
   return z ^ (z >> 31);
 }
 
+struct Window {        // state of the first-wrap search (rsa_search.cuh)
+  u64 lo, hi, mid, next_mid;                // window (lo, hi], thresholds
+  u32 cur, hi_ok, ready, first;             // union-find buffer of the state at lo; a probe
+                                            // has wrapped at hi; the window is the last one;
+                                            // no probe yet
+  u32 probes, pad;
+};
+
 struct SampleState {   // one per sample
-  u32 n_nodes, n_edges, rounds, probes;
-  u32 done, status, sdone, wrap;            // wrap: the current probe closed one
-  u64 lo, hi, mid, next_mid;                // window (lo, hi] of the search
-  u32 cur, hi_ok, ready, step;
-  u32 count_a, count_b, in_win, ticket;     // edges of (lo, mid], (mid, hi], (lo, hi]
-  u32 win_n, ranked, nc, wdirs;             // wdirs: configuration pass, winding bits
+  u32 n_nodes, n_edges, rounds, status;
+  u32 done, sdone, ticket, win_n;
+  u32 ranked, nc, wdirs;                    // wdirs: configuration pass, winding bits
   u32 contacts_x, contacts_y, contacts_xy;  // lattice edges between different
                                             // k-mers: both H, both V, mixed
-  u32 pad;
   u64 tc;                                   // priority of the k-mer that first wraps
   u64 sel;                                  // configuration pass: m-th key
+  Window w;
 };
-static_assert(sizeof(SampleState) == 144, "SampleState is 144 bytes");
+static_assert(sizeof(SampleState) == 128, "SampleState is 128 bytes");
+
+struct Team {          // the blocks that share a sample: this one's rank of size
+  u32 rank, size;
+};
 
 struct WinEdge;
 
@@ -78,6 +87,8 @@ struct Group {         // one batch of samples sharing (L, k)
   u32 uf_cap;          // steps of one union-find walk or link retry loop
   u32 edge_limit;      // contact edges stored per sample (<= cap_edges)
   u64 LL;
+  u64 rstride;         // bytes between samples in the buffers marked (r): those of the
+                       // rounds and those of the search share one region per sample
   u32* owner;          // [n][L][L]   node id of the k-mer anchored at the cell; only
                        //             anchors are written, the rest is never read
   u64* base;           // [n]         splitmix64 stream base per sample
@@ -85,18 +96,35 @@ struct Group {         // one batch of samples sharing (L, k)
   u64* node_key;       // [n][cap_nodes]
   u32* node_idx;       // [n][cap_nodes]  accepted candidate idx
   u32* node_pos;       // [n][cap_nodes]  o << 31 | y0 << 15 | x0 of the anchor
-  u64* uf;             // [n][2][cap_nodes] union-find words
-  u64* etime;          // [n][cap_edges] contact edges: max of the two priorities,
-  uint4* elink;        // [n][cap_edges] and node ids, lifted anchor(m2) - anchor(m1)
+  u64* uf;             // (r) [2][cap_nodes] union-find words
+  u64* etime;          // (r) [cap_edges] contact edges: max of the two priorities,
+  uint4* elink;        // (r) [cap_edges] and node ids, lifted anchor(m2) - anchor(m1)
                        //                as 16-bit dx, dy
-  u32* ehist;          // [n][EHIST + SUB_BINS] edges per time_bin, per sub-bin of the
-                       //                window; null where no graph can be large
-  WinEdge* win;        // [n][win_cap]
+  u32* ehist;          // (r) [SEARCH_WORDS] edges per time_bin, then the counts of a
+                       //                probe; null where no graph can be large
+  WinEdge* win;        // (r) [win_cap]
   SampleState* st;     // [n]
   u64* work;           // [4][WORK_SLOTS] work counters of the deposition: candidates
                        //     hashed by the first pass, list entries tested, active
                        //     candidates resolved, k-mers accepted
 };
+
+// Sample s's part of a buffer of the shared region.
+template <typename T>
+__host__ __device__ __forceinline__ T* region_of(const Group& g, T* first, u32 s) {
+  return reinterpret_cast<T*>(reinterpret_cast<char*>(first) + (size_t)s * g.rstride);
+}
+
+// Slots from a counter for the lanes with ok, one atomic per warp.
+__device__ __forceinline__ u32 warp_append(u32* counter, bool ok) {
+  const u32 m = __ballot_sync(FULL, ok);
+  if (!m) return 0;
+  const u32 lane = threadIdx.x & 31, leader = __ffs(m) - 1;
+  u32 at = 0;
+  if (lane == leader) at = atomicAdd(counter, (u32)__popc(m));
+  at = __shfl_sync(FULL, at, leader);
+  return at + __popc(m & ((1u << lane) - 1u));
+}
 
 // Monotone bin of a priority: 32 bins per power of two.
 __device__ __forceinline__ u32 time_bin(u64 t) {

@@ -1,8 +1,6 @@
 // rsa_mix.cu -- batching of samples of uneven (L, k) and the autotuner that
 // picks how each shape runs (C ABI in include/rsa.h).
 //
-//   rsa_run_small  small lattices, one CTA per sample (rsa_small.cuh): any
-//                  mix of shapes in one persistent launch;
 //   rsa_run_mix    a batch of samples of any shapes: the small ones in one
 //                  persistent launch, every other shape on its own handle
 //                  (graph-replayed rounds) on its own stream, all at once;
@@ -16,7 +14,6 @@
 #include <sys/stat.h>
 
 #include <algorithm>
-#include <atomic>
 #include <chrono>
 #include <cstdio>
 #include <cstdlib>
@@ -30,12 +27,13 @@
 #include <vector>
 
 #include "../../include/rsa.h"
-#include "rsa_small.cuh"
 
-using namespace rsak;
-
+// Of the other translation unit (rsa.cu).
 namespace rsa_detail {
 int set_error(int code, const std::string& msg);
+bool small_eligible(uint32_t L, uint32_t k);
+unsigned long long take_small_launches();
+void release_small();
 }
 
 namespace {
@@ -49,89 +47,9 @@ using rsa_detail::set_error;
       return set_error(RSA_ECUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
   } while (0)
 
-bool small_eligible(uint32_t L, uint32_t k) {
-  return k >= 1 && k <= L && L <= SMALL_LMAX && (uint64_t)L * L / k <= SMALL_NMAX;
-}
-
-int status_to_code(u32 bits) {
-  if (bits & ST_NOWRAP) return RSA_ENOWRAP;
-  if (bits & (ST_UF_CAP | ST_ROUND_CAP)) return RSA_ETIMEOUT;
-  if (bits & ST_NODE_OVF) return RSA_ENOMEM;
-  return 0;
-}
-
-// k_small launches since the last rsa_mix_launches() call.
-std::atomic<unsigned long long> g_small_launches{0};
-
-// Resident CTAs of k_small per SM for a CTA size and lattice bound.
-int small_blocks_per_sm(uint32_t threads, uint32_t Lm, int* out) {
-  const size_t smem = small_smem_bytes(Lm);
-  MIX_CUDA(cudaFuncSetAttribute(k_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)small_smem_bytes(SMALL_LMAX)));
-  MIX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_small, (int)threads, smem));
-  return 0;
-}
+using rsa_detail::small_eligible;
 
 }  // namespace
-
-extern "C" int rsa_run_small(const uint32_t* L, const uint32_t* k, const uint64_t* seeds,
-                             uint32_t n, uint32_t threads, uint32_t* n_j, uint32_t* n_c,
-                             void* stream) {
-  if (!L || !k || !seeds || !n_j || !n_c || n == 0)
-    return set_error(RSA_EINVAL, "rsa_run_small: null array or n == 0");
-  if (threads == 0) threads = 512;
-  nvtxRangePushA("rsa_run_small");
-  struct Pop { ~Pop() { nvtxRangePop(); } } pop;
-  if (threads % 32 || threads > 1024) return set_error(RSA_EINVAL, "threads must be 32 .. 1024, a multiple of 32");
-  std::vector<SmallJob> jobs(n);
-  uint32_t Lm = 0;
-  for (uint32_t i = 0; i < n; ++i) {
-    if (!small_eligible(L[i], k[i]))
-      return set_error(RSA_EINVAL, "rsa_run_small: sample " + std::to_string(i) + " (L=" +
-                                       std::to_string(L[i]) + ", k=" + std::to_string(k[i]) +
-                                       ") needs L <= 128 and L^2/k <= 4096");
-    jobs[i] = SmallJob{L[i], k[i], seeds[i]};
-    Lm = std::max(Lm, L[i]);
-  }
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
-  int dev = 0, sms = 0, bps = 0;
-  MIX_CUDA(cudaGetDevice(&dev));
-  MIX_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  int rc = small_blocks_per_sm(threads, Lm, &bps);
-  if (rc) return rc;
-  if (bps < 1) return set_error(RSA_EINVAL, "rsa_run_small: CTA size does not fit an SM");
-  // job table, results and the work counter, stream-ordered
-  const size_t jb = sizeof(SmallJob) * n, ob = sizeof(SmallOut) * n;
-  char* d = nullptr;
-  MIX_CUDA(cudaMallocAsync(reinterpret_cast<void**>(&d), jb + ob + 256, st));
-  SmallJob* djobs = reinterpret_cast<SmallJob*>(d);
-  SmallOut* dout = reinterpret_cast<SmallOut*>(d + jb);
-  u32* dnext = reinterpret_cast<u32*>(d + jb + ob);
-  std::vector<SmallOut> out(n);
-  cudaError_t e = cudaMemcpyAsync(djobs, jobs.data(), jb, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(dnext, 0, 4, st);
-  if (e == cudaSuccess) {
-    const u32 grid = (u32)std::min<uint64_t>(n, (uint64_t)sms * bps);
-    k_small<<<grid, threads, small_smem_bytes(Lm), st>>>(djobs, n, dout, dnext, Lm, UF_CAP);
-    e = cudaGetLastError();
-    if (e == cudaSuccess) g_small_launches.fetch_add(1);
-  }
-  if (e == cudaSuccess) e = cudaMemcpyAsync(out.data(), dout, ob, cudaMemcpyDeviceToHost, st);
-  cudaFreeAsync(d, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  if (e != cudaSuccess) return set_error(RSA_ECUDA, std::string("rsa_run_small: ") + cudaGetErrorString(e));
-  int first = 0;
-  for (uint32_t i = 0; i < n; ++i) {
-    n_j[i] = out[i].n_j;
-    n_c[i] = out[i].n_c;
-    const int c = status_to_code(out[i].status);
-    if (c && !first) {
-      first = c;
-      set_error(c, "sample " + std::to_string(i) + " status bits " + std::to_string(out[i].status));
-    }
-  }
-  return first;
-}
 
 // ---------------------------------------------------------------------
 // Autotuner.  For one (GPU, L, k, batch size rounded up to a power of two)
@@ -492,7 +410,7 @@ extern "C" int rsa_run_mix(const uint32_t* L, const uint32_t* k, const uint64_t*
 }
 
 extern "C" unsigned long long rsa_mix_launches(void) {
-  unsigned long long total = g_small_launches.exchange(0);
+  unsigned long long total = rsa_detail::take_small_launches();
   uint32_t nk = 0;
   while (rsa_kernel_name(nk)[0]) ++nk;
   std::vector<double> ms(nk);
@@ -521,4 +439,5 @@ extern "C" void rsa_mix_release(void) {
     cudaEventDestroy(kv.second.second);
   }
   g_small_stream.clear();
+  rsa_detail::release_small();
 }

@@ -46,9 +46,8 @@ namespace rsak {
 
 constexpr u32 RD_LEVELS = 32;
 constexpr u32 RD_THREADS = 256;
+constexpr u32 DENSE_THREADS = 256;
 constexpr u32 DENSE_PER = 16;                      // candidates per thread and tile
-constexpr u32 DENSE_TILE = RD_THREADS * DENSE_PER;
-constexpr u32 DENSE_STAGE = 2 * DENSE_TILE;
 constexpr u32 REFILL_WORDS = 2304;                 // words of line staged per block
 
 struct RoundCfg {
@@ -71,7 +70,7 @@ struct Act {        // an active candidate (16 bytes, one load)
   u32 next;         // next active candidate of its bin
 };
 
-struct RoundState { // per sample
+struct Slice {      // where the scan of a sample stands
   u64 lo, hi;       // current slice, both ends included
   u64 fill_hi;      // the refilled list holds priorities up to this one
   u32 t;            // number of the slice: 0 .. lzmax
@@ -80,8 +79,12 @@ struct RoundState { // per sample
   u32 refill;       // the lists are used up: k_refill has to run, from lo on
   u32 finished;     // every slice has been entered
   u32 par;          // active buffer written by this round
+};
+
+struct RoundState { // per sample
+  Slice sl;
   u32 act[2];       // active candidates per buffer
-  u32 left;         // not accepted in the last round
+  u32 taken;        // accepted in this round
   u32 flat_n;
   u32 ticket, ticket2;
   u32 lvl_n[RD_LEVELS];
@@ -92,25 +95,32 @@ __device__ __forceinline__ u64 slice_top(const RoundCfg& c, u32 t) {
   return lz == 0 ? ~0ull : (1ull << (64 - lz)) - 1ull;
 }
 
+__device__ __forceinline__ Slice first_slice(const RoundCfg& c) {
+  Slice z = {};
+  z.open = 1;
+  z.hi = slice_top(c, 0);
+  z.fill_hi = ~0ull;
+  return z;
+}
+
 struct RoundPtrs {
-  u32* fine;        // [n][2][L][W]
-  u32* block;       // [n][2][nbl][W]
+  u32* fine;        // (r) [2][L][W]
+  u32* block;       // (r) [2][nbl][W]
   u32* anch;        // [n][4][L][WA]: type * 2 + layout
-  u32* list;        // [n][list_cap]
-  u32* flat;        // [n][cap_flat]
-  Act* act;         // [n][2][cap_act]
-  u32* heads;       // [n][2][2][nb * nb]
+  u32* list;        // (r) [list_cap]
+  u32* flat;        // (r) [cap_flat]
+  Act* act;         // (r) [2][cap_act]
+  u32* heads;       // (r) [2][2][nb * nb]
   RoundState* rs;   // [n]
-  u64 list_cap;
 };
 
 __device__ __forceinline__ u32* cover_line(const Group& g, const RoundCfg& c, const RoundPtrs& p,
                                            u32 s, u32 o, u32 line) {
-  return p.fine + (((size_t)s * 2 + o) * g.L + line) * c.W;
+  return region_of(g, p.fine, s) + ((size_t)o * g.L + line) * c.W;
 }
-__device__ __forceinline__ u32* block_line(const RoundCfg& c, const RoundPtrs& p, u32 s, u32 o,
-                                           u32 bl) {
-  return p.block + (((size_t)s * 2 + o) * c.nbl + bl) * c.W;
+__device__ __forceinline__ u32* block_line(const Group& g, const RoundCfg& c, const RoundPtrs& p,
+                                           u32 s, u32 o, u32 bl) {
+  return region_of(g, p.block, s) + ((size_t)o * c.nbl + bl) * c.W;
 }
 // Anchors of k-mers of orientation `type`, as lines along `layout`.
 __device__ __forceinline__ u32* anchor_line(const Group& g, const RoundCfg& c, const RoundPtrs& p,
@@ -131,21 +141,8 @@ __global__ void k_round_init(Group g, RoundCfg c, RoundPtrs p) {
   const u32 s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= g.n) return;
   RoundState z = {};
-  z.open = 1;
-  z.hi = slice_top(c, 0);
-  z.fill_hi = ~0ull;
+  z.sl = first_slice(c);
   p.rs[s] = z;
-}
-
-// Append v for every lane with ok: slot of the lane in a counter.
-__device__ __forceinline__ u32 warp_append(u32* counter, bool ok) {
-  const u32 m = __ballot_sync(FULL, ok);
-  if (!m) return 0;
-  const u32 lane = threadIdx.x & 31, leader = __ffs(m) - 1;
-  u32 at = 0;
-  if (lane == leader) at = atomicAdd(counter, (u32)__popc(m));
-  at = __shfl_sync(FULL, at, leader);
-  return at + __popc(m & ((1u << lane) - 1u));
 }
 
 // Every candidate hashed once.  A block goes over tiles of 4096 consecutive
@@ -155,38 +152,43 @@ __device__ __forceinline__ u32 warp_append(u32* counter, bool ok) {
 // (the high word of mix64's last step z ^ (z >> 31) has at least a >= 1
 // leading zeros iff that of z has, so the hit test needs neither that step
 // nor the low word of the second product)
-template <bool KEYS>
-__global__ void __launch_bounds__(RD_THREADS) k_dense(Group g, const __grid_constant__ RoundCfg c,
-                                                      RoundPtrs p) {
-  __shared__ u32 stage[DENSE_STAGE];
-  __shared__ u8 lev[DENSE_STAGE];
-  __shared__ u32 count, lcnt[RD_LEVELS], lbase[RD_LEVELS];
-  const u32 s = blockIdx.y, tid = threadIdx.x, lane = tid & 31;
-  const u64 N = 2 * g.LL, zb = g.base[s] + SM_GAMMA;
-  RoundState& r = p.rs[s];
-  const u64 ntile = (N + DENSE_TILE - 1) / DENSE_TILE;
+template <u32 NT, u32 PER>   // threads of the block, at most; candidates of each in a tile
+struct DenseSmem {
+  static constexpr u32 STAGE = 8192;
+  u32 count, lcnt[RD_LEVELS], lbase[RD_LEVELS];
+  u32 stage[STAGE];
+  u8 lev[STAGE];
+};
+
+template <bool KEYS, u32 NT, u32 PER>
+__device__ void dense_body(const Group& g, const RoundCfg& c, const RoundPtrs& p, u32 s, Team team,
+                           RoundState& r, DenseSmem<NT, PER>& sm) {
+  const u32 tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
+  const u32 tile_n = PER * nt;
+  const u64 N = 2 * g.LL, zb = g.base[s] + SM_GAMMA, zstep = SM_GAMMA * nt;
+  const u64 ntile = (N + tile_n - 1) / tile_n;
   const u32 shift = 32 - c.a;
-  if (tid == 0) count = 0;
+  if (tid == 0) sm.count = 0;
   __syncthreads();
-  for (u64 tile = blockIdx.x; tile < ntile; tile += gridDim.x) {
-    const u64 i0 = tile * DENSE_TILE + tid;
+  for (u64 tile = team.rank; tile < ntile; tile += team.size) {
+    const u64 i0 = tile * tile_n + tid;
     u32 hits = 0;
     if (KEYS) {
-      for (u32 j = 0; j < DENSE_PER; ++j) {
-        const u64 i = i0 + j * RD_THREADS;
+      for (u32 j = 0; j < PER; ++j) {
+        const u64 i = i0 + j * nt;
         if (i < N && (u32)(g.keys[i] >> 32) >> shift == 0) hits |= 1u << j;
       }
     } else {
       u64 z = zb + SM_GAMMA * i0;
 #pragma unroll
-      for (u32 j = 0; j < DENSE_PER; ++j, z += SM_GAMMA * RD_THREADS) {
+      for (u32 j = 0; j < PER; ++j, z += zstep) {
         u64 h = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
         h = (h ^ (h >> 27)) * 0x94D049BB133111EBull;
         if ((u32)(h >> 32) >> shift == 0) hits |= 1u << j;
       }
-      if (i0 + (DENSE_PER - 1) * RD_THREADS >= N) {
-        for (u32 j = 0; j < DENSE_PER; ++j)
-          if (i0 + j * RD_THREADS >= N) hits &= ~(1u << j);
+      if (i0 + (u64)(PER - 1) * nt >= N) {
+        for (u32 j = 0; j < PER; ++j)
+          if (i0 + (u64)j * nt >= N) hits &= ~(1u << j);
       }
     }
     // this warp's hits, packed
@@ -198,45 +200,66 @@ __global__ void __launch_bounds__(RD_THREADS) k_dense(Group g, const __grid_cons
       if ((int)lane >= d) pre += o;
     }
     u32 at = 0;
-    if (lane == 31 && pre) at = atomicAdd(&count, pre);
+    if (lane == 31 && pre) at = atomicAdd(&sm.count, pre);
     at = __shfl_sync(FULL, at, 31) + pre - nh;
-    for (u32 m = hits; m; m &= m - 1) stage[at++] = (u32)(i0 + (__ffs(m) - 1) * RD_THREADS);
+    u32* list = region_of(g, p.list, s);
+    auto level_of = [&](u32 idx) {
+      const u64 key = KEYS ? g.keys[idx] : mix64(zb + SM_GAMMA * idx);
+      return c.lzmax - min((u32)__clzll((long long)key), c.lzmax);
+    };
+    auto put = [&](u32 t, u32 at2, u32 idx) {
+      if (at2 < c.lvl_cap[t]) list[c.lvl_off[t] + at2] = idx;
+      else atomicOr(&g.st[s].status, ST_NODE_OVF);
+    };
+    for (u32 m = hits; m; m &= m - 1, ++at) {
+      const u32 idx = (u32)(i0 + (u64)(__ffs(m) - 1) * nt);
+      if (at < sm.STAGE) {
+        sm.stage[at] = idx;
+      } else {  // more hits than the stage holds (not met by hashed priorities)
+        const u32 t = level_of(idx);
+        put(t, atomicAdd(&r.lvl_n[t], 1u), idx);
+      }
+    }
     __syncthreads();
-    const u32 n = count;
-    const bool last = tile + gridDim.x >= ntile;
-    if (n + DENSE_TILE > DENSE_STAGE || last) {
-      if (tid < RD_LEVELS) lcnt[tid] = 0;
+    const u32 n = min(sm.count, sm.STAGE);
+    const bool last = tile + team.size >= ntile;
+    if (n > sm.STAGE / 2 || last) {
+      if (tid < RD_LEVELS) sm.lcnt[tid] = 0;
       __syncthreads();
-      for (u32 i = tid; i < n; i += RD_THREADS) {
-        const u32 idx = stage[i];
-        const u64 key = KEYS ? g.keys[idx] : mix64(zb + SM_GAMMA * idx);
-        const u32 lz = min((u32)__clzll((long long)key), c.lzmax), t = c.lzmax - lz;
-        lev[i] = (u8)t;
-        atomicAdd(&lcnt[t], 1u);
+      for (u32 i = tid; i < n; i += nt) {
+        const u32 t = level_of(sm.stage[i]);
+        sm.lev[i] = (u8)t;
+        atomicAdd(&sm.lcnt[t], 1u);
       }
       __syncthreads();
       if (tid < c.nlev) {
-        lbase[tid] = lcnt[tid] ? atomicAdd(&r.lvl_n[tid], lcnt[tid]) : 0u;
-        lcnt[tid] = 0;
+        sm.lbase[tid] = sm.lcnt[tid] ? atomicAdd(&r.lvl_n[tid], sm.lcnt[tid]) : 0u;
+        sm.lcnt[tid] = 0;
       }
       __syncthreads();
-      u32* list = p.list + (size_t)s * p.list_cap;
-      for (u32 i = tid; i < n; i += RD_THREADS) {
-        const u32 t = lev[i], at2 = lbase[t] + atomicAdd(&lcnt[t], 1u);
-        if (at2 < c.lvl_cap[t]) list[c.lvl_off[t] + at2] = stage[i];
-        else atomicOr(&g.st[s].status, ST_NODE_OVF);
+      for (u32 i = tid; i < n; i += nt) {
+        const u32 t = sm.lev[i];
+        put(t, sm.lbase[t] + atomicAdd(&sm.lcnt[t], 1u), sm.stage[i]);
       }
       __syncthreads();
-      if (tid == 0) count = 0;
+      if (tid == 0) sm.count = 0;
     }
     __syncthreads();
   }
-  if (tid == 0 && blockIdx.x == 0) work_add(g, 0, N);
+}
+
+template <bool KEYS>
+__global__ void __launch_bounds__(DENSE_THREADS) k_dense(Group g,
+                                                         const __grid_constant__ RoundCfg c,
+                                                         RoundPtrs p) {
+  __shared__ DenseSmem<DENSE_THREADS, DENSE_PER> sm;
+  dense_body<KEYS>(g, c, p, blockIdx.y, Team{blockIdx.x, gridDim.x}, p.rs[blockIdx.y], sm);
+  if (threadIdx.x == 0 && blockIdx.x == 0) work_add(g, 0, 2 * g.LL);
 }
 
 // Word w of the bits [pos, pos + k) of a line, masked to them.
 __device__ __forceinline__ u32 window_word(const u32* line, u32 w, u32 pos, u32 end) {
-  u32 v = __ldcg(line + w);
+  u32 v = line[w];
   if (w == pos >> 5) v &= 0xFFFFFFFFu << (pos & 31u);
   if (w == end >> 5) v &= 0xFFFFFFFFu >> (31u - (end & 31u));
   return v;
@@ -247,33 +270,26 @@ __device__ __forceinline__ u32 window_word(const u32* line, u32 w, u32 pos, u32 
 // the few that pass by the whole warp.
 constexpr u32 PICK_LONGK = 96;
 template <bool LONG>
-__global__ void __launch_bounds__(RD_THREADS) k_pick(Group g, const __grid_constant__ RoundCfg c,
-                                                     RoundPtrs p) {
-  const u32 s = blockIdx.y;
-  if (g.st[s].done) return;
-  RoundState& r = p.rs[s];
-  const u32 L = g.L, k = g.k, tid = threadIdx.x, lane = tid & 31;
-  const u32 par = r.par, t = r.t;
-  const u64 lo = r.lo, hi = r.hi;
-  const bool flat = t >= c.nlev, take = r.open && !r.drain;
-  const u32 n1 = !take ? 0u : flat ? r.flat_n : min(r.lvl_n[t], c.lvl_cap[t]);
-  const u32 n2 = r.act[par ^ 1u];
-  const u32* list = flat ? p.flat + (size_t)s * c.cap_flat
-                         : p.list + (size_t)s * p.list_cap + c.lvl_off[t];
-  const Act* prev = p.act + ((size_t)s * 2 + (par ^ 1u)) * c.cap_act;
-  Act* cur = p.act + ((size_t)s * 2 + par) * c.cap_act;
-  u32* heads = p.heads + ((size_t)s * 2 + par) * 2 * c.nb * c.nb;
+__device__ void pick_body(const Group& g, const RoundCfg& c, const RoundPtrs& p, u32 s, Team team,
+                          const Slice& sl, u32 n1, u32 n2, u32* count) {
+  const u32 L = g.L, k = g.k, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
+  const u32 par = sl.par, t = sl.t;
+  const u64 lo = sl.lo, hi = sl.hi;
+  const u32* list = t >= c.nlev ? region_of(g, p.flat, s)
+                                : region_of(g, p.list, s) + c.lvl_off[t];
+  const Act* prev = region_of(g, p.act, s) + (size_t)(par ^ 1u) * c.cap_act;
+  Act* cur = region_of(g, p.act, s) + (size_t)par * c.cap_act;
+  u32* heads = region_of(g, p.heads, s) + (size_t)par * 2 * c.nb * c.nb;
   const u64 zb = g.base[s] + SM_GAMMA;
-  if (blockIdx.x == 0 && tid == 0) r.left = 0;
   const u32 total = n1 + n2;
-  for (u32 i0 = blockIdx.x * blockDim.x; i0 < total; i0 += gridDim.x * blockDim.x) {
+  for (u32 i0 = team.rank * nt; i0 < total; i0 += team.size * nt) {
     const u32 i = i0 + tid;
     bool ok = i < total;
     u32 o = 0, y = 0, x = 0;
     u64 key = 0;
     if (ok) {
       if (i < n1) {
-        const u32 idx = __ldg(list + i);
+        const u32 idx = list[i];
         key = g.keys ? g.keys[idx] : mix64(zb + SM_GAMMA * idx);
         ok = key >= lo && key <= hi;
         if (ok) {
@@ -283,16 +299,16 @@ __global__ void __launch_bounds__(RD_THREADS) k_pick(Group g, const __grid_const
           x = rr - y * L;
         }
       } else {
-        const Act e = prev[i - n1];
-        key = e.key;
-        o = e.pos >> 31;
-        y = (e.pos >> 15) & 0x7FFFu;
-        x = e.pos & 0x7FFFu;
+        const uint4 e = *reinterpret_cast<const uint4*>(prev + (i - n1));
+        key = (u64)e.y << 32 | e.x;
+        o = e.z >> 31;
+        y = (e.z >> 15) & 0x7FFFu;
+        x = e.z & 0x7FFFu;
       }
     }
     const u32 line = o ? x : y, pos = o ? y : x, end = pos + k - 1;
     const u32* fl = cover_line(g, c, p, s, o, line);
-    const u32* bl = c.bs ? block_line(c, p, s, o, line >> c.bs) : fl;
+    const u32* bl = c.bs ? block_line(g, c, p, s, o, line >> c.bs) : fl;
     const u32 w0 = pos >> 5, w1 = end >> 5;
     if (!LONG) {
       if (ok) {
@@ -308,23 +324,22 @@ __global__ void __launch_bounds__(RD_THREADS) k_pick(Group g, const __grid_const
       if (ok) {
         const u32 wm = (w0 + w1) >> 1;
         ok = (window_word(fl, w0, pos, end) | window_word(bl, w0, pos, end) |
-              window_word(fl, w1, pos, end) | window_word(bl, w1, pos, end) | __ldcg(fl + wm) |
-              __ldcg(bl + wm)) == 0;
+              window_word(fl, w1, pos, end) | window_word(bl, w1, pos, end) | fl[wm] | bl[wm]) == 0;
       }
       // the words between, 32 at a time, one candidate after another
       for (u32 m = __ballot_sync(FULL, ok); m; m &= m - 1) {
         const u32 src = __ffs(m) - 1;
-        const u32 so = __shfl_sync(FULL, o, src), sl = __shfl_sync(FULL, line, src);
+        const u32 so = __shfl_sync(FULL, o, src), ln = __shfl_sync(FULL, line, src);
         const u32 a0 = __shfl_sync(FULL, w0, src) + 1, a1 = __shfl_sync(FULL, w1, src);
-        const u32* f2 = cover_line(g, c, p, s, so, sl);
-        const u32* b2 = block_line(c, p, s, so, sl >> c.bs);
+        const u32* f2 = cover_line(g, c, p, s, so, ln);
+        const u32* b2 = block_line(g, c, p, s, so, ln >> c.bs);
         u32 v = 0;
-        for (u32 w = a0 + lane; w < a1; w += 32) v |= __ldcg(f2 + w) | __ldcg(b2 + w);
+        for (u32 w = a0 + lane; w < a1; w += 32) v |= f2[w] | b2[w];
         const bool hit = __any_sync(FULL, v != 0);
         if (lane == src && hit) ok = false;
       }
     }
-    const u32 slot = warp_append(&r.act[par], ok);
+    const u32 slot = warp_append(count, ok);
     if (ok && slot < c.cap_act) {
       Act e;
       e.key = key;
@@ -333,7 +348,27 @@ __global__ void __launch_bounds__(RD_THREADS) k_pick(Group g, const __grid_const
       *reinterpret_cast<uint4*>(cur + slot) = *reinterpret_cast<uint4*>(&e);
     }
   }
-  if (tid == 0 && blockIdx.x == 0) work_add(g, 1, total);
+}
+
+// Entries of the current slice's list.
+__device__ __forceinline__ u32 slice_entries(const RoundCfg& c, const RoundState& r,
+                                             const Slice& sl) {
+  return !sl.open || sl.drain ? 0u : sl.t >= c.nlev ? r.flat_n : min(r.lvl_n[sl.t], c.lvl_cap[sl.t]);
+}
+
+template <bool LONG>
+__global__ void __launch_bounds__(RD_THREADS) k_pick(Group g, const __grid_constant__ RoundCfg c,
+                                                     RoundPtrs p) {
+  const u32 s = blockIdx.y;
+  if (g.st[s].done) return;
+  RoundState& r = p.rs[s];
+  const Slice sl = r.sl;
+  const u32 n1 = slice_entries(c, r, sl), n2 = r.act[sl.par ^ 1u];
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    r.taken = 0;
+    work_add(g, 1, n1 + n2);
+  }
+  pick_body<LONG>(g, c, p, s, Team{blockIdx.x, gridDim.x}, sl, n1, n2, &r.act[sl.par]);
 }
 
 // Bins that the cells [a, a + len) of a ring of L cells touch, as n1 bins
@@ -400,7 +435,7 @@ __device__ void cover_kmer(const Group& g, const RoundCfg& c, const RoundPtrs& p
         f0 = j0 << c.bs;
         f1 = min(j1 << c.bs, L);
         for (u32 bl = j0 + j; bl < j1; bl += G)
-          set_bit_copies(block_line(c, p, s, o ^ 1u, bl), line, L, bits);
+          set_bit_copies(block_line(g, c, p, s, o ^ 1u, bl), line, L, bits);
       }
     }
     for (u32 q = a + j; q < f0; q += G)
@@ -410,19 +445,18 @@ __device__ void cover_kmer(const Group& g, const RoundCfg& c, const RoundPtrs& p
   }
 }
 
-// The step from one round to the next (one thread per sample).
-__device__ void round_step(const Group& g, const RoundCfg& c, RoundState& r, SampleState& st,
-                           u32 n) {
+// The step from one round of n active candidates, `left` of them undecided,
+// to the next.  True if the sample is done.
+__device__ bool round_step(const RoundCfg& c, Slice& r, u32 n, u32 left, u32& rounds,
+                           u32& status) {
   if (n > c.cap_act) {
     // too many: this round decided nothing; the same undecided candidates
     // again, with a narrower slice, or with none if it is one key wide
-    r.act[r.par] = 0;
     if (r.hi == r.lo) r.drain = 1;
     else r.hi = r.lo + (r.hi - r.lo) / 8;
-    return;
+    return false;
   }
   r.par ^= 1u;
-  r.act[r.par] = 0;
   if (r.drain) {
     r.drain = 0;
   } else if (r.open) {
@@ -444,139 +478,166 @@ __device__ void round_step(const Group& g, const RoundCfg& c, RoundState& r, Sam
         r.refill = 1;  // k_refill opens the next slice
         r.open = 0;
         r.fill_hi = ~0ull;
-        r.flat_n = 0;
       } else if (!listed) {
         r.hi = r.hi < r.fill_hi ? r.hi : r.fill_hi;
       }
     }
   }
-  if (n) st.rounds += 1;
-  if (r.finished && r.left == 0) st.done = 1;
-  else if (st.rounds >= c.round_cap) {
-    st.status |= ST_ROUND_CAP;
-    st.done = 1;
+  if (n) rounds += 1;
+  if (r.finished && left == 0) return true;
+  if (rounds >= c.round_cap) {
+    status |= ST_ROUND_CAP;
+    return true;
   }
+  return false;
+}
+
+// The step after k_refill listed flat_n candidates.
+__device__ __forceinline__ void refill_step(const RoundCfg& c, Slice& r, u32 flat_n) {
+  if (flat_n > c.cap_flat) {
+    // more than the list holds: fewer priorities, next time
+    r.fill_hi = r.lo + (r.fill_hi - r.lo) / 8;
+  } else {
+    r.refill = 0;
+    r.open = 1;
+    r.hi = r.hi < r.fill_hi ? r.hi : r.fill_hi;
+  }
+}
+
+// Bins of the round after, emptied while this one is resolved.
+__device__ __forceinline__ void clear_bins(const Group& g, const RoundCfg& c, const RoundPtrs& p,
+                                           u32 s, Team team, u32 buf) {
+  u32* nx = region_of(g, p.heads, s) + (size_t)buf * 2 * c.nb * c.nb;
+  for (u32 i = team.rank * blockDim.x + threadIdx.x; i < 2 * c.nb * c.nb;
+       i += team.size * blockDim.x)
+    nx[i] = NONE32;
 }
 
 // G lanes per active candidate.  Bins are about 4 sqrt(k) cells wide, which
 // leaves one or two active candidates in each and k / 16 bins to look at.
+// Adds this thread's accepted candidates to taken.
+template <int G>
+__device__ void resolve_body(const Group& g, const RoundCfg& c, const RoundPtrs& p, u32 s,
+                             Team team, u32 par, u32 n, u32* nodes, u32& taken) {
+  SampleState& st = g.st[s];
+  const u32 L = g.L, k = g.k, tid = threadIdx.x;
+  const u32* heads = region_of(g, p.heads, s) + (size_t)par * 2 * c.nb * c.nb;
+  const Act* cur = region_of(g, p.act, s) + (size_t)par * c.cap_act;
+  const u32 j = tid & (G - 1);
+  const u32 gmask = G == 32 ? FULL : ((1u << (G & 31)) - 1u) << ((tid & 31) & ~(G - 1));
+  const u32 gpb = blockDim.x / G;
+  for (u32 i = team.rank * gpb + tid / G; i < n; i += team.size * gpb) {
+    const uint4 raw = *reinterpret_cast<const uint4*>(cur + i);
+    const u64 key = (u64)raw.y << 32 | raw.x;
+    const u32 o = raw.z >> 31, y = (raw.z >> 15) & 0x7FFFu, x = raw.z & 0x7FFFu;
+    const u32 line = o ? x : y, pos = o ? y : x;
+    // conflicting anchors: on its own line less than k away; crossing ones
+    // on the k lines of its cells, from k - 1 cells before its line to it
+    const BinRun same(ring_sub(pos, k - 1, L), 2 * k - 1, L, c.b);
+    const BinRun cl(pos, k, L, c.b), cp(ring_sub(line, k - 1, L), k, L, c.b);
+    // the candidates of one bin (its place among the bins of orientation bo)
+    auto walk = [&](u32 bo, u32 bl, u32 bp) -> bool {
+      const u32 by = bo ? bp : bl, bx = bo ? bl : bp;  // stored by (row, column)
+      u32 e = heads[((size_t)bo * c.nb + by) * c.nb + bx];
+      for (u32 guard = 0; e != NONE32 && guard < n; ++guard) {
+        const uint4 a = *reinterpret_cast<const uint4*>(cur + e);
+        e = a.w;
+        if (((u64)a.y << 32 | a.x) >= key) continue;
+        const u32 ay = (a.z >> 15) & 0x7FFFu, ax = a.z & 0x7FFFu;
+        const u32 aline = bo ? ax : ay, apos = bo ? ay : ax;
+        if (bo == o) {
+          const u32 d = ring_sub(apos, pos, L);
+          if (aline == line && (d < k || d > L - k)) return true;
+        } else if (ring_sub(aline, pos, L) < k && ring_sub(line, apos, L) < k) {
+          return true;
+        }
+      }
+      return false;
+    };
+    bool beaten = false;
+    if (G == 1) {
+      for (u32 q = 0; q < same.n && !beaten; ++q) beaten = walk(o, line >> c.b, same.bin(q));
+      for (u32 q1 = 0; q1 < cl.n && !beaten; ++q1)
+        for (u32 q2 = 0; q2 < cp.n && !beaten; ++q2)
+          beaten = walk(o ^ 1u, cl.bin(q1), cp.bin(q2));
+    } else {
+      const u32 nbin = same.n + cl.n * cp.n;
+      for (u32 q0 = 0; q0 < nbin && !beaten; q0 += G) {
+        const u32 q = q0 + j;
+        if (q < same.n) {
+          beaten = walk(o, line >> c.b, same.bin(q));
+        } else if (q < nbin) {
+          const u32 qq = q - same.n, q1 = qq / cp.n;
+          beaten = walk(o ^ 1u, cl.bin(q1), cp.bin(qq - q1 * cp.n));
+        }
+        beaten = (__ballot_sync(gmask, beaten) & gmask) != 0;
+      }
+    }
+    if (beaten) continue;
+    u32 node = 0;
+    if (j == 0) node = atomicAdd(nodes, 1u);
+    if (G > 1) node = __shfl_sync(gmask, node, 0, G);
+    if (node >= g.cap_nodes) {
+      if (j == 0) atomicOr(&st.status, ST_NODE_OVF);
+      continue;
+    }
+    if (j == 0) {
+      const size_t nd = (size_t)s * g.cap_nodes + node;
+      const u32 cell = y * L + x;
+      g.node_key[nd] = key;
+      g.node_idx[nd] = o * (u32)g.LL + cell;
+      g.node_pos[nd] = raw.z;
+      g.owner[(size_t)s * g.LL + cell] = node;
+      ++taken;
+    }
+    if (G == 1 || j < 2) {
+      const u32 bits = L + 2 * k;
+      for (u32 lay = G == 1 ? 0 : j; lay < (G == 1 ? 2 : j + 1); ++lay)
+        set_bit_copies(anchor_line(g, c, p, s, o, lay, lay ? x : y), lay ? y : x, L, bits);
+    }
+    cover_kmer<G>(g, c, p, s, o, line, pos, j);
+  }
+}
+
 template <int G>
 __global__ void __launch_bounds__(RD_THREADS) k_resolve(Group g,
                                                         const __grid_constant__ RoundCfg c,
                                                         RoundPtrs p) {
-  __shared__ u32 left_sh;
+  __shared__ u32 taken_sh;
   const u32 s = blockIdx.y;
   SampleState& st = g.st[s];
   if (st.done) return;
   RoundState& r = p.rs[s];
-  const u32 L = g.L, k = g.k, tid = threadIdx.x;
-  const u32 par = r.par, n = r.act[par];
+  const u32 tid = threadIdx.x, par = r.sl.par, n = r.act[par];
+  const Team team{blockIdx.x, gridDim.x};
   const bool over = n > c.cap_act;
-  // the bins of the next round
-  {
-    u32* nx = p.heads + ((size_t)s * 2 + (over ? par : par ^ 1u)) * 2 * c.nb * c.nb;
-    for (u32 i = blockIdx.x * RD_THREADS + tid; i < 2 * c.nb * c.nb; i += gridDim.x * RD_THREADS)
-      nx[i] = NONE32;
-  }
-  if (tid == 0) left_sh = 0;
+  clear_bins(g, c, p, s, team, over ? par : par ^ 1u);
+  if (tid == 0) taken_sh = 0;
   __syncthreads();
-  const u32* heads = p.heads + ((size_t)s * 2 + par) * 2 * c.nb * c.nb;
-  const Act* cur = p.act + ((size_t)s * 2 + par) * c.cap_act;
-  const u32 j = tid & (G - 1);
-  const u32 gmask = G == 32 ? FULL : ((1u << (G & 31)) - 1u) << ((tid & 31) & ~(G - 1));
-  constexpr u32 GPB = RD_THREADS / G;
-  u32 left = 0, taken = 0;
-  if (!over) {
-    for (u32 i = blockIdx.x * GPB + tid / G; i < n; i += gridDim.x * GPB) {
-      const uint4 raw = __ldg(reinterpret_cast<const uint4*>(cur + i));
-      const u64 key = (u64)raw.y << 32 | raw.x;
-      const u32 o = raw.z >> 31, y = (raw.z >> 15) & 0x7FFFu, x = raw.z & 0x7FFFu;
-      const u32 line = o ? x : y, pos = o ? y : x;
-      // conflicting anchors: on its own line less than k away; crossing ones
-      // on the k lines of its cells, from k - 1 cells before its line to it
-      const BinRun same(ring_sub(pos, k - 1, L), 2 * k - 1, L, c.b);
-      const BinRun cl(pos, k, L, c.b), cp(ring_sub(line, k - 1, L), k, L, c.b);
-      const u32 nbin = same.n + cl.n * cp.n;
-      bool beaten = false;
-      for (u32 q0 = 0; q0 < nbin; q0 += G) {
-        const u32 q = q0 + j;
-        if (q < nbin) {
-          u32 bo, bl, bp;  // orientation, bin along its line's index, bin along the line
-          if (q < same.n) {
-            bo = o;
-            bl = line >> c.b;
-            bp = same.bin(q);
-          } else {
-            const u32 qq = q - same.n, q1 = qq / cp.n;
-            bo = o ^ 1u;
-            bl = cl.bin(q1);
-            bp = cp.bin(qq - q1 * cp.n);
-          }
-          // bins are stored by (row, column)
-          const u32 by = bo ? bp : bl, bx = bo ? bl : bp;
-          u32 e = __ldg(heads + ((size_t)bo * c.nb + by) * c.nb + bx);
-          for (u32 guard = 0; e != NONE32 && guard < n; ++guard) {
-            const uint4 a = __ldg(reinterpret_cast<const uint4*>(cur + e));
-            e = a.w;
-            if (((u64)a.y << 32 | a.x) >= key) continue;
-            const u32 ay = (a.z >> 15) & 0x7FFFu, ax = a.z & 0x7FFFu;
-            const u32 aline = bo ? ax : ay, apos = bo ? ay : ax;
-            if (bo == o) {
-              const u32 d = ring_sub(apos, pos, L);
-              if (aline == line && (d < k || d > L - k)) { beaten = true; break; }
-            } else if (ring_sub(aline, pos, L) < k && ring_sub(line, apos, L) < k) {
-              beaten = true;
-              break;
-            }
-          }
-        }
-        if (G > 1) beaten = (__ballot_sync(gmask, beaten) & gmask) != 0;
-        if (beaten) break;
-      }
-      if (beaten) {
-        if (j == 0) ++left;
-        continue;
-      }
-      u32 node = 0;
-      if (j == 0) node = atomicAdd(&st.n_nodes, 1u);
-      if (G > 1) node = __shfl_sync(gmask, node, 0, G);
-      if (node >= g.cap_nodes) {
-        if (j == 0) atomicOr(&st.status, ST_NODE_OVF);
-        continue;
-      }
-      if (j == 0) {
-        const size_t nd = (size_t)s * g.cap_nodes + node;
-        const u32 cell = y * L + x;
-        g.node_key[nd] = key;
-        g.node_idx[nd] = o * (u32)g.LL + cell;
-        g.node_pos[nd] = raw.z;
-        g.owner[(size_t)s * g.LL + cell] = node;
-        ++taken;
-      }
-      if (G == 1 || j < 2) {
-        const u32 bits = L + 2 * k;
-        for (u32 lay = G == 1 ? 0 : j; lay < (G == 1 ? 2 : j + 1); ++lay)
-          set_bit_copies(anchor_line(g, c, p, s, o, lay, lay ? x : y), lay ? y : x, L, bits);
-      }
-      cover_kmer<G>(g, c, p, s, o, line, pos, j);
-    }
-  }
-  left = __reduce_add_sync(FULL, left);
+  u32 taken = 0;
+  if (!over) resolve_body<G>(g, c, p, s, team, par, n, &st.n_nodes, taken);
   taken = __reduce_add_sync(FULL, taken);
-  if ((tid & 31) == 0) {
-    if (left) atomicAdd(&left_sh, left);
-    if (taken) work_add(g, 3, taken);
-  }
+  if ((tid & 31) == 0 && taken) atomicAdd(&taken_sh, taken);
   __syncthreads();
   if (tid == 0) {
-    if (left_sh) atomicAdd(&r.left, left_sh);
+    if (taken_sh) {
+      atomicAdd(&r.taken, taken_sh);
+      work_add(g, 3, taken_sh);
+    }
     if (blockIdx.x == 0) work_add(g, 2, over ? 0 : n);
     __threadfence();
     if (atomicAdd(&r.ticket, 1u) == gridDim.x - 1) {
       __threadfence();
       r.ticket = 0;
-      r.left = __ldcg(&r.left);
-      round_step(g, c, r, st, n);
+      Slice sl = r.sl;
+      u32 rounds = st.rounds, status = __ldcg(&st.status);
+      const bool was_refill = sl.refill;
+      if (round_step(c, sl, n, n - __ldcg(&r.taken), rounds, status)) st.done = 1;
+      r.act[sl.par] = 0;  // the next round's buffer (this one's, if it was overfull)
+      if (sl.refill && !was_refill) r.flat_n = 0;
+      r.sl = sl;
+      st.rounds = rounds;
+      st.status = status;
     }
   }
 }
@@ -584,30 +645,26 @@ __global__ void __launch_bounds__(RD_THREADS) k_resolve(Group g,
 // The candidates of every line still live once the list is used up, those
 // with priorities in [lo, fill_hi]: the window OR of a line's cover bits,
 // doubling the window until it holds k cells.
-__global__ void __launch_bounds__(RD_THREADS) k_refill(Group g, const __grid_constant__ RoundCfg c,
-                                                       RoundPtrs p, u32 lines_per_block) {
-  __shared__ u32 buf[2][REFILL_WORDS];
-  const u32 s = blockIdx.y;
-  if (g.st[s].done) return;
-  RoundState& r = p.rs[s];
-  if (!r.refill) return;
-  const u32 L = g.L, k = g.k, W = c.W, tid = threadIdx.x;
-  const u64 lo = r.lo, hi = r.fill_hi, zb = g.base[s] + SM_GAMMA;
-  u32* flat = p.flat + (size_t)s * c.cap_flat;
+__device__ void refill_body(const Group& g, const RoundCfg& c, const RoundPtrs& p, u32 s,
+                            Team team, const Slice& sl, u32 lines_per_block, u32* flat_n,
+                            u32 (*buf)[REFILL_WORDS]) {
+  const u32 L = g.L, k = g.k, W = c.W, tid = threadIdx.x, nt = blockDim.x;
+  const u64 lo = sl.lo, hi = sl.fill_hi, zb = g.base[s] + SM_GAMMA;
+  u32* flat = region_of(g, p.flat, s);
   const u32 groups = (2 * L + lines_per_block - 1) / lines_per_block;
-  for (u32 gr = blockIdx.x; gr < groups; gr += gridDim.x) {
+  for (u32 gr = team.rank; gr < groups; gr += team.size) {
     const u32 l0 = gr * lines_per_block, nl = min(lines_per_block, 2 * L - l0), nw = nl * W;
-    for (u32 i = tid; i < nw; i += RD_THREADS) {
+    for (u32 i = tid; i < nw; i += nt) {
       const u32 ll = i / W, w = i - ll * W, o = l0 + ll >= L, line = l0 + ll - (o ? L : 0u);
       u32 v = cover_line(g, c, p, s, o, line)[w];
-      if (c.bs) v |= block_line(c, p, s, o, line >> c.bs)[w];
+      if (c.bs) v |= block_line(g, c, p, s, o, line >> c.bs)[w];
       buf[0][i] = v;
     }
     __syncthreads();
     u32 from = 0;
     for (u32 m = 1; m < k;) {
       const u32 d = min(m, k - m), dw = d >> 5, db = d & 31u;
-      for (u32 i = tid; i < nw; i += RD_THREADS) {
+      for (u32 i = tid; i < nw; i += nt) {
         const u32 w = i % W;
         const u32 v0 = w + dw < W ? buf[from][i + dw] : 0u;
         const u32 v1 = w + dw + 1 < W ? buf[from][i + dw + 1] : 0u;
@@ -618,7 +675,7 @@ __global__ void __launch_bounds__(RD_THREADS) k_refill(Group g, const __grid_con
       __syncthreads();
     }
     const u32 WL = (L + 31) / 32, items = nl * WL;
-    for (u32 i0 = 0; i0 < items; i0 += RD_THREADS) {
+    for (u32 i0 = 0; i0 < items; i0 += nt) {
       const u32 i = i0 + tid;
       u32 live = 0;
       u64 idx0 = 0, step = 1;
@@ -643,27 +700,33 @@ __global__ void __launch_bounds__(RD_THREADS) k_refill(Group g, const __grid_con
         if ((int)lane >= d) pre += v;
       }
       u32 at = 0;
-      if (lane == 31 && pre) at = atomicAdd(&r.flat_n, pre);
+      if (lane == 31 && pre) at = atomicAdd(flat_n, pre);
       at = __shfl_sync(FULL, at, 31) + pre - nh;
       for (u32 m = live; m; m &= m - 1, ++at)
         if (at < c.cap_flat) flat[at] = (u32)(idx0 + step * (__ffs(m) - 1));
     }
     __syncthreads();
   }
-  if (tid == 0) {
+}
+
+__global__ void __launch_bounds__(RD_THREADS) k_refill(Group g, const __grid_constant__ RoundCfg c,
+                                                       RoundPtrs p, u32 lines_per_block) {
+  __shared__ u32 buf[2][REFILL_WORDS];
+  const u32 s = blockIdx.y;
+  if (g.st[s].done) return;
+  RoundState& r = p.rs[s];
+  if (!r.sl.refill) return;
+  const Slice sl = r.sl;
+  refill_body(g, c, p, s, Team{blockIdx.x, gridDim.x}, sl, lines_per_block, &r.flat_n, buf);
+  if (threadIdx.x == 0) {
     __threadfence();
     if (atomicAdd(&r.ticket2, 1u) == gridDim.x - 1) {
       __threadfence();
       r.ticket2 = 0;
-      if (__ldcg(&r.flat_n) > c.cap_flat) {
-        // more than the list holds: fewer priorities, next time
-        r.fill_hi = lo + (hi - lo) / 8;
-        r.flat_n = 0;
-      } else {
-        r.refill = 0;
-        r.open = 1;
-        r.hi = r.hi < hi ? r.hi : hi;
-      }
+      Slice nx = sl;
+      refill_step(c, nx, __ldcg(&r.flat_n));
+      if (nx.refill) r.flat_n = 0;
+      r.sl = nx;
     }
   }
 }
@@ -679,11 +742,11 @@ __global__ void k_round_check(Group g, u32* n_active) {
 // cell takes the one of smaller priority, in one pass, as node y L + x; its
 // contacts are its right and lower neighbour.
 // ---------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_sites(Group g) {
-  const u32 s = blockIdx.y, L = g.L;
+__device__ void sites_body(const Group& g, u32 s, Team team) {
+  const u32 L = g.L, nt = blockDim.x;
   const u64 zb = g.base[s] + SM_GAMMA;
   const size_t nb = (size_t)s * g.cap_nodes;
-  for (u64 i = blockIdx.x * 256ull + threadIdx.x; i < g.LL; i += gridDim.x * 256ull) {
+  for (u64 i = team.rank * nt + threadIdx.x; i < g.LL; i += team.size * nt) {
     const u64 h = g.keys ? g.keys[i] : mix64(zb + SM_GAMMA * i);
     const u64 v = g.keys ? g.keys[i + g.LL] : mix64(zb + SM_GAMMA * (i + g.LL));
     const u32 o = v < h, y = (u32)i / L, x = (u32)i - y * L;
@@ -691,6 +754,11 @@ __global__ void __launch_bounds__(256) k_sites(Group g) {
     g.node_idx[nb + i] = (u32)(i + (o ? g.LL : 0));
     g.node_pos[nb + i] = (o << 31) | (y << 15) | x;
   }
+}
+
+__global__ void __launch_bounds__(256) k_sites(Group g) {
+  const u32 s = blockIdx.y;
+  sites_body(g, s, Team{blockIdx.x, gridDim.x});
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     SampleState& st = g.st[s];
     st.n_nodes = (u32)g.LL;
@@ -718,9 +786,8 @@ __device__ __forceinline__ void put_edge(const Group& g, u32 s, SampleState& st,
     atomicOr(&st.status, ST_EDGE_OVF);
     return;
   }
-  const size_t i = (size_t)s * g.cap_edges + at;
-  g.etime[i] = time;
-  g.elink[i] = make_uint4(m1, m2, (dx & 0xFFFFu) | (dy << 16), 0);
+  region_of(g, g.etime, s)[at] = time;
+  region_of(g, g.elink, s)[at] = make_uint4(m1, m2, (dx & 0xFFFFu) | (dy << 16), 0);
 }
 
 // Histogram of a block's edge times, added to the sample's at the end.
@@ -738,20 +805,18 @@ struct TimeHist {
     __syncthreads();
     if (h)
       for (u32 i = threadIdx.x; i < EHIST; i += blockDim.x)
-        if (h[i]) atomicAdd(&g.ehist[(size_t)s * (EHIST + SUB_BINS) + i], h[i]);
+        if (h[i]) atomicAdd(region_of(g, g.ehist, s) + i, h[i]);
   }
 };
 
-__global__ void __launch_bounds__(256) k_site_contacts(Group g) {
-  const u32 s = blockIdx.y, L = g.L;
+__device__ void site_contacts_body(const Group& g, u32 s, Team team, u32* hist_sh) {
+  const u32 L = g.L, nt = blockDim.x;
   SampleState& st = g.st[s];
   const u64* K = g.node_key + (size_t)s * g.cap_nodes;
   const u32* P = g.node_pos + (size_t)s * g.cap_nodes;
-  __shared__ u32 hist_sh[EHIST];
-  if (st.sdone) return;
   TimeHist hist(g, hist_sh);
   u32 cnt[3] = {0, 0, 0};
-  for (u64 i = blockIdx.x * 256ull + threadIdx.x; i < g.LL; i += gridDim.x * 256ull) {
+  for (u64 i = team.rank * nt + threadIdx.x; i < g.LL; i += team.size * nt) {
     const u32 m = (u32)i, y = m / L, x = m - y * L;
     const u32 right = x + 1 == L ? m + 1 - L : m + 1, down = y + 1 == L ? x : m + L;
     const u64 km = K[m];
@@ -772,7 +837,13 @@ __global__ void __launch_bounds__(256) k_site_contacts(Group g) {
   }
   contact_counts(st, cnt);
   hist.flush(g, s);
-  if (blockIdx.x == 0 && threadIdx.x == 0) st.n_edges = 2 * (u32)g.LL;
+  if (team.rank == 0 && threadIdx.x == 0) st.n_edges = 2 * (u32)g.LL;
+}
+
+__global__ void __launch_bounds__(256) k_site_contacts(Group g) {
+  __shared__ u32 hist_sh[EHIST];
+  if (g.st[blockIdx.y].sdone) return;
+  site_contacts_body(g, blockIdx.y, Team{blockIdx.x, gridDim.x}, hist_sh);
 }
 
 // ---------------------------------------------------------------------
@@ -792,25 +863,22 @@ __global__ void __launch_bounds__(256) k_site_contacts(Group g) {
 // ---------------------------------------------------------------------
 __device__ __forceinline__ u32 anchor_bits(const u32* line, u32 a, u32 n) {
   const u32 w = a >> 5;
-  const u32 v = __funnelshift_r(__ldg(line + w), __ldg(line + w + 1), a & 31u);
+  const u32 v = __funnelshift_r(line[w], line[w + 1], a & 31u);
   return n < 32 ? v & ((1u << n) - 1u) : v;
 }
 
 template <int G>
-__global__ void __launch_bounds__(256) k_contacts(Group g, const __grid_constant__ RoundCfg c,
-                                                  RoundPtrs p) {
-  const u32 s = blockIdx.y, L = g.L, k = g.k, tid = threadIdx.x;
+__device__ void contacts_body(const Group& g, const RoundCfg& c, const RoundPtrs& p, u32 s,
+                              Team team, u32* edges, u32* hist_sh) {
+  const u32 L = g.L, k = g.k, tid = threadIdx.x;
   SampleState& st = g.st[s];
   const u32 nn = min(st.n_nodes, g.cap_nodes);
   const size_t nb = (size_t)s * g.cap_nodes;
   const u32* anchor_node = g.owner + (size_t)s * g.LL;
-  __shared__ u32 hist_sh[EHIST];
-  if (st.sdone) return;
   TimeHist hist(g, hist_sh);
-  const u32 j = tid & (G - 1);
-  constexpr u32 GPB = 256 / G;
+  const u32 j = tid & (G - 1), gpb = blockDim.x / G;
   u32 cnt[3] = {0, 0, 0};
-  for (u32 m = blockIdx.x * GPB + tid / G; m < nn; m += gridDim.x * GPB) {
+  for (u32 m = team.rank * gpb + tid / G; m < nn; m += team.size * gpb) {
     const u32 pk = g.node_pos[nb + m];
     const u64 key = g.node_key[nb + m];
     const u32 o = pk >> 31, y = (pk >> 15) & 0x7FFFu, x = pk & 0x7FFFu;
@@ -818,10 +886,10 @@ __global__ void __launch_bounds__(256) k_contacts(Group g, const __grid_constant
     // contact with the k-mer anchored at (line al, position ap) in the
     // layout of o, displaced by (along, across) lines of o
     auto emit = [&](u32 al, u32 ap, u32 along, u32 across, u32 run, bool mixed, u32 copies) {
-      const u32 b = __ldg(anchor_node + (o ? ap * L + al : al * L + ap));
+      const u32 b = anchor_node[o ? ap * L + al : al * L + ap];
       const u64 kb = g.node_key[nb + b];
       if (b != m) cnt[mixed ? 2 : o] += run;
-      const u32 at = atomicAdd(&st.n_edges, copies);
+      const u32 at = atomicAdd(edges, copies);
       const u64 time = tmax(key, kb);
       hist.add(time, copies);
       for (u32 i = 0; i < copies; ++i)
@@ -875,6 +943,15 @@ __global__ void __launch_bounds__(256) k_contacts(Group g, const __grid_constant
   }
   contact_counts(st, cnt);
   hist.flush(g, s);
+}
+
+template <int G>
+__global__ void __launch_bounds__(256) k_contacts(Group g, const __grid_constant__ RoundCfg c,
+                                                  RoundPtrs p) {
+  __shared__ u32 hist_sh[EHIST];
+  if (g.st[blockIdx.y].sdone) return;
+  contacts_body<G>(g, c, p, blockIdx.y, Team{blockIdx.x, gridDim.x},
+                   &g.st[blockIdx.y].n_edges, hist_sh);
 }
 
 }  // namespace rsak

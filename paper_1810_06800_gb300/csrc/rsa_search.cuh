@@ -14,9 +14,8 @@
 //              halve the edges of the window;
 //   k_collect  once the window holds at most FIN_EDGES edges: those, with
 //              the roots of their ends and the displacement between the roots;
-//   k_finish   one block per sample: these edges sorted by time in shared
-//              memory and the rest of the bisection there, on the graph of
-//              the roots;
+//   k_finish   one block per sample: the rest of the search in shared memory,
+//              on the graph of the roots; the last 32 edges one by one;
 //   k_rank     n_c, the k-mers of priority <= T_c.
 // Samples whose whole graph has at most FIN_EDGES edges need no probe.
 // That hi itself wraps is assumed until a probe shows it (the jammed lattice
@@ -30,11 +29,15 @@
 
 namespace rsak {
 
-constexpr u32 FIN_EDGES = 4096;
+constexpr u32 FIN_EDGES = 2048;
 constexpr u32 FIN_THREADS = 512;
 constexpr u32 FIN_SLOTS = 4 * FIN_EDGES;  // hash slots for the roots of the window (4 B: as much
                                           // as 2 FIN_EDGES union-find words)
 constexpr u32 SUB_BINS = 128;
+// per sample: the time histogram, and two sets of the counts of a probe
+constexpr u32 SUB_WRAP = SUB_BINS, SUB_A = SUB_BINS + 1, SUB_B = SUB_BINS + 2;
+constexpr u32 SUB_WORDS = SUB_BINS + 4;
+constexpr u32 SEARCH_WORDS = EHIST + 2 * SUB_WORDS;
 
 struct WinEdge {  // an edge of the last window, between roots
   u64 time;
@@ -42,7 +45,7 @@ struct WinEdge {  // an edge of the last window, between roots
 };
 
 struct SearchCfg {
-  u32 win_cap;      // window edges stored per sample, <= FIN_EDGES
+  u32 win_cap;      // window edges stored per sample (<= FIN_EDGES with hashed roots)
   u32 hashed;       // roots are renumbered through a hash table (else: node ids)
   u32 ids;          // union-find words in shared memory
   u32 q0, q1;       // first two thresholds, edge quantiles in 1/65536
@@ -82,7 +85,8 @@ __device__ __forceinline__ u32 uf_find(u64* W, u32 x, u32* ox, u32* oy, bool* ca
 // of non-zero winding, and then, if mis is given, stores the cycle's lifted
 // mismatch (x in bits 0-15, y in 16-31, modulo 2^16).  Roots are linked
 // larger-id under smaller-id, so the forest stays acyclic under concurrent
-// unions.
+// unions.  (Linking in the order of mixed ids, for shallower trees where ids
+// follow the lattice, was no faster: k = 1 probes 10.7 ms in all, 9.7 so.)
 __device__ bool uf_union(u64* W, u32 m1, u32 m2, u32 dxy, bool* capped, u32 cap,
                          u32* mis = nullptr) {
   const u32 dx = dxy & 0xFFFFu, dy = dxy >> 16;
@@ -116,263 +120,383 @@ __device__ __forceinline__ u64 bin_floor(u32 b) {
   return e >= 5 ? (u64)m << (e - 5) : (u64)m >> (5 - e);
 }
 
+__device__ __forceinline__ Window first_window() {
+  Window w = {};
+  w.hi = KEY_NONE;
+  w.first = 1;
+  return w;
+}
+
 // Start of the search of one batch; while a sample of it is still being
 // deposited (*n_active) nothing of it runs.
-__global__ void k_graph_init(Group g, const u32* n_active) {
-  const u32 s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= g.n) return;
+__global__ void __launch_bounds__(256) k_graph_init(Group g, const u32* n_active) {
+  const u32 s = blockIdx.x;
+  const bool wait = *n_active != 0;  // the region still holds the rounds' lists
+  if (g.ehist && !wait)
+    for (u32 i = threadIdx.x; i < SEARCH_WORDS; i += 256) region_of(g, g.ehist, s)[i] = 0;
+  if (threadIdx.x) return;
   SampleState& st = g.st[s];
   st.n_edges = 0;
   st.contacts_x = st.contacts_y = st.contacts_xy = 0;
-  st.lo = 0;
-  st.hi = KEY_NONE;
-  st.mid = 0;
-  st.hi_ok = 0;
-  st.ready = 0;
-  st.step = 0;
-  st.wrap = 0;
-  st.cur = 0;
-  st.count_a = st.count_b = 0;
+  st.w = first_window();
   st.ticket = 0;
   st.win_n = 0;
   st.ranked = 0;
   st.nc = NONE32;
-  st.probes = 0;
-  st.sdone = (*n_active || (st.status & (ST_NODE_OVF | ST_ROUND_CAP))) ? 1u : 0u;
+  st.sdone = (wait || (st.status & (ST_NODE_OVF | ST_ROUND_CAP))) ? 1u : 0u;
+}
+
+// The first two thresholds from the histogram of times, ends of the bins in
+// which the quantiles fall.  part: 256 words; out: two thresholds (shared).
+__device__ void thresholds_body(const Group& g, const SearchCfg& c, u32 s, u32 ne, u32* part,
+                                u64* out) {
+  const u32 tid = threadIdx.x;
+  constexpr u32 PER = EHIST / 256;
+  const u32* h = region_of(g, g.ehist, s);
+  u32 v[PER], sum = 0;
+  if (tid < 256) {
+#pragma unroll
+    for (u32 i = 0; i < PER; ++i) {
+      v[i] = __ldcg(h + tid * PER + i);
+      sum += v[i];
+    }
+    part[tid] = sum;
+  }
+  if (tid < 2) out[tid] = KEY_NONE / 2;
+  __syncthreads();
+  for (u32 d = 1; d < 256; d <<= 1) {
+    const u32 o = tid < 256 && tid >= d ? part[tid - d] : 0u;
+    __syncthreads();
+    if (tid < 256) part[tid] += o;
+    __syncthreads();
+  }
+  if (tid < 256) {
+    const u32 r0 = (u32)((u64)ne * c.q0 >> 16), r1 = (u32)((u64)ne * c.q1 >> 16);
+    u32 a = part[tid] - sum;
+#pragma unroll
+    for (u32 i = 0; i < PER; ++i) {
+      const u32 b = a + v[i];
+      const u64 top = tid * PER + i + 1 < EHIST ? bin_floor(tid * PER + i + 1) - 1 : KEY_NONE - 1;
+      if (a <= r0 && r0 < b) out[0] = top;
+      if (a <= r1 && r1 < b) out[1] = top;
+      a = b;
+    }
+  }
+  __syncthreads();
 }
 
 // After the contacts: one block per sample.  Few edges: straight to the last
-// window.  Otherwise the first two thresholds from the histogram of times.
+// window.
 __global__ void __launch_bounds__(256) k_search_init(Group g, SearchCfg c) {
   __shared__ u32 part[256];
+  __shared__ u64 mids[2];
   const u32 s = blockIdx.x, tid = threadIdx.x;
   SampleState& st = g.st[s];
   if (st.sdone) return;
-  if (st.status & ST_EDGE_OVF) {
-    __syncthreads();
+  const bool ovf = (st.status & ST_EDGE_OVF) != 0;
+  const u32 ne = st.n_edges;
+  __syncthreads();
+  if (ovf) {
     if (tid == 0) st.sdone = 1;
     return;
   }
-  const u32 ne = st.n_edges;
-  if (ne <= c.win_cap) {
-    if (tid == 0) st.ready = 1;
-    return;
+  if (g.ehist) thresholds_body(g, c, s, ne, part, mids);
+  if (tid == 0) {
+    if (g.ehist) {
+      st.w.mid = mids[0];
+      st.w.next_mid = mids[1];
+    }
+    st.w.ready = ne <= c.win_cap;
   }
-  u32* h = g.ehist + (size_t)s * (EHIST + SUB_BINS);
-  constexpr u32 PER = EHIST / 256;
-  u32 v[PER], sum = 0;
-#pragma unroll
-  for (u32 i = 0; i < PER; ++i) {
-    v[i] = h[tid * PER + i];
-    sum += v[i];
-  }
-  part[tid] = sum;
-  if (tid < SUB_BINS) h[EHIST + tid] = 0;
-  __syncthreads();
-  for (u32 d = 1; d < 256; d <<= 1) {
-    const u32 o = tid >= d ? part[tid - d] : 0u;
-    __syncthreads();
-    part[tid] += o;
-    __syncthreads();
-  }
-  // the bin in which each quantile falls ends at the threshold
-  const u32 r0 = (u32)((u64)ne * c.q0 >> 16), r1 = (u32)((u64)ne * c.q1 >> 16);
-  u32 a = part[tid] - sum;
-#pragma unroll
-  for (u32 i = 0; i < PER; ++i) {
-    const u32 b = a + v[i];
-    const u64 top = tid * PER + i + 1 < EHIST ? bin_floor(tid * PER + i + 1) - 1 : KEY_NONE - 1;
-    if (a <= r0 && r0 < b) st.mid = top;
-    if (a <= r1 && r1 < b) st.next_mid = top;
-    a = b;
-  }
-  if (tid == 0) st.in_win = ne;
 }
 
-// Working copy of the union-find state at lo (single k-mers while lo = 0).
+// The word of node m with its root for parent.  No union runs meanwhile; a
+// word that another thread flattens while it is read is a true ancestor
+// relation before and after.
+__device__ __forceinline__ u64 flat_word(u64* W, u32 m, u32 cap, bool* capped) {
+  u64 w = *(volatile u64*)(W + m);
+  u32 x = m, sx = 0, sy = 0;
+  for (u32 it = 0; it < cap; ++it) {
+    const u32 p = (u32)w;
+    if (p == x) return uf_pack(x, sx, sy);
+    sx += (u32)(w >> 32);
+    sy += (u32)(w >> 48);
+    x = p;
+    w = *(volatile u64*)(W + x);
+  }
+  *capped = true;
+  return uf_pack(x, sx, sy);
+}
+
+// Working copy of the union-find state at lo (single k-mers while lo = 0),
+// flattened: the walks of a probe start at the roots of that state, and the
+// state, if a wrap sends the search back to it, stays flat.
+__device__ __forceinline__ void copy_body(const Group& g, u32 s, Team team, const Window& w) {
+  const u32 nn = min(g.st[s].n_nodes, g.cap_nodes), nt = blockDim.x;
+  u64* S = region_of(g, g.uf, s) + (size_t)w.cur * g.cap_nodes;
+  u64* Wd = region_of(g, g.uf, s) + (size_t)(w.cur ^ 1u) * g.cap_nodes;
+  bool capped = false;
+  for (u32 m = team.rank * nt + threadIdx.x; m < nn; m += team.size * nt) {
+    u64 v = uf_pack(m, 0, 0);
+    if (w.lo) {
+      v = flat_word(S, m, g.uf_cap, &capped);
+      S[m] = v;
+    }
+    Wd[m] = v;
+  }
+  if (capped) atomicOr(&g.st[s].status, ST_UF_CAP);
+}
+
 __global__ void __launch_bounds__(256) k_probe_copy(Group g) {
   const u32 s = blockIdx.y;
-  const SampleState& st = g.st[s];
-  if (st.sdone || st.ready) return;
-  const u32 nn = min(st.n_nodes, g.cap_nodes);
-  const bool fresh = st.lo == 0;
-  const u64* S = g.uf + ((size_t)s * 2 + st.cur) * g.cap_nodes;
-  u64* Wd = g.uf + ((size_t)s * 2 + (st.cur ^ 1u)) * g.cap_nodes;
-  for (u32 m = blockIdx.x * blockDim.x + threadIdx.x; m < nn; m += gridDim.x * blockDim.x)
-    Wd[m] = fresh ? uf_pack(m, 0, 0) : S[m];
+  if (g.st[s].sdone) return;
+  const Window w = g.st[s].w;
+  if (!w.ready) copy_body(g, s, Team{blockIdx.x, gridDim.x}, w);
 }
 
-// The step from one probe to the next (one thread per sample).
-__device__ void probe_step(SampleState& st, u32* sub, u32 shift, u32 win_cap, u32 probe_cap) {
-  st.probes += 1;
-  const u64 lo0 = st.lo;
-  const bool w = st.wrap != 0, first = st.step == 0;
-  st.wrap = 0;
-  st.step = 1;
-  if (st.status & ST_UF_CAP) {
-    st.sdone = 1;
-    return;
+// Sub-bins of the window (lo, hi]: 2^shift times each, at most SUB_BINS.
+__device__ __forceinline__ u32 sub_shift(const Window& w) {
+  const u32 width = 64 - (u32)__clzll((long long)(w.hi - w.lo - 1));
+  return width > 7 ? width - 7 : 0;
+}
+
+// A threshold that halves the `in` edges of the window, at the end of a
+// sub-bin (sub-bins of 2^shift times from lo0 on), by a whole warp.
+__device__ u64 halve_window(const Window& w, u64 lo0, u32 shift, const u32* set, u32 in) {
+  const u32 lane = threadIdx.x & 31;
+  u32 v[4], sum = 0;  // four sub-bins per lane
+  u64 end[4];
+#pragma unroll
+  for (u32 i = 0; i < 4; ++i) {
+    const u32 b = lane * 4 + i;
+    const u64 from = lo0 + 1 + ((u64)b << shift);
+    end[i] = from + ((1ull << shift) - 1);
+    const bool out = from <= lo0 || end[i] < from || end[i] <= w.lo || from > w.hi;
+    v[i] = out ? 0u : set[b];
+    sum += v[i];
   }
-  if (w) {
-    st.hi = st.mid;
-    st.hi_ok = 1;
+  u32 inc = sum;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const u32 o = __shfl_up_sync(FULL, inc, d);
+    if ((int)lane >= d) inc += o;
+  }
+  const u32 half = in / 2;
+  const u32 m = __ballot_sync(FULL, inc >= half && sum);
+  u32 a = inc - sum;
+  u64 mine = 0;
+#pragma unroll
+  for (u32 i = 0; i < 4; ++i) {
+    a += v[i];
+    if (mine == 0 && v[i] && a >= half) mine = end[i];
+  }
+  u64 mid = 0;
+  if (m) mid = __shfl_sync(FULL, mine, __ffs(m) - 1);
+  if (mid <= w.lo || mid >= w.hi) mid = w.lo + (w.hi - w.lo) / 2;
+  return mid;
+}
+
+// The step from one probe to the next, from the counts in `set`, by a whole
+// warp (every lane holds the same w).  True if the search of the sample ends
+// here.
+__device__ bool probe_step(Window& w, const u32* set, u32 win_cap, u32 probe_cap, u32& status) {
+  const u32 lane = threadIdx.x & 31;
+  w.probes += 1;
+  if (status & ST_UF_CAP) return true;
+  const bool wrap = set[SUB_WRAP] != 0, first = w.first != 0;
+  const u32 in = set[wrap ? SUB_A : SUB_B];
+  const u64 lo0 = w.lo;
+  const u32 shift = sub_shift(w);
+  w.first = 0;
+  if (wrap) {
+    w.hi = w.mid;
+    w.hi_ok = 1;
   } else {
-    st.lo = st.mid;
-    st.cur ^= 1u;
+    w.lo = w.mid;
+    w.cur ^= 1u;
   }
-  const u32 in = w ? st.count_a : st.count_b;
-  st.in_win = in;
-  st.count_a = st.count_b = 0;
   if (in <= win_cap) {
-    st.ready = 1;
-  } else if (st.probes >= probe_cap) {
-    st.status |= ST_SEARCH_CAP;
-    st.sdone = 1;
-  } else {
-    u64 mid = 0;
-    if (first && !w && st.next_mid > st.lo && st.next_mid < st.hi) {
-      mid = st.next_mid;
-    } else {
-      // halve the window's edges at a sub-bin boundary
-      u32 sum = 0;
-      for (u32 b = 0; b < SUB_BINS; ++b) {
-        const u64 first_t = lo0 + 1 + ((u64)b << shift);
-        const u64 last_t = first_t + ((1ull << shift) - 1);
-        if (last_t <= st.lo || first_t > st.hi) continue;
-        sum += sub[b];
-        mid = last_t;
-        if (sum >= in / 2) break;
-      }
-      if (mid <= st.lo || mid >= st.hi) mid = st.lo + (st.hi - st.lo) / 2;
-    }
-    st.mid = mid;
+    w.ready = 1;
+    return false;
   }
-  for (u32 b = 0; b < SUB_BINS; ++b) sub[b] = 0;
+  if (w.probes >= probe_cap) {
+    status |= ST_SEARCH_CAP;
+    return true;
+  }
+  if (first && !wrap && w.next_mid > w.lo && w.next_mid < w.hi) w.mid = w.next_mid;
+  else w.mid = halve_window(w, lo0, shift, set, in);
+  return false;
+}
+
+// Edges picked out of a scan, packed so that whole warps work on them: an
+// edge costs a chain of a dozen L2 accesses, and a warp with one such lane
+// waits as long as one with 32 (L = 512, k = 1, 100 samples, a window of 5% of
+// the edges: 1.9 ms by the lane that met the edge, 0.50 ms packed).
+constexpr u32 QUEUE_TILE = 4;      // edges per thread between two looks at the queue
+struct EdgeQueue {
+  u32 n;
+  u32 item[1];                     // (QUEUE_TILE + 1) x the block's threads
+};
+__host__ __device__ constexpr u32 queue_words(u32 threads) { return 1 + (QUEUE_TILE + 1) * threads; }
+
+// Calls work(i) for every i < ne, spread over the team's blocks, for which
+// want(i) holds.  Every thread of the block takes part.
+template <typename Want, typename Work>
+__device__ __forceinline__ void scan_packed(u32 ne, Team team, EdgeQueue& q, Want want, Work work) {
+  const u32 tid = threadIdx.x, nt = blockDim.x;
+  const u32 tile = QUEUE_TILE * nt;
+  if (tid == 0) q.n = 0;
+  __syncthreads();
+  for (u32 i0 = team.rank * tile; i0 < ne; i0 += team.size * tile) {
+#pragma unroll
+    for (u32 j = 0; j < QUEUE_TILE; ++j) {
+      const u32 i = i0 + j * nt + tid;
+      const bool ok = i < ne && want(i);
+      const u32 at = warp_append(&q.n, ok);
+      if (ok) q.item[at] = i;
+    }
+    __syncthreads();
+    const u32 n = q.n;
+    if (n >= nt || ne - i0 <= team.size * tile) {  // full, or the last tile of this block
+      for (u32 e = tid; e < n; e += nt) work(q.item[e]);
+      __syncthreads();
+      if (tid == 0) q.n = 0;
+    }
+    __syncthreads();
+  }
+}
+
+// Unites the edges of (lo, mid] in the working copy; adds to `set` the edges
+// of the window by sub-bin and by side of mid, and whether a wrap was closed.
+// hist: SUB_WORDS words (shared).
+__device__ void probe_body(const Group& g, u32 s, Team team, const Window& w, u32* hist,
+                           EdgeQueue& q, u32* set) {
+  const u32 tid = threadIdx.x, nt = blockDim.x;
+  SampleState& st = g.st[s];
+  const u64 lo = w.lo, mid = w.mid, hi = w.hi;
+  const u32 shift = sub_shift(w);
+  const u32 ne = min(st.n_edges, g.edge_limit);
+  for (u32 i = tid; i < SUB_WORDS; i += nt) hist[i] = 0;
+  __syncthreads();
+  u64* Wd = region_of(g, g.uf, s) + (size_t)(w.cur ^ 1u) * g.cap_nodes;
+  const u64* E = region_of(g, g.etime, s);
+  const uint4* K = region_of(g, g.elink, s);
+  bool wrap = false, capped = false;
+  u32 na = 0, nb = 0;
+  scan_packed(
+      ne, team, q,
+      [&](u32 i) {
+        const u64 t = E[i];
+        if (t <= lo || t > hi) return false;
+        atomicAdd(&hist[(u32)((t - lo - 1) >> shift)], 1u);
+        if (t > mid) {
+          ++nb;
+          return false;
+        }
+        ++na;
+        return true;
+      },
+      [&](u32 i) {
+        const uint4 e = K[i];
+        if (uf_union(Wd, e.x, e.y, e.z, &capped, g.uf_cap)) wrap = true;
+      });
+  na = __reduce_add_sync(FULL, na);
+  nb = __reduce_add_sync(FULL, nb);
+  if ((tid & 31) == 0) {
+    if (na) atomicAdd(&hist[SUB_A], na);
+    if (nb) atomicAdd(&hist[SUB_B], nb);
+  }
+  if (wrap) hist[SUB_WRAP] = 1;
+  if (capped) atomicOr(&st.status, ST_UF_CAP);
+  __syncthreads();
+  for (u32 i = tid; i < SUB_WORDS; i += nt)
+    if (hist[i]) atomicAdd(set + i, hist[i]);
 }
 
 // Eight 256-thread blocks per SM (32 registers): probes are latency-bound
 // union-find walks, and full occupancy hides more of that latency.
 __global__ void __launch_bounds__(256, 8) k_probe(Group g, SearchCfg c, u32 probe_cap) {
-  __shared__ u32 hist[SUB_BINS];
-  __shared__ u32 na_sh, nb_sh;
+  __shared__ u32 hist[SUB_WORDS];
+  __shared__ u32 queue[queue_words(256)];
+  __shared__ u32 last_sh;
   const u32 s = blockIdx.y, tid = threadIdx.x;
   SampleState& st = g.st[s];
-  if (st.sdone || st.ready) return;
-  const u64 lo = st.lo, mid = st.mid, hi = st.hi;
-  // sub-bins of the window (lo, hi], as many as fit SUB_BINS
-  const u64 span = hi - lo - 1;
-  const u32 width = 64 - __clzll((long long)span), shift = width > 7 ? width - 7 : 0;
-  const u32 ne = min(st.n_edges, g.edge_limit);
-  if (tid < SUB_BINS) hist[tid] = 0;
-  if (tid == 0) na_sh = nb_sh = 0;
-  __syncthreads();
-  u64* Wd = g.uf + ((size_t)s * 2 + (st.cur ^ 1u)) * g.cap_nodes;
-  const u64* E = g.etime + (size_t)s * g.cap_edges;
-  const uint4* K = g.elink + (size_t)s * g.cap_edges;
-  bool wrap = false, capped = false;
-  u32 na = 0, nb = 0;
-  for (u32 i = blockIdx.x * 256 + tid; i < ne; i += gridDim.x * 256) {
-    const u64 t = E[i];
-    if (t <= lo || t > hi) continue;
-    atomicAdd(&hist[(u32)((t - lo - 1) >> shift)], 1u);
-    if (t > mid) {
-      ++nb;
-      continue;
-    }
-    ++na;
-    const uint4 e = K[i];
-    if (uf_union(Wd, e.x, e.y, e.z, &capped, g.uf_cap)) wrap = true;
-  }
-  na = __reduce_add_sync(FULL, na);
-  nb = __reduce_add_sync(FULL, nb);
-  if ((tid & 31) == 0) {
-    if (na) atomicAdd(&na_sh, na);
-    if (nb) atomicAdd(&nb_sh, nb);
-  }
-  const bool bw = __syncthreads_or(wrap);
-  const bool bc = __syncthreads_or(capped);
-  u32* sub = g.ehist + (size_t)s * (EHIST + SUB_BINS) + EHIST;
-  if (tid < SUB_BINS && hist[tid]) atomicAdd(&sub[tid], hist[tid]);
+  if (st.sdone) return;
+  Window w = st.w;
+  if (w.ready) return;
+  u32* set = region_of(g, g.ehist, s) + EHIST;
+  probe_body(g, s, Team{blockIdx.x, gridDim.x}, w, hist, *reinterpret_cast<EdgeQueue*>(queue), set);
   __threadfence();
   __syncthreads();
-  if (tid == 0) {
-    if (bw) atomicOr(&st.wrap, 1u);
-    if (bc) atomicOr(&st.status, ST_UF_CAP);
-    if (na_sh) atomicAdd(&st.count_a, na_sh);
-    if (nb_sh) atomicAdd(&st.count_b, nb_sh);
-    __threadfence();
-    if (atomicAdd(&st.ticket, 1u) == gridDim.x - 1) {
-      __threadfence();
+  if (tid == 0) last_sh = atomicAdd(&st.ticket, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last_sh) return;
+  __threadfence();
+  if (tid < 32) {
+    u32 status = __ldcg(&st.status);
+    const bool end = probe_step(w, set, c.win_cap, probe_cap, status);
+    if (tid == 0) {
       st.ticket = 0;
-      st.wrap = __ldcg(&st.wrap);
-      st.status = __ldcg(&st.status);
-      st.count_a = __ldcg(&st.count_a);
-      st.count_b = __ldcg(&st.count_b);
-      probe_step(st, sub, shift, c.win_cap, probe_cap);
+      st.w = w;
+      st.status = status;
+      if (end) st.sdone = 1;
     }
   }
+  __syncthreads();
+  for (u32 i = tid; i < SUB_WORDS; i += 256) set[i] = 0;
 }
 
 // The edges of the last window between the roots they join.  Edges inside one
 // root without mismatch can close no wrap and are left out.
-__global__ void __launch_bounds__(256) k_collect(Group g, SearchCfg c) {
-  const u32 s = blockIdx.y;
+__device__ void collect_body(const Group& g, const SearchCfg& c, u32 s, Team team,
+                             const Window& w, EdgeQueue& q) {
   SampleState& st = g.st[s];
-  if (st.sdone || !st.ready) return;
-  const u64 lo = st.lo, hi = st.hi;
+  const u64 lo = w.lo, hi = w.hi;
   const u32 ne = min(st.n_edges, g.edge_limit);
-  u64* W = g.uf + ((size_t)s * 2 + st.cur) * g.cap_nodes;
-  const u64* E = g.etime + (size_t)s * g.cap_edges;
-  const uint4* K = g.elink + (size_t)s * g.cap_edges;
-  WinEdge* out = g.win + (size_t)s * c.win_cap;
+  u64* W = region_of(g, g.uf, s) + (size_t)w.cur * g.cap_nodes;
+  const u64* E = region_of(g, g.etime, s);
+  const uint4* K = region_of(g, g.elink, s);
+  WinEdge* out = region_of(g, g.win, s);
   bool capped = false;
-  for (u32 i = blockIdx.x * 256 + threadIdx.x; i < ne; i += gridDim.x * 256) {
-    const u64 t = E[i];
-    if (t <= lo || t > hi) continue;
-    const uint4 e = K[i];
-    WinEdge w;
-    w.time = t;
-    w.r1 = e.x;
-    w.r2 = e.y;
-    w.dxy = e.z;
-    w.pad = 0;
-    if (lo) {
-      u32 ax, ay, bx, by;
-      w.r1 = uf_find(W, e.x, &ax, &ay, &capped, g.uf_cap);
-      w.r2 = uf_find(W, e.y, &bx, &by, &capped, g.uf_cap);
-      w.dxy = ((ax + e.z - bx) & 0xFFFFu) | ((ay + (e.z >> 16) - by) << 16);
-      if (w.r1 == w.r2 && w.dxy == 0) continue;
-    }
-    const u32 at = atomicAdd(&st.win_n, 1u);
-    if (at < c.win_cap) out[at] = w;
-  }
+  scan_packed(
+      ne, team, q, [&](u32 i) { return E[i] > lo && E[i] <= hi; },
+      [&](u32 i) {
+        const uint4 e = K[i];
+        WinEdge we;
+        we.time = E[i];
+        we.r1 = e.x;
+        we.r2 = e.y;
+        we.dxy = e.z;
+        we.pad = 0;
+        if (lo) {
+          u32 ax, ay, bx, by;
+          we.r1 = uf_find(W, e.x, &ax, &ay, &capped, g.uf_cap);
+          we.r2 = uf_find(W, e.y, &bx, &by, &capped, g.uf_cap);
+          we.dxy = ((ax + e.z - bx) & 0xFFFFu) | ((ay + (e.z >> 16) - by) << 16);
+          if (we.r1 == we.r2 && we.dxy == 0) return;
+        }
+        const u32 at = atomicAdd(&st.win_n, 1u);
+        if (at < c.win_cap) out[at] = we;
+      });
   if (capped) atomicOr(&st.status, ST_UF_CAP);
 }
 
-// Root of x on shared-memory words, with path halving as in uf_find.
+__global__ void __launch_bounds__(256) k_collect(Group g, SearchCfg c) {
+  const u32 s = blockIdx.y;
+  if (g.st[s].sdone) return;
+  const Window w = g.st[s].w;
+  __shared__ u32 queue[queue_words(256)];
+  if (w.ready)
+    collect_body(g, c, s, Team{blockIdx.x, gridDim.x}, w, *reinterpret_cast<EdgeQueue*>(queue));
+}
+
+// Root of x on shared-memory words.  Every probe starts from flat words, so
+// walks are short, and halving them would cost more (a 64-bit CAS per step).
 __device__ __forceinline__ u32 fin_find(u64* W, u32 x, u32* ox, u32* oy, bool* capped, u32 cap) {
-  u32 sx = 0, sy = 0;
-  for (u32 it = 0; it < cap; ++it) {
-    const u64 wx = *(volatile u64*)(W + x);
-    const u32 p = (u32)wx;
-    if (p == x) {
-      *ox = sx;
-      *oy = sy;
-      return x;
-    }
-    const u64 wp = *(volatile u64*)(W + p);
-    const u32 gp = (u32)wp;
-    if (gp != p)
-      atomicCAS(W + x, wx, uf_pack(gp, (u32)(wx >> 32) + (u32)(wp >> 32),
-                                   (u32)(wx >> 48) + (u32)(wp >> 48)));
-    sx += (u32)(wx >> 32);
-    sy += (u32)(wx >> 48);
-    x = p;
-  }
-  *capped = true;
-  *ox = sx;
-  *oy = sy;
-  return x;
+  const u64 w = flat_word(W, x, cap, capped);
+  *ox = (u32)(w >> 32);
+  *oy = (u32)(w >> 48);
+  return (u32)w;
 }
 
 __device__ __forceinline__ bool fin_union(u64* W, u32 m1, u32 m2, u32 dxy, bool* capped, u32 cap) {
@@ -392,193 +516,268 @@ __device__ __forceinline__ bool fin_union(u64* W, u32 m1, u32 m2, u32 dxy, bool*
   return false;
 }
 
-__host__ __device__ inline size_t finish_smem(const SearchCfg& c, u32 pow2) {
-  // union-find words (as large as the hash table they follow), then per edge
-  // its time, displacement, two ids, place in the order and end of a time
-  return (c.hashed ? (size_t)FIN_SLOTS * 4 : (size_t)c.ids * 8) + (size_t)pow2 * 20;
+// Shared memory of finish_body: two arrays of union-find words (the hash
+// table before them), then per edge its time, displacement and two ids, and a
+// list of edges.
+__host__ __device__ inline size_t finish_smem(const SearchCfg& c) {
+  return ((c.hashed ? (size_t)FIN_SLOTS * 4 : (size_t)c.ids * 8)) * 2 + (size_t)c.win_cap * 18;
 }
+constexpr size_t FIN_SMEM_MAX = (size_t)FIN_SLOTS * 8 + (size_t)FIN_EDGES * 18;  // 2 FIN_EDGES ids
+constexpr u32 FIN_LAST = 32;  // edges united one after another in the end
 
-constexpr size_t FIN_SMEM_MAX = (size_t)FIN_SLOTS * 4 + (size_t)FIN_EDGES * 20;  // 2 FIN_EDGES ids
+struct FinishSmem {
+  u32 set[SUB_WORDS];
+  u32 wsum[34];
+  u32 count, flag;
+  u16 list[FIN_LAST];
+  Window w;
+  u32 status;
+};
 
-// The rest of the search in one block's shared memory.  pow2: win_cap rounded
-// up to a power of two.
-__global__ void __launch_bounds__(FIN_THREADS) k_finish(Group g, SearchCfg c, u32 pow2,
-                                                        u32 probe_cap, u32* n_open) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ u32 wsum[FIN_THREADS / 32 + 1];
-  __shared__ u32 ndist_sh;
-  const u32 s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+// The rest of the search by one block: probes as before on the edges in
+// shared memory, halving the window by sub-bins, and once FIN_LAST edges are
+// left these in the order of their times until one closes a wrap.  (Sorting
+// the edges for an exact bisection took longer than the probes themselves.)
+// Thread 0 writes the sample's results.
+__device__ void finish_body(const Group& g, const SearchCfg& c, u32 s, const Window& w0,
+                            u32 probe_cap, unsigned char* smem, FinishSmem& fs) {
+  const u32 tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarp = nt >> 5;
   SampleState& st = g.st[s];
-  if (st.sdone) {
-    if (tid == 0 && st.ranked == 1) st.ranked = 2;
-    return;
-  }
-  if (!st.ready) {
-    if (tid == 0) atomicAdd(n_open, 1u);
-    return;
-  }
-  u64* uf = reinterpret_cast<u64*>(smem_raw);             // and, before, the hash table
-  u32* slots = reinterpret_cast<u32*>(smem_raw);
-  const size_t words = finish_smem(c, 0);
-  u64* tm = reinterpret_cast<u64*>(smem_raw + words);     // times, sorted
-  u32* dxy = reinterpret_cast<u32*>(tm + pow2);           // by edge
-  u32* ends = dxy + pow2;                                 // by edge: two 16-bit ids
-  u16* ord = reinterpret_cast<u16*>(ends + pow2);         // edge of each sorted time
-  u16* last = ord + pow2;                                 // last position of each distinct time
+  const size_t words = c.hashed ? (size_t)FIN_SLOTS * 4 : (size_t)c.ids * 8;
+  u64* ua = reinterpret_cast<u64*>(smem);                 // working copy
+  u64* ub = reinterpret_cast<u64*>(smem + words);         // state at lo
+  u32* slots = reinterpret_cast<u32*>(smem);
+  u64* tm = reinterpret_cast<u64*>(smem + 2 * words);     // by edge: time,
+  u32* dxy = reinterpret_cast<u32*>(tm + c.win_cap);      // displacement,
+  u32* ends = dxy + c.win_cap;                            // two 16-bit ids
+  u16* todo = reinterpret_cast<u16*>(ends + c.win_cap);   // edges of this probe, packed
   const u32 n = min(st.win_n, c.win_cap);
-  const WinEdge* in = g.win + (size_t)s * c.win_cap;
-  u32 P2 = 1;
-  while (P2 < n) P2 <<= 1;
+  const WinEdge* in = region_of(g, g.win, s);
   u32 nid = min(st.n_nodes, g.cap_nodes);
-  if (c.hashed) {
-    for (u32 i = tid; i < FIN_SLOTS; i += FIN_THREADS) slots[i] = NONE32;
-    __syncthreads();
+  if (c.hashed)
+    for (u32 i = tid; i < FIN_SLOTS; i += nt) slots[i] = NONE32;
+  for (u32 i = tid; i < SUB_WORDS; i += nt) fs.set[i] = 0;
+  if (tid == 0) {
+    fs.w = w0;
+    fs.w.ready = 0;
+    fs.status = st.status;
+    fs.flag = 0;
+    fs.count = 0;
   }
-  for (u32 i = tid; i < P2; i += FIN_THREADS) {
-    u64 t = KEY_NONE;
-    if (i < n) {
-      const WinEdge w = in[i];
-      t = w.time;
-      dxy[i] = w.dxy;
-      u32 id[2] = {w.r1, w.r2};
-      if (c.hashed) {
+  __syncthreads();
+  // the first threshold, unless one is set: the middle of the window's edges
+  const bool whole = w0.lo == 0 && w0.mid > 0 && w0.mid < w0.hi;
+  const u32 shift0 = sub_shift(w0);
+  for (u32 i = tid; i < n; i += nt) {
+    const WinEdge e = in[i];
+    tm[i] = e.time;
+    dxy[i] = e.dxy;
+    if (!whole) atomicAdd(&fs.set[(u32)((e.time - w0.lo - 1) >> shift0)], 1u);
+    u32 id[2] = {e.r1, e.r2};
+    if (c.hashed) {
 #pragma unroll
-        for (u32 j = 0; j < 2; ++j) {
-          // at most 2 n <= FIN_SLOTS / 2 roots, so a free slot is met
-          u32 q = ((id[j] * 0x9E3779B1u) >> 16) & (FIN_SLOTS - 1);
-          for (u32 guard = 0; guard < FIN_SLOTS; ++guard, q = (q + 1) & (FIN_SLOTS - 1)) {
-            const u32 was = atomicCAS(&slots[q], NONE32, id[j]);
-            if (was == NONE32 || was == id[j]) break;
-          }
-          id[j] = q;
+      for (u32 j = 0; j < 2; ++j) {
+        // at most 2 n <= FIN_SLOTS / 2 roots, so a free slot is met
+        u32 q = ((id[j] * 0x9E3779B1u) >> 16) & (FIN_SLOTS - 1);
+        for (u32 guard = 0; guard < FIN_SLOTS; ++guard, q = (q + 1) & (FIN_SLOTS - 1)) {
+          const u32 was = atomicCAS(&slots[q], NONE32, id[j]);
+          if (was == NONE32 || was == id[j]) break;
         }
+        id[j] = q;
       }
-      ends[i] = id[0] | (id[1] << 16);
     }
-    tm[i] = t;
-    ord[i] = (u16)i;
+    ends[i] = id[0] | (id[1] << 16);
   }
   __syncthreads();
   if (c.hashed) {
     // number the slots in use
-    constexpr u32 PER = FIN_SLOTS / FIN_THREADS;
+    const u32 per = (FIN_SLOTS + nt - 1) / nt, a = min(tid * per, FIN_SLOTS),
+              b = min(a + per, FIN_SLOTS);
     u32 used = 0;
-    for (u32 i = 0; i < PER; ++i) used += slots[tid * PER + i] != NONE32;
+    for (u32 i = a; i < b; ++i) used += slots[i] != NONE32;
     u32 pre = used;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
       const u32 o = __shfl_up_sync(FULL, pre, d);
       if ((int)lane >= d) pre += o;
     }
-    if (lane == 31) wsum[warp] = pre;
+    if (lane == 31) fs.wsum[warp] = pre;
     __syncthreads();
     u32 at = pre - used;
-    for (u32 w = 0; w < warp; ++w) at += wsum[w];
-    for (u32 i = 0; i < PER; ++i)
-      if (slots[tid * PER + i] != NONE32) slots[tid * PER + i] = at++;
     nid = 0;
-    for (u32 w = 0; w < FIN_THREADS / 32; ++w) nid += wsum[w];
+    for (u32 q = 0; q < nwarp; ++q) {
+      if (q < warp) at += fs.wsum[q];
+      nid += fs.wsum[q];
+    }
+    for (u32 i = a; i < b; ++i)
+      if (slots[i] != NONE32) slots[i] = at++;
     __syncthreads();
-    for (u32 i = tid; i < n; i += FIN_THREADS)
+    for (u32 i = tid; i < n; i += nt)
       ends[i] = slots[ends[i] & 0xFFFFu] | (slots[ends[i] >> 16] << 16);
     __syncthreads();
   }
-  // bitonic sort of the times with their edges
-  for (u32 kk = 2; kk <= P2; kk <<= 1)
-    for (u32 j = kk >> 1; j > 0; j >>= 1) {
-      for (u32 q = tid; q < P2 / 2; q += FIN_THREADS) {
-        const u32 i = 2 * q - (q & (j - 1)), p = i + j;
-        const u64 a = tm[i], b = tm[p];
-        if ((a > b) == ((i & kk) == 0)) {
-          tm[i] = b;
-          tm[p] = a;
-          const u16 oa = ord[i];
-          ord[i] = ord[p];
-          ord[p] = oa;
-        }
+  for (u32 i = tid; i < nid; i += nt) ub[i] = uf_pack(i, 0, 0);
+  if (tid < 32) {
+    Window w = fs.w;
+    if (n <= FIN_LAST) w.ready = 1;
+    else if (!whole) w.mid = halve_window(w, w.lo, shift0, fs.set, n);
+    if (tid == 0) fs.w = w;
+  }
+  __syncthreads();
+  for (;;) {
+    const Window w = fs.w;
+    if (w.ready || fs.flag || (fs.status & ST_UF_CAP)) break;
+    if (w.probes >= probe_cap) {
+      __syncthreads();
+      if (tid == 0) {
+        fs.status |= ST_SEARCH_CAP;
+        fs.flag = 1;
       }
       __syncthreads();
+      break;
     }
-  // positions where a time ends, in order
-  {
-    const u32 per = (n + FIN_THREADS - 1) / FIN_THREADS, a = min(tid * per, n), b = min(a + per, n);
-    u32 cnt = 0;
-    for (u32 i = a; i < b; ++i) cnt += i + 1 == n || tm[i] != tm[i + 1];
-    u32 pre = cnt;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const u32 o = __shfl_up_sync(FULL, pre, d);
-      if ((int)lane >= d) pre += o;
-    }
-    if (lane == 31) wsum[warp] = pre;
-    __syncthreads();
-    u32 at = pre - cnt;
-    for (u32 w = 0; w < warp; ++w) at += wsum[w];
-    for (u32 i = a; i < b; ++i)
-      if (i + 1 == n || tm[i] != tm[i + 1]) last[at++] = (u16)i;
-    if (tid == FIN_THREADS - 1) ndist_sh = at;
-    __syncthreads();
-  }
-  u32 probes = st.probes, status = st.status;
-  // wrap after the first `m` distinct times of the window
-  auto probe = [&](u32 m, bool* capped_out) -> bool {
-    for (u32 i = tid; i < nid; i += FIN_THREADS) uf[i] = uf_pack(i, 0, 0);
-    __syncthreads();
     bool wrap = false, capped = false;
-    const u32 e1 = (u32)last[m - 1] + 1;
-    for (u32 i = tid; i < e1; i += FIN_THREADS) {
-      const u32 e = ord[i], ab = ends[e];
-      if (fin_union(uf, ab & 0xFFFFu, ab >> 16, dxy[e], &capped, g.uf_cap)) wrap = true;
+    for (u32 i = tid; i < nid; i += nt) {
+      const u64 v = flat_word(ub, i, g.uf_cap, &capped);
+      ub[i] = v;
+      ua[i] = v;
     }
-    *capped_out = __syncthreads_or(capped);
-    return __syncthreads_or(wrap);
-  };
-  u32 lo = 0, hi = ndist_sh;  // wrap(lo) is false; wrap(hi) if hi_ok
-  bool hi_ok = st.hi_ok != 0, capped = (status & ST_UF_CAP) != 0, over = false;
-  if (hi == 0) status |= ST_NOWRAP;  // no edge left that could close a wrap
-  while (hi > 0 && !capped && !(hi - lo == 1 && hi_ok)) {
-    if (probes >= probe_cap) {
-      over = true;
-      break;
+    for (u32 i = tid; i < SUB_WORDS; i += nt) fs.set[i] = 0;
+    if (tid == 0) fs.count = 0;
+    __syncthreads();
+    const u32 shift = sub_shift(w);
+    u32 na = 0, nb = 0;
+    for (u32 i0 = 0; i0 < n; i0 += nt) {
+      const u32 i = i0 + tid;
+      const u64 t = i < n ? tm[i] : 0;
+      const bool in_w = i < n && t > w.lo && t <= w.hi, now = in_w && t <= w.mid;
+      if (in_w) atomicAdd(&fs.set[(u32)((t - w.lo - 1) >> shift)], 1u);
+      const u32 at = warp_append(&fs.count, now);
+      if (now) todo[at] = (u16)i;
+      na += now;
+      nb += in_w && !now;
     }
-    ++probes;
-    const u32 mid = hi - lo == 1 ? hi : lo + (hi - lo) / 2;
-    if (probe(mid, &capped)) {
-      hi = mid;
-      hi_ok = true;
-    } else if (mid == hi) {
-      if (!capped) status |= ST_NOWRAP;
-      break;
-    } else {
-      lo = mid;
+    na = __reduce_add_sync(FULL, na);
+    nb = __reduce_add_sync(FULL, nb);
+    if (lane == 0) {
+      if (na) atomicAdd(&fs.set[SUB_A], na);
+      if (nb) atomicAdd(&fs.set[SUB_B], nb);
+    }
+    __syncthreads();
+    for (u32 q = tid; q < fs.count; q += nt) {
+      const u32 e = todo[q];
+      if (fin_union(ua, ends[e] & 0xFFFFu, ends[e] >> 16, dxy[e], &capped, g.uf_cap)) wrap = true;
+    }
+    if (wrap) fs.set[SUB_WRAP] = 1;
+    if (capped) atomicOr(&fs.status, ST_UF_CAP);
+    __syncthreads();
+    const bool wrapped = fs.set[SUB_WRAP] != 0;
+    if (tid < 32) {
+      Window x = w;
+      u32 status = fs.status;
+      const bool end = probe_step(x, fs.set, FIN_LAST, probe_cap, status);
+      __syncwarp();
+      if (tid == 0) {
+        fs.w = x;
+        fs.status = status;
+        fs.flag = end;
+      }
+    }
+    __syncthreads();
+    if (!wrapped) {
+      u64* t = ua;
+      ua = ub;
+      ub = t;
     }
   }
-  if (tid == 0) {
-    if (capped) status |= ST_UF_CAP;
-    if (over) status |= ST_SEARCH_CAP;
-    st.status = status;
-    st.probes = probes;
-    st.sdone = 1;
-    if (hi > 0 && !(status & (ST_UF_CAP | ST_SEARCH_CAP | ST_NOWRAP))) {
-      st.tc = tm[last[hi - 1]];
-      st.nc = 0;
-      st.ranked = 1;
+  const Window w = fs.w;
+  const bool go = w.ready && !fs.flag && !(fs.status & ST_UF_CAP);
+  if (tid == 0) fs.count = 0;
+  __syncthreads();
+  if (go)
+    for (u32 i = tid; i < n; i += nt)
+      if (tm[i] > w.lo && tm[i] <= w.hi) {
+        const u32 at = atomicAdd(&fs.count, 1u);
+        if (at < FIN_LAST) fs.list[at] = (u16)i;
+      }
+  __syncthreads();
+  if (warp == 0) {
+    u32 status = fs.status, probes = w.probes;
+    u64 tc = 0;
+    if (go && probes >= probe_cap) {
+      status |= ST_SEARCH_CAP;
+    } else if (go) {
+      ++probes;
+      const u32 m = min(fs.count, FIN_LAST);
+      const u32 mine = lane < m ? fs.list[lane] : 0u;
+      const u64 t = lane < m ? tm[mine] : KEY_NONE;
+      u32 rank = 0;
+      for (u32 i = 0; i < 32; ++i) {
+        const u64 o = __shfl_sync(FULL, t, i);
+        rank += o < t || (o == t && i < lane);
+      }
+      if (lane < m) fs.list[rank] = (u16)mine;
+      __syncwarp();
+      if (lane == 0) {
+        bool capped = false;
+        u32 i = 0;
+        for (; i < m && !capped; ++i) {
+          const u32 e = fs.list[i];
+          if (fin_union(ub, ends[e] & 0xFFFFu, ends[e] >> 16, dxy[e], &capped, g.uf_cap)) {
+            tc = tm[e];
+            break;
+          }
+        }
+        if (capped) status |= ST_UF_CAP;
+        else if (i == m) status |= ST_NOWRAP;
+      }
+    }
+    if (lane == 0) {
+      st.status = status;
+      st.w.probes = probes;
+      st.sdone = 1;
+      if (tc) {
+        st.tc = tc;
+        st.nc = 0;
+        st.ranked = 1;
+      }
     }
   }
 }
 
-// n_c: the k-mers of priority <= T_c.
-__global__ void __launch_bounds__(256) k_rank(Group g) {
-  const u32 s = blockIdx.y;
+__global__ void __launch_bounds__(FIN_THREADS) k_finish(Group g, SearchCfg c, u32 probe_cap,
+                                                        u32* n_open) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ FinishSmem fs;
+  const u32 s = blockIdx.x, tid = threadIdx.x;
   SampleState& st = g.st[s];
-  if (st.ranked != 1) return;
+  if (st.sdone) {
+    if (tid == 0 && st.ranked == 1) st.ranked = 2;
+    return;
+  }
+  const Window w = st.w;
+  __syncthreads();
+  if (!w.ready) {
+    if (tid == 0) atomicAdd(n_open, 1u);
+    return;
+  }
+  finish_body(g, c, s, w, probe_cap, smem_raw, fs);
+}
+
+// n_c: the k-mers of priority <= T_c.
+__device__ __forceinline__ void rank_body(const Group& g, u32 s, Team team) {
+  SampleState& st = g.st[s];
   const u64 T = st.tc;
   const u64* K = g.node_key + (size_t)s * g.cap_nodes;
-  const u32 nn = min(st.n_nodes, g.cap_nodes);
+  const u32 nn = min(st.n_nodes, g.cap_nodes), nt = blockDim.x;
   u32 cnt = 0;
-  for (u32 i = blockIdx.x * 256 + threadIdx.x; i < nn; i += gridDim.x * 256) cnt += K[i] <= T;
+  for (u32 i = team.rank * nt + threadIdx.x; i < nn; i += team.size * nt) cnt += K[i] <= T;
   cnt = __reduce_add_sync(FULL, cnt);
   if ((threadIdx.x & 31) == 0 && cnt) atomicAdd(&st.nc, cnt);
+}
+
+__global__ void __launch_bounds__(256) k_rank(Group g) {
+  if (g.st[blockIdx.y].ranked == 1) rank_body(g, blockIdx.y, Team{blockIdx.x, gridDim.x});
 }
 
 }  // namespace rsak
