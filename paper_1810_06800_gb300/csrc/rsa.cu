@@ -256,7 +256,9 @@ Layout layout_of(u32 L, u32 k, u32 n, bool with_keys, const Geometry& G) {
   l.rs = take(G.sites ? 0 : (size_t)n * sizeof(RoundState));
   l.st = take((size_t)n * sizeof(SampleState));
   l.seeds = take((size_t)n * 8);
-  l.counters = take(READ_BYTES);  // loop counters, then the work counters
+  // loop counters, work counters, key bins of the configuration passes: zeroed
+  // together
+  l.counters = take(READ_BYTES + CFG_BINS * 4);
   l.work = l.counters + ALIGN;
   l.keys = take(with_keys ? 2 * LL * 8 : 0);
   l.total = off;
@@ -307,6 +309,7 @@ struct rsa {
   void* ws = nullptr;
   Layout lay{};
   u32 last_n = 0;
+  std::vector<SampleState> states;  // of the last run, once read (fetch_states)
   bool with_keys = false;
   cudaStream_t stream = nullptr;
   u32* h_counter = nullptr;  // pinned, READ_BYTES: loop and work counters, configuration bits
@@ -431,8 +434,8 @@ cudaEvent_t prof_begin(Prof& p, int kind, cudaStream_t st) {
   return e1;
 }
 
-template <typename K, typename... Args>
-void launch(rsa_t* h, int kind, K kernel, dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+template <typename... KArgs, typename... Args>
+void launch(rsa_t* h, int kind, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
             Args... args) {
   Prof& p = h->prof;
   cudaEvent_t e1 = prof_begin(p, kind, st);
@@ -529,6 +532,7 @@ int run_impl(rsa_t* h, const uint64_t* seeds, u32 n, const uint64_t* keys, cudaS
   if ((rc = ensure_workspace(h, n, h->with_keys))) return rc;
   h->stream = stream;
   h->last_n = n;
+  h->states.clear();
   Group g = group_of(h, n);
   const Geometry& G = h->geo;
   const Layout& l = h->lay;
@@ -590,7 +594,7 @@ int run_impl(rsa_t* h, const uint64_t* seeds, u32 n, const uint64_t* keys, cudaS
   // the whole deposition: every slice once, and three more rounds for the
   // candidates left undecided by the last ones
   auto deposit = [&](cudaStream_t st) {
-    check(cudaMemsetAsync(b + l.counters, 0, READ_BYTES, st));
+    check(cudaMemsetAsync(b + l.counters, 0, READ_BYTES + CFG_BINS * 4, st));
     launch(h, KD_INIT, k_init, init_grid, dim3(128), 0, st, g, (const u64*)d_seeds);
     if (G.sites) {
       launch(h, KD_SITES, k_sites, grid_x((LL + 255) / 256, 32), dim3(256), 0, st, g);
@@ -664,7 +668,7 @@ int run_impl(rsa_t* h, const uint64_t* seeds, u32 n, const uint64_t* keys, cudaS
   CUDA_TRY(cudaFuncSetAttribute(k_sample, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMP_MAX));
   auto whole = [&](cudaStream_t st) {
     if (by_sample) {
-      check(cudaMemsetAsync(b + l.counters, 0, READ_BYTES, st));
+      check(cudaMemsetAsync(b + l.counters, 0, READ_BYTES + CFG_BINS * 4, st));
       launch(h, KD_SAMPLE, k_sample, dim3(std::min(n, (u32)h->sm_count)), dim3(SMP_THREADS),
              sample_smem(shape), st, shape, (const u64*)d_seeds);
       return;
@@ -710,13 +714,18 @@ int status_code(u32 bits) {
   return 0;
 }
 
-int fetch_states(rsa_t* h, std::vector<SampleState>& out) {
+// The sample states of the last run, read from the device once per run.
+int fetch_states(rsa_t* h, const std::vector<SampleState>** out) {
   if (!h->ws || h->last_n == 0) return fail(RSA_ESTATE, "no run to read");
-  out.resize(h->last_n);
-  const char* b = static_cast<const char*>(h->ws);
-  CUDA_TRY(cudaStreamSynchronize(h->stream));
-  CUDA_TRY(cudaMemcpy(out.data(), b + h->lay.st, sizeof(SampleState) * h->last_n,
-                      cudaMemcpyDeviceToHost));
+  if (h->states.size() != h->last_n) {
+    std::vector<SampleState> v(h->last_n);
+    const char* b = static_cast<const char*>(h->ws);
+    CUDA_TRY(cudaMemcpyAsync(v.data(), b + h->lay.st, sizeof(SampleState) * h->last_n,
+                             cudaMemcpyDeviceToHost, h->stream));
+    CUDA_TRY(cudaStreamSynchronize(h->stream));
+    h->states.swap(v);
+  }
+  *out = &h->states;
   return 0;
 }
 
@@ -788,9 +797,10 @@ int configuration(rsa_t* h, uint32_t sample, uint32_t m, uint32_t* counts, uint3
   if (!h) return fail(RSA_EINVAL, "null handle");
   if (sample >= h->last_n) return fail(RSA_EINVAL, "sample out of range");
   if (counts && cap < (u64)m + 1) return fail(RSA_EINVAL, "counts needs m + 1 entries");
-  std::vector<SampleState> st;
-  int rc = fetch_states(h, st);
+  const std::vector<SampleState>* states = nullptr;
+  int rc = fetch_states(h, &states);
   if (rc) return rc;
+  const std::vector<SampleState>& st = *states;
   if ((rc = status_code(st[sample].status))) {
     g_err = "sample " + std::to_string(sample) + " has no valid result";
     return rc;
@@ -802,36 +812,44 @@ int configuration(rsa_t* h, uint32_t sample, uint32_t m, uint32_t* counts, uint3
   if (m == 0) return 0;
   cudaStream_t stream = h->stream;
   Group g = group_of(h, h->last_n);
-  const u32 bx = (u32)std::min<u64>(((u64)g.cap_edges + 255) / 256, 2048);
+  const u32 bx = (u32)std::min<u64>(((u64)st[sample].n_edges + 1023) / 1024 + 1, 2048);
   const u32 nb = (u32)std::min<u64>(((u64)nj + 256) / 256, 1024);
   const bool at_wrap = m == st[sample].nc;
-  if (!at_wrap) {
-    u64* keys_out = cfg_uf(g, sample);
-    if (g.cap_nodes >= EHIST) {
-      u32* bins = cfg_size(g, sample);
-      const u32 kb = std::min(nb, 152u);
-      CUDA_TRY(cudaMemsetAsync(bins, 0, (EHIST + 4) * 4, stream));
-      k_key_bins<<<kb, 256, 0, stream>>>(g, sample, m, bins);
-      k_key_select<<<kb, 256, 0, stream>>>(g, sample, m, bins, keys_out);
-    } else {
-      k_key_select<<<1, 256, 0, stream>>>(g, sample, m, nullptr, keys_out);
-    }
-  }
-  k_cfg_init<<<nb, 256, 0, stream>>>(g, sample, at_wrap);
-  k_cfg_union<<<bx, 256, 0, stream>>>(g, sample);
-  if (counts) {
-    k_cfg_count<<<nb, 256, 0, stream>>>(g, sample);
-    k_cfg_hist<<<nb, 256, 0, stream>>>(g, sample);
-  }
-  CUDA_TRY(cudaGetLastError());
   const char* b = static_cast<const char*>(h->ws);
-  const size_t so = h->lay.st + (size_t)sample * sizeof(SampleState);
-  CUDA_TRY(cudaMemcpyAsync(h->h_counter + 12, b + so + offsetof(SampleState, wdirs), 4,
-                           cudaMemcpyDeviceToHost, stream));
-  if (counts)
-    CUDA_TRY(cudaMemcpyAsync(counts + 1, cfg_hist(g, sample), (size_t)m * sizeof(uint32_t),
+  if (g.cap_nodes <= CFG_NODES) {
+    const size_t smem = cfg_block_smem(g.cap_nodes);
+    CUDA_TRY(cudaFuncSetAttribute(k_cfg_block, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)cfg_block_smem(CFG_NODES)));
+    k_cfg_block<<<1, CFG_THREADS, smem, stream>>>(g, sample, m, at_wrap, counts != nullptr);
+    CUDA_TRY(cudaGetLastError());
+    u32* to = counts ? counts : h->h_counter + 12;
+    CUDA_TRY(cudaMemcpyAsync(to, cfg_size(g, sample), (counts ? (size_t)m + 1 : 1) * sizeof(u32),
                              cudaMemcpyDeviceToHost, stream));
-  CUDA_TRY(cudaStreamSynchronize(stream));
+    CUDA_TRY(cudaStreamSynchronize(stream));
+    h->h_counter[12] = to[0];
+    if (counts) counts[0] = 0;
+  } else {
+    if (!at_wrap) {
+      u32* bins = reinterpret_cast<u32*>(const_cast<char*>(b) + h->lay.counters + READ_BYTES);
+      const u32 kb = std::min(nb, 152u);
+      k_key_bins<<<kb, 256, 0, stream>>>(g, sample, m, bins);
+      k_key_select<<<kb, SEL_THREADS, 0, stream>>>(g, sample, bins);
+    }
+    k_cfg_init<<<nb, 256, 0, stream>>>(g, sample, at_wrap);
+    k_cfg_union<<<bx, 256, 0, stream>>>(g, sample);
+    if (counts) {
+      k_cfg_count<<<nb, 256, 0, stream>>>(g, sample);
+      k_cfg_hist<<<nb, 256, 0, stream>>>(g, sample);
+    }
+    CUDA_TRY(cudaGetLastError());
+    const size_t so = h->lay.st + (size_t)sample * sizeof(SampleState);
+    CUDA_TRY(cudaMemcpyAsync(h->h_counter + 12, b + so + offsetof(SampleState, wdirs), 4,
+                             cudaMemcpyDeviceToHost, stream));
+    if (counts)
+      CUDA_TRY(cudaMemcpyAsync(counts + 1, cfg_hist(g, sample), (size_t)m * sizeof(uint32_t),
+                               cudaMemcpyDeviceToHost, stream));
+    CUDA_TRY(cudaStreamSynchronize(stream));
+  }
   const u32 w = h->h_counter[12];
   if (w & CFG_CAPPED) return fail(RSA_ETIMEOUT, "union-find walk cap reached");
   *wdirs = w & 3u;
@@ -1079,9 +1097,10 @@ int rsa_run_static(uint32_t L, uint32_t k, const uint64_t* seeds, uint32_t n, ui
 int rsa_results(rsa_t* h, uint32_t* n_j, uint32_t* n_c, uint32_t n) {
   if (!h) return fail(RSA_EINVAL, "null handle");
   if (n > h->last_n) return fail(RSA_EINVAL, "n exceeds samples of the last run");
-  std::vector<SampleState> st;
-  int rc = fetch_states(h, st);
+  const std::vector<SampleState>* states = nullptr;
+  int rc = fetch_states(h, &states);
   if (rc) return rc;
+  const std::vector<SampleState>& st = *states;
   int first = 0;
   for (u32 i = 0; i < n; ++i) {
     if (n_j) n_j[i] = st[i].n_nodes;
@@ -1099,9 +1118,10 @@ int rsa_sample_stats(rsa_t* h, uint32_t* rounds, uint32_t* probes, uint32_t* edg
                      int32_t* status, uint32_t n) {
   if (!h) return fail(RSA_EINVAL, "null handle");
   if (n > h->last_n) return fail(RSA_EINVAL, "n exceeds samples of the last run");
-  std::vector<SampleState> st;
-  int rc = fetch_states(h, st);
+  const std::vector<SampleState>* states = nullptr;
+  int rc = fetch_states(h, &states);
   if (rc) return rc;
+  const std::vector<SampleState>& st = *states;
   for (u32 i = 0; i < n; ++i) {
     if (rounds) rounds[i] = st[i].rounds;
     if (probes) probes[i] = st[i].w.probes;
@@ -1114,9 +1134,10 @@ int rsa_sample_stats(rsa_t* h, uint32_t* rounds, uint32_t* probes, uint32_t* edg
 int rsa_contacts(rsa_t* h, uint32_t* n_x, uint32_t* n_y, uint32_t* n_xy, uint32_t n) {
   if (!h) return fail(RSA_EINVAL, "null handle");
   if (n > h->last_n) return fail(RSA_EINVAL, "n exceeds samples of the last run");
-  std::vector<SampleState> st;
-  int rc = fetch_states(h, st);
+  const std::vector<SampleState>* states = nullptr;
+  int rc = fetch_states(h, &states);
   if (rc) return rc;
+  const std::vector<SampleState>& st = *states;
   for (u32 i = 0; i < n; ++i) {
     if (n_x) n_x[i] = st[i].contacts_x;
     if (n_y) n_y[i] = st[i].contacts_y;
@@ -1128,9 +1149,10 @@ int rsa_contacts(rsa_t* h, uint32_t* n_x, uint32_t* n_y, uint32_t* n_xy, uint32_
 int rsa_accepted(rsa_t* h, uint32_t sample, uint32_t* idx, uint32_t cap, uint32_t* count) {
   if (!h || !count) return fail(RSA_EINVAL, "null argument");
   if (sample >= h->last_n) return fail(RSA_EINVAL, "sample out of range");
-  std::vector<SampleState> st;
-  int rc = fetch_states(h, st);
+  const std::vector<SampleState>* states = nullptr;
+  int rc = fetch_states(h, &states);
   if (rc) return rc;
+  const std::vector<SampleState>& st = *states;
   const u32 cn = cap_nodes_of(h->L, h->k);
   const u32 nj = std::min(st[sample].n_nodes, cn);
   std::vector<uint32_t> v(nj);

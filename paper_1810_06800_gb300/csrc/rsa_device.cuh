@@ -145,7 +145,6 @@ __device__ __forceinline__ u64 cand_key(const Group& g, u32 s, u64 idx) {
 template <typename T> __device__ __forceinline__ T tmin(T a, T b) { return b < a ? b : a; }
 template <typename T> __device__ __forceinline__ T tmax(T a, T b) { return b > a ? b : a; }
 
-// Shared by the engine and the small-lattice kernel.
 // Position of cell (cy, cx) inside the k-mer whose anchor is packed as
 // o << 31 | y0 << 15 | x0; *o receives the orientation.
 __device__ __forceinline__ u32 pos_in_kmer(u32 pos, u32 cy, u32 cx, u32 L, u32* o) {

@@ -29,8 +29,8 @@
 
 namespace rsak {
 
-constexpr u32 FIN_EDGES = 2048;
-constexpr u32 FIN_THREADS = 512;
+constexpr u32 FIN_EDGES = 4096;
+constexpr u32 FIN_THREADS = 1024;
 constexpr u32 FIN_SLOTS = 4 * FIN_EDGES;  // hash slots for the roots of the window (4 B: as much
                                           // as 2 FIN_EDGES union-find words)
 constexpr u32 SUB_BINS = 128;
@@ -51,34 +51,45 @@ struct SearchCfg {
   u32 q0, q1;       // first two thresholds, edge quantiles in 1/65536
 };
 
-// Root of x and x's offset from it.  Path halving by CAS; a failed CAS is
-// harmless because every stored (parent, offset) pair stays a true ancestor
-// relation.  Loads bypass L1 (other SMs write these words).
-__device__ __forceinline__ u32 uf_find(u64* W, u32 x, u32* ox, u32* oy, bool* capped, u32 cap) {
-  u32 sx = 0, sy = 0;
-  for (u32 it = 0; it < cap; ++it) {
-    const u64 wx = __ldcg(W + x);
-    const u32 p = (u32)wx;
-    if (p == x) {
-      *ox = sx;
-      *oy = sy;
-      return x;
+// Root of x and x's offset from it, halving the path: every node passed gets
+// its grandparent for parent by a plain store.  A node that is no root never
+// becomes one, and every word stored for it is a true ancestor relation, so
+// stores may overtake one another.  Global words are read from L2 (other SMs
+// write them).
+template <bool GLOBAL>
+__device__ __forceinline__ u32 find_root(u64* W, u32 x, u32* ox, u32* oy, bool* capped, u32 cap) {
+  auto load = [&](u32 i) { return GLOBAL ? __ldcg(W + i) : *(volatile u64*)(W + i); };
+  u32 sx = 0, sy = 0, steps = 0;
+  u64 w = load(x);
+  for (;;) {
+    const u32 p = (u32)w;
+    if (p == x) break;
+    if (++steps >= cap) {
+      *capped = true;
+      break;
     }
-    const u64 wp = __ldcg(W + p);
-    const u32 gp = (u32)wp;
-    if (gp != p) {
-      const u64 nw = uf_pack(gp, (u32)(wx >> 32) + (u32)(wp >> 32),
-                             (u32)(wx >> 48) + (u32)(wp >> 48));
-      atomicCAS(W + x, wx, nw);
+    const u64 wp = load(p);
+    const u32 gp = (u32)wp, dx = (u32)(w >> 32), dy = (u32)(w >> 48);
+    if (gp == p) {
+      sx += dx;
+      sy += dy;
+      x = p;
+      break;
     }
-    sx += (u32)(wx >> 32);
-    sy += (u32)(wx >> 48);
-    x = p;
+    const u64 nw = uf_pack(gp, dx + (u32)(wp >> 32), dy + (u32)(wp >> 48));
+    *(volatile u64*)(W + x) = nw;
+    sx += (u32)(nw >> 32);
+    sy += (u32)(nw >> 48);
+    x = gp;
+    w = load(x);
   }
-  *capped = true;
   *ox = sx;
   *oy = sy;
   return x;
+}
+
+__device__ __forceinline__ u32 uf_find(u64* W, u32 x, u32* ox, u32* oy, bool* capped, u32 cap) {
+  return find_root<true>(W, x, ox, oy, capped, cap);
 }
 
 // Add edge "anchor(m2) = anchor(m1) + d"; returns true if it closes a cycle
@@ -490,23 +501,18 @@ __global__ void __launch_bounds__(256) k_collect(Group g, SearchCfg c) {
     collect_body(g, c, s, Team{blockIdx.x, gridDim.x}, w, *reinterpret_cast<EdgeQueue*>(queue));
 }
 
-// Root of x on shared-memory words.  Every probe starts from flat words, so
-// walks are short, and halving them would cost more (a 64-bit CAS per step).
-__device__ __forceinline__ u32 fin_find(u64* W, u32 x, u32* ox, u32* oy, bool* capped, u32 cap) {
-  const u64 w = flat_word(W, x, cap, capped);
-  *ox = (u32)(w >> 32);
-  *oy = (u32)(w >> 48);
-  return (u32)w;
-}
-
-__device__ __forceinline__ bool fin_union(u64* W, u32 m1, u32 m2, u32 dxy, bool* capped, u32 cap) {
+__device__ __forceinline__ bool fin_union(u64* W, u32 m1, u32 m2, u32 dxy, bool* capped, u32 cap,
+                                          u32* mis = nullptr) {
   for (u32 it = 0; it < cap; ++it) {
     u32 ax, ay, bx, by;
-    const u32 r1 = fin_find(W, m1, &ax, &ay, capped, cap);
-    const u32 r2 = fin_find(W, m2, &bx, &by, capped, cap);
+    const u32 r1 = find_root<false>(W, m1, &ax, &ay, capped, cap);
+    const u32 r2 = find_root<false>(W, m2, &bx, &by, capped, cap);
     if (*capped) return false;
     const u32 Dx = ax + dxy - bx, Dy = ay + (dxy >> 16) - by;
-    if (r1 == r2) return ((Dx | Dy) & 0xFFFFu) != 0;
+    if (r1 == r2) {
+      if (mis) *mis = (Dx & 0xFFFFu) | ((Dy & 0xFFFFu) << 16);
+      return ((Dx | Dy) & 0xFFFFu) != 0;
+    }
     const u32 hi = r1 < r2 ? r2 : r1;
     const u64 want = uf_pack(hi, 0, 0);
     const u64 link = r1 < r2 ? uf_pack(r1, Dx, Dy) : uf_pack(r2, 0u - Dx, 0u - Dy);
