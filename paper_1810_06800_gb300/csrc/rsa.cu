@@ -75,7 +75,6 @@ struct Geometry {
   size_t list_cap;  // listed candidates per sample
   SearchCfg sc;
   SearchCfg ssc;    // the same for a sample in one block (rsa_sample.cuh)
-  u32 lines;        // lines per block of k_refill
   u32 probes;       // probes that bring the window of a large graph to the last
   Shape hot;        // what of it a block keeps in shared memory (offsets only)
   bool one_block;   // that fits
@@ -169,6 +168,7 @@ Geometry plan(u32 L, u32 k) {
   const u64 N = 2ull * L * L, D = (u64)k * k + 2 * k;
   const u32 lk = log2_floor(k);
   c.W = (L + k + 31) / 32 + 1;
+  c.inv_L = ((1ull << 45) + L - 1) / L;
   c.WA = (L + 2 * k + 31) / 32 + 1;
   // lines per block line: 2^bs + k / 2^bs updates per k-mer, least at sqrt(k)
   c.bs = k < 16 ? 0 : std::max(3u, lk / 2);
@@ -200,7 +200,6 @@ Geometry plan(u32 L, u32 k) {
   // takes a narrower slice and the run only takes longer
   c.cap_flat = (u32)std::min<u64>(N, N / 4 + 32);
   c.cap_act = (u32)std::min<u64>(N, std::max(cap_nodes_of(L, k) / 2, c.lvl_cap[0]) + 32);
-  G.lines = std::max(1u, std::min(1024u, REFILL_WORDS) / c.W);
   plan_hot(L, G);
   return G;
 }
@@ -453,7 +452,6 @@ Shape shape_of(const Geometry& G, const Group& g, const RoundCfg& c, const Round
   s.p = p;
   s.sc = G.ssc;
   s.probe_cap = probe_cap;
-  s.lines = G.lines;
   s.sites = G.sites;
   return s;
 }
@@ -564,12 +562,17 @@ int run_impl(rsa_t* h, const uint64_t* seeds, u32 n, const uint64_t* keys, cudaS
   };
   const dim3 init_grid((n + 127) / 128);
   // Lanes per active candidate in k_resolve.  Long k has many bins to look at
-  // (L = 8192, k = 512, 32 samples: 4.9 ms with 32 lanes, 7.4 with 8, 7.6 with
-  // 1).  For short k one lane does the least work in all, which counts once
-  // the candidates fill the GPU (L = 1024, k = 32, 1000 samples: 10.4 ms with
-  // 1, 11.5 with 8), and eight lanes have the shortest chain of loads, which
-  // counts when they do not (L = 128, k = 8, 32 samples: 0.49 and 0.18 ms).
-  const u32 lanes = h->k > 128 ? 32 : (u64)n * g.cap_nodes >= (2u << 20) ? 1 : 8;
+  // (L = 8192, k = 512, 32 samples: the run takes 14.6 ms with 16 lanes, 15.8
+  // with 8, 15.1 with 32; L = 32768, k = 4096: 20.5 and 20.2 with 16 and 32).
+  // For short k one lane does the least work in all, which counts once the
+  // candidates fill the GPU (L = 1024, k = 32, 1000 samples: 19.8 ms, with 8
+  // lanes 24.1), and eight lanes have the shortest chain of loads, which
+  // counts when they do not (L = 128, k = 8, 32 samples: 0.18 ms of k_resolve
+  // against 0.49).
+  const u32 lanes = h->k >= 2048                             ? 32
+                    : h->k > 128                             ? 16
+                    : (u64)n * g.cap_nodes >= (2u << 20) ? 1
+                                                             : 8;
   auto round = [&](cudaStream_t st) {
     const dim3 pg = grid_x((c.lvl_cap[c.nlev - 1] + RD_THREADS - 1) / RD_THREADS, 16);
     if (h->k <= PICK_LONGK)
@@ -580,12 +583,14 @@ int run_impl(rsa_t* h, const uint64_t* seeds, u32 n, const uint64_t* keys, cudaS
     switch (lanes) {
       case 1: launch(h, KD_RESOLVE, k_resolve<1>, rg, dim3(RD_THREADS), 0, st, g, c, rp); break;
       case 8: launch(h, KD_RESOLVE, k_resolve<8>, rg, dim3(RD_THREADS), 0, st, g, c, rp); break;
+      case 16: launch(h, KD_RESOLVE, k_resolve<16>, rg, dim3(RD_THREADS), 0, st, g, c, rp); break;
       default: launch(h, KD_RESOLVE, k_resolve<32>, rg, dim3(RD_THREADS), 0, st, g, c, rp); break;
     }
   };
   auto refill = [&](cudaStream_t st) {
-    launch(h, KD_REFILL, k_refill, grid_x((2ull * h->L + G.lines - 1) / G.lines, 16),
-           dim3(RD_THREADS), 0, st, g, c, rp, G.lines);
+    const u32 warps = std::min(RD_THREADS / 32, REFILL_WORDS / c.W);
+    launch(h, KD_REFILL, k_refill, grid_x((2ull * h->L + warps - 1) / warps, 16), dim3(RD_THREADS),
+           0, st, g, c, rp);
   };
   auto count_active = [&](cudaStream_t st) {
     check(cudaMemsetAsync(d_counter, 0, 4, st));
@@ -624,7 +629,7 @@ int run_impl(rsa_t* h, const uint64_t* seeds, u32 n, const uint64_t* keys, cudaS
   const SearchCfg& sc = G.sc;
   // blocks per sample over its k-mers and its edges
   const dim3 node_grid = grid_x(((u64)g.cap_nodes + 255) / 256, 32);
-  const dim3 edge_grid = grid_x(((u64)g.cap_edges + 1023) / 1024, 16);
+  const dim3 edge_grid = grid_x(((u64)g.cap_edges + 255) / 256, 16);
   const size_t fin_smem = finish_smem(sc);
   // the same limit for every shape: handles run on several threads at once
   CUDA_TRY(cudaFuncSetAttribute(k_finish, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -812,7 +817,7 @@ int configuration(rsa_t* h, uint32_t sample, uint32_t m, uint32_t* counts, uint3
   if (m == 0) return 0;
   cudaStream_t stream = h->stream;
   Group g = group_of(h, h->last_n);
-  const u32 bx = (u32)std::min<u64>(((u64)st[sample].n_edges + 1023) / 1024 + 1, 2048);
+  const u32 bx = (u32)std::min<u64>(((u64)st[sample].n_edges + 255) / 256 + 1, 2048);
   const u32 nb = (u32)std::min<u64>(((u64)nj + 256) / 256, 1024);
   const bool at_wrap = m == st[sample].nc;
   const char* b = static_cast<const char*>(h->ws);

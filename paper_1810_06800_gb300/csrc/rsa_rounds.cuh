@@ -48,7 +48,8 @@ constexpr u32 RD_LEVELS = 32;
 constexpr u32 RD_THREADS = 256;
 constexpr u32 DENSE_THREADS = 256;
 constexpr u32 DENSE_PER = 16;                      // candidates per thread and tile
-constexpr u32 REFILL_WORDS = 2304;                 // words of line staged per block
+constexpr u32 REFILL_WORDS = 9472;                 // words of line staged per block: 8 lines of
+                                                   // L = 32768, k = 4096; at least one of any shape
 
 struct RoundCfg {
   u32 W;            // words of a cover line, (L + k) bits and one spare
@@ -61,6 +62,7 @@ struct RoundCfg {
   u32 cap_act;      // active candidates per sample
   u32 cap_flat;     // entries of the refilled list
   u32 round_cap;
+  u64 inv_L;        // ceil(2^45 / L)
   u32 lvl_off[RD_LEVELS], lvl_cap[RD_LEVELS];
 };
 
@@ -103,6 +105,12 @@ __device__ __forceinline__ Slice first_slice(const RoundCfg& c) {
   return z;
 }
 
+// r / L for r < L^2 (L <= 2^15): the product with ceil(2^45 / L) is at most
+// r / 2^45 < 1 / L above 2^45 r / L.
+__device__ __forceinline__ u32 row_of(const RoundCfg& c, u32 r) {
+  return (u32)(((u64)r * c.inv_L) >> 45);
+}
+
 struct RoundPtrs {
   u32* fine;        // (r) [2][L][W]
   u32* block;       // (r) [2][nbl][W]
@@ -116,11 +124,11 @@ struct RoundPtrs {
 
 __device__ __forceinline__ u32* cover_line(const Group& g, const RoundCfg& c, const RoundPtrs& p,
                                            u32 s, u32 o, u32 line) {
-  return region_of(g, p.fine, s) + ((size_t)o * g.L + line) * c.W;
+  return region_of(g, p.fine, s) + (o * g.L + line) * c.W;  // < 2^28 words
 }
 __device__ __forceinline__ u32* block_line(const Group& g, const RoundCfg& c, const RoundPtrs& p,
                                            u32 s, u32 o, u32 bl) {
-  return region_of(g, p.block, s) + ((size_t)o * c.nbl + bl) * c.W;
+  return region_of(g, p.block, s) + (o * c.nbl + bl) * c.W;
 }
 // Anchors of k-mers of orientation `type`, as lines along `layout`.
 __device__ __forceinline__ u32* anchor_line(const Group& g, const RoundCfg& c, const RoundPtrs& p,
@@ -275,29 +283,33 @@ __device__ void pick_body(const Group& g, const RoundCfg& c, const RoundPtrs& p,
   const u32 L = g.L, k = g.k, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31;
   const u32 par = sl.par, t = sl.t;
   const u64 lo = sl.lo, hi = sl.hi;
-  const u32* list = t >= c.nlev ? region_of(g, p.flat, s)
-                                : region_of(g, p.list, s) + c.lvl_off[t];
+  const bool flat = t >= c.nlev;
+  const u32* list = flat ? region_of(g, p.flat, s) : region_of(g, p.list, s) + c.lvl_off[t];
   const Act* prev = region_of(g, p.act, s) + (size_t)(par ^ 1u) * c.cap_act;
   Act* cur = region_of(g, p.act, s) + (size_t)par * c.cap_act;
   u32* heads = region_of(g, p.heads, s) + (size_t)par * 2 * c.nb * c.nb;
   const u64 zb = g.base[s] + SM_GAMMA;
+  auto key_of = [&](u32 idx) { return g.keys ? g.keys[idx] : mix64(zb + SM_GAMMA * idx); };
   const u32 total = n1 + n2;
   for (u32 i0 = team.rank * nt; i0 < total; i0 += team.size * nt) {
     const u32 i = i0 + tid;
     bool ok = i < total;
-    u32 o = 0, y = 0, x = 0;
+    u32 o = 0, y = 0, x = 0, idx = 0;
     u64 key = 0;
     if (ok) {
       if (i < n1) {
-        const u32 idx = list[i];
-        key = g.keys ? g.keys[idx] : mix64(zb + SM_GAMMA * idx);
-        ok = key >= lo && key <= hi;
-        if (ok) {
-          u32 rr = idx;
-          if (rr >= (u32)g.LL) { o = 1; rr -= (u32)g.LL; }
-          y = rr / L;
-          x = rr - y * L;
+        // a refilled list holds all later slices: first whether the entry is of
+        // this one; of a slice's own list most entries are dead: first whether
+        // it is live, and its priority only then
+        idx = list[i];
+        if (flat) {
+          key = key_of(idx);
+          ok = key >= lo && key <= hi;
         }
+        u32 rr = idx;
+        if (rr >= (u32)g.LL) { o = 1; rr -= (u32)g.LL; }
+        y = row_of(c, rr);
+        x = rr - y * L;
       } else {
         const uint4 e = *reinterpret_cast<const uint4*>(prev + (i - n1));
         key = (u64)e.y << 32 | e.x;
@@ -338,6 +350,10 @@ __device__ void pick_body(const Group& g, const RoundCfg& c, const RoundPtrs& p,
         const bool hit = __any_sync(FULL, v != 0);
         if (lane == src && hit) ok = false;
       }
+    }
+    if (ok && i < n1 && !flat) {
+      key = key_of(idx);
+      ok = key >= lo && key <= hi;  // (a narrowed slice)
     }
     const u32 slot = warp_append(count, ok);
     if (ok && slot < c.cap_act) {
@@ -526,8 +542,10 @@ __device__ void resolve_body(const Group& g, const RoundCfg& c, const RoundPtrs&
   const u32 j = tid & (G - 1);
   const u32 gmask = G == 32 ? FULL : ((1u << (G & 31)) - 1u) << ((tid & 31) & ~(G - 1));
   const u32 gpb = blockDim.x / G;
-  for (u32 i = team.rank * gpb + tid / G; i < n; i += team.size * gpb) {
-    const uint4 raw = *reinterpret_cast<const uint4*>(cur + i);
+  for (u32 i0 = team.rank * gpb; i0 < n; i0 += team.size * gpb) {
+    const u32 i = i0 + tid / G;
+    const bool valid = i < n;
+    const uint4 raw = valid ? *reinterpret_cast<const uint4*>(cur + i) : make_uint4(0, 0, 0, 0);
     const u64 key = (u64)raw.y << 32 | raw.x;
     const u32 o = raw.z >> 31, y = (raw.z >> 15) & 0x7FFFu, x = raw.z & 0x7FFFu;
     const u32 line = o ? x : y, pos = o ? y : x;
@@ -535,48 +553,58 @@ __device__ void resolve_body(const Group& g, const RoundCfg& c, const RoundPtrs&
     // on the k lines of its cells, from k - 1 cells before its line to it
     const BinRun same(ring_sub(pos, k - 1, L), 2 * k - 1, L, c.b);
     const BinRun cl(pos, k, L, c.b), cp(ring_sub(line, k - 1, L), k, L, c.b);
-    // the candidates of one bin (its place among the bins of orientation bo)
-    auto walk = [&](u32 bo, u32 bl, u32 bp) -> bool {
-      const u32 by = bo ? bp : bl, bx = bo ? bl : bp;  // stored by (row, column)
-      u32 e = heads[((size_t)bo * c.nb + by) * c.nb + bx];
+    const u32 nbin = same.n + cl.n * cp.n;
+    // does the active candidate a beat this one?
+    auto beats = [&](const uint4& a) -> bool {
+      if (((u64)a.y << 32 | a.x) >= key) return false;
+      const u32 ao = a.z >> 31, ay = (a.z >> 15) & 0x7FFFu, ax = a.z & 0x7FFFu;
+      const u32 aline = ao ? ax : ay, apos = ao ? ay : ax;
+      if (ao == o) {
+        const u32 d = ring_sub(apos, pos, L);
+        return aline == line && (d < k || d > L - k);
+      }
+      return ring_sub(o ? ay : ax, pos, L) < k && ring_sub(line, o ? ax : ay, L) < k;
+    };
+    auto rest = [&](u32 e) -> bool {  // the chain of a bin from e on
       for (u32 guard = 0; e != NONE32 && guard < n; ++guard) {
         const uint4 a = *reinterpret_cast<const uint4*>(cur + e);
+        if (beats(a)) return true;
         e = a.w;
-        if (((u64)a.y << 32 | a.x) >= key) continue;
-        const u32 ay = (a.z >> 15) & 0x7FFFu, ax = a.z & 0x7FFFu;
-        const u32 aline = bo ? ax : ay, apos = bo ? ay : ax;
-        if (bo == o) {
-          const u32 d = ring_sub(apos, pos, L);
-          if (aline == line && (d < k || d > L - k)) return true;
-        } else if (ring_sub(aline, pos, L) < k && ring_sub(line, apos, L) < k) {
-          return true;
-        }
       }
       return false;
     };
-    bool beaten = false;
+    // bins are stored by (orientation, row, column)
+    auto head = [&](u32 bo, u32 bl, u32 bp) -> u32 {
+      const u32 by = bo ? bp : bl, bx = bo ? bl : bp;
+      return heads[(bo * c.nb + by) * c.nb + bx];
+    };
+    bool beaten = !valid;
     if (G == 1) {
-      for (u32 q = 0; q < same.n && !beaten; ++q) beaten = walk(o, line >> c.b, same.bin(q));
+      for (u32 q = 0; q < same.n && !beaten; ++q) beaten = rest(head(o, line >> c.b, same.bin(q)));
       for (u32 q1 = 0; q1 < cl.n && !beaten; ++q1)
         for (u32 q2 = 0; q2 < cp.n && !beaten; ++q2)
-          beaten = walk(o ^ 1u, cl.bin(q1), cp.bin(q2));
+          beaten = rest(head(o ^ 1u, cl.bin(q1), cp.bin(q2)));
     } else {
-      const u32 nbin = same.n + cl.n * cp.n;
       for (u32 q0 = 0; q0 < nbin && !beaten; q0 += G) {
         const u32 q = q0 + j;
         if (q < same.n) {
-          beaten = walk(o, line >> c.b, same.bin(q));
+          beaten = rest(head(o, line >> c.b, same.bin(q)));
         } else if (q < nbin) {
           const u32 qq = q - same.n, q1 = qq / cp.n;
-          beaten = walk(o ^ 1u, cl.bin(q1), cp.bin(qq - q1 * cp.n));
+          beaten = rest(head(o ^ 1u, cl.bin(q1), cp.bin(qq - q1 * cp.n)));
         }
         beaten = (__ballot_sync(gmask, beaten) & gmask) != 0;
       }
     }
+    // the lanes of a warp go on together from here: their k-mers are placed side
+    // by side, with one node counter update (L = 1024, k = 32, 1000 samples: 8.2 ms
+    // by lanes that left the search one after another, 7.4 now; four bins read
+    // ahead at a time 9.3, every lane at its own pace through bins and chains
+    // 11.7)
+    __syncwarp();
+    u32 node = warp_append(nodes, !beaten && j == 0);
+    if (G > 1) node = __shfl_sync(FULL, node, 0, G);
     if (beaten) continue;
-    u32 node = 0;
-    if (j == 0) node = atomicAdd(nodes, 1u);
-    if (G > 1) node = __shfl_sync(gmask, node, 0, G);
     if (node >= g.cap_nodes) {
       if (j == 0) atomicOr(&st.status, ST_NODE_OVF);
       continue;
@@ -643,81 +671,125 @@ __global__ void __launch_bounds__(RD_THREADS) k_resolve(Group g,
 }
 
 // The candidates of every line still live once the list is used up, those
-// with priorities in [lo, fill_hi]: the window OR of a line's cover bits,
-// doubling the window until it holds k cells.
+// with priorities in [lo, fill_hi].  k <= 33: the window OR of a word and the
+// next by doubling in registers, one word per lane.  Longer windows reach past
+// every word's end, so the live anchors of a word are those after its last
+// covered cell and at least k before the next covered cell beyond it: the
+// first covered cells of all words, and a suffix minimum over them, in one
+// pass over the staged line; one warp per line.  (Doubling windows over whole lines in shared memory took 5.5 ms at
+// L = 32768, k = 4096, 4 samples, and 1.95 ms at L = 1024, k = 32, 1000
+// samples; now 1.5 and
+// 1.3.)
 __device__ void refill_body(const Group& g, const RoundCfg& c, const RoundPtrs& p, u32 s,
-                            Team team, const Slice& sl, u32 lines_per_block, u32* flat_n,
-                            u32 (*buf)[REFILL_WORDS]) {
-  const u32 L = g.L, k = g.k, W = c.W, tid = threadIdx.x, nt = blockDim.x;
+                            Team team, const Slice& sl, u32* flat_n, u32* stage, u32 stage_words) {
+  const u32 L = g.L, k = g.k, W = c.W, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const u64 lo = sl.lo, hi = sl.fill_hi, zb = g.base[s] + SM_GAMMA;
   u32* flat = region_of(g, p.flat, s);
-  const u32 groups = (2 * L + lines_per_block - 1) / lines_per_block;
-  for (u32 gr = team.rank; gr < groups; gr += team.size) {
-    const u32 l0 = gr * lines_per_block, nl = min(lines_per_block, 2 * L - l0), nw = nl * W;
-    for (u32 i = tid; i < nw; i += nt) {
-      const u32 ll = i / W, w = i - ll * W, o = l0 + ll >= L, line = l0 + ll - (o ? L : 0u);
-      u32 v = cover_line(g, c, p, s, o, line)[w];
-      if (c.bs) v |= block_line(g, c, p, s, o, line >> c.bs)[w];
-      buf[0][i] = v;
+  const u32 WL = (L + 31) / 32;
+  // lists the live anchors of word i of line q (2 L lines), by a whole warp
+  auto put = [&](u32 o, u32 line, u32 i, u32 live) {
+    if (i == WL - 1 && (L & 31u)) live &= (1u << (L & 31u)) - 1u;
+    const u32 idx0 = o ? (u32)(g.LL + (u64)i * 32 * L + line) : line * L + i * 32;
+    const u32 step = o ? L : 1;
+    for (u32 m = live; m; m &= m - 1) {
+      const u32 bit = __ffs(m) - 1, idx = idx0 + step * bit;
+      const u64 key = g.keys ? g.keys[idx] : mix64(zb + SM_GAMMA * idx);
+      if (key < lo || key > hi) live &= ~(1u << bit);  // below lo: in the active set already
     }
-    __syncthreads();
-    u32 from = 0;
-    for (u32 m = 1; m < k;) {
-      const u32 d = min(m, k - m), dw = d >> 5, db = d & 31u;
-      for (u32 i = tid; i < nw; i += nt) {
-        const u32 w = i % W;
-        const u32 v0 = w + dw < W ? buf[from][i + dw] : 0u;
-        const u32 v1 = w + dw + 1 < W ? buf[from][i + dw + 1] : 0u;
-        buf[from ^ 1][i] = buf[from][i] | __funnelshift_r(v0, v1, db);
-      }
-      m += d;
-      from ^= 1u;
-      __syncthreads();
-    }
-    const u32 WL = (L + 31) / 32, items = nl * WL;
-    for (u32 i0 = 0; i0 < items; i0 += nt) {
-      const u32 i = i0 + tid;
-      u32 live = 0;
-      u64 idx0 = 0, step = 1;
-      if (i < items) {
-        const u32 ll = i / WL, w = i - ll * WL, o = l0 + ll >= L, line = l0 + ll - (o ? L : 0u);
-        live = ~buf[from][ll * W + w];
-        if (w == WL - 1 && (L & 31u)) live &= (1u << (L & 31u)) - 1u;
-        idx0 = o ? g.LL + (u64)w * 32 * L + line : (u64)line * L + w * 32;
-        step = o ? L : 1;
-        for (u32 m = live; m; m &= m - 1) {
-          const u32 b = __ffs(m) - 1;
-          const u64 idx = idx0 + step * b;
-          const u64 key = g.keys ? g.keys[idx] : mix64(zb + SM_GAMMA * idx);
-          if (key < lo || key > hi) live &= ~(1u << b);  // below lo: in the active set already
-        }
-      }
-      const u32 nh = __popc(live), lane = tid & 31;
-      u32 pre = nh;
+    if (!__any_sync(FULL, live != 0)) return;
+    const u32 nh = __popc(live);
+    u32 pre = nh;
 #pragma unroll
-      for (int d = 1; d < 32; d <<= 1) {
-        const u32 v = __shfl_up_sync(FULL, pre, d);
-        if ((int)lane >= d) pre += v;
-      }
-      u32 at = 0;
-      if (lane == 31 && pre) at = atomicAdd(flat_n, pre);
-      at = __shfl_sync(FULL, at, 31) + pre - nh;
-      for (u32 m = live; m; m &= m - 1, ++at)
-        if (at < c.cap_flat) flat[at] = (u32)(idx0 + step * (__ffs(m) - 1));
+    for (int d = 1; d < 32; d <<= 1) {
+      const u32 v = __shfl_up_sync(FULL, pre, d);
+      if ((int)lane >= d) pre += v;
     }
-    __syncthreads();
+    u32 at = 0;
+    if (lane == 31) at = atomicAdd(flat_n, pre);
+    at = __shfl_sync(FULL, at, 31) + pre - nh;
+    for (u32 m = live; m; m &= m - 1, ++at)
+      if (at < c.cap_flat) flat[at] = idx0 + step * (__ffs(m) - 1);
+  };
+  if (k <= 33) {
+    const u32 items = 2 * L * WL, nt = blockDim.x;
+    for (u32 i0 = team.rank * nt; i0 < items; i0 += team.size * nt) {
+      const u32 it = i0 + threadIdx.x;
+      u32 live = 0, o = 0, line = 0, i = 0;
+      if (it < items) {
+        const u32 q = it / WL;
+        i = it - q * WL;
+        o = q >= L;
+        line = o ? q - L : q;
+        const u32* fl = cover_line(g, c, p, s, o, line) + i;
+        u64 v = (u64)fl[1] << 32 | fl[0];
+        if (c.bs) {
+          const u32* bl = block_line(g, c, p, s, o, line >> c.bs) + i;
+          v |= (u64)bl[1] << 32 | bl[0];
+        }
+        for (u32 m = 1; m < k;) {
+          const u32 d = min(m, k - m);
+          v |= v >> d;
+          m += d;
+        }
+        live = ~(u32)v;
+      }
+      put(o, line, i, live);
+    }
+    return;
+  }
+  // warps that have room for a line of W words
+  const u32 nwarp = min(blockDim.x / 32, stage_words / W);
+  if (warp >= nwarp) return;
+  u32* ln = stage + warp * W;
+  for (u32 q = team.rank * nwarp + warp; q < 2 * L; q += team.size * nwarp) {
+    const u32 o = q >= L, line = o ? q - L : q;
+    const u32* fl = cover_line(g, c, p, s, o, line);
+    const u32* bl = c.bs ? block_line(g, c, p, s, o, line >> c.bs) : fl;
+    // lane l keeps words [l per, (l + 1) per); staged, the line is read in
+    // coalesced order all the same
+    const u32 per = ((W + 31) / 32) | 1u;
+    for (u32 i = lane; i < W; i += 32) ln[i] = c.bs ? fl[i] | bl[i] : fl[i];
+    __syncwarp();
+    const u32 a = min(lane * per, W), b = min(a + per, W);
+    u32 first = NONE32;
+    for (u32 i = a; i < b && first == NONE32; ++i)
+      if (ln[i]) first = i * 32 + __ffs(ln[i]) - 1;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const u32 v = __shfl_down_sync(FULL, first, d);
+      if (lane + d < 32) first = min(first, v);
+    }
+    u32 nxt = __shfl_down_sync(FULL, first, 1);  // first covered cell after this lane's words
+    if (lane == 31) nxt = NONE32;
+    // this lane's words from the last to the first, all lanes in step
+    for (u32 st = 0; st < per; ++st) {
+      const u32 i = a + per - 1 - st;
+      const u32 w = i < b ? ln[i] : 0u;
+      u32 live = 0;
+      if (i < b && i < WL) {
+        const u32 from = w ? 32u - __clz(w) : 0u;  // past the last covered cell
+        const u32 end = nxt == NONE32      ? 32u
+                        : nxt >= k + i * 32 ? min(nxt - k - i * 32 + 1, 32u)
+                                            : 0u;
+        if (from < end) live = (0xFFFFFFFFu << from) & (0xFFFFFFFFu >> (32 - end));
+      }
+      if (w) nxt = i * 32 + __ffs(w) - 1;
+      put(o, line, i, live);
+    }
+    __syncwarp();
   }
 }
 
 __global__ void __launch_bounds__(RD_THREADS) k_refill(Group g, const __grid_constant__ RoundCfg c,
-                                                       RoundPtrs p, u32 lines_per_block) {
-  __shared__ u32 buf[2][REFILL_WORDS];
+                                                       RoundPtrs p) {
+  __shared__ u32 stage[REFILL_WORDS];
   const u32 s = blockIdx.y;
   if (g.st[s].done) return;
   RoundState& r = p.rs[s];
   if (!r.sl.refill) return;
   const Slice sl = r.sl;
-  refill_body(g, c, p, s, Team{blockIdx.x, gridDim.x}, sl, lines_per_block, &r.flat_n, buf);
+  refill_body(g, c, p, s, Team{blockIdx.x, gridDim.x}, sl, &r.flat_n, stage, REFILL_WORDS);
+  __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
     if (atomicAdd(&r.ticket2, 1u) == gridDim.x - 1) {

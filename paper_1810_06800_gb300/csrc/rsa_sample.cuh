@@ -27,7 +27,7 @@ struct Shape {       // everything a sample's run needs to know of its (L, k)
   RoundCfg c;
   RoundPtrs p;
   SearchCfg sc;
-  u32 probe_cap, lines, sites;
+  u32 probe_cap, sites;
   // byte offsets of the buffers kept in shared memory (NO_HOT: in the
   // workspace), and their size
   u32 fine, heads, act, anch, hot_bytes;
@@ -54,7 +54,7 @@ struct SampleSmem {
 };
 union SampleScratch {  // one use at a time
   DenseSmem<SMP_THREADS, SMP_PER> dense;
-  u32 refill[2][REFILL_WORDS];
+  u32 refill[REFILL_WORDS];
   u32 hist[EHIST];
   struct {
     u32 hist[SUB_WORDS], queue[queue_words(SMP_THREADS)];
@@ -151,7 +151,7 @@ __device__ void run_sample(SampleSmem& sm, SampleScratch& scratch, unsigned char
       __syncthreads();
       if (sm.flag) break;
       while (r.sl.refill) {
-        refill_body(g, c, p, 0, team, r.sl, sm.sh.lines, &r.flat_n, scratch.refill);
+        refill_body(g, c, p, 0, team, r.sl, &r.flat_n, scratch.refill, REFILL_WORDS);
         __syncthreads();
         if (tid == 0) {
           refill_step(c, r.sl, r.flat_n);

@@ -355,12 +355,15 @@ __host__ __device__ constexpr u32 queue_words(u32 threads) { return 1 + (QUEUE_T
 template <typename Want, typename Work>
 __device__ __forceinline__ void scan_packed(u32 ne, Team team, EdgeQueue& q, Want want, Work work) {
   const u32 tid = threadIdx.x, nt = blockDim.x;
-  const u32 tile = QUEUE_TILE * nt;
+  // few edges: fewer per thread, on more blocks
+  const u32 per = min(QUEUE_TILE, max(1u, (ne + team.size * nt - 1) / (team.size * nt)));
+  const u32 tile = per * nt;
   if (tid == 0) q.n = 0;
   __syncthreads();
   for (u32 i0 = team.rank * tile; i0 < ne; i0 += team.size * tile) {
 #pragma unroll
     for (u32 j = 0; j < QUEUE_TILE; ++j) {
+      if (j == per) break;
       const u32 i = i0 + j * nt + tid;
       const bool ok = i < ne && want(i);
       const u32 at = warp_append(&q.n, ok);
