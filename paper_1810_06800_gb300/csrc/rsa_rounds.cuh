@@ -175,7 +175,7 @@ __device__ void dense_body(const Group& g, const RoundCfg& c, const RoundPtrs& p
   const u32 tile_n = PER * nt;
   const u64 N = 2 * g.LL, zb = g.base[s] + SM_GAMMA, zstep = SM_GAMMA * nt;
   const u64 ntile = (N + tile_n - 1) / tile_n;
-  const u32 shift = 32 - c.a;
+  const u32 limit = 1u << (32 - c.a);
   if (tid == 0) sm.count = 0;
   __syncthreads();
   for (u64 tile = team.rank; tile < ntile; tile += team.size) {
@@ -184,7 +184,7 @@ __device__ void dense_body(const Group& g, const RoundCfg& c, const RoundPtrs& p
     if (KEYS) {
       for (u32 j = 0; j < PER; ++j) {
         const u64 i = i0 + j * nt;
-        if (i < N && (u32)(g.keys[i] >> 32) >> shift == 0) hits |= 1u << j;
+        if (i < N && (u32)(g.keys[i] >> 32) < limit) hits |= 1u << j;
       }
     } else {
       u64 z = zb + SM_GAMMA * i0;
@@ -192,7 +192,7 @@ __device__ void dense_body(const Group& g, const RoundCfg& c, const RoundPtrs& p
       for (u32 j = 0; j < PER; ++j, z += zstep) {
         u64 h = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
         h = (h ^ (h >> 27)) * 0x94D049BB133111EBull;
-        if ((u32)(h >> 32) >> shift == 0) hits |= 1u << j;
+        if ((u32)(h >> 32) < limit) hits |= 1u << j;
       }
       if (i0 + (u64)(PER - 1) * nt >= N) {
         for (u32 j = 0; j < PER; ++j)
@@ -676,10 +676,9 @@ __global__ void __launch_bounds__(RD_THREADS) k_resolve(Group g,
 // every word's end, so the live anchors of a word are those after its last
 // covered cell and at least k before the next covered cell beyond it: the
 // first covered cells of all words, and a suffix minimum over them, in one
-// pass over the staged line; one warp per line.  (Doubling windows over whole lines in shared memory took 5.5 ms at
-// L = 32768, k = 4096, 4 samples, and 1.95 ms at L = 1024, k = 32, 1000
-// samples; now 1.5 and
-// 1.3.)
+// pass over the staged line; one warp per line.  (Doubling windows over whole
+// lines in shared memory took 5.5 ms at L = 32768, k = 4096, 4 samples, and
+// 1.95 ms at L = 1024, k = 32, 1000 samples; now 1.2 and 1.3.)
 __device__ void refill_body(const Group& g, const RoundCfg& c, const RoundPtrs& p, u32 s,
                             Team team, const Slice& sl, u32* flat_n, u32* stage, u32 stage_words) {
   const u32 L = g.L, k = g.k, W = c.W, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1017,8 +1016,12 @@ __device__ void contacts_body(const Group& g, const RoundCfg& c, const RoundPtrs
   hist.flush(g, s);
 }
 
+// Six blocks per SM: the pass waits for owner lookups in L2 (issue slots 16%
+// busy), and the registers that six leave per thread suffice.  L = 32768,
+// k = 4096, 4 samples 1.53 -> 1.26 ms; L = 1024, k = 32, 1000 samples 2.07 ->
+// 2.03.
 template <int G>
-__global__ void __launch_bounds__(256) k_contacts(Group g, const __grid_constant__ RoundCfg c,
+__global__ void __launch_bounds__(256, 6) k_contacts(Group g, const __grid_constant__ RoundCfg c,
                                                   RoundPtrs p) {
   __shared__ u32 hist_sh[EHIST];
   if (g.st[blockIdx.y].sdone) return;
