@@ -3,15 +3,15 @@
 
 Workload (default): the large-k batch, L = 32768 periodic lattice, k = 4096,
 8 samples with seeds 1..8 per step (per rank under torchrun; rank r uses
-seeds r*8 + 1 ..), 78 GB held on the device.  One step runs the whole path
-for the batch: the parallel greedy rounds to jamming (n_j), the contact
-graph, and the first-wrap bisection (n_c).  Prints one JSON line.
+seeds r*8 + 1 ..), 59 GB held on the device.  One step runs the whole path
+for the batch: deposition to jamming by priority slices (n_j), the contact
+graph, and the search for the first wrap (n_c).  Prints one JSON line.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
                   [--workload NAME]
 
-`value` is timed on the product path (graph-replayed round and probe loops,
-no per-kernel events).  A separate profiled pass of the same steps records a
+`value` is timed on the product path (one graph per run, no per-kernel
+events).  A separate profiled pass of the same steps records a
 CUDA event pair around every launch for the per-kernel shares and the
 roofline of the dominant kernel.  `--impl reference` times the CPU oracle (a
 plain sequential scan plus union-find in C) on the host cores, on a bounded
@@ -54,75 +54,28 @@ MIX_WORKLOADS = {
 }
 METRIC = "jammed samples/s (n_j and n_c per sample, bit-exact to the oracle)"
 
-# Algorithmic bytes per processed lattice cell of each round kernel, from
-# the byte model of the method's unfused steps: rowmin reads a priority and
-# writes a cell minimum (8 + 8); colmin reads a priority and the row minimum
-# and writes their minimum (8 + 8 + 8); accept reads the cell minimum along
-# both orientations and both priorities (2 x 8 + 16); kill reads occupancy
-# (1).  A kernel that carries out several of these steps is credited with
-# their sum over the cells it processed; where two kernels split one step,
-# each is credited with the part it does.  Priorities are recomputed rather
-# than stored and minima are kept as short argmin codes, so the kernels move
-# far fewer DRAM bytes than this (ncu "traffic").
-STEP_BYTES = {"rowmin": 16.0, "colmin": 24.0, "accept": 32.0, "kill": 1.0}
-KERNEL_STEPS = {
-    # 32 x 32 tile path: one pass both window minima, one pass acceptance
-    "k_tile_cmin": (("rowmin", "colmin"), 40.0),
-    "k_tile_accept": (("accept", "kill"), 33.0),
-    # long-k line path: horizontal windows (rowmin); vertical windows (the
-    # window part of colmin, 16 of its 24 bytes); the per-cell combine of
-    # the two minima (the remaining 8); acceptance along rows / columns (half
-    # of accept + kill each)
-    "k_line_cmin_h": (("rowmin",), 16.0),
-    "k_line_cmin_v": (("colmin",), 16.0),
-    "k_line_codes": (("colmin",), 8.0),
-    "k_line_combine": (("colmin",), 8.0),
-    "k_line_accept_h": (("accept", "kill"), 16.5),
-    "k_line_accept_v": (("accept", "kill"), 16.5),
-    # long-k lines of whole k-blocks: the same split with argmin offsets
-    "k_lwin_h": (("rowmin",), 16.0),
-    "k_lwin_v": (("colmin",), 16.0),
-    "k_lcomb": (("colmin",), 8.0),
-    "k_lacc_h": (("accept", "kill"), 16.5),
-    "k_lacc_v": (("accept", "kill"), 16.5),
-    # general path
-    "k_row_cmin": (("rowmin",), 16.0),
-    "k_col_cmin": (("colmin",), 24.0),
-    "k_row_accept": (("accept", "kill"), 16.5),
-    "k_col_accept": (("accept", "kill"), 16.5),
-}
-# Processed cells per kernel: (work counter, share of it).  Tile path
-# counters: 0 cmin cells, 1 cmin keys, 2 accept cells, 3 accept keys; long-k
-# path: 0 / 1 horizontal / vertical window cells, 2 acceptance cells (both
-# orientations), 3 combine cells.  The general path has no counters: every
-# cell of every round.
-WORK_CELLS = {"k_tile_cmin": (0, 1.0), "k_tile_accept": (2, 1.0),
-              "k_line_cmin_h": (0, 1.0), "k_line_cmin_v": (1, 1.0),
-              "k_line_codes": (3, 1.0), "k_line_combine": (3, 1.0),
-              "k_line_accept_h": (2, 0.5), "k_line_accept_v": (2, 0.5),
-              "k_lwin_h": (0, 1.0), "k_lwin_v": (1, 1.0), "k_lcomb": (3, 1.0),
-              "k_lacc_h": (2, 0.5), "k_lacc_v": (2, 0.5)}
-# A second view of the tile kernels, which are bound by integer issue:
-# algorithmic 32-bit lane operations (a 64-bit minimum is 4 ops plus 1 when
-# the argmin is tracked, a window minimum is 3 minima per cell, a liveness
-# test 4 ops, a splitmix64 priority 20 ops) against 128 integer lanes per SM
-# per clock.
-OPS_PER_KEY = 20
-OPS_PER_CELL = {"k_tile_cmin": 2 * 3 * 5 + 6 + 2 * 4, "k_tile_accept": 2 * 3}
-TILE_KEYS = {"k_tile_cmin": 1, "k_tile_accept": 3}
+# The deposition's arithmetic is one splitmix64 priority for each of the 2 L^2
+# candidates of a sample, in the pass that hashes them all (k_dense): about 18
+# integer instructions each (a 64-bit addition, two xor-shifts and products,
+# of the last product the high word only, a compare).  Its roofline is the
+# integer rate of 128 lanes per SM and clock.  The kernels after it work on
+# lists of a few per cent of the candidates and on the accepted k-mers; they
+# wait for L2 and have no byte or operation model.
+OPS_PER_CANDIDATE = 18
 ALU_LANES_PER_SM = 128
+
+# Byte model of a whole-lattice round pass (rowmin reads a priority and writes a
+# cell minimum, 8 + 8 bytes per cell): for recorded figures of such a pass.
+KERNEL_STEPS = {"k_lwin_h": (("rowmin",), 16.0)}
+WORK_CELLS = {"k_lwin_h": (0, 1.0)}
 
 # The source file that holds each kernel: a DRAM-traffic figure measured by
 # ncu is used only while that file is unchanged.
-KERNEL_FILE = {"k_tile_cmin": "rsa_tile.cuh", "k_tile_accept": "rsa_tile.cuh",
-               "k_line_cmin_h": "rsa_line.cuh", "k_line_cmin_v": "rsa_line.cuh",
-               "k_line_codes": "rsa_line.cuh", "k_line_accept_h": "rsa_line.cuh",
-               "k_line_accept_v": "rsa_line.cuh", "k_lwin_h": "rsa_lwin.cuh",
-               "k_lwin_v": "rsa_lwin.cuh", "k_lcomb": "rsa_lwin.cuh",
-               "k_lacc_h": "rsa_lwin.cuh", "k_lacc_v": "rsa_lwin.cuh",
-               "k_row_cmin": "rsa_kernels.cuh",
-               "k_col_cmin": "rsa_kernels.cuh", "k_row_accept": "rsa_kernels.cuh",
-               "k_col_accept": "rsa_kernels.cuh"}
+KERNEL_FILE = {"k_dense": "rsa_rounds.cuh", "k_pick": "rsa_rounds.cuh",
+               "k_resolve": "rsa_rounds.cuh", "k_refill": "rsa_rounds.cuh",
+               "k_edges": "rsa_rounds.cuh", "k_probe": "rsa_search.cuh",
+               "k_sample": "rsa_sample.cuh",
+               "k_lwin_h": "rsa_lwin.cuh", "k_tile_cmin": "rsa_tile.cuh"}
 
 
 def src_digest(kernel: str) -> str:
@@ -131,6 +84,8 @@ def src_digest(kernel: str) -> str:
     edits keep a measurement valid while any code change voids it."""
     import re
     f = os.path.join(ROOT, "paper_1810_06800_gb300", "csrc", KERNEL_FILE.get(kernel, "rsa.cu"))
+    if not os.path.exists(f):  # a kernel that is no longer there
+        return ""
     with open(f) as fh:
         lines = [re.sub(r"//.*$", "", ln).rstrip() for ln in fh]
     code = "\n".join(ln for ln in lines if ln)
@@ -317,6 +272,15 @@ def roofline(dom, kstats, work, passes, L, n_cells_round, hbm_peak, peak_kind, s
     `window_threads` is the window-pass CTA size the run asked for (0: the
     library's default, not known here)."""
     dom_ms, dom_launches = kstats[dom]
+    if dom == "k_dense" and dom_ms > 0:
+        n_cand = work["raw"][0]
+        peak = sm_count * ALU_LANES_PER_SM * sm_mhz * 1e6 / 1e9
+        got = n_cand * OPS_PER_CANDIDATE / (dom_ms / 1e3) / 1e9
+        return {"bound": "alu", "kernel": dom, "unit": "Gop/s", "peak": peak,
+                "peak_source": f"{sm_count} SMs x {ALU_LANES_PER_SM} int lanes x {sm_mhz:.0f} MHz",
+                "achieved": got, "frac": got / peak, "candidates": n_cand,
+                "candidates_per_s": n_cand / (dom_ms / 1e3), "ops_per_candidate": OPS_PER_CANDIDATE,
+                "avg_launch_ms": dom_ms / dom_launches, "traffic": None}
     if dom in WORK_CELLS:
         ctr, share = WORK_CELLS[dom]
         cells = work["raw"][ctr] * share
@@ -348,15 +312,6 @@ def roofline(dom, kstats, work, passes, L, n_cells_round, hbm_peak, peak_kind, s
     if fresh and "window_threads" in ent:
         fresh = ent["window_threads"] == window_threads
     out["traffic"] = (ent["bytes_per_cell"] * cells / dom_launches) if fresh else None
-    if dom in OPS_PER_CELL:
-        keys = work["raw"][TILE_KEYS[dom]]
-        ops = cells * OPS_PER_CELL[dom] + keys * OPS_PER_KEY
-        peak = sm_count * ALU_LANES_PER_SM * sm_mhz * 1e6 / 1e9
-        got = ops / (dom_ms / 1e3) / 1e9
-        out["alu_view"] = {"bound": "alu", "achieved": got, "peak": peak, "unit": "Gop/s",
-                           "frac": got / peak,
-                           "peak_source": f"{sm_count} SMs x {ALU_LANES_PER_SM} int lanes x "
-                                          f"{sm_mhz:.0f} MHz"}
     return out
 
 
@@ -561,9 +516,9 @@ def main():
     ap.add_argument("--profile-steps", type=int, default=2,
                     help="steps of the separate pass with per-kernel CUDA events")
     ap.add_argument("--window-threads", type=int, default=0,
-                    help="CTA size of the long-k window pass (128 or 256; 0 = the library default)")
+                    help="a former setting, checked and without effect (128 or 256; 0 = not set)")
     ap.add_argument("--rounds-per-check", type=int, default=0,
-                    help="greedy rounds per captured chunk (0 = the library default)")
+                    help="rounds per host check after the run's first graph (0 = the library default)")
     ap.add_argument("--cpu-seconds", type=float, default=10.0)
     ap.add_argument("--no-cpu-baseline", action="store_true")
     args = ap.parse_args()
@@ -695,11 +650,11 @@ def main():
     # the same figures for every round kernel with a byte model
     roof_all = {}
     for nm in ours:
-        if nm in KERNEL_STEPS:
+        if nm == "k_dense":
             r = roofline(nm, ours, work, passes, L, L * L, hbm_peak, peak_kind, sm_count, sm_mhz,
                          args.window_threads)
-            roof_all[nm] = {k2: r.get(k2) for k2 in ("achieved", "frac", "alg_bytes_per_cell",
-                                                      "avg_launch_ms", "traffic")}
+            roof_all[nm] = {k2: r.get(k2) for k2 in ("bound", "unit", "achieved", "frac",
+                                                      "candidates_per_s", "avg_launch_ms")}
     total_ms = sum(x[0] for x in ours.values())
     kernel_table = {nm: {"ms": round(v[0], 3), "launches": v[1],
                          "share": round(v[0] / total_ms, 4)} for nm, v in ours.items()}

@@ -56,8 +56,9 @@ int rsa_create(uint32_t L, uint32_t k, uint64_t seed, rsa_t **out);
 /* Run n_samples samples (seeds seed .. seed + n_samples - 1) to jamming and
  * find each first-wrap count, on `stream`.  Device memory is allocated on
  * first use (or taken from a bound workspace).  The call returns once the
- * work is enqueued; it synchronises `stream` a few times while running the
- * data-dependent round and bisection loops.  Results stay on the device
+ * work is enqueued; where shapes do not run in one launch it synchronises
+ * `stream`, once as a rule and again only for samples that need more rounds or
+ * probes than the run's graph holds.  Results stay on the device
  * until rsa_results(). */
 int rsa_run_batch(rsa_t *h, uint32_t n_samples, void *stream);
 
@@ -170,7 +171,7 @@ int rsa_set_window_threads(rsa_t *h, uint32_t threads);
 int rsa_results(rsa_t *h, uint32_t *n_j, uint32_t *n_c, uint32_t n);
 
 /* Per-sample diagnostics of the last run (any pointer may be NULL, arrays of
- * length n): rounds of the parallel greedy, bisection probes, contact edges
+ * length n): rounds of the deposition, probes of the first-wrap search, contact edges
  * of the k-mer graph, and the status code. */
 int rsa_sample_stats(rsa_t *h, uint32_t *rounds, uint32_t *probes, uint32_t *edges,
                      int32_t *status, uint32_t n);
@@ -222,7 +223,7 @@ int rsa_accepted(rsa_t *h, uint32_t sample, uint32_t *idx, uint32_t cap, uint32_
  *              RSA_ETIMEOUT from rsa_results;
  *   uf_steps   steps of one union-find walk and retries of one link (default
  *              2^20): a walk that runs out stops its probe, RSA_ETIMEOUT;
- *   probe_cap  bisection probes per sample (default 40), RSA_ETIMEOUT;
+ *   probe_cap  probes of the first-wrap search per sample (default 96), RSA_ETIMEOUT;
  *   edge_cap   contact edges stored per sample (default: the buffer's
  *              capacity, min(2 L^2, 6 L^2/k + 4 L) + 64): more edges than
  *              that stop the sample with RSA_ENOMEM, and nothing is written

@@ -1,9 +1,10 @@
 """Build the in-tree CUDA library ``_lib/librsa_gb300.so`` for sm_103a.
 
 The library has two translation units, compiled in parallel and linked
-together: ``csrc/rsa.cu`` (the engine: handles, round, contact-graph and
-first-wrap kernels) and ``csrc/rsa_mix.cu`` (samples of uneven shapes: the
-small-lattice one-CTA-per-sample kernel, mixed batches, the autotuner)."""
+together: ``csrc/rsa.cu`` (the engine and every kernel: handles, deposition,
+contact graph, first wrap, configurations, small lattices) and
+``csrc/rsa_mix.cu`` (host code for samples of uneven shapes: mixed batches,
+the autotuner)."""
 from __future__ import annotations
 
 import os

@@ -4,16 +4,14 @@
 // viable-list deposition tries each (orientation, y, x) candidate once in
 // uniformly random order and accepts it iff its k cells are free.  With the
 // order fixed by distinct 64-bit priorities this is the lexicographically
-// first maximal independent set of the candidate conflict graph, which is
-// reached in rounds: a live candidate whose priority is the smallest over
-// every live candidate sharing a cell with it is accepted, and candidates
-// touching the newly occupied cells die.  Per round and per cell:
-//   cmin(cell) = min over live candidates covering the cell of key,
-//   accept c   iff min over c's k cells of cmin == key(c).
-// Both minima are sliding-window minima of width k along rows (horizontal
-// candidates) and columns (vertical ones), computed with the van Herk /
-// Gil-Werman split into k-aligned blocks (segmented prefix and suffix
-// minima), so the cost per cell does not depend on k.
+// first maximal independent set of the candidate conflict graph.  The
+// priorities are taken in slices, smallest first (rsa_rounds.cuh): of a
+// slice's candidates those still live against the accepted k-mers are put in
+// a list, and a listed candidate whose priority is the smallest of all listed
+// ones sharing a cell with it is accepted, round by round, until the slice is
+// empty.  rsa_search.cuh builds the contact graph and finds the first wrap,
+// rsa_sample.cuh runs a whole sample in one block with the same bodies, and
+// rsa_config.cuh answers for the configuration at m k-mers.
 //
 // Priorities are recomputed from (seed, idx) wherever they are needed
 // instead of being stored: splitmix64 costs a few integer instructions,
@@ -38,15 +36,13 @@ constexpr unsigned FULL = 0xFFFFFFFFu;
 constexpr u32 WORK_SLOTS = 32;
 constexpr u32 EHIST = 2048;  // bins of time_bin
 
-
 // status bits (per sample), mapped to RSA_E* codes by the host
 constexpr u32 ST_NODE_OVF = 1u;     // more accepted k-mers than L^2/k (bug)
 constexpr u32 ST_EDGE_OVF = 2u;     // contact-edge buffer too small
 constexpr u32 ST_UF_CAP = 4u;       // union-find retry cap hit
 constexpr u32 ST_NOWRAP = 8u;       // no wrap at jamming
-constexpr u32 ST_SEARCH_CAP = 16u;  // bisection did not converge
+constexpr u32 ST_SEARCH_CAP = 16u;  // search did not converge
 constexpr u32 ST_ROUND_CAP = 32u;   // round loop cap hit
-constexpr u32 ST_SEARCH_BAD = 64u;  // inconsistent bisection counts
 
 // splitmix64 output finaliser (Stafford "Mix13"), Steele/Lea/Flood 2014.
 __device__ __forceinline__ u64 mix64(u64 z) {
@@ -137,22 +133,7 @@ __device__ __forceinline__ void work_add(const Group& g, u32 c, u64 v) {
   atomicAdd(g.work + c * WORK_SLOTS + (blockIdx.x & (WORK_SLOTS - 1)), v);
 }
 
-__device__ __forceinline__ u64 cand_key(const Group& g, u32 s, u64 idx) {
-  if (g.keys) return g.keys[idx];
-  return mix64(g.base[s] + SM_GAMMA * (idx + 1));
-}
-
-template <typename T> __device__ __forceinline__ T tmin(T a, T b) { return b < a ? b : a; }
 template <typename T> __device__ __forceinline__ T tmax(T a, T b) { return b > a ? b : a; }
-
-// Position of cell (cy, cx) inside the k-mer whose anchor is packed as
-// o << 31 | y0 << 15 | x0; *o receives the orientation.
-__device__ __forceinline__ u32 pos_in_kmer(u32 pos, u32 cy, u32 cx, u32 L, u32* o) {
-  const u32 oo = pos >> 31, y0 = (pos >> 15) & 0x7FFFu, x0 = pos & 0x7FFFu;
-  *o = oo;
-  const u32 d = oo == 0 ? cx - x0 : cy - y0;
-  return (int)d < 0 ? d + L : d;
-}
 
 __device__ __forceinline__ u64 uf_pack(u32 p, u32 dx, u32 dy) {
   return (u64)p | ((u64)(dx & 0xFFFFu) << 32) | ((u64)(dy & 0xFFFFu) << 48);

@@ -3,10 +3,10 @@
 //
 //   rsa_run_mix    a batch of samples of any shapes: the small ones in one
 //                  persistent launch, every other shape on its own handle
-//                  (graph-replayed rounds) on its own stream, all at once;
-//   rsa_tune       per (GPU, L, k, batch size): small mode and its CTA size,
-//                  or the global path and its rounds per host check, by
-//                  timing each candidate once; kept in a JSON-lines cache.
+//                  on its own stream, all at once;
+//   rsa_tune       per (GPU, L, k, batch size): small mode, or a handle and its
+//                  rounds per host check, by timing each candidate once; kept
+//                  in a JSON-lines cache.
 // Everything here runs the library's own kernels through its public calls;
 // results never depend on the choices made (tested).
 #include <cuda_runtime.h>

@@ -311,7 +311,6 @@ __device__ u64 halve_window(const Window& w, u64 lo0, u32 shift, const u32* set,
 // warp (every lane holds the same w).  True if the search of the sample ends
 // here.
 __device__ bool probe_step(Window& w, const u32* set, u32 win_cap, u32 probe_cap, u32& status) {
-  const u32 lane = threadIdx.x & 31;
   w.probes += 1;
   if (status & ST_UF_CAP) return true;
   const bool wrap = set[SUB_WRAP] != 0, first = w.first != 0;

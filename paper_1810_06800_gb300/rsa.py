@@ -298,9 +298,10 @@ def rsa_kernel_stats(h):
 
 
 def rsa_work_stats(h):
-    """Round-pass work since the previous call: the four counters under their
-    tile-path names, and as ``raw`` (their long-k path meaning differs; see
-    include/rsa.h)."""
+    """Work of the deposition since the previous call: the four counters of
+    include/rsa.h as ``raw`` (candidates hashed by the first pass, list entries
+    tested, active candidates resolved, k-mers accepted), and the same four
+    under the names of former round passes, kept for callers that read them."""
     out = np.zeros(4, dtype=np.uint64)
     _check(load().rsa_work_stats(h, out.ctypes.data, 4))
     return dict(cmin_cells=int(out[0]), cmin_keys=int(out[1]), accept_cells=int(out[2]),
