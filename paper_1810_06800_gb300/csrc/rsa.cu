@@ -672,7 +672,8 @@ int run_impl(rsa_t* h, const uint64_t* seeds, u32 n, const uint64_t* keys, cudaS
   // One block per sample for the small lattices, and for those that still fit
   // a block when there are enough samples to fill the GPU with blocks
   // (L = 256, k = 16: 256 samples 0.72 ms, over the whole grid 1.11; 4 samples
-  // 0.36 and 0.30), or when every launch costs the host (runs without graphs:
+  // 0.36 and 0.30; L = 160, k = 10, 4 samples 0.260 and 0.264, L = 192, k = 12, 4
+  // samples 0.300 and 0.267), or when every launch costs the host (runs without graphs:
   // 4 samples 0.39 against 0.43).
   const bool by_sample =
       G.one_block && (h->L <= 160 || n >= (u32)h->sm_count / 2 || !h->use_graphs);

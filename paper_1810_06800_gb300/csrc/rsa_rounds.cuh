@@ -153,7 +153,10 @@ __global__ void k_round_init(Group g, RoundCfg c, RoundPtrs p) {
   p.rs[s] = z;
 }
 
-// Every candidate hashed once.  A block goes over tiles of 4096 consecutive
+// Every candidate hashed once: bound by integer issue (L = 1024, k = 32: issue
+// slots 74% busy, ALU pipe 60%, 40 instructions per candidate with one in 8 to
+// be staged; 1000 samples, 2.1 G candidates, in 2.9 ms.  L = 32768, k = 4096, 4
+// samples, 8.6 G candidates, in 8.1 ms).  A block goes over tiles of 4096 consecutive
 // candidates; a thread keeps its 16 hits of a tile as a bit mask, so the
 // inner loop is the hash and one compare.  Hits are staged in shared memory
 // and leave by level, one global counter update per level and flush.
@@ -273,10 +276,16 @@ __device__ __forceinline__ u32 window_word(const u32* line, u32 w, u32 pos, u32 
   return v;
 }
 
-// The active set of this round.  Windows of up to LONGK cells are tested by
-// the lane that holds the candidate; longer ones first at three words, and
-// the few that pass by the whole warp.
-constexpr u32 PICK_LONGK = 96;
+// The active set of this round.  Bound by the loads of the cover words, which
+// lie anywhere on the lattice (issue slots 38 to 67% busy).  Windows of up to
+// PICK_LONGK cells are tested word by word by the lane that holds the
+// candidate, which stops at the first covered word; longer ones at three
+// words, at seven more, and the few that pass by the whole warp.  The line:
+// k_pick of L = 2048, k = 128, 32 samples 0.39 ms by lanes and 0.51 by warps,
+// L = 8192, k = 512, 32 samples 2.56 and 2.66, k = 1024, 8 samples 0.83 and
+// 0.72, L = 32768, k = 4096, 4 samples 4.87 and 3.72 (3.07 with the seven
+// words).
+constexpr u32 PICK_LONGK = 768;
 template <bool LONG>
 __device__ void pick_body(const Group& g, const RoundCfg& c, const RoundPtrs& p, u32 s, Team team,
                           const Slice& sl, u32 n1, u32 n2, u32* count) {
@@ -337,6 +346,13 @@ __device__ void pick_body(const Group& g, const RoundCfg& c, const RoundPtrs& p,
         const u32 wm = (w0 + w1) >> 1;
         ok = (window_word(fl, w0, pos, end) | window_word(bl, w0, pos, end) |
               window_word(fl, w1, pos, end) | window_word(bl, w1, pos, end) | fl[wm] | bl[wm]) == 0;
+      }
+      if (ok) {
+        const u32 step = (w1 - w0) >> 3;  // >= 3: whole words inside the window
+        u32 v = 0;
+#pragma unroll
+        for (u32 i = 1; i < 8; ++i) v |= fl[w0 + i * step] | bl[w0 + i * step];
+        ok = v == 0;
       }
       // the words between, 32 at a time, one candidate after another
       for (u32 m = __ballot_sync(FULL, ok); m; m &= m - 1) {
@@ -531,6 +547,9 @@ __device__ __forceinline__ void clear_bins(const Group& g, const RoundCfg& c, co
 
 // G lanes per active candidate.  Bins are about 4 sqrt(k) cells wide, which
 // leaves one or two active candidates in each and k / 16 bins to look at.
+// Bound by the latency of the chain counter - bin head - candidate - its next
+// (L = 1024, k = 32, 1000 samples: 30 of 41 resident warps wait for a load,
+// issue slots 21 to 28% busy, 7.6 ms in all rounds).
 // Adds this thread's accepted candidates to taken.
 template <int G>
 __device__ void resolve_body(const Group& g, const RoundCfg& c, const RoundPtrs& p, u32 s,

@@ -1,6 +1,6 @@
 """Deposition by priority slices against the CPU oracle where it can go wrong:
 sides one off a bit word, k at the borders of its variants (block lines from
-16 on, whole-warp window tests from 97, lanes per candidate at 129), lattices
+16 on, whole-warp window tests from 769, lanes per candidate at 129), lattices
 barely longer than k, where windows and bins meet themselves round the torus,
 and priority orders that fill the active set and the refilled list past their
 capacities, so that slices are narrowed and refills repeated."""
@@ -32,6 +32,16 @@ def test_slice_shapes(L, k):
         _same(lat, i, nj[i], nc[i], L, k, keys)
         acc, _ = oracle.scan(L, k, keys)
         assert (int(nx[i]), int(ny[i]), int(nxy[i])) == oracle.contacts(L, k, acc)
+    lat.close()
+
+
+@pytest.mark.parametrize("L,k", [(800, 768), (801, 769), (769, 769), (1100, 1055)])
+def test_long_windows(L, k):
+    seeds = [31, 32]
+    lat = rsa.Lattice(L, k)
+    nj, nc = lat.run(seeds)
+    for i, s in enumerate(seeds):
+        _same(lat, i, nj[i], nc[i], L, k, oracle.keys(L, s))
     lat.close()
 
 
