@@ -646,10 +646,16 @@ __device__ void resolve_body(const Group& g, const RoundCfg& c, const RoundPtrs&
   }
 }
 
+// With 16 and 32 lanes eight blocks per SM (32 registers, 8 bytes spilled): the
+// more candidates wait at once, the better (L = 8192, k = 512, 32 samples 4.5 ->
+// 3.7 ms, L = 32768, k = 4096, 4 samples 4.7 -> 4.5).  One lane gains nothing (7.6
+// and 7.6 ms at L = 1024, k = 32, 1000 samples) and eight lanes, used where the
+// GPU is not full, lose (one such sample 0.19 -> 0.20 ms): the compiler's choice
+// stays (0 sets no bound; 1 would let it take 72 and 88 registers, L = 777,
+// k = 100, 16 samples 0.57 -> 0.63 ms in all).
 template <int G>
-__global__ void __launch_bounds__(RD_THREADS) k_resolve(Group g,
-                                                        const __grid_constant__ RoundCfg c,
-                                                        RoundPtrs p) {
+__global__ void __launch_bounds__(RD_THREADS, G >= 16 ? 8 : 0)
+k_resolve(Group g, const __grid_constant__ RoundCfg c, RoundPtrs p) {
   __shared__ u32 taken_sh;
   const u32 s = blockIdx.y;
   SampleState& st = g.st[s];
