@@ -3,7 +3,7 @@
 
 Workload (default): the large-k batch, L = 32768 periodic lattice, k = 4096,
 8 samples with seeds 1..8 per step (per rank under torchrun; rank r uses
-seeds r*8 + 1 ..), 59 GB held on the device.  One step runs the whole path
+seeds r*8 + 1 ..), 60 GB held on the device.  One step runs the whole path
 for the batch: deposition to jamming by priority slices (n_j), the contact
 graph, and the search for the first wrap (n_c).  Prints one JSON line.
 
