@@ -12,10 +12,12 @@
 //              below and above where T_c is expected (k-mers at the first wrap
 //              over k-mers at jamming: 0.59 + 0.0225 log2 k), later ones
 //              halve the edges of the window;
-//   k_collect  once the window holds at most FIN_EDGES edges: those, with
-//              the roots of their ends and the displacement between the roots;
+//   k_collect  once the window holds at most FIN_EDGES edges (or edges of one
+//              time only): those, with the roots of their ends and the
+//              displacement between the roots;
 //   k_finish   one block per sample: the rest of the search in shared memory,
-//              on the graph of the roots; the last 32 edges one by one;
+//              on the graph of the roots; the last 32 edges one by one, unless
+//              the window has come down to one time, which then is T_c;
 //   k_rank     n_c, the k-mers of priority <= T_c.
 // Samples whose whole graph has at most FIN_EDGES edges need no probe.
 // That hi itself wraps is assumed until a probe shows it (the jammed lattice
@@ -271,18 +273,22 @@ __device__ __forceinline__ u32 sub_shift(const Window& w) {
   return width > 7 ? width - 7 : 0;
 }
 
-// A threshold that halves the `in` edges of the window, at the end of a
-// sub-bin (sub-bins of 2^shift times from lo0 on), by a whole warp.
+// A threshold that halves the `in` edges of the window, at an end of a sub-bin
+// (sub-bins of 2^shift times from lo0 on), by a whole warp.  Of the last
+// sub-bin that is its lower end: the window then shrinks to that sub-bin or
+// loses half of its edges, so about three probes take seven bits off a window
+// whose edges all share one time, where its middle would take one.
 __device__ u64 halve_window(const Window& w, u64 lo0, u32 shift, const u32* set, u32 in) {
   const u32 lane = threadIdx.x & 31;
+  const u64 span = (1ull << shift) - 1;
   u32 v[4], sum = 0;  // four sub-bins per lane
-  u64 end[4];
+  u64 from[4];
 #pragma unroll
   for (u32 i = 0; i < 4; ++i) {
     const u32 b = lane * 4 + i;
-    const u64 from = lo0 + 1 + ((u64)b << shift);
-    end[i] = from + ((1ull << shift) - 1);
-    const bool out = from <= lo0 || end[i] < from || end[i] <= w.lo || from > w.hi;
+    from[i] = lo0 + 1 + ((u64)b << shift);
+    const u64 end = from[i] + span < from[i] ? KEY_NONE : from[i] + span;
+    const bool out = from[i] <= lo0 || end <= w.lo || from[i] > w.hi;
     v[i] = out ? 0u : set[b];
     sum += v[i];
   }
@@ -295,16 +301,32 @@ __device__ u64 halve_window(const Window& w, u64 lo0, u32 shift, const u32* set,
   const u32 half = in / 2;
   const u32 m = __ballot_sync(FULL, inc >= half && sum);
   u32 a = inc - sum;
-  u64 mine = 0;
+  u64 mine = 0;  // start of the sub-bin (at least 1)
 #pragma unroll
   for (u32 i = 0; i < 4; ++i) {
     a += v[i];
-    if (mine == 0 && v[i] && a >= half) mine = end[i];
+    if (mine == 0 && v[i] && a >= half) mine = from[i];
   }
   u64 mid = 0;
-  if (m) mid = __shfl_sync(FULL, mine, __ffs(m) - 1);
+  if (m) {
+    mine = __shfl_sync(FULL, mine, __ffs(m) - 1);
+    mid = mine + span;
+    if (mid < mine || mid >= w.hi) mid = mine - 1;
+  }
   if (mid <= w.lo || mid >= w.hi) mid = w.lo + (w.hi - w.lo) / 2;
   return mid;
+}
+
+// The edges of a k-mer to its earlier neighbours all have its priority for
+// time (2 k of them where it meets the ends of others all along its sides), so
+// a window of one time can hold any number of edges.  Once a probe has wrapped
+// there, that time is T_c.
+__device__ __forceinline__ bool one_time(const Window& w) { return w.hi - w.lo == 1 && w.hi_ok; }
+
+// The next threshold of a window that is not the last one.
+__device__ __forceinline__ u64 next_threshold(const Window& w, u64 lo0, u32 shift, const u32* set,
+                                              u32 in) {
+  return w.hi - w.lo == 1 ? w.hi : halve_window(w, lo0, shift, set, in);
 }
 
 // The step from one probe to the next, from the counts in `set`, by a whole
@@ -325,7 +347,7 @@ __device__ bool probe_step(Window& w, const u32* set, u32 win_cap, u32 probe_cap
     w.lo = w.mid;
     w.cur ^= 1u;
   }
-  if (in <= win_cap) {
+  if (in <= win_cap || one_time(w)) {
     w.ready = 1;
     return false;
   }
@@ -334,7 +356,7 @@ __device__ bool probe_step(Window& w, const u32* set, u32 win_cap, u32 probe_cap
     return true;
   }
   if (first && !wrap && w.next_mid > w.lo && w.next_mid < w.hi) w.mid = w.next_mid;
-  else w.mid = halve_window(w, lo0, shift, set, in);
+  else w.mid = next_threshold(w, lo0, shift, set, in);
   return false;
 }
 
@@ -627,8 +649,8 @@ __device__ void finish_body(const Group& g, const SearchCfg& c, u32 s, const Win
   for (u32 i = tid; i < nid; i += nt) ub[i] = uf_pack(i, 0, 0);
   if (tid < 32) {
     Window w = fs.w;
-    if (n <= FIN_LAST) w.ready = 1;
-    else if (!whole) w.mid = halve_window(w, w.lo, shift0, fs.set, n);
+    if (n <= FIN_LAST || one_time(w)) w.ready = 1;
+    else if (!whole) w.mid = next_threshold(w, w.lo, shift0, fs.set, n);
     if (tid == 0) fs.w = w;
   }
   __syncthreads();
@@ -712,7 +734,9 @@ __device__ void finish_body(const Group& g, const SearchCfg& c, u32 s, const Win
   if (warp == 0) {
     u32 status = fs.status, probes = w.probes;
     u64 tc = 0;
-    if (go && probes >= probe_cap) {
+    if (go && one_time(w)) {
+      tc = w.hi;
+    } else if (go && probes >= probe_cap) {
       status |= ST_SEARCH_CAP;
     } else if (go) {
       ++probes;
