@@ -24,6 +24,9 @@
  *     holds a message (thread-local, valid until the next call on the thread);
  *   - `stream` is a cudaStream_t passed as void* (NULL = legacy default);
  *   - host pointers are caller-owned and only read/written during the call;
+ *   - rsa_results, rsa_sample_stats, rsa_contacts and rsa_accepted may be called
+ *     on one handle from several threads at once, after its run has returned;
+ *     any other call needs the handle for itself;
  *   - no call traps the GPU: device-side failures are recorded in a status
  *     word per sample and reported by rsa_results().
  *   - 1 <= k <= L <= 32768.

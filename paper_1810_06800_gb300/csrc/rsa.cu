@@ -16,6 +16,7 @@
 #include <cmath>
 #include <cstddef>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <cstdio>
 #include <cstring>
@@ -313,7 +314,10 @@ struct rsa {
   void* ws = nullptr;
   Layout lay{};
   u32 last_n = 0;
-  std::vector<SampleState> states;  // of the last run, once read (fetch_states)
+  // sample states of the last run, once read (fetch_states): readers on several
+  // threads share them
+  std::mutex states_mu;
+  std::shared_ptr<const std::vector<SampleState>> states;
   bool with_keys = false;
   cudaStream_t stream = nullptr;
   u32* h_counter = nullptr;  // pinned, READ_BYTES: loop and work counters, configuration bits
@@ -535,7 +539,10 @@ int run_impl(rsa_t* h, const uint64_t* seeds, u32 n, const uint64_t* keys, cudaS
   if ((rc = ensure_workspace(h, n, h->with_keys))) return rc;
   h->stream = stream;
   h->last_n = n;
-  h->states.clear();
+  {
+    std::lock_guard<std::mutex> lock(h->states_mu);
+    h->states.reset();
+  }
   Group g = group_of(h, n);
   const Geometry& G = h->geo;
   const Layout& l = h->lay;
@@ -726,18 +733,22 @@ int status_code(u32 bits) {
   return 0;
 }
 
-// The sample states of the last run, read from the device once per run.
-int fetch_states(rsa_t* h, const std::vector<SampleState>** out) {
+typedef std::shared_ptr<const std::vector<SampleState>> States;
+
+// The sample states of the last run, read from the device once per run.  A
+// reader keeps the ones it was given while it walks over them.
+int fetch_states(rsa_t* h, States* out) {
   if (!h->ws || h->last_n == 0) return fail(RSA_ESTATE, "no run to read");
-  if (h->states.size() != h->last_n) {
-    std::vector<SampleState> v(h->last_n);
+  std::lock_guard<std::mutex> lock(h->states_mu);
+  if (!h->states) {
+    auto v = std::make_shared<std::vector<SampleState>>(h->last_n);
     const char* b = static_cast<const char*>(h->ws);
-    CUDA_TRY(cudaMemcpyAsync(v.data(), b + h->lay.st, sizeof(SampleState) * h->last_n,
+    CUDA_TRY(cudaMemcpyAsync(v->data(), b + h->lay.st, sizeof(SampleState) * h->last_n,
                              cudaMemcpyDeviceToHost, h->stream));
     CUDA_TRY(cudaStreamSynchronize(h->stream));
-    h->states.swap(v);
+    h->states = std::move(v);
   }
-  *out = &h->states;
+  *out = h->states;
   return 0;
 }
 
@@ -809,7 +820,7 @@ int configuration(rsa_t* h, uint32_t sample, uint32_t m, uint32_t* counts, uint3
   if (!h) return fail(RSA_EINVAL, "null handle");
   if (sample >= h->last_n) return fail(RSA_EINVAL, "sample out of range");
   if (counts && cap < (u64)m + 1) return fail(RSA_EINVAL, "counts needs m + 1 entries");
-  const std::vector<SampleState>* states = nullptr;
+  States states;
   int rc = fetch_states(h, &states);
   if (rc) return rc;
   const std::vector<SampleState>& st = *states;
@@ -1109,7 +1120,7 @@ int rsa_run_static(uint32_t L, uint32_t k, const uint64_t* seeds, uint32_t n, ui
 int rsa_results(rsa_t* h, uint32_t* n_j, uint32_t* n_c, uint32_t n) {
   if (!h) return fail(RSA_EINVAL, "null handle");
   if (n > h->last_n) return fail(RSA_EINVAL, "n exceeds samples of the last run");
-  const std::vector<SampleState>* states = nullptr;
+  States states;
   int rc = fetch_states(h, &states);
   if (rc) return rc;
   const std::vector<SampleState>& st = *states;
@@ -1130,7 +1141,7 @@ int rsa_sample_stats(rsa_t* h, uint32_t* rounds, uint32_t* probes, uint32_t* edg
                      int32_t* status, uint32_t n) {
   if (!h) return fail(RSA_EINVAL, "null handle");
   if (n > h->last_n) return fail(RSA_EINVAL, "n exceeds samples of the last run");
-  const std::vector<SampleState>* states = nullptr;
+  States states;
   int rc = fetch_states(h, &states);
   if (rc) return rc;
   const std::vector<SampleState>& st = *states;
@@ -1146,7 +1157,7 @@ int rsa_sample_stats(rsa_t* h, uint32_t* rounds, uint32_t* probes, uint32_t* edg
 int rsa_contacts(rsa_t* h, uint32_t* n_x, uint32_t* n_y, uint32_t* n_xy, uint32_t n) {
   if (!h) return fail(RSA_EINVAL, "null handle");
   if (n > h->last_n) return fail(RSA_EINVAL, "n exceeds samples of the last run");
-  const std::vector<SampleState>* states = nullptr;
+  States states;
   int rc = fetch_states(h, &states);
   if (rc) return rc;
   const std::vector<SampleState>& st = *states;
@@ -1161,7 +1172,7 @@ int rsa_contacts(rsa_t* h, uint32_t* n_x, uint32_t* n_y, uint32_t* n_xy, uint32_
 int rsa_accepted(rsa_t* h, uint32_t sample, uint32_t* idx, uint32_t cap, uint32_t* count) {
   if (!h || !count) return fail(RSA_EINVAL, "null argument");
   if (sample >= h->last_n) return fail(RSA_EINVAL, "sample out of range");
-  const std::vector<SampleState>* states = nullptr;
+  States states;
   int rc = fetch_states(h, &states);
   if (rc) return rc;
   const std::vector<SampleState>& st = *states;
