@@ -121,17 +121,7 @@ void plan_search(u32 L, u32 k, Geometry& G) {
   // edges per k-mer of capacity: 2 at k = 1, 1.7 at k = 4, 1 from 32 on
   const double edges = (double)cn * (k == 1 ? 2.0 : k <= 8 ? 1.7 : 1.0) * 0.16 * f;
   G.probes = ce <= c.win_cap ? 0 : 3 + (u32)std::max(0.0, std::ceil(std::log2(edges / c.win_cap)));
-  // in one block: as many edges as fit beside the union-find words of all
-  // k-mers, so that most graphs need no probe at all
   G.ssc = c;
-  if (!c.hashed || cn <= 4 * FIN_EDGES) {
-    SearchCfg w = c;
-    w.hashed = 0;
-    w.ids = cn;
-    const size_t room = SMP_MAX - SMP_FIXED - (size_t)cn * 16;
-    w.win_cap = (u32)std::min<size_t>(ce, room / 18 / 8 * 8);
-    if (w.win_cap >= c.win_cap) G.ssc = w;
-  }
 }
 
 // Shared memory of a sample in one block: cover bits, bins and active
@@ -161,6 +151,18 @@ void plan_hot(u32 L, Geometry& G) {
     h.anch = NO_HOT;
   }
   h.hot_bytes = (u32)off;
+}
+
+// The search of a sample in one block: as many edges as fit beside the
+// union-find words of all k-mers, so that most graphs need no probe at all.
+void plan_block_search(u32 L, u32 k, Geometry& G) {
+  const size_t cn = cap_nodes_of(L, k), room = SMP_MAX - SMP_FIXED;
+  if (!G.one_block || cn * 16 >= room) return;
+  SearchCfg w = G.sc;
+  w.hashed = 0;
+  w.ids = (u32)cn;
+  w.win_cap = (u32)std::min<size_t>(cap_edges_of(L, k), (room - cn * 16) / 18 / 8 * 8);
+  if (w.win_cap >= G.sc.win_cap) G.ssc = w;
 }
 
 Geometry plan(u32 L, u32 k) {
@@ -207,6 +209,7 @@ Geometry plan(u32 L, u32 k) {
   c.cap_flat = (u32)std::min<u64>(N, N / 4 + 32);
   c.cap_act = (u32)std::min<u64>(N, std::max(cap_nodes_of(L, k) / 2, c.lvl_cap[0]) + 32);
   plan_hot(L, G);
+  plan_block_search(L, k, G);
   return G;
 }
 
