@@ -892,24 +892,35 @@ int configuration(rsa_t* h, uint32_t sample, uint32_t m, uint32_t* counts, uint3
 constexpr u64 SMALL_LMAX = 128, SMALL_NMAX = 4096;
 constexpr unsigned long long SMALL_POOL_KEEP = 512ull << 20;
 std::atomic<unsigned long long> g_small_launches{0};
+// By device and context: the pool of a context that cudaDeviceReset has
+// destroyed is gone with it, and its handle is never used again.
 std::mutex g_pool_mu;
-cudaMemPool_t g_pool[MAX_DEVICES] = {};
+std::map<std::pair<int, unsigned long long>, cudaMemPool_t> g_pools;
 
 int small_pool(int dev, cudaMemPool_t* out) {
-  if (dev < 0 || dev >= MAX_DEVICES) return fail(RSA_EINVAL, "device ordinal out of range");
   std::lock_guard<std::mutex> lock(g_pool_mu);
-  if (!g_pool[dev]) {
+  unsigned long long ctx = current_context_id();
+  if (!ctx) {
+    CUDA_TRY(cudaSetDevice(dev));  // makes the device's context current
+    ctx = current_context_id();
+  }
+  if (!ctx) {  // no ids to tell contexts apart: the device's own pool
+    CUDA_TRY(cudaDeviceGetDefaultMemPool(out, dev));
+    return 0;
+  }
+  cudaMemPool_t& pool = g_pools[{dev, ctx}];
+  if (!pool) {
     cudaMemPoolProps props = {};
     props.allocType = cudaMemAllocationTypePinned;
     props.location.type = cudaMemLocationTypeDevice;
     props.location.id = dev;
-    cudaMemPool_t pool = nullptr;
-    CUDA_TRY(cudaMemPoolCreate(&pool, &props));
+    cudaMemPool_t made = nullptr;
+    CUDA_TRY(cudaMemPoolCreate(&made, &props));
     unsigned long long keep = SMALL_POOL_KEEP;
-    cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
-    g_pool[dev] = pool;
+    cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep);
+    pool = made;
   }
-  *out = g_pool[dev];
+  *out = pool;
   return 0;
 }
 
@@ -1007,8 +1018,15 @@ bool small_eligible(uint32_t L, uint32_t k) {
 unsigned long long take_small_launches() { return g_small_launches.exchange(0); }
 void release_small() {
   std::lock_guard<std::mutex> lock(g_pool_mu);
-  for (cudaMemPool_t p : g_pool)
-    if (p) cudaMemPoolTrimTo(p, 0);
+  int dev = 0, now = -1;
+  unsigned long long ctx = 0;
+  if (g_pools.empty() || cudaGetDevice(&dev) != cudaSuccess) return;
+  for (auto& p : g_pools) {  // ordered by device
+    if (p.first.first != now && cudaSetDevice(now = p.first.first) == cudaSuccess)
+      ctx = current_context_id();
+    if (p.second && p.first.second == ctx) cudaMemPoolTrimTo(p.second, 0);
+  }
+  cudaSetDevice(dev);
 }
 }  // namespace rsa_detail
 
