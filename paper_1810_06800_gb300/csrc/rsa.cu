@@ -968,7 +968,7 @@ int run_small(const uint32_t* L, const uint32_t* k, const uint64_t* seeds, uint3
   int rc = small_pool(dev, &pool);
   if (rc) return rc;
   CUDA_TRY(cudaFuncSetAttribute(k_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMP_MAX));
-  const u32 grid = std::min(n, (u32)sms);
+  u32 grid = std::min(n, (u32)sms);
   // shapes and jobs in one copy; then results, work counters, job counter, slots
   const size_t sb = align_up(sizeof(Shape) * shapes.size()), jb = align_up(sizeof(SmallJob) * n);
   const size_t ob = align_up(sizeof(SmallOut) * n), wb = 4 * WORK_SLOTS * 8 + ALIGN;
@@ -977,9 +977,18 @@ int run_small(const uint32_t* L, const uint32_t* k, const uint64_t* seeds, uint3
   std::memcpy(in.data() + sb, jobs.data(), sizeof(SmallJob) * n);
   std::vector<SmallOut> out(n);
   char* d = nullptr;
-  CUDA_TRY(cudaMallocFromPoolAsync(reinterpret_cast<void**>(&d), sb + jb + ob + wb + grid * slot, pool, st));
+  cudaError_t e;
+  // where a slot for every block does not fit the free memory, fewer blocks take
+  // more samples each
+  for (;; grid = (grid + 1) / 2) {
+    e = cudaMallocFromPoolAsync(reinterpret_cast<void**>(&d), sb + jb + ob + wb + grid * slot, pool, st);
+    if (e == cudaSuccess) break;
+    cudaGetLastError();
+    if (e != cudaErrorMemoryAllocation || grid == 1)
+      return fail(RSA_ECUDA, std::string("rsa_run_small: ") + cudaGetErrorString(e));
+  }
   char* work = d + sb + jb + ob;
-  cudaError_t e = cudaMemcpyAsync(d, in.data(), in.size(), cudaMemcpyHostToDevice, st);
+  e = cudaMemcpyAsync(d, in.data(), in.size(), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(work, 0, wb, st);
   if (e == cudaSuccess) {
     k_small<<<grid, threads, smem, st>>>(
