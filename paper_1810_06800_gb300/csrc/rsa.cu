@@ -968,7 +968,18 @@ int run_small(const uint32_t* L, const uint32_t* k, const uint64_t* seeds, uint3
   int rc = small_pool(dev, &pool);
   if (rc) return rc;
   CUDA_TRY(cudaFuncSetAttribute(k_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMP_MAX));
-  u32 grid = std::min(n, (u32)sms);
+  if (!threads) {
+    // One sample per SM at a time: as many threads as a block takes.  More
+    // samples than that: smaller blocks, as many as shared memory holds beside
+    // each other (5000 samples of L = 16, k = 2: 0.77 ms by 256 threads, 1.25 by
+    // 512, 2.40 by 1024; of L = 128, k = 128, two blocks per SM: 4.51, 4.36 and
+    // 7.96; of L = 64, k = 4, one block: 5.28, 4.23 and 3.99).
+    const size_t fit = n > (u32)sms ? (SMP_MAX + 1024) / (smem + 1024) : 1;
+    threads = fit >= 4 ? SMP_THREADS / 4 : fit >= 2 ? SMP_THREADS / 2 : SMP_THREADS;
+  }
+  int per_sm = 0;
+  CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_small, (int)threads, smem));
+  u32 grid = (u32)std::min<u64>(n, (u64)sms * std::max(per_sm, 1));
   // shapes and jobs in one copy; then results, work counters, job counter, slots
   const size_t sb = align_up(sizeof(Shape) * shapes.size()), jb = align_up(sizeof(SmallJob) * n);
   const size_t ob = align_up(sizeof(SmallOut) * n), wb = 4 * WORK_SLOTS * 8 + ALIGN;
@@ -1048,7 +1059,7 @@ int rsa_run_small(const uint32_t* L, const uint32_t* k, const uint64_t* seeds, u
   if (threads % 32 || threads > 1024)
     return fail(RSA_EINVAL, "threads must be 32 .. 1024, a multiple of 32");
   // the search's set-up needs 256 threads
-  threads = threads == 0 ? SMP_THREADS : std::max(threads, 256u);
+  if (threads) threads = std::max(threads, 256u);
   return run_small(L, k, seeds, n, threads, n_j, n_c, static_cast<cudaStream_t>(stream));
 }
 
