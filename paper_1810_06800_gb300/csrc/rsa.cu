@@ -842,7 +842,7 @@ int configuration(rsa_t* h, uint32_t sample, uint32_t m, uint32_t* counts, uint3
   const u32 nb = (u32)std::min<u64>(((u64)nj + 256) / 256, 1024);
   const bool at_wrap = m == st[sample].nc;
   const char* b = static_cast<const char*>(h->ws);
-  if (g.cap_nodes <= CFG_NODES) {
+  if (g.cap_nodes <= CFG_NODES && st[sample].n_edges <= CFG_EDGES) {
     const size_t smem = cfg_block_smem(g.cap_nodes);
     CUDA_TRY(cudaFuncSetAttribute(k_cfg_block, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)cfg_block_smem(CFG_NODES)));

@@ -25,9 +25,12 @@
 // in the first half of its uf slot; sizes (u32) in the third quarter and the
 // histogram (u32, entry s - 1 for size s) in the fourth; for the select, the
 // keys of one bin in the first half.
-// A sample of few k-mers goes through all of it in one block (k_cfg_block):
-// a call is bound by its launches and copies then (L = 2048, k = 256: 147 us
-// by six launches, 100 us by one).
+// A sample of few edges goes through all of it in one block (k_cfg_block): a
+// call is bound by its launches and copies then.  The line lies at CFG_EDGES
+// edges, where the walks of one block take as long as the launches: cluster
+// sizes of 0.9 n_j k-mers, one block and several launches, 60 and 84 us at
+// L = 256, k = 12 (6717 edges), 73 and 76 at L = 64, k = 1 (8192), 85 and 77 at
+// L = 72, k = 1 (10368), 152 and 132 at L = 256, k = 4 (27307).
 #pragma once
 #include "rsa_search.cuh"
 
@@ -242,6 +245,7 @@ __global__ void k_cfg_hist(Group g, u32 s) {
 constexpr u32 CFG_THREADS = 1024;
 __host__ __device__ inline size_t cfg_block_smem(u32 cap_nodes) { return (size_t)cap_nodes * 12; }
 constexpr u32 CFG_NODES = 18500;  // cap_nodes that fit beside the bins
+constexpr u32 CFG_EDGES = 8192;
 
 __global__ void __launch_bounds__(CFG_THREADS) k_cfg_block(Group g, u32 s, u32 m, bool at_wrap,
                                                            bool sizes) {
