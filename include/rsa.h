@@ -147,7 +147,8 @@ typedef struct {
 /* The choice for (L, k) and a batch of n samples on the current GPU.  Looked
  * up in a per-process table backed by a JSON-lines file ($RSA_TUNE_CACHE,
  * else $HOME/.cache/rsa_gb300/tune.jsonl), keyed by (GPU name, L, k, n
- * rounded up to a power of two).  If absent and `measure` is non-zero, every
+ * rounded up to a power of two); lines measured on earlier kernels (another
+ * "kernels" number, or none) do not count.  If absent and `measure` is non-zero, every
  * candidate (small mode at 256 / 512 / 1024 threads where the shape fits it;
  * the global path at 2 / 4 / 8 rounds per check) is timed once on seeds
  * 1 .. n (at most 8 GB of workspace) and the fastest is kept and appended

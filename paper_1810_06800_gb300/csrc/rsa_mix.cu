@@ -58,8 +58,13 @@ using rsa_detail::small_eligible;
 // at 2, 4 and 8 rounds per host check -- on seeds 1 .. n, and keeps
 // the fastest.  Results go to a JSON-lines cache ($RSA_TUNE_CACHE, else
 // $HOME/.cache/rsa_gb300/tune.jsonl), read back on the next process start.
+// A line counts only for the kernels it was measured on (TUNE_KERNELS).
 // ---------------------------------------------------------------------
 namespace {
+
+// Raised by changes of the kernels that may change which way is the fastest.
+// Lines without it are of the kernels before the deposition by slices.
+constexpr uint32_t TUNE_KERNELS = 2;
 
 std::mutex g_tune_mu;
 std::map<std::tuple<std::string, uint32_t, uint32_t, uint32_t>, rsa_tune_t> g_tune;
@@ -99,7 +104,9 @@ void tune_load_locked() {
   char buf[1024];
   while (std::fgets(buf, sizeof(buf), f)) {
     const std::string line(buf);
-    std::string gpu, L, k, n, mode, thr, rpc, ms, wt;
+    std::string gpu, L, k, n, mode, thr, rpc, ms, wt, kv;
+    if (!json_field(line, "kernels", &kv) || std::strtoul(kv.c_str(), nullptr, 10) != TUNE_KERNELS)
+      continue;
     if (!json_field(line, "gpu", &gpu) || !json_field(line, "L", &L) || !json_field(line, "k", &k) ||
         !json_field(line, "n", &n) || !json_field(line, "mode", &mode) ||
         !json_field(line, "threads", &thr) || !json_field(line, "rounds_per_check", &rpc) ||
@@ -133,9 +140,9 @@ void tune_store_locked(const std::string& gpu, uint32_t L, uint32_t k, uint32_t 
   std::fprintf(f,
                "{\"gpu\": \"%s\", \"L\": %u, \"k\": %u, \"n\": %u, \"mode\": \"%s\", "
                "\"threads\": %u, \"rounds_per_check\": %u, \"window_threads\": %u, "
-               "\"ms_per_sample\": %.6g}\n",
+               "\"ms_per_sample\": %.6g, \"kernels\": %u}\n",
                gpu.c_str(), L, k, nb, c.mode == RSA_MODE_SMALL ? "small" : "global", c.threads,
-               c.rounds_per_check, c.window_threads, c.ms_per_sample);
+               c.rounds_per_check, c.window_threads, c.ms_per_sample, TUNE_KERNELS);
   std::fclose(f);
 }
 
