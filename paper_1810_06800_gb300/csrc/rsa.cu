@@ -55,7 +55,7 @@ int fail(int code, const std::string& msg) {
   } while (0)
 
 constexpr size_t ALIGN = 256;
-constexpr u32 ROUND_CHECK = 4;   // rounds between host checks once every slice is entered (default)
+constexpr u32 ROUND_CHECK = 4;   // added rounds per graph and host check (default)
 constexpr u32 PROBE_CAP = 96;    // a threshold bisection of 64-bit times, at its worst, and the last window
 
 // The loop counters and, behind them, the work counters.
@@ -328,15 +328,15 @@ struct rsa {
   int device = -1;
   int sm_count = 0;
   Prof prof;
-  // CUDA graphs of a chunk of greedy rounds and of bisection probes, captured
-  // once per (workspace, batch size, key source) on a private stream and
-  // replayed on the run's stream
+  // CUDA graphs of a whole run, of added rounds, of the search after them and of
+  // added probes, captured once per (workspace, batch size, key source, caps) on
+  // a private stream and replayed on the run's stream
   bool use_graphs = true;
   cudaStream_t cap_stream = nullptr;
   // rounds after the last slice in the run's first graph: more once a run
   // has needed more
   u32 drain = 3;
-  u32 round_check = ROUND_CHECK;  // greedy rounds per graph chunk / host check
+  u32 round_check = ROUND_CHECK;  // added rounds per graph and host check
   // test-only lowered caps of the device loops (0 = default; rsa_test_caps)
   u32 t_round = 0, t_uf = 0, t_probe = 0, t_edges = 0;
   struct GraphSlot {
@@ -680,11 +680,17 @@ int run_impl(rsa_t* h, const uint64_t* seeds, u32 n, const uint64_t* keys, cudaS
     probes(st);
   };
   // One block per sample for the small lattices, and for those that still fit
-  // a block when there are enough samples to fill the GPU with blocks
-  // (L = 256, k = 16: 256 samples 0.72 ms, over the whole grid 1.11; 4 samples
-  // 0.36 and 0.30; L = 160, k = 10, 4 samples 0.260 and 0.264, L = 192, k = 12, 4
-  // samples 0.300 and 0.267), or when every launch costs the host (runs without graphs:
-  // 4 samples 0.39 against 0.43).
+  // a block when there are enough samples to fill half of the GPU with blocks.
+  // ms in one block / over the grid:
+  //   4 samples    L = 160, k = 10  0.260 / 0.264, L = 192, k = 12  0.300 / 0.267
+  //   76 samples   L = 256, k = 16  0.39 / 0.53, L = 512, k = 64  0.72 / 0.74
+  //   152 samples  L = 256, k = 16  0.40 / 0.75, L = 512, k = 64  0.73 / 1.04
+  //   400 samples  L = 256, k = 16  1.05 / 1.42, L = 512, k = 64  2.02 / 2.12
+  // Of 43 such batches (L = 170 .. 512) five are slower in one block, the worst of
+  // them L = 400, k = 100, 400 samples, 1.72 / 1.32 (a third wave of blocks).  Runs without
+  // graphs pay for every launch on the host and take one block wherever it fits:
+  // 4 samples L = 256, k = 16  0.40 / 0.42, L = 320, k = 320  0.33 / 0.50; the
+  // grid would be better from L = 320 on for short k (L = 512, k = 64  0.68 / 0.50).
   const bool by_sample =
       G.one_block && (h->L <= 160 || n >= (u32)h->sm_count / 2 || !h->use_graphs);
   const Shape shape = shape_of(G, g, c, rp, probe_cap);
@@ -1275,7 +1281,7 @@ int rsa_test_caps(rsa_t* h, uint32_t round_cap, uint32_t uf_steps, uint32_t prob
 int rsa_set_rounds_per_check(rsa_t* h, uint32_t rounds) {
   if (!h) return fail(RSA_EINVAL, "null handle");
   if (rounds < 1 || rounds > 64) return fail(RSA_EINVAL, "rounds per check must be in 1 .. 64");
-    h->round_check = rounds;
+  h->round_check = rounds;
   return 0;
 }
 

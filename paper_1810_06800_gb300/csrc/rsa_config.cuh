@@ -23,8 +23,8 @@
 // wind along x", whatever order the edges are united in.
 // Scratch (the sample's search state is no longer needed): union-find words
 // in the first half of its uf slot; sizes (u32) in the third quarter and the
-// histogram (u32, entry s - 1 for size s) in the fourth; for the select, the
-// keys of one bin in the first half.
+// histogram (u32, entry s - 1 for size s) in the fourth; for the select, before
+// these, the keys of one bin in the second half.
 // A sample of few edges goes through all of it in one block (k_cfg_block): a
 // call is bound by its launches and copies then.  The line lies at CFG_EDGES
 // edges, where the walks of one block take as long as the launches: cluster
@@ -152,8 +152,8 @@ __device__ u64 select_key(const u64* keys, u32 cnt, u32 rank, u32* sh) {
   return pre;
 }
 
-// The keys of that bin into the sample's first uf half (identity words
-// afterwards), the m-th key of all, T_m, into st.sel by the last block.
+// The keys of that bin into the second half of the sample's uf slot (sizes and
+// histogram afterwards), the m-th key of all, T_m, into st.sel by the last block.
 constexpr u32 SEL_THREADS = 1024;
 __global__ void __launch_bounds__(SEL_THREADS) k_key_select(Group g, u32 s, u32* bins) {
   __shared__ u32 sh[260];

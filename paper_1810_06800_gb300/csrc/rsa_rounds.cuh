@@ -226,7 +226,10 @@ __device__ void dense_body(const Group& g, const RoundCfg& c, const RoundPtrs& p
       const u32 idx = (u32)(i0 + (u64)(__ffs(m) - 1) * nt);
       if (at < sm.STAGE) {
         sm.stage[at] = idx;
-      } else {  // more hits than the stage holds (not met by hashed priorities)
+      } else {
+        // more hits than the stage holds: one atomic per hit.  Hashed priorities
+        // meet it where one block tiles 16384 candidates and half of them are
+        // hits (rsa_sample.cuh, k = 2 and 3); a tile of k_dense has 4096
         const u32 t = level_of(idx);
         put(t, atomicAdd(&r.lvl_n[t], 1u), idx);
       }

@@ -120,8 +120,8 @@ __device__ void run_sample(SampleSmem& sm, SampleScratch& scratch, unsigned char
     for (;;) {
       const Slice sl = r.sl;
       const u32 n1 = slice_entries(c, r, sl), n2 = r.act[sl.par ^ 1u];
-      if (k <= PICK_LONGK) pick_body<false>(g, c, p, 0, team, sl, n1, n2, &r.act[sl.par]);
-      else pick_body<true>(g, c, p, 0, team, sl, n1, n2, &r.act[sl.par]);
+      // (k > PICK_LONGK: 300 KB of cover bits and more, never in one block)
+      pick_body<false>(g, c, p, 0, team, sl, n1, n2, &r.act[sl.par]);
       __syncthreads();
       const u32 n = r.act[sl.par];
       const bool over = n > c.cap_act;

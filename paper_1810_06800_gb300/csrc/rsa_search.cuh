@@ -36,10 +36,10 @@ constexpr u32 FIN_THREADS = 1024;
 constexpr u32 FIN_SLOTS = 4 * FIN_EDGES;  // hash slots for the roots of the window (4 B: as much
                                           // as 2 FIN_EDGES union-find words)
 constexpr u32 SUB_BINS = 128;
-// per sample: the time histogram, and two sets of the counts of a probe
+// per sample: the time histogram, and the counts of a probe
 constexpr u32 SUB_WRAP = SUB_BINS, SUB_A = SUB_BINS + 1, SUB_B = SUB_BINS + 2;
 constexpr u32 SUB_WORDS = SUB_BINS + 4;
-constexpr u32 SEARCH_WORDS = EHIST + 2 * SUB_WORDS;
+constexpr u32 SEARCH_WORDS = EHIST + SUB_WORDS;
 
 struct WinEdge {  // an edge of the last window, between roots
   u64 time;
