@@ -108,8 +108,9 @@ int rsa_run_static(uint32_t L, uint32_t k, const uint64_t *seeds, uint32_t n, ui
  * L^2 / k <= 4096 (RSA_EINVAL otherwise).  threads: CTA size, a multiple of
  * 32 up to 1024 (0 = the library's choice; at least 256 run).  Its job table
  * and workspaces come stream-ordered on `stream` from a memory pool that
- * keeps them between calls (rsa_mix_release gives them back); synchronises
- * `stream`; returns the first per-sample error code. */
+ * keeps them between calls (rsa_mix_release gives them back); where the free
+ * memory does not hold a workspace for every block, fewer blocks run.
+ * Synchronises `stream`; returns the first per-sample error code. */
 int rsa_run_small(const uint32_t *L, const uint32_t *k, const uint64_t *seeds, uint32_t n,
                   uint32_t threads, uint32_t *n_j, uint32_t *n_c, void *stream);
 
