@@ -116,7 +116,8 @@ int rsa_run_small(const uint32_t *L, const uint32_t *k, const uint64_t *seeds, u
 
 /* A batch of samples of uneven shapes (same arrays as rsa_run_small, any
  * 1 <= k <= L <= 32768): samples are grouped by shape, each shape runs the
- * way rsa_tune picks for it, the small-lattice groups together in one
+ * way rsa_tune picks for it (small mode without a measurement: at the CTA size
+ * rsa_run_small chooses), the small-lattice groups together in one
  * persistent launch and every other shape on its own handle and stream, all
  * concurrently (one host thread per such shape).  Work queued on `stream`
  * before the call runs first, work queued after it runs after the batch.

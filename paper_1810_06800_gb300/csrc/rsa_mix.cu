@@ -331,7 +331,10 @@ extern "C" int rsa_run_mix(const uint32_t* L, const uint32_t* k, const uint64_t*
       const uint64_t work = (uint64_t)gkv.first.first * gkv.first.first * gkv.second.size();
       if (work > small_work) {
         small_work = work;
-        small_threads = c.threads;
+        // an unmeasured default leaves the size to rsa_run_small, which knows how
+        // many samples there are (20000 samples of L = 8, k = 2: 2.40 ms, with
+        // 512 threads 3.73)
+        small_threads = c.ms_per_sample > 0 ? c.threads : 0;
       }
     } else {
       global.push_back(Job{gkv.first.first, gkv.first.second, c.rounds_per_check ? c.rounds_per_check : 4u,
